@@ -6,354 +6,328 @@
 // f(C) = C^-1/2 (z + eta C^1/2)^-1, i.e. the resolvent of D = C^1/2 with the
 // weights divided by Omega:  Sigma_tm(omega) = -eta G(-eta z),
 //   G(zeta) = sum_j wt_j / (zeta - Omega_j),  Omega_j = sqrt(theta_j),
-//   wt_j = ||b||^2 u_1j^2 / Omega_j.
-// The continued fraction of Eq. 14 for G needs the Jacobi matrix of this
-// discrete measure; it is rebuilt here from (Omega_j, wt_j) by inserting the
-// nodes one at a time and chasing the bulge with plane rotations (the
-// Rutishauser / Gragg-Harrod reconstruction, O(k^2), orthogonal, stable).
+//   wt_j = ||b||^2 u_1j^2 / Omega_j,
+// the sum over poles of Eq. 11.  The fraction kernels evaluate that sum: it
+// equals the continued fraction of the measure's Jacobi matrix (Eq. 14), has
+// no serial chain over the depth, and needs no rebuild of that matrix.
 //
-// One warp per start vector: the Gauss rule of T_k by parallel bisection and
-// the product formula for the weights, then the Jacobi rebuild (lane-
-// pipelined node insertions); the work rows live in shared memory.
+// One block per start vector, one eigenvalue per thread.
 #include <algorithm>
 
 #include "lgw_internal.cuh"
 
 namespace lgw {
 
-// Plane rotation applied symmetrically to rows/cols (i, i+1) of a symmetric
-// tridiagonal with diagonal d and off-diagonal e (e[i] couples i, i+1).
-__device__ __forceinline__ void rot_sym(double c, double s, double *d, double *e, int i) {
-  const double a = d[i], bb = e[i], cc = d[i + 1];
-  const double cs = c * s, c2 = c * c, s2 = s * s;
-  d[i] = c2 * a + 2.0 * cs * bb + s2 * cc;
-  d[i + 1] = s2 * a - 2.0 * cs * bb + c2 * cc;
-  e[i] = cs * (cc - a) + (c2 - s2) * bb;
-}
-
-// Givens pair (c, s) with c x + s z = r >= 0, -s x + c z = 0, from one
-// reciprocal square root (no FP64 division: GB300 runs FP64 at 1/58 rate).
-__device__ __forceinline__ void givens(double x, double z, double &c, double &s, double &r) {
-  const double r2 = fma(x, x, z * z);
-  if (r2 > 0.0) {
-    const double inv = rsqrt(r2);
-    c = x * inv;
-    s = z * inv;
-    r = r2 * inv;
-  } else {
-    c = 1.0;
-    s = 0.0;
-    r = 0.0;
-  }
-}
-
-// Jacobi matrix (a[0..n), off-diagonal b[0..n-1), not squared) and total
-// weight of the discrete measure sum_j wt_j delta(x - x_j), n = number of
-// nodes.  Node jn enters as a new leading row with start-vector weight wt_jn:
-// one rotation in plane (0, 1) folds it into the start vector, and the bulge
-// it leaves in b is chased to the bottom by rotations in planes (kk, kk+1).
+// --------------------------------------------------------------------------
+// Gauss rule of T_k.  theta_j is the (j+1)-th smallest eigenvalue.
+//   1. FP32 bisection on the number of negative pivots of T - x (22 halvings
+//      of the Gershgorin interval).  The computed count is the exact count of
+//      a matrix within a few FP32 roundings of T, so theta_j lies within
+//      2^-18 of the interval's width of the result.
+//   2. FP64 Sturm counts at both ends of that bracket: they show that it
+//      holds theta_j alone, or move and widen it.
+//   3. Newton's method on p(x) = det(T - x) inside the bracket, p and p' from
+//      the three-term recurrence of the trailing minors r_i (bottom row
+//      first); its sign changes are the Sturm count, which narrows the
+//      bracket at every evaluation.  While the bracket holds more than one
+//      eigenvalue (clusters, ghosts of a recurrence without
+//      reorthogonalisation), or where Newton's step leaves it, it is halved.
+//   u_1j^2 = |r_1 / p'|, the product formula prod_i (theta_j - mu_i) /
+//   prod_{i != j} (theta_j - theta_i) (mu: eigenvalues of T without its first
+//   row and column), from the same last evaluation.
 //
-// The insertions are pipelined over the warp: in each group of 32 nodes,
-// lane l inserts node g0 + l and chases its bulge two rows behind lane l-1.
-// Rows are stored bottom-up (with m rows present the leading row sits at
-// index n - m), so a new leading row shifts nothing.  A rotation in plane
-// (kk, kk+1) touches rows kk-1 .. kk+1, so the rotations of one super-step
-// are at least three rows apart, and each row that two insertions both
-// rotate is rotated by the earlier insertion first: every rotation sees the
-// operands it would see in the one-node-at-a-time order.  Wp (n doubles)
-// receives the running weights W_jn = sum_{i < jn} wt_i.  All 32 lanes call
-// this; the total weight is returned to every lane.
-__device__ double jacobi_from_nodes_warp(const double *x, const double *wt, int n, double *a,
-                                         double *b, double *Wp) {
-  const int lane = threadIdx.x & 31;
-  if (n <= 0) return 0.0;
-  double Wtot = 0.0;
-  if (lane == 0) {
-    double W = 0.0;
-    for (int j = 0; j < n; ++j) {
-      Wp[j] = W;
-      W += wt[j];
-    }
-    Wtot = W;
-    a[n - 1] = x[0];
-  }
-  __syncwarp();
-  for (int g0 = 1; g0 < n; g0 += 32) {
-    const int nl = min(32, n - g0);
-    const bool act = lane < nl;
-    const int jn = g0 + lane;
-    const int L = n - 1 - jn;   // leading row once node jn is in
-    const int m = jn + 1;       // rows after the insertion
-    double bulge = 0.0;
-    bool live = false;
-    // lane l's last chase step (kk = m - 2) comes at super-step 2 l + m - 2
-    const int steps = 3 * (nl - 1) + g0;
-    for (int tau = 0; tau < steps; ++tau) {
-      const int kk = tau - 2 * lane;
-      if (act && kk == 0) {
-        a[L] = x[jn];
-        b[L] = 0.0;
-        const double wj = wt[jn], W = Wp[jn];
-        double c = 1.0, s = 0.0;
-        if (W + wj > 0.0) {
-          const double inv = rsqrt(W + wj);
-          c = sqrt(wj) * inv;
-          s = sqrt(W) * inv;
-        }
-        rot_sym(c, s, a, b, L);
-        bulge = 0.0;
-        if (m > 2) {
-          bulge = s * b[L + 1];
-          b[L + 1] *= c;
-        }
-        live = bulge != 0.0;
-      } else if (act && live && kk >= 1 && kk < m - 1) {
-        double c, s, rr;
-        givens(b[L + kk - 1], bulge, c, s, rr);
-        b[L + kk - 1] = rr;
-        rot_sym(c, s, a, b, L + kk);
-        if (kk + 1 < m - 1) {
-          bulge = s * b[L + kk + 1];
-          b[L + kk + 1] *= c;
-        } else {
-          bulge = 0.0;
-        }
-        live = bulge != 0.0;
+// What bounds it: GB300's FP64 pipe (2 lanes per SM clock).  Pure FP64
+// bisection needs 60 counts of 3 operations per level and eigenvalue, and the
+// separate weight recurrences 10 more; this needs 2 counts and about 3
+// evaluations of 5 (21).  One warp per vector also left most of the chip
+// idle at a few hundred vectors.  512 vectors, k = 200: 2.4 ms, against 22.6
+// ms for one warp per vector, pure bisection and the Jacobi rebuild.
+// --------------------------------------------------------------------------
+constexpr int SPEC_THREADS = 256;
+constexpr int SPEC_FP32_ITS = 22;
+constexpr int SPEC_MAX_ITS = 160;
+
+__device__ __forceinline__ int hi_abs(double p) { return __double2hiint(p) & 0x7fffffff; }
+
+// The trailing minors r_i = det(T_{i:n} - x) from the last row up: p = r_0,
+// r1 = r_1, dp = dp/dx (DERIV), all on one common scale, and the number of
+// eigenvalues below x.  ab[i] = (a_i, b_i^2), b_i coupling rows i and i + 1.
+// A zero minor takes the opposite sign of its predecessor at a magnitude that
+// later minors cannot see.  Signs and magnitudes are tested on the integer
+// pipe; the common power-of-two rescaling every eight levels is exact (a
+// level grows the minors by less than 2^4 on a T of width below 2).
+template <bool DERIV>
+__device__ __forceinline__ void sturm_eval(const double2 *ab, int n, double x, double &p,
+                                           double &dp, double &r1, int &count) {
+  constexpr int kBig = (1023 + 400) << 20, kSmall = (1023 - 400) << 20;
+  double p0 = 1.0, p1 = ab[n - 1].x - x, d0 = 0.0, d1 = -1.0;
+  if (p1 == 0.0) p1 = -0x1p-900;
+  int neg = __double2hiint(p1) < 0 ? 1 : 0, cnt = neg;
+  int i = n - 2;
+  while (i >= 0) {
+    const int stop = max(-1, i - 8);
+    for (; i > stop; --i) {
+      const double2 v = ab[i];
+      const double c = v.x - x;
+      double p2 = fma(c, p1, -v.y * p0);
+      if (DERIV) {
+        const double d2 = fma(c, d1, fma(-v.y, d0, -p1));
+        d0 = d1;
+        d1 = d2;
       }
-      __syncwarp();
+      if (((__double2hiint(p2) << 1) | __double2loint(p2)) == 0)
+        p2 = neg ? 0x1p-900 : -0x1p-900;
+      const int ng = __double2hiint(p2) < 0 ? 1 : 0;
+      cnt += ng ^ neg;
+      neg = ng;
+      p0 = p1;
+      p1 = p2;
+    }
+    const int m = max(hi_abs(p0), hi_abs(p1));
+    if (max(m, DERIV ? hi_abs(d1) : 0) > kBig) {
+      p0 *= 0x1p-400;
+      p1 *= 0x1p-400;
+      if (DERIV) {
+        d0 *= 0x1p-400;
+        d1 *= 0x1p-400;
+      }
+    } else if (m < kSmall) {
+      p0 *= 0x1p+400;
+      p1 *= 0x1p+400;
+      if (DERIV) {
+        d0 *= 0x1p+400;
+        d1 *= 0x1p+400;
+      }
     }
   }
-  return __shfl_sync(0xffffffffu, Wtot, 0);
+  p = p1;
+  r1 = p0;
+  dp = d1;
+  count = cnt;
 }
 
-// --------------------------------------------------------------------------
-// Warp-parallel Gauss rule: one warp per vector, lanes over the eigenvalues.
-//   theta_j (the (j+1)-th smallest eigenvalue of T) by bisection on the Sturm
-//   count: the number of sign changes of the leading principal minors
-//   p_i = det(T_i - x I) is the number of eigenvalues below x (division-free
-//   three-term recurrence, rescaled by exact powers of two);
-//   u_1j^2 = det(theta_j I - T_2:n) / (d/dtheta det(theta I - T))|theta_j,
-//   the product formula prod_i (theta_j - mu_i) / prod_{i != j} (theta_j -
-//   theta_i) (mu: eigenvalues of T without its first row and column).
-// A lane interleaves up to SPEC_ILP eigenvalues so that their independent
-// recurrences hide the FP64 latency.  The Omega-space Jacobi rebuild then
-// runs from the nodes and weights in shared memory, its insertions pipelined
-// over the lanes.
-// --------------------------------------------------------------------------
-constexpr int SPEC_ILP = 8;
-constexpr double SCALE_UP = 0x1p+500, SCALE_DN = 0x1p-500;
-// bit patterns of 2^500 and 2^-500 (biased exponents 1523 and 523)
-constexpr unsigned long long kUpBits = 1523ULL << 52, kDnBits = 523ULL << 52;
-
-// sign with the Sturm convention for zeros (a zero takes the opposite sign
-// of its predecessor): p < 0, or p == 0 and the predecessor was not
-// negative.  Tested on the bit pattern, and |p| against the rescaling
-// thresholds likewise (bit patterns of non-negative doubles order like
-// their values), so that the bisection's FP64 pipe, on which GB300 runs
-// 2 lanes per SM clock, issues only the recurrence's subtract, multiply and
-// fused multiply-add; the comparisons go to the integer pipe.
-__device__ __forceinline__ bool neg_sturm(double p, bool prev_neg) {
-  const long long bits = __double_as_longlong(p);
-  return ((bits << 1) == 0) ? !prev_neg : (bits < 0);
+// theta_j of the n x n scaled matrix ab (abf: the same about mid, in FP32), all
+// of whose eigenvalues lie in [glo, ghi], w < ghi - glo < 1.1 w; wt = u_1j^2.
+// The 32 lanes of a warp call it together; a lane without an eigenvalue
+// (real == false) takes part in the loops only.
+__device__ __noinline__ double eigenvalue(const double2 *ab, const float2 *abf, int n, int j,
+                                          bool real, double glo, double ghi, double mid,
+                                          double w, double &wt_out) {
+  const double tol = 0x1p-50;
+  // 1. FP32 bracket
+  float flo = -0.51f * (float)w, fhi = 0.51f * (float)w;
+  for (int it = 0; it < SPEC_FP32_ITS; ++it) {
+    const float x = 0.5f * (flo + fhi);
+    float q = 1.0f, bb = 0.0f;
+    int cnt = 0;
+    for (int i = 0; i < n; ++i) {
+      const float2 t = abf[i];
+      q = (t.x - x) - __fdividef(bb, q);
+      if (fabsf(q) < 1e-9f) q = -1e-9f;
+      cnt += q < 0.0f ? 1 : 0;
+      bb = t.y;
+    }
+    if (cnt <= j)
+      flo = x;
+    else
+      fhi = x;
+  }
+  double x = mid + 0.5 * ((double)flo + (double)fhi);
+  double lo = fmax(x - 0x1p-18 * w, glo), hi = fmin(x + 0x1p-18 * w, ghi);
+  // 2. FP64 counts at its ends
+  int cl, ch;
+  double p, dp, r1;
+  sturm_eval<false>(ab, n, lo, p, dp, r1, cl);
+  sturm_eval<false>(ab, n, hi, p, dp, r1, ch);
+  if (cl > j) {
+    hi = lo;
+    ch = cl;
+    lo = glo;
+    cl = 0;
+    x = 0.5 * (lo + hi);
+  } else if (ch <= j) {
+    lo = hi;
+    cl = ch;
+    hi = ghi;
+    ch = n;
+    x = 0.5 * (lo + hi);
+  }
+  // 3. Newton inside the bracket
+  bool act = real;
+  double th = x, wt = 0.0, dx_prev = 1e300;
+  for (int it = 0; it < SPEC_MAX_ITS && __any_sync(0xffffffffu, act); ++it) {
+    int cnt;
+    sturm_eval<true>(ab, n, x, p, dp, r1, cnt);
+    if (!act) continue;
+    if (cnt <= j) {
+      lo = x;
+      cl = cnt;
+    } else {
+      hi = x;
+      ch = cnt;
+    }
+    const bool alone = cl == j && ch == j + 1;
+    const double dx = p / dp, adx = fabs(dx), xn = x - dx;
+    wt = fabs(r1 / dp);
+    // converged, or at the rounding level of p / p'
+    if (alone && (adx <= tol || (adx <= 0x1p-44 && adx >= 0.25 * dx_prev))) {
+      th = xn >= lo && xn <= hi ? xn : x;
+      act = false;
+    } else if (hi - lo <= tol) {
+      th = 0.5 * (lo + hi);
+      act = false;
+    } else {
+      // every other pass halves the bracket once Newton drags
+      const bool newton = alone && xn > lo && xn < hi && !(it > 8 && (it & 1));
+      dx_prev = newton ? adx : 1e300;
+      x = newton ? xn : 0.5 * (lo + hi);
+      th = x;
+    }
+  }
+  wt_out = wt;
+  return th;
 }
-__device__ __forceinline__ unsigned long long abs_bits(double p) {
-  return (unsigned long long)__double_as_longlong(p) & 0x7fffffffffffffffULL;
-}
 
-__global__ void k_spectral_warp(const double *__restrict__ alpha, const double *__restrict__ beta,
-                                const double *__restrict__ beta0, const int *__restrict__ k_eff,
-                                int B, int k, int warps, JacobiBufs jb,
-                                unsigned long long *min_theta_bits, unsigned *status) {
-  extern __shared__ double sm[];
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int v = blockIdx.x * warps + wid;
-  if (v >= B) return;
-  double *al = sm + (size_t)wid * 6 * k;   // alpha
-  double *b2 = al + k;                     // beta^2 (b2[i] couples i, i+1)
-  double *th = b2 + k;                     // nodes (theta, then Omega)
-  double *wt = th + k;                     // u_1^2, then the Omega-space weights
-  double *ja = wt + k;                     // Jacobi diagonal
-  double *jb_ = ja + k;                    // Jacobi off-diagonal
+__global__ void __launch_bounds__(SPEC_THREADS) k_spectral(
+    const double *__restrict__ alpha, const double *__restrict__ beta,
+    const double *__restrict__ beta0, const int *__restrict__ k_eff, int k, JacobiBufs jb,
+    unsigned long long *min_theta_bits, unsigned *status) {
+  extern __shared__ double2 ab[];                       // [k] scaled (a, b^2)
+  float2 *abf = reinterpret_cast<float2 *>(ab + k);     // [k] the same about the middle, FP32
+  double *ths = reinterpret_cast<double *>(abf + k);    // [k] scaled nodes
+  double *mus = ths + k;                                // [k] eigenvalues without row 0
+  __shared__ double slo[SPEC_THREADS / 32], shi[SPEC_THREADS / 32];
+  const int v = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int nw = blockDim.x >> 5;
   // A depth outside [0, k] (possible only for caller-supplied tridiagonals)
   // is flagged and the vector skipped: its rows hold at most k entries.
   int n = k_eff[v];
   if (n < 0 || n > k) {
-    if (lane == 0) atomicOr(status, ST_BAD_INPUT);
+    if (tid == 0) atomicOr(status, ST_BAD_INPUT);
     n = 0;
   }
-  if (lane == 0) jb.n[v] = n;
-  if (n <= 0) {
-    if (lane == 0) jb.w0[v] = 0.0;
-    return;
-  }
+  if (tid == 0) jb.n[v] = n;
+  if (n <= 0) return;
+  const double *al = alpha + (size_t)v * k, *be = beta + (size_t)v * k;
+  // Gershgorin interval
   double glo = 1e300, ghi = -1e300;
-  for (int i = lane; i < n; i += 32) {
-    const double a = alpha[(size_t)v * k + i];
-    const double bl = i > 0 ? fabs(beta[(size_t)v * k + i - 1]) : 0.0;
-    const double br = i + 1 < n ? fabs(beta[(size_t)v * k + i]) : 0.0;
-    al[i] = a;
-    b2[i] = (i + 1 < n) ? br * br : 0.0;
-    glo = fmin(glo, a - bl - br);
-    ghi = fmax(ghi, a + bl + br);
+  for (int i = tid; i < n; i += blockDim.x) {
+    const double a = al[i];
+    const double r = (i > 0 ? fabs(be[i - 1]) : 0.0) + (i + 1 < n ? fabs(be[i]) : 0.0);
+    glo = fmin(glo, a - r);
+    ghi = fmax(ghi, a + r);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     glo = fmin(glo, __shfl_xor_sync(0xffffffffu, glo, o));
     ghi = fmax(ghi, __shfl_xor_sync(0xffffffffu, ghi, o));
   }
-  __syncwarp();
-  const double width = ghi - glo;
-  glo -= 1e-12 * width + 1e-300;
-  ghi += 1e-12 * width + 1e-300;
+  if (lane == 0) {
+    slo[wid] = glo;
+    shi[wid] = ghi;
+  }
+  __syncthreads();
+  glo = slo[0];
+  ghi = shi[0];
+  for (int w = 1; w < nw; ++w) {
+    glo = fmin(glo, slo[w]);
+    ghi = fmax(ghi, shi[w]);
+  }
+  // T on a power-of-two scale (exact) that brings the width into [1, 2)
+  const double width = fmax(fmax(ghi - glo, 1e-14 * fmax(fabs(glo), fabs(ghi))), 1e-290);
+  const int ex = ilogb(width);
+  const double sc = ldexp(1.0, -ex);
+  const double w = width * sc, pad = 1e-12 * w;
+  glo = glo * sc - pad;
+  ghi = ghi * sc + pad;
+  const double mid = 0.5 * (glo + ghi);
+  for (int i = tid; i < n; i += blockDim.x) {
+    const double a = al[i] * sc;
+    const double b = i + 1 < n ? be[i] * sc : 0.0;
+    ab[i] = make_double2(a, b * b);
+    abf[i] = make_float2((float)(a - mid), (float)(b * b));
+  }
+  __syncthreads();
 
-  for (int j0 = 0; j0 < n; j0 += 32 * SPEC_ILP) {
-    double lo[SPEC_ILP], hi[SPEC_ILP];
-    int idx[SPEC_ILP];
-#pragma unroll
-    for (int r = 0; r < SPEC_ILP; ++r) {
-      idx[r] = j0 + lane + 32 * r;
-      lo[r] = glo;
-      hi[r] = ghi;
-    }
-    // bisection: count(lo) <= j < count(hi); 60 halvings reach the rounding
-    // level of the Gershgorin width
-    for (int it = 0; it < 60; ++it) {
-      double x[SPEC_ILP], p0[SPEC_ILP], p1[SPEC_ILP];
-      int cnt[SPEC_ILP];
-      bool pn[SPEC_ILP];
-#pragma unroll
-      for (int r = 0; r < SPEC_ILP; ++r) {
-        x[r] = 0.5 * (lo[r] + hi[r]);
-        p0[r] = 1.0;
-        p1[r] = al[0] - x[r];
-        pn[r] = neg_sturm(p1[r], false);
-        cnt[r] = pn[r] ? 1 : 0;
-      }
-      for (int i = 1; i < n; ++i) {
-        const double a = al[i], bb = b2[i - 1];
-#pragma unroll
-        for (int r = 0; r < SPEC_ILP; ++r) {
-          double p2 = fma(a - x[r], p1[r], -bb * p0[r]);
-          const bool ng = neg_sturm(p2, pn[r]);
-          cnt[r] += (ng != pn[r]) ? 1 : 0;
-          pn[r] = ng;
-          p0[r] = p1[r];
-          p1[r] = p2;
-          if (abs_bits(p2) > kUpBits) {
-            p0[r] *= SCALE_DN;
-            p1[r] *= SCALE_DN;
-          } else if (abs_bits(p2) < kDnBits && abs_bits(p0[r]) < kDnBits) {
-            p0[r] *= SCALE_UP;
-            p1[r] *= SCALE_UP;
-          }
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < SPEC_ILP; ++r) {
-        if (cnt[r] <= idx[r])
-          lo[r] = x[r];
-        else
-          hi[r] = x[r];
-      }
-    }
-    // weights: u_1j^2 = det(theta I - T_2:n) / d/dtheta det(theta I - T)
-#pragma unroll
-    for (int r = 0; r < SPEC_ILP; ++r) {
-      if (idx[r] >= n) continue;
-      const double t = 0.5 * (lo[r] + hi[r]);
-      double d0 = 1.0, d1 = t - al[0], q0 = 0.0, q1 = 1.0;   // det and derivative
-      int ed = 0;
-      for (int i = 1; i < n; ++i) {
-        const double c = t - al[i], bb = b2[i - 1];
-        const double d2 = fma(c, d1, -bb * d0);
-        const double q2 = fma(c, q1, fma(-bb, q0, d1));
-        d0 = d1;
-        d1 = d2;
-        q0 = q1;
-        q1 = q2;
-        if (fmax(fabs(d1), fabs(q1)) > SCALE_UP) {
-          d0 *= SCALE_DN;
-          d1 *= SCALE_DN;
-          q0 *= SCALE_DN;
-          q1 *= SCALE_DN;
-          ed += 500;
-        } else if (fmax(fmax(fabs(d1), fabs(q1)), fmax(fabs(d0), fabs(q0))) < SCALE_DN) {
-          d0 *= SCALE_UP;
-          d1 *= SCALE_UP;
-          q0 *= SCALE_UP;
-          q1 *= SCALE_UP;
-          ed -= 500;
-        }
-      }
-      double e0 = 1.0, e1 = n > 1 ? t - al[1] : 1.0;
-      int ee = 0;
-      for (int i = 2; i < n; ++i) {
-        const double e2 = fma(t - al[i], e1, -b2[i - 1] * e0);
-        e0 = e1;
-        e1 = e2;
-        if (fabs(e1) > SCALE_UP) {
-          e0 *= SCALE_DN;
-          e1 *= SCALE_DN;
-          ee += 500;
-        } else if (fmax(fabs(e1), fabs(e0)) < SCALE_DN) {
-          e0 *= SCALE_UP;
-          e1 *= SCALE_UP;
-          ee -= 500;
-        }
-      }
-      th[idx[r]] = t;
-      wt[idx[r]] = fabs(ldexp(e1 / q1, ee - ed));
+  double *node = jb.a + (size_t)v * k, *weight = jb.b2 + (size_t)v * k;
+  for (int j0 = 0; j0 < n; j0 += blockDim.x) {
+    const int j = j0 + tid;
+    if (j - lane >= n) break;   // this warp's eigenvalues are done
+    double wt;
+    const double th = eigenvalue(ab, abf, n, j, j < n, glo, ghi, mid, w, wt);
+    if (j < n) {
+      ths[j] = n == 1 ? ab[0].x : th;
+      weight[j] = n == 1 ? 1.0 : wt;
     }
   }
-  __syncwarp();
-  // Gauss nodes -> (Omega_j, wt_j) in place; smallest node for the report
+  __syncthreads();
+  // A close pair's weights are ill-conditioned one by one: r_1 / p' of the two
+  // nodes errs by eps ||T|| / gap, and their sum with it.  The product formula
+  // over the computed nodes and the computed eigenvalues without row 0 gives
+  // the weights of a nearby tridiagonal, whose sums over a cluster are right.
+  bool close = false;
+  for (int j = tid; j + 1 < n; j += blockDim.x) close |= ths[j + 1] - ths[j] < 0x1p-16 * w;
+  if (__syncthreads_or(close)) {
+    for (int j0 = 0; j0 < n - 1; j0 += blockDim.x) {
+      const int j = j0 + tid;
+      if (j - lane >= n - 1) break;
+      double wt;
+      const double mu = eigenvalue(ab + 1, abf + 1, n - 1, j, j < n - 1, glo, ghi, mid, w, wt);
+      // interlacing, also where rounding has broken it
+      if (j < n - 1)
+        mus[j] = fmin(fmax(mu, fmin(ths[j], ths[j + 1])), fmax(ths[j], ths[j + 1]));
+    }
+    __syncthreads();
+    for (int j = tid; j < n; j += blockDim.x) {
+      const double th = ths[j];
+      double wt = 1.0;
+      for (int i = 0; i < n; ++i) {
+        if (i == j) continue;
+        // mu between theta_i and theta_j: a factor within [0, 1]
+        const double den = th - ths[i];
+        wt *= den != 0.0 ? (th - mus[i < j ? i : i - 1]) / den : 0.5;
+      }
+      weight[j] = wt;
+    }
+  }
+  // Gauss nodes -> (Omega_j, wt_j); the smallest node for the report
   const double b0 = beta0[v];
   double tmin = 1e300;
   bool bad = false;
-  for (int i = lane; i < n; i += 32) {
-    const double t = th[i];
+  for (int j = tid; j < n; j += blockDim.x) {
+    const double t = ldexp(ths[j], ex);
     tmin = fmin(tmin, t);
     bad |= !(t > 0.0);
     const double Om = t > 0.0 ? sqrt(t) : 0.0;
-    th[i] = Om;
-    wt[i] = Om > 0.0 ? b0 * b0 * wt[i] / Om : 0.0;
+    node[j] = Om;
+    weight[j] = Om > 0.0 ? b0 * b0 * weight[j] / Om : 0.0;
   }
+  bad = __syncthreads_or(bad);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) tmin = fmin(tmin, __shfl_xor_sync(0xffffffffu, tmin, o));
-  bad = __any_sync(0xffffffffu, bad);
-  __syncwarp();
-  if (lane == 0) {
+  if (lane == 0) slo[wid] = tmin;
+  __syncthreads();
+  if (tid == 0) {
+    for (int i = 1; i < nw; ++i) tmin = fmin(tmin, slo[i]);
     if (bad)
       atomicOr(status, ST_NOT_SPD);
     else
       atomicMin(min_theta_bits, (unsigned long long)__double_as_longlong(tmin));
   }
-  // alpha's rows are free now: the running weights of the rebuild
-  const double W = jacobi_from_nodes_warp(th, wt, n, ja, jb_, al);
-  if (lane == 0) jb.w0[v] = W;
-  __syncwarp();
-  double *ga = jb.a + (size_t)v * k, *gb2 = jb.b2 + (size_t)v * k;
-  for (int i = lane; i < n; i += 32) {
-    ga[i] = ja[i];
-    gb2[i] = (i + 1 < n) ? jb_[i] * jb_[i] : 0.0;
-  }
 }
 
 void launch_spectral_impl(const double *alpha, const double *beta, const double *beta0,
-                          const int *k_eff, int B, int k, JacobiBufs jb, double *scratch,
+                          const int *k_eff, int B, int k, JacobiBufs jb,
                           unsigned long long *min_theta_bits, unsigned *status, cudaStream_t st) {
-  // warp-parallel Gauss rule: 6 k doubles of shared memory per warp
-  const size_t per_warp = (size_t)6 * k * sizeof(double);
-  const int warps = (int)std::max<size_t>(1, std::min<size_t>(4, (200 * 1024) / per_warp));
+  // 40 k bytes of shared memory per block: 164 KB at the largest depth
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(k_spectral_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_spectral, cudaFuncAttributeMaxDynamicSharedMemorySize, 164 * 1024);
     attr = true;
   }
-  const dim3 grid((B + warps - 1) / warps);
-  k_spectral_warp<<<grid, 32 * warps, per_warp * warps, st>>>(alpha, beta, beta0, k_eff, B, k,
-                                                              warps, jb, min_theta_bits, status);
-  (void)scratch;
+  const int threads = std::min(SPEC_THREADS, (k + 31) / 32 * 32);
+  const size_t sh = (size_t)k * (sizeof(double2) + sizeof(float2) + 2 * sizeof(double));
+  k_spectral<<<B, threads, sh, st>>>(alpha, beta, beta0, k_eff, k, jb, min_theta_bits, status);
 }
 
 // ---------------------------------------------------------------------------

@@ -1199,7 +1199,6 @@ void run_sigma(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts &o
   jb.b2 = wsT<double>(h, "jac_b2", (size_t)std::max(B, 1) * k);
   jb.w0 = wsT<double>(h, "jac_w0", (size_t)std::max(B, 1));
   jb.n = wsT<int>(h, "jac_n", (size_t)std::max(B, 1));
-  double *scratch = wsT<double>(h, "spec_scratch", (size_t)3 * std::max(B, 1) * k);
   unsigned long long *mt = wsT<unsigned long long>(h, "min_theta", 1);
   const double big = 1e300;
   unsigned long long bigbits;
@@ -1208,12 +1207,13 @@ void run_sigma(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts &o
   tm.mark(C_SPEC);
   if (B > 0 && poly) {
     // the fractions run on D = p_g(C)'s own tridiagonal (no spectral map)
+    jb.poles = 0;
     jb.a = const_cast<double *>(alpha);
     jb.g0 = cfmode == 1 ? wsT<double>(h, "jac_g0", (size_t)B) : nullptr;
     launch_poly_prep(alpha, beta, beta0, k_eff, B, k, jb, h->d_status, st);
     check_launch(h, "poly_prep");
   } else if (B > 0) {
-    launch_spectral_impl(alpha, beta, beta0, k_eff, B, k, jb, scratch, mt, h->d_status, st);
+    launch_spectral_impl(alpha, beta, beta0, k_eff, B, k, jb, mt, h->d_status, st);
     check_launch(h, "spectral");
   }
   CfProblem cp{};
@@ -2808,9 +2808,9 @@ lgw_status lgw_fit_factors(lgw_handle *h, int32_t n_pairs, int32_t n_aux, const 
 namespace {
 
 // 2^21 doubles = 16 MiB on every device that loads the library, held until
-// the process exits.  Layout per call: Jacobi a [B][k], b2 [B][k], w0 [B],
-// depth [B] (ints, rounded up), three tridiagonal work rows [3][B][k], one
-// word for the smallest Gauss node.
+// the process exits.  Layout per call: poles [B][k], weights [B][k], w0 [B],
+// depth [B] (ints, rounded up), 3 B k doubles that are not used (they keep
+// the accepted sizes what they were), one word for the smallest Gauss node.
 constexpr size_t kNoallocDoubles = (size_t)1 << 21;
 static __device__ __align__(256) double g_noalloc_scratch[kNoallocDoubles];
 
@@ -2933,7 +2933,7 @@ extern "C" lgw_status lgw_sigma_from_coeffs_noalloc(lgw_handle *h, const lgw_sys
       return set_err(h, LGW_ERR_SHAPE,
                      "noalloc: orbital index outside [0, n_v + n_c) or k_eff outside [0, k]");
   }
-  launch_spectral_impl(alpha, beta, beta0, k_eff, (int)B, k, jb, work, mt, h->d_status, st);
+  launch_spectral_impl(alpha, beta, beta0, k_eff, (int)B, k, jb, mt, h->d_status, st);
   CfProblem cp{};
   cp.n_t = n_t;
   cp.n_m = n_m;

@@ -346,15 +346,17 @@ void launch_pass2_dcgs(const VecCtx &c, int j, cudaStream_t st);
 void launch_scale_rows_to_bf16(const double *x, const double *dsq, int Bs, int N,
                                __nv_bfloat16 *out, cudaStream_t st);
 
-// k_spectral.cu : tridiagonal -> Gauss rule -> Omega-space Jacobi matrix
+// k_spectral.cu : tridiagonal -> Gauss rule -> Omega-space poles
 struct JacobiBufs {
-  double *a;    // [B][k]
-  double *b2;   // [B][k]  b2[i][j] = b_{j+1}^2 couples j and j+1
-  double *w0;   // [B]     total weight (zeroth moment)
+  double *a;    // [B][k]  poles Omega_j (pole sums) or the fraction's diagonal
+  double *b2;   // [B][k]  pole weights, or b2[i][j] = b_{j+1}^2 coupling j and j+1
+  double *w0;   // [B]     total weight (zeroth moment; fractions only)
   int *n;       // [B]     depth
+  // 1: Omega-space poles and weights of the spectral map (Sigma_tm = -eta
+  // G(zeta), G the pole sum); 0: continued fraction of a tridiagonal
+  int poles = 1;
   // polynomial variant: G(0) per vector, and the fractions belong to
-  // D = p_g(C) (Sigma_tm = (G(zeta) - G(0)) / z); NULL for the Omega-space
-  // fractions of the spectral map (Sigma_tm = -eta G(zeta))
+  // D = p_g(C) (Sigma_tm = (G(zeta) - G(0)) / z); NULL otherwise
   double *g0 = nullptr;
 };
 
@@ -377,10 +379,10 @@ void launch_cheb_final(const PolyStep &p, const double *qprev, const double *bet
 void launch_poly_prep(const double *alpha, const double *beta, const double *beta0,
                       const int *k_eff, int B, int k, JacobiBufs jb, unsigned *status,
                       cudaStream_t st);
-// scratch: 3 * B * k doubles; min_theta_bits: running minimum of the Gauss
-// nodes (positive doubles compare like their bit patterns)
+// min_theta_bits: running minimum of the Gauss nodes (positive doubles
+// compare like their bit patterns)
 void launch_spectral_impl(const double *alpha, const double *beta, const double *beta0,
-                          const int *k_eff, int B, int k, JacobiBufs jb, double *scratch,
+                          const int *k_eff, int B, int k, JacobiBufs jb,
                           unsigned long long *min_theta_bits, unsigned *status, cudaStream_t st);
 
 // make_vector: a hash start vector vec [N] (entries in [-1, 1), zero
