@@ -5,8 +5,10 @@
 // gemm1: Y = L^T (Delta^1/2 X), split over the pair dimension (long K).
 // gemm2: U = L Y with the Lanczos epilogue w = Delta^2 q + c_K Delta^1/2 U -
 //        beta_j q_{j-1} and per-tile partial sums of alpha_j = q_j . w.
-// These run on the FP64 pipe (about 1.2 TFLOP/s on GB300); they are the
-// plain FP64 path and the FP64 coupling-vector product V = L M.
+// These run on the FP64 pipe (about 1.2 TFLOP/s on GB300).  The FP64 path
+// takes the tensor-core products of k_gemm_oz.cu (20 TFLOP/s) where a system
+// holds the digits of L; these remain for systems without them: no memory for
+// the digits, a handle with a workspace limit, Inf or NaN in L.
 #include "lgw_internal.cuh"
 
 namespace lgw {

@@ -1,0 +1,658 @@
+// FP64 matrix products on the tensor cores by error-free slicing (the scheme
+// of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59 (2012) 95).
+//
+// GB300 executes FP64 at 2 lanes per SM clock (1.2 TFLOP/s); its BF16 tensor
+// cores multiply small integers exactly and add them exactly in FP32 up to
+// 2^24.  Each operand row (along the contraction) is scaled by a power of two
+// above its largest magnitude, x = 2^e sum_s d_s 2^(-6-7s), into 8 signed
+// 7-bit digits d_s in [-64, 64]: a resolution of 2^-56 of the row's largest
+// element, where FP64's own rounding of that element is 2^-53.  Then
+//   sum_k x_k y_k = 2^(ex+ey-12) sum_t 2^(-7t) S_t,  S_t = sum_{i+j=t} d_i . d_j
+// over t = 0..8 (43 digit products; the dropped ones are below 2^-62 of the
+// largest product).  Products are at most 2^12, so over 1024 terms S_0..S_3
+// are exact multiples of their unit below 2^24 of it; the others carry weights
+// of 2^-28 and less and may round.  Every 1024 terms the sums are joined in
+// 64-bit integers and rounded once to FP64.  The digits of a product thus lose
+// less than an FP64 dot product's own roundings do
+// (tests/test_gpu_f64_products.py; against exact sums, B = C R with 1024 terms
+// errs by 2.6e-16 of its norm, the FP64 FMA chain by 1.08e-15).
+//
+// N_vc 32768, N_aux 1024, 64 vectors: L^T x 207 us and L y 272 us, against 3.6
+// and 4.1 ms on the FP64 pipe (2 x 32768 x 1024 x 64 flops: 20 TFLOP/s in FP64
+// terms).  The tensor pipe is 37% busy there, DRAM at 2.6 TB/s: an MMA of few
+// columns costs more than its share, and a tile's sums are joined with the
+// tensor pipe idle (TMEM holds one tile).
+//
+// Layout: digits as BF16, [slice][K block of 64][row][64], so a TMA box (64
+// elements by rows) is one contiguous run, as for the other contractions.  A
+// CTA owns 128 rows of A by NT rows of B and keeps S_0 .. S_7 as 8 NT TMEM
+// columns: digit i of A against the stacked digits 0..7-i of B is one product
+// of N = (8-i) NT columns that lands in S_i .. S_7, so an A tile is read once
+// however many digits of B it meets.  An MMA whose columns cross a multiple of
+// 256 gives wrong sums, so at NT = 64 the product is split there.  Digit s is
+// stored with its weight 2^(-7s) (BF16 is a float), so S_8 is simply added to
+// S_7's columns.  B's eight tiles of a K block have two buffers, A's go through
+// a ring of single tiles.
+#include <cudaTypedefs.h>
+
+#include <algorithm>
+#include <cstdio>
+
+#include "tc_ptx.cuh"
+
+namespace lgw {
+namespace oz {
+
+using namespace tc;
+
+constexpr int S = OZ_SLICES;
+constexpr int BM = 128;
+constexpr int KB = 64;          // K elements per block: one 128-byte swizzle row
+constexpr int CHUNK_KB = 16;    // 1024 terms per exact sum
+constexpr int NTHREADS = 192;
+
+template <int NT>
+struct Cfg {
+  static constexpr int A_BYTES = BM * KB * 2;
+  static constexpr int B_BYTES = S * NT * KB * 2;
+  static constexpr int A_STAGES = NT == 64 ? 6 : 8;
+  static constexpr int BOX = NT == 64 ? 4 : 8;   // B's slices per box (32 KB at most)
+  static constexpr int BAR_BYTES = 256;
+  static constexpr int SMEM = 1024 + 2 * B_BYTES + A_STAGES * A_BYTES + BAR_BYTES;
+  static constexpr uint32_t TMEM_COLS = S * NT;
+};
+
+__device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *tm, uint64_t *bar, int x,
+                                            int y, int z, int w) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(tm)), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z), "r"(w)
+      : "memory");
+}
+// 8 consecutive FP32 columns of this thread's TMEM lane (no wait)
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&r)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+      : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]),
+        "=f"(r[7])
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld_wait() {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ int hi_abs(double p) { return __double2hiint(p) & 0x7fffffff; }
+
+// d * 2^sh for a finite d: on the exponent field while argument and result
+// are normal (FP64 multiplications load the narrow FP64 pipe).
+__device__ __forceinline__ double scale_pow2(double d, int sh) {
+  const int hi = __double2hiint(d), f = ((hi >> 20) & 0x7ff) + sh;
+  if (d == 0.0) return 0.0;
+  if (f >= 1 && f <= 2046 && (hi & 0x7ff00000) != 0) return __hiloint2double(hi + (sh << 20), __double2loint(d));
+  return scalbn(d, sh);
+}
+
+// sum_t 2^(40 - 7t) S_t from the weighted sums s[t] = 2^(-7t) S_t: a 64-bit
+// integer below 2^62.3 in magnitude, and what is left below its unit where the
+// double has room for it.
+__device__ __forceinline__ double join_sums(const float (&s)[8]) {
+  const int h = __float2int_rn(s[0]) * 128 + __float2int_rn(s[1] * 0x1p+7f);
+  const int g = __float2int_rn(s[2] * 0x1p+14f) * 128 + __float2int_rn(s[3] * 0x1p+21f);
+  const float low = (s[6] + s[7]) * 0x1p+40f;
+  const int il = __float2int_rn(low);
+  const int f = __float2int_rn(s[5] * 0x1p+35f) * 32 + il;
+  const long long t = ((long long)h << 33) + (long long)g * (1 << 19) +
+                      (long long)__float2int_rn(s[4] * 0x1p+28f) * 4096 + f;
+  double d = __ll2double_rn(t);
+  if (hi_abs(d) < ((1023 + 55) << 20)) d += (double)(low - (float)il);
+  return d;
+}
+
+// out[col * ldo + row] of the tile's products; the epilogues of the FP64
+// contractions (k_gemm_f64.cu), and plain or accumulated output.
+struct Epi {
+  int mode;
+  const int *ea, *eb;      // exponent fields of A's and B's rows
+  double *out;             // OZ_PART: [split][Ncols][ldo]; else [Ncols][ldo]
+  int ldo;
+  double scale;            // OZ_ADD: out += scale * product
+  const double *Delta2, *dsq, *cd, *q, *qprev, *betaj;
+  double *alpha_part;      // [M / 64][Ncols] partials of q . w, or NULL
+  unsigned *status;
+};
+
+template <int NT>
+__global__ void __launch_bounds__(NTHREADS, 1)
+    k_oz_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+              int M, int Ncols, int num_kb, int kb_per_split, Epi e) {
+  using C = Cfg<NT>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = reinterpret_cast<uint8_t *>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  uint8_t *bbuf = smem, *aring = smem + 2 * C::B_BYTES;
+  uint64_t *afull = reinterpret_cast<uint64_t *>(aring + C::A_STAGES * C::A_BYTES);
+  uint64_t *aempty = afull + C::A_STAGES;
+  uint64_t *bfull = aempty + C::A_STAGES;   // [2]
+  uint64_t *bempty = bfull + 2;             // [2]
+  uint64_t *tfull = bempty + 2;             // the eight sums of a chunk are complete
+  uint64_t *tempty = tfull + 1;             // and have been read
+  uint64_t *mdone = tempty + 1;             // every MMA issued by the CTA has completed
+  uint32_t *tslot = reinterpret_cast<uint32_t *>(mdone + 1);
+  // alpha partials per epilogue warp, over the B buffers once their last
+  // MMAs are done
+  double(*red)[NT] = reinterpret_cast<double(*)[NT]>(bbuf);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // N tiles fastest: the CTAs that share A's tiles run together
+  const int m_tile = blockIdx.y, n_tile = blockIdx.x, split = blockIdx.z;
+  const int kb0 = split * kb_per_split, kb1 = min(num_kb, kb0 + kb_per_split);
+  const int nk = max(0, kb1 - kb0);
+  const int chunks = (nk + CHUNK_KB - 1) / CHUNK_KB;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < C::A_STAGES; ++s) {
+      mbar_init(&afull[s], 1);
+      mbar_init(&aempty[s], 1);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&bfull[s], 1);
+      mbar_init(&bempty[s], 1);
+    }
+    mbar_init(tfull, 1);
+    mbar_init(tempty, 4);   // one arrival per epilogue warp
+    mbar_init(mdone, 1);
+    fence_barrier_init();
+  }
+  if (warp == 1) tmem_alloc(tslot, C::TMEM_COLS);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tslot;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int na = 0, nb = 0;   // tiles issued
+      bool ok = true;
+      for (int it = 0; it < nk && ok; ++it) {
+        const int bs = it & 1;
+        if (!mbar_wait(&bempty[bs], ((it >> 1) & 1) ^ 1, e.status)) break;
+        mbar_expect_tx(&bfull[bs], C::B_BYTES);
+        for (int p = 0; p < S; p += C::BOX)
+          tma_load_4d(bbuf + bs * C::B_BYTES + p * (NT * KB * 2), &tmB, &bfull[bs], 0, n_tile * NT,
+                      kb0 + it, p);
+        nb = it + 1;
+        for (int i = 0; i < S; ++i, ++na) {
+          const int as = na % C::A_STAGES;
+          if (!mbar_wait(&aempty[as], ((na / C::A_STAGES) & 1) ^ 1, e.status)) {
+            ok = false;
+            break;
+          }
+          mbar_expect_tx(&afull[as], C::A_BYTES);
+          tma_load_4d(aring + as * C::A_BYTES, &tmA, &afull[as], 0, m_tile * BM, kb0 + it, i);
+        }
+      }
+      // every issued copy must have landed before the CTA may exit
+      for (int i = max(0, na - C::A_STAGES); i < na; ++i)
+        mbar_wait(&afull[i % C::A_STAGES], (i / C::A_STAGES) & 1, e.status);
+      for (int i = max(0, nb - 2); i < nb; ++i) mbar_wait(&bfull[i & 1], (i >> 1) & 1, e.status);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      int na = 0;
+      bool ok = true;
+      for (int c = 0; c < chunks && ok; ++c) {
+        if (c > 0 && !mbar_wait(tempty, (c - 1) & 1, e.status)) break;
+        tc_fence_after();
+        const int it1 = min(nk, (c + 1) * CHUNK_KB);
+        for (int it = c * CHUNK_KB; it < it1 && ok; ++it) {
+          const int bs = it & 1;
+          if (!mbar_wait(&bfull[bs], (it >> 1) & 1, e.status)) {
+            ok = false;
+            break;
+          }
+          const uint64_t db = make_sdesc(smem_u32(bbuf + bs * C::B_BYTES));
+#pragma unroll 1
+          for (int i = 0; i < S; ++i, ++na) {
+            const int as = na % C::A_STAGES;
+            if (!mbar_wait(&afull[as], (na / C::A_STAGES) & 1, e.status)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint64_t da = make_sdesc(smem_u32(aring + as * C::A_BYTES));
+            // columns i NT .. 8 NT, split at 256: lo columns from B's first
+            // rows, hi columns from the rows after them
+            const int c0 = i * NT, hi0 = max(c0, 256);
+            const int lo = max(0, min(256, S * NT) - c0), hi = max(0, S * NT - hi0);
+            const uint32_t idlo = make_idesc(BM, lo), idhi = make_idesc(BM, hi);
+            const uint64_t dbhi = db + (uint64_t)((hi0 - c0) * 128 >> 4);
+            const uint64_t db8 = db + (uint64_t)((S - i) * NT * 128 >> 4);
+#pragma unroll
+            for (int kk = 0; kk < KB / 16; ++kk) {
+              const uint32_t acc = (it > c * CHUNK_KB || i > 0 || kk > 0) ? 1u : 0u;
+              if (lo > 0) umma_bf16(tmem + (uint32_t)c0, da + 2 * kk, db + 2 * kk, idlo, acc);
+              if (hi > 0) umma_bf16(tmem + (uint32_t)hi0, da + 2 * kk, dbhi + 2 * kk, idhi, acc);
+              // t = 8: digit 8 - i of B, into S_7
+              if (i > 0)
+                umma_bf16(tmem + 7 * NT, da + 2 * kk, db8 + 2 * kk, make_idesc(BM, NT), 1u);
+            }
+            umma_commit(&aempty[as]);
+          }
+          if (ok) umma_commit(&bempty[bs]);
+        }
+        if (ok) umma_commit(tfull);
+      }
+      // no MMA may still write TMEM when it is freed (also after a timeout)
+      umma_commit(mdone);
+      mbar_wait(mdone, 0, e.status);
+    }
+  } else {
+    // ------------------------------ epilogue ------------------------------
+    const int qd = warp & 3;
+    const int row = m_tile * BM + qd * 32 + lane;
+    const bool rok = row < M;
+    const int fa = rok ? e.ea[row] : 1;
+    double d2 = 0.0, cdr = 0.0;
+    if (rok && (e.mode == OZ_LANCZOS || e.mode == OZ_APPLY)) {
+      d2 = e.Delta2[row];
+      cdr = e.cd[row];
+    } else if (rok && e.mode == OZ_START) {
+      cdr = e.dsq[row];
+    }
+    double *out = e.out + (e.mode == OZ_PART ? (size_t)split * Ncols * e.ldo : 0);
+    for (int c = 0; c < chunks; ++c) {
+      if (!mbar_wait(tfull, c & 1, e.status)) break;
+      tc_fence_after();
+      const bool last = c + 1 == chunks;
+#pragma unroll 1
+      for (int c8 = 0; c8 < NT; c8 += 8) {
+        const int col0 = n_tile * NT + c8;
+        const uint32_t tc0 = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)c8;
+        if (col0 >= Ncols) break;
+        float s[S][8];
+#pragma unroll
+        for (int t = 0; t < S; ++t)
+          tmem_ld8(tc0 + (uint32_t)(t * NT), s[t]);
+        tmem_ld_wait();
+        double part[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int col = col0 + i;
+          part[i] = 0.0;
+          if (!rok || col >= Ncols) continue;
+          const int fb = e.eb[col];
+          float v8[S];
+#pragma unroll
+          for (int t = 0; t < S; ++t) v8[t] = s[t][i];
+          // row scales 2^(field - 1022); a non-finite row gives NaN
+          double v = (fa >= 2047 || fb >= 2047)
+                         ? __longlong_as_double(0x7ff8000000000000LL)
+                         : scale_pow2(join_sums(v8), max(fa, 1) + max(fb, 1) - 2044 - 52);
+          double *o = out + (size_t)col * e.ldo + row;
+          if (e.mode == OZ_ADD) {
+            *o = fma(e.scale, v, *o);
+            continue;
+          }
+          if (c > 0) v += *o;
+          if (!last || e.mode == OZ_PART) {
+            *o = v;
+          } else if (e.mode == OZ_START) {
+            *o = cdr * v;
+          } else {
+            const size_t oi = (size_t)col * e.ldo + row;
+            const double qv = e.q[oi];
+            double w = fma(d2, qv, cdr * v);
+            if (e.mode == OZ_LANCZOS && e.qprev != nullptr)
+              w = fma(-e.betaj[col], e.qprev[oi], w);
+            *o = w;
+            part[i] = qv * w;
+          }
+        }
+        if (e.alpha_part != nullptr && last) {
+          // the eight columns' sums over the warp's rows: a transposed
+          // butterfly (lane bits 2..0 pick the column), then bits 3 and 4
+#pragma unroll
+          for (int off = 4; off >= 1; off >>= 1) {
+            const bool up = (lane & off) != 0;
+#pragma unroll
+            for (int i = 0; i < off; ++i) {
+              const double send = up ? part[i] : part[i + off];
+              const double keep = up ? part[i + off] : part[i];
+              part[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+            }
+          }
+          part[0] += __shfl_xor_sync(0xffffffffu, part[0], 8);
+          part[0] += __shfl_xor_sync(0xffffffffu, part[0], 16);
+          if (lane < 8) red[qd][c8 + lane] = part[0];
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tempty);
+    }
+    if (e.alpha_part != nullptr && chunks > 0) {
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      for (int i = threadIdx.x - 64; i < 2 * NT; i += 128) {
+        const int half = i / NT, col = i % NT, b = n_tile * NT + col;
+        if (b < Ncols && m_tile * BM + 64 * half < M)
+          e.alpha_part[(size_t)(2 * m_tile + half) * Ncols + b] =
+              red[2 * half][col] + red[2 * half + 1][col];
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, C::TMEM_COLS);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Digits of an operand
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+// x on the grid 2^(f - 1022 - 55) of a row whose largest exponent field is f,
+// biased so that the base-128 digits come out as 64 + d_s.
+__device__ __forceinline__ unsigned long long fixed56(double x, int f) {
+  constexpr unsigned long long bias =
+      64ULL * ((1ULL << 49) + (1ULL << 42) + (1ULL << 35) + (1ULL << 28) + (1ULL << 21) +
+               (1ULL << 14) + (1ULL << 7) + 1ULL);
+  const long long b = __double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  long long m = b & 0xfffffffffffffLL;
+  if (ex != 0) m |= 1LL << 52;
+  const int sh = max(ex, 1) - f + 2;   // at most 2: |x| < 2^(f - 1022)
+  long long v = 0;
+  if (sh >= 0)
+    v = m << sh;
+  else if (sh > -56)
+    v = (m + (1LL << (-sh - 1))) >> -sh;
+  if (b < 0) v = -v;
+  return (unsigned long long)v + bias;
+}
+// BF16 bits of 2^(-7s) times digit s (an integer in [-64, 64]) of the biased
+// fixed point
+__device__ __forceinline__ uint32_t digit_bf16(unsigned long long u, int s) {
+  const uint32_t t = s == 0 ? (uint32_t)(u >> 49) : (uint32_t)(u >> (49 - 7 * s)) & 127u;
+  const float w = __uint_as_float((uint32_t)(127 - 7 * s) << 23);   // 2^(-7s)
+  return __float_as_uint((__uint_as_float(0x4B000000u | t) - 8388672.0f) * w) >> 16;
+}
+// 16 consecutive K elements of one operand row into its eight digit planes
+__device__ __forceinline__ void store_digits16(const unsigned long long (&u)[16], uint16_t *dst,
+                                               size_t plane) {
+#pragma unroll
+  for (int s = 0; s < S; ++s) {
+    uint32_t w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      w[i] = digit_bf16(u[2 * i], s) | (digit_bf16(u[2 * i + 1], s) << 16);
+    uint4 *o = reinterpret_cast<uint4 *>(dst + s * plane);
+    o[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    o[1] = make_uint4(w[4], w[5], w[6], w[7]);
+  }
+}
+
+// A matrix in memory: element (r, c) = x[r * ld + c] * (scale ? scale[c] : 1)
+// inside [nr][nc], zero outside.
+struct Src {
+  const double *x, *scale;
+  size_t ld;
+  int nr, nc;
+  __device__ __forceinline__ double at(int r, int c) const {
+    if (r >= nr || c >= nc) return 0.0;
+    const double v = x[(size_t)r * ld + c];
+    return scale ? scale[c] * v : v;
+  }
+};
+
+// Largest exponent field of each operand row: the operand's rows are the
+// matrix's rows (COLS = false, contraction along c) or its columns.
+template <bool COLS>
+__global__ void __launch_bounds__(256) k_oz_max(Src src, int *__restrict__ e) {
+  const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
+  if (COLS) {
+    const int c = c0 + (threadIdx.x & 63);
+    int m = 0;
+    for (int r = r0 + (threadIdx.x >> 6); r < r0 + 64; r += 4) m = max(m, exp_field(src.at(r, c)));
+    if (m > 0) atomicMax(&e[c], m);
+  } else {
+    const int r = r0 + (threadIdx.x >> 2), cc = c0 + (threadIdx.x & 3) * 16;
+    int m = 0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) m = max(m, exp_field(src.at(r, cc + i)));
+    m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+    m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+    if ((threadIdx.x & 3) == 0 && m > 0) atomicMax(&e[r], m);
+  }
+}
+
+// Digits of a 64 x 64 tile; the operand has `rows` rows and nkb K blocks.
+template <bool COLS>
+__global__ void __launch_bounds__(256) k_oz_slice(Src src, const int *__restrict__ e,
+                                                  uint16_t *__restrict__ out, int rows, int nkb) {
+  __shared__ double tile[COLS ? 64 : 1][65];
+  const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
+  const int i = threadIdx.x >> 2, k0 = (threadIdx.x & 3) * 16;   // row and K offset in the tile
+  if (COLS) {
+    for (int r = threadIdx.x >> 6; r < 64; r += 4)
+      tile[r][threadIdx.x & 63] = src.at(r0 + r, c0 + (threadIdx.x & 63));
+    __syncthreads();
+  }
+  const int row = (COLS ? c0 : r0) + i, kb = COLS ? blockIdx.y : blockIdx.x;
+  if (row >= rows || kb >= nkb) return;
+  const int f = max(e[row], 1);
+  unsigned long long u[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k)
+    u[k] = fixed56(COLS ? tile[k0 + k][i] : src.at(row, c0 + k0 + k), f);
+  store_digits16(u, out + ((size_t)kb * rows + row) * 64 + k0, (size_t)nkb * rows * 64);
+}
+
+// One operand row per block, up to OZ_ROW_MAX elements: the sum of `splits`
+// partials (fixed order, optionally stored to y), its exponent and its digits.
+__global__ void __launch_bounds__(256) k_oz_rows(const double *__restrict__ x, int splits,
+                                                 size_t part, Src src, double *__restrict__ y,
+                                                 int *__restrict__ e, uint16_t *__restrict__ out,
+                                                 int rows, int nkb) {
+  extern __shared__ double v[];
+  __shared__ int wmax[8];
+  const int r = blockIdx.x;
+  int m = 0;
+  for (int i = threadIdx.x; i < nkb * 64; i += 256) {
+    double s = 0.0;
+    if (r < src.nr && i < src.nc) {
+      const size_t o = (size_t)r * src.ld + i;
+      for (int p = 0; p < splits; ++p) s += x[(size_t)p * part + o];
+      if (src.scale) s *= src.scale[i];
+      if (y) y[o] = s;
+    }
+    v[i] = s;
+    m = max(m, exp_field(s));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
+  __syncthreads();
+  for (int w = 0; w < 8; ++w) m = max(m, wmax[w]);
+  if (threadIdx.x == 0) e[r] = m;
+  m = max(m, 1);
+  for (int g = threadIdx.x; g < nkb * 4; g += 256) {
+    unsigned long long u[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) u[k] = fixed56(v[g * 16 + k], m);
+    store_digits16(u, out + ((size_t)(g >> 2) * rows + r) * 64 + (g & 3) * 16,
+                   (size_t)nkb * rows * 64);
+  }
+}
+
+// *bad != 0 if an exponent field says Inf or NaN
+__global__ void k_oz_check(const int *__restrict__ e, int n, unsigned *bad) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n && e[i] >= 2047) atomicOr(bad, 1u);
+}
+
+static PFN_cuTensorMapEncodeTiled_v12000 encoder() {
+  static PFN_cuTensorMapEncodeTiled_v12000 f = [] {
+    void *p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
+                                         &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      p = nullptr;
+    return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+  }();
+  return f;
+}
+
+// Map of an operand's digits: (64 elements, rows, K blocks, slices)
+static bool encode(CUtensorMap *tm, const OzOperand &o, int box_rows, int box_slices) {
+  auto enc = encoder();
+  if (!enc) return false;
+  cuuint64_t dims[4] = {64, (cuuint64_t)o.rows, (cuuint64_t)o.nkb, (cuuint64_t)S};
+  cuuint64_t strides[3] = {128, (cuuint64_t)o.rows * 128, (cuuint64_t)o.nkb * o.rows * 128};
+  cuuint32_t box[4] = {64, (cuuint32_t)box_rows, 1, (cuuint32_t)box_slices};
+  cuuint32_t es[4] = {1, 1, 1, 1};
+  return enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<uint16_t *>(o.d), dims, strides,
+             box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int NT>
+static void launch(const CUtensorMap &A, const CUtensorMap &B, int M, int Ncols, int nkb, int per,
+                   int splits, const Epi &e, cudaStream_t st) {
+  static bool attr = false;
+  if (!attr) {
+    cudaFuncSetAttribute(k_oz_gemm<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         Cfg<NT>::SMEM);
+    attr = true;
+  }
+  const dim3 grid((Ncols + NT - 1) / NT, (M + BM - 1) / BM, splits);
+  k_oz_gemm<NT><<<grid, NTHREADS, Cfg<NT>::SMEM, st>>>(A, B, M, Ncols, nkb, per, e);
+}
+
+static void launch_rows(const double *x, int splits, size_t part, const Src &src, double *y,
+                        const OzOperand &o, cudaStream_t st) {
+  static bool attr = false;
+  if (!attr) {
+    cudaFuncSetAttribute(k_oz_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         OZ_ROW_MAX * (int)sizeof(double));
+    attr = true;
+  }
+  k_oz_rows<<<o.rows, 256, (size_t)o.nkb * 64 * sizeof(double), st>>>(x, splits, part, src, y, o.e,
+                                                                      o.d, o.rows, o.nkb);
+}
+
+static int sm_count() {
+  static int n = [] {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    return v > 0 ? v : 152;
+  }();
+  return n;
+}
+
+// Columns of B per tile: as many as fill the chip with up to `splits` K splits
+// (an A tile is loaded once per column tile, so wide tiles load less), no
+// wider than B.
+static int tile_cols(int m_tiles, int ncols, int splits) {
+  int nt = ncols >= 64 ? 64 : (ncols >= 32 ? 32 : 16);
+  while (nt > 16 && m_tiles * ((ncols + nt - 1) / nt) * splits * 2 <= sm_count()) nt /= 2;
+  return nt;
+}
+
+}  // namespace oz
+
+// K splits of A's M rows by ncols columns over nkb K blocks: the count with
+// the fewest K blocks in sequence, a CTA's fixed cost (pipeline fill, eight
+// sums joined and stored) standing for four of them.
+int oz_splits(int M, int ncols, int nkb) {
+  const int m_tiles = (M + oz::BM - 1) / oz::BM;
+  const int nt = oz::tile_cols(m_tiles, ncols, std::min(64, nkb));
+  const int tiles = m_tiles * ((ncols + nt - 1) / nt), nsm = oz::sm_count();
+  int best = 1;
+  long long best_cost = 1LL << 60;
+  for (int s = 1; s <= std::min(64, nkb); ++s) {
+    const int per = (nkb + s - 1) / s, real = (nkb + per - 1) / per;
+    const long long waves = ((long long)tiles * real + nsm - 1) / nsm;
+    const long long cost = waves * (per + 4 * ((per + oz::CHUNK_KB - 1) / oz::CHUNK_KB));
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = real;
+    }
+  }
+  return best;
+}
+
+bool launch_oz_gemm(const OzOperand &A, const OzOperand &B, int M, int Ncols, int splits,
+                    const OzOut &o, unsigned *status, cudaStream_t st) {
+  oz::Epi e{};
+  e.mode = o.mode;
+  e.ea = A.e;
+  e.eb = B.e;
+  e.out = o.out;
+  e.ldo = o.ldo;
+  e.scale = o.scale;
+  e.Delta2 = o.Delta2;
+  e.dsq = o.dsq;
+  e.cd = o.cd;
+  e.q = o.q;
+  e.qprev = o.qprev;
+  e.betaj = o.betaj;
+  e.alpha_part = o.alpha_part;
+  e.status = status;
+  const int nkb = A.nkb, per = (nkb + splits - 1) / splits;
+  const int m_tiles = (M + oz::BM - 1) / oz::BM;
+  const int nt = oz::tile_cols(m_tiles, Ncols, o.mode == OZ_PART ? std::min(64, nkb) : 1);
+  CUtensorMap ta, tb;
+  if (A.rows < oz::BM || B.rows < nt || A.nkb != B.nkb || !oz::encode(&ta, A, oz::BM, 1) ||
+      !oz::encode(&tb, B, nt, nt == 64 ? oz::Cfg<64>::BOX : OZ_SLICES))
+    return false;
+  if (nt == 64)
+    oz::launch<64>(ta, tb, M, Ncols, nkb, per, splits, e, st);
+  else if (nt == 32)
+    oz::launch<32>(ta, tb, M, Ncols, nkb, per, splits, e, st);
+  else
+    oz::launch<16>(ta, tb, M, Ncols, nkb, per, splits, e, st);
+  return true;
+}
+
+// Digits of x [nr][nc] (row stride ld, optional column scale): operand rows
+// are x's rows, or its columns.  o.rows covers them (more rows become zeros).
+void launch_oz_slice(const double *x, size_t ld, int nr, int nc, const double *scale, bool cols,
+                     const OzOperand &o, cudaStream_t st) {
+  const oz::Src src{x, scale, ld, nr, nc};
+  // short rows: one kernel, a block per row (4 us at 160 rows of 256); longer
+  // ones spread each row over many blocks (64 rows of 32768: 32 us in two
+  // kernels, where a block per row would take about 60)
+  if (!cols && o.nkb * 64 <= 4096) {
+    oz::launch_rows(x, 1, 0, src, nullptr, o, st);
+    return;
+  }
+  cudaMemsetAsync(o.e, 0, sizeof(int) * o.rows, st);
+  const int kr = cols ? o.nkb : (o.rows + 63) / 64, kc = cols ? (o.rows + 63) / 64 : o.nkb;
+  const dim3 grid(kc, kr), data((nc + 63) / 64, (nr + 63) / 64);
+  if (cols) {
+    oz::k_oz_max<true><<<data, 256, 0, st>>>(src, o.e);
+    oz::k_oz_slice<true><<<grid, 256, 0, st>>>(src, o.e, o.d, o.rows, o.nkb);
+  } else {
+    oz::k_oz_max<false><<<data, 256, 0, st>>>(src, o.e);
+    oz::k_oz_slice<false><<<grid, 256, 0, st>>>(src, o.e, o.d, o.rows, o.nkb);
+  }
+}
+
+// y [rows][len] = sum of the split partials, and its digits (len <= OZ_ROW_MAX)
+void launch_oz_reduce(const double *part, int splits, int nr, int len, double *y,
+                      const OzOperand &o, cudaStream_t st) {
+  const oz::Src src{part, nullptr, (size_t)len, nr, len};
+  oz::launch_rows(part, splits, (size_t)nr * len, src, y, o, st);
+}
+
+void launch_oz_check(const OzOperand &o, unsigned *bad, cudaStream_t st) {
+  oz::k_oz_check<<<(o.rows + 255) / 256, 256, 0, st>>>(o.e, o.rows, bad);
+}
+
+}  // namespace lgw

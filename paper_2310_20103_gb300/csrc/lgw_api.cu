@@ -46,6 +46,7 @@ struct lgw_handle {
   // with its own workspace namespace (ws_prefix)
   std::vector<cudaStream_t> lanes;
   std::string ws_prefix;
+  std::vector<lgw_system *> sliced;   // systems that hold digits of L (k_gemm_oz.cu)
   void drop_graphs() {
     for (auto &kv : graphs)
       if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
@@ -63,6 +64,10 @@ struct lgw_system {
   // Tamm-Dancoff view (A = Delta + (c_K/2) L L^T in place of C), made on first use
   SysDev tda{};
   void *tda_buf = nullptr;
+  // digits of L for the FP64 products: 1 made, -1 not (no memory, or L holds
+  // Inf or NaN), 0 not asked for yet
+  int oz_state = 0;
+  void *oz_buf = nullptr;
 };
 
 // ---------------------------------------------------------------------------
@@ -106,9 +111,41 @@ void check_launch(lgw_handle *h, const char *what) {
   }
 }
 
-void *ws(lgw_handle *h, const std::string &name, size_t bytes) {
+void free_digits(lgw_system *sys) {
+  if (sys->oz_buf) cudaFree(sys->oz_buf);
+  sys->oz_buf = nullptr;
+  sys->s.ozA = sys->s.ozT = sys->tda.ozA = sys->tda.ozT = OzOperand{};
+  sys->oz_state = -1;
+}
+
+// Gives back every system's digits of L and the workspace of the digits
+// (oz_* buffers); the FP64 products then run on the CUDA cores.  False if
+// there was nothing to give back.
+bool drop_digits(lgw_handle *h) {
+  bool any = !h->sliced.empty();
+  for (auto &kv : h->bufs) any = any || (kv.first.find("oz_") != std::string::npos && kv.second.p);
+  if (!any) return false;
+  cudaDeviceSynchronize();
+  for (lgw_system *sys : h->sliced) free_digits(sys);
+  h->sliced.clear();
+  for (auto &kv : h->bufs)
+    if (kv.first.find("oz_") != std::string::npos && kv.second.p) {
+      cudaFree(kv.second.p);
+      h->ws_bytes -= kv.second.n;
+      kv.second = lgw_handle::Buf{};
+    }
+  h->ws_gen++;
+  h->drop_graphs();
+  return true;
+}
+
+// A workspace buffer of at least `bytes`.  optional (the digits of the FP64
+// products): NULL where the device's memory does not allow it, and on a
+// handle with a byte limit, which is kept for the buffers every call needs.
+void *ws(lgw_handle *h, const std::string &name, size_t bytes, bool optional = false) {
   auto &b = h->bufs[h->ws_prefix + name];
   if (bytes == 0) bytes = 8;
+  if (optional && h->ws_limit) return nullptr;
   if (b.n < bytes) {
     // the handle's byte limit is checked before anything is freed, so a
     // refused request leaves the workspace as it was
@@ -127,8 +164,13 @@ void *ws(lgw_handle *h, const std::string &name, size_t bytes) {
     }
     void *p = nullptr;
     cudaError_t e = cudaMalloc(&p, bytes);
+    if (e == cudaErrorMemoryAllocation && !optional && drop_digits(h)) {
+      cudaGetLastError();
+      e = cudaMalloc(&p, bytes);
+    }
     if (e != cudaSuccess) {
       cudaGetLastError();
+      if (optional) return nullptr;
       set_err(h, LGW_ERR_OOM, "cudaMalloc(%zu bytes) for %s failed: %s", bytes, name.c_str(),
               cudaGetErrorString(e));
       throw Fail{LGW_ERR_OOM};
@@ -401,6 +443,51 @@ void make_fp8(lgw_handle *h, SysDev &s, const double *src, int ld, int nr, int n
   s.sL = sc;
 }
 
+// Digits of L for the FP64 products (32 bytes per element of L), made on the
+// first FP64 request.  They may take a third of the free memory at most, and
+// are given back when a workspace allocation fails (drop_digits); without
+// them the products run on the CUDA cores.  One synchronisation, once.
+void ensure_digits(lgw_handle *h, lgw_system *sys) {
+  if (sys->oz_state != 0) return;
+  SysDev &s = sys->s;
+  sys->oz_state = -1;
+  if (!s.L64 || !tc_available() || s.A > OZ_ROW_MAX) return;
+  const size_t plane = OzOperand::digits((size_t)s.N, (size_t)s.A / 64) * sizeof(uint16_t);
+  const size_t ints = ((size_t)s.N + s.A + 64) * sizeof(int);
+  size_t fr = 0, tot = 0;
+  LGW_TRY_CUDA(h, cudaMemGetInfo(&fr, &tot));
+  if (2 * plane + ints > fr / 3) return;
+  void *p = nullptr;
+  if (cudaMalloc(&p, 2 * plane + ints) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  sys->oz_buf = p;
+  uint16_t *d = static_cast<uint16_t *>(p);
+  int *e = reinterpret_cast<int *>(static_cast<uint8_t *>(p) + 2 * plane);
+  const OzOperand a{d, e, s.N, s.A / 64};
+  const OzOperand t{d + plane / sizeof(uint16_t), e + s.N, s.A, s.N / 64};
+  unsigned *bad = reinterpret_cast<unsigned *>(e + s.N + s.A);
+  cudaStream_t st = h->stream;
+  LGW_TRY_CUDA(h, cudaMemsetAsync(bad, 0, sizeof(unsigned), st));
+  launch_oz_slice(s.L64, s.A, s.N, s.A, nullptr, false, a, st);
+  launch_oz_slice(s.L64, s.A, s.N, s.A, nullptr, true, t, st);
+  launch_oz_check(t, bad, st);
+  check_launch(h, "oz_slice(L)");
+  h->launches--;   // the system's preparation, not this call's
+  unsigned hb = 1;
+  LGW_TRY_CUDA(h, cudaMemcpyAsync(&hb, bad, sizeof hb, cudaMemcpyDeviceToHost, st));
+  LGW_TRY_CUDA(h, cudaStreamSynchronize(st));
+  if (hb != 0) {
+    free_digits(sys);
+    return;
+  }
+  s.ozA = a;
+  s.ozT = t;
+  sys->oz_state = 1;
+  h->sliced.push_back(sys);
+}
+
 // The copies of L a request needs must exist; the E4M3 copies are made on
 // the first FP8 request for a system that keeps its FP64 copy.
 void ensure_copies(lgw_handle *h, const lgw_system *csys, const Opts &o) {
@@ -413,6 +500,7 @@ void ensure_copies(lgw_handle *h, const lgw_system *csys, const Opts &o) {
     set_err(h, LGW_ERR_UNSUPPORTED, "the system keeps no BF16 copy of L (LGW_SYS_NO_BF16)");
     throw Fail{LGW_ERR_UNSUPPORTED};
   }
+  if (o.precision == LGW_FP64) ensure_digits(h, const_cast<lgw_system *>(csys));
   if ((o.precision != LGW_FP8 && o.precision != LGW_FP8_DEQ) || cs.L8) return;
   if (!cs.L64) {
     set_err(h, LGW_ERR_UNSUPPORTED, "no E4M3 copy of L and no FP64 copy to make it from");
@@ -509,6 +597,180 @@ PolyOp make_poly(int g, double lo, double hi) {
   }
   p.c[0] *= 0.5;
   return p;
+}
+
+// ---------------------------------------------------------------------------
+// FP64 contractions: on the tensor cores where the system holds digits of L
+// and the operands' digits fit the workspace, else on the CUDA cores.
+// ---------------------------------------------------------------------------
+constexpr int F64_ROWS = 1024;   // vectors sliced at a time
+
+struct F64Work {
+  OzOperand x, y;        // digits of the vectors and of y = L^T (Delta^1/2 x); d NULL: none
+  double *part = nullptr;
+  int rows = 0;
+};
+
+F64Work f64_work(lgw_handle *h, const SysDev &s, int rows) {
+  F64Work f;
+  f.rows = rows;
+  size_t part = (size_t)gemm1_f64_splits(s, rows) * rows * s.A;
+  if (s.ozA.d) {
+    const int r = std::min(rows, F64_ROWS);
+    const size_t nx = OzOperand::digits(r, s.N / 64), ny = OzOperand::digits(r, s.A / 64);
+    uint16_t *d = static_cast<uint16_t *>(ws(h, "oz_xy", (nx + ny) * sizeof(uint16_t), true));
+    int *e = d ? static_cast<int *>(ws(h, "oz_e", 2 * (size_t)r * sizeof(int), true)) : nullptr;
+    const size_t op = (size_t)oz_splits(s.A, r, s.N / 64) * r * s.A;
+    double *pp = e ? static_cast<double *>(ws(h, "yp64", std::max(part, op) * sizeof(double), true))
+                   : nullptr;
+    if (pp) {
+      f.x = OzOperand{d, e, r, s.N / 64};
+      f.y = OzOperand{d + nx, e + r, r, s.A / 64};
+      f.part = pp;
+      return f;
+    }
+  }
+  f.part = wsT<double>(h, "yp64", part);
+  return f;
+}
+
+void oz_gemm(lgw_handle *h, const OzOperand &A, const OzOperand &B, int M, int Ncols, int splits,
+             const OzOut &o, const char *what) {
+  if (!launch_oz_gemm(A, B, M, Ncols, splits, o, h->d_status, h->stream)) {
+    set_err(h, LGW_ERR_CUDA, "tensor map of %s failed", what);
+    throw Fail{LGW_ERR_CUDA};
+  }
+  check_launch(h, what);
+}
+
+// Y [rows][A] = (Delta^1/2 q) L; with digits, those of Y too (of the last
+// F64_ROWS rows) for f64_contract2.
+void f64_contract1(lgw_handle *h, const SysDev &s, const F64Work &f, const double *q, int rows,
+                   double *Y) {
+  cudaStream_t st = h->stream;
+  if (!f.x.d || !s.ozT.d) {
+    const int splits = gemm1_f64_splits(s, rows);
+    launch_gemm1_f64(s, q, rows, f.part, splits, st);
+    check_launch(h, "gemm1_f64");
+    launch_reduce_y_f64(f.part, splits, rows, s.A, Y, st);
+    check_launch(h, "reduce_y_f64");
+    return;
+  }
+  for (int r0 = 0; r0 < rows; r0 += F64_ROWS) {
+    const int nr = std::min(F64_ROWS, rows - r0);
+    OzOperand x = f.x, y = f.y;
+    x.rows = y.rows = nr;
+    launch_oz_slice(q + (size_t)r0 * s.N, (size_t)s.N, nr, s.N, s.dsq, false, x, st);
+    check_launch(h, "oz_slice(x)");
+    const int splits = oz_splits(s.A, nr, s.N / 64);
+    OzOut o;
+    o.mode = OZ_PART;
+    o.out = f.part;
+    o.ldo = s.A;
+    oz_gemm(h, s.ozT, x, s.A, nr, splits, o, "oz_gemm1");
+    launch_oz_reduce(f.part, splits, nr, s.A, Y + (size_t)r0 * s.A, y, st);
+    check_launch(h, "oz_reduce(y)");
+  }
+}
+
+// The FP64 GEMM2 and its epilogue; fresh: Y comes straight from f64_contract1
+// (its digits are in place).
+void f64_contract2(lgw_handle *h, const SysDev &s, const F64Work &f, const double *Y, bool fresh,
+                   int Bs, int epi, const double *q, const double *qprev, const double *betaj,
+                   double *w, double *alpha_part) {
+  cudaStream_t st = h->stream;
+  if (!f.y.d || !s.ozA.d || Bs > F64_ROWS) {
+    launch_gemm2_f64(s, Y, Bs, epi, q, qprev, betaj, w, alpha_part, st);
+    check_launch(h, "gemm2_f64");
+    return;
+  }
+  OzOperand y = f.y;
+  y.rows = Bs;
+  if (!fresh) {
+    launch_oz_reduce(Y, 1, Bs, s.A, nullptr, y, st);
+    check_launch(h, "oz_slice(y)");
+  }
+  OzOut o;
+  o.mode = epi;
+  o.out = w;
+  o.ldo = s.N;
+  o.Delta2 = s.Delta2;
+  o.dsq = s.dsq;
+  o.cd = s.cd;
+  o.q = q;
+  o.qprev = qprev;
+  o.betaj = betaj;
+  o.alpha_part = epi == EPI_START ? nullptr : alpha_part;
+  oz_gemm(h, s.ozA, y, s.N, Bs, 1, o, "oz_gemm2");
+}
+
+// S [Ni][Nmu] += scale * X^T Y over R rows (X row stride ldx, Y row stride
+// ldy), 1024 rows at a time on the tensor cores.
+void f64_atb(lgw_handle *h, const double *X, int ldx, const double *Y, int ldy, int R, int Ni,
+             int Nmu, double *S, double scale = 1.0) {
+  cudaStream_t st = h->stream;
+  constexpr int RC = 1024;
+  const int ra = std::max(128, round_up(Nmu, 16)), rb = std::max(64, round_up(Ni, 16));
+  const int kb = (std::min(R, RC) + 63) / 64;
+  const size_t na = OzOperand::digits(ra, kb), nb = OzOperand::digits(rb, kb);
+  uint16_t *d = nullptr;
+  int *e = nullptr;
+  if (tc_available()) {
+    d = static_cast<uint16_t *>(ws(h, "oz_atb", (na + nb) * sizeof(uint16_t), true));
+    if (d) e = static_cast<int *>(ws(h, "oz_atb_e", (size_t)(ra + rb) * sizeof(int), true));
+  }
+  if (!e) {
+    launch_atb_f64(X, ldx, Y, ldy, R, Ni, Nmu, S, st, scale);
+    check_launch(h, "atb_f64");
+    return;
+  }
+  for (int r0 = 0; r0 < R; r0 += RC) {
+    const int nr = std::min(RC, R - r0), nkb = (nr + 63) / 64;
+    const OzOperand a{d, e, ra, nkb}, b{d + na, e + ra, rb, nkb};
+    launch_oz_slice(Y + (size_t)r0 * ldy, (size_t)ldy, nr, Nmu, nullptr, true, a, st);
+    launch_oz_slice(X + (size_t)r0 * ldx, (size_t)ldx, nr, Ni, nullptr, true, b, st);
+    check_launch(h, "oz_slice(atb)");
+    OzOut o;
+    o.mode = OZ_ADD;
+    o.out = S;
+    o.ldo = Nmu;
+    o.scale = scale;
+    oz_gemm(h, a, b, Nmu, Ni, 1, o, "oz_gemm(atb)");
+  }
+}
+
+// B [n_pairs][n] = C [n_pairs][n] R [n][n], 8192 pairs at a time on the
+// tensor cores.
+void f64_fit(lgw_handle *h, const double *C, const double *R, int n_pairs, int n, double *B) {
+  cudaStream_t st = h->stream;
+  constexpr int PC = 8192;
+  const int ra = std::max(128, round_up(n, 16)), nkb = (n + 63) / 64;
+  const int rb = std::max(64, round_up(std::min(n_pairs, PC), 16));
+  const size_t na = OzOperand::digits(ra, nkb), nb = OzOperand::digits(rb, nkb);
+  uint16_t *d = nullptr;
+  int *e = nullptr;
+  if (tc_available() && n <= OZ_ROW_MAX) {
+    d = static_cast<uint16_t *>(ws(h, "oz_fit", (na + nb) * sizeof(uint16_t), true));
+    if (d) e = static_cast<int *>(ws(h, "oz_fit_e", (size_t)(ra + rb) * sizeof(int), true));
+  }
+  if (!e) {
+    launch_gemm_nn_f64(C, R, n_pairs, n, n, B, st);
+    check_launch(h, "gemm_nn_f64");
+    return;
+  }
+  const OzOperand a{d, e, ra, nkb}, b{d + na, e + ra, rb, nkb};
+  launch_oz_slice(R, (size_t)n, n, n, nullptr, true, a, st);
+  check_launch(h, "oz_slice(R)");
+  for (int p0 = 0; p0 < n_pairs; p0 += PC) {
+    const int np = std::min(PC, n_pairs - p0);
+    launch_oz_slice(C + (size_t)p0 * n, (size_t)n, np, n, nullptr, false, b, st);
+    check_launch(h, "oz_slice(C)");
+    OzOut o;
+    o.mode = OZ_PART;
+    o.out = B + (size_t)p0 * n;
+    o.ldo = n;
+    oz_gemm(h, a, b, n, np, 1, o, "oz_gemm(fit)");
+  }
 }
 
 // keep_basis stores all k + 1 FP64 basis vectors of a sub-batch (slot j of
@@ -630,8 +892,8 @@ void run_lanczos(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts 
 
   // contraction buffers
   double *Y64 = wsT<double>(h, "y64", (size_t)Bs * s.A);
-  const int splits64 = gemm1_f64_splits(s, Bs);
-  double *Yp64 = tc ? nullptr : wsT<double>(h, "yp64", (size_t)splits64 * Bs * s.A);
+  F64Work f64;
+  if (!tc) f64 = f64_work(h, s, Bs);
   TcPlan *plan = nullptr;
   uint8_t *x8 = nullptr, *y8 = nullptr;
   uint16_t *x16 = nullptr, *y16 = nullptr;
@@ -730,12 +992,8 @@ void run_lanczos(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts 
       launch_gemm2_tc_split(plan, ucd_buf, h->d_status, st);
       check_launch(h, "gemm2_tc");
     } else {
-      launch_gemm1_f64(s, bsrc, Bs, Yp64, splits64, st);
-      check_launch(h, "gemm1_f64");
-      launch_reduce_y_f64(Yp64, splits64, Bs, s.A, Y64, st);
-      check_launch(h, "reduce_y_f64");
-      launch_gemm2_f64(s, Y64, Bs, EPI_APPLY, bsrc, nullptr, nullptr, pT, nullptr, st);
-      check_launch(h, "gemm2_f64");
+      f64_contract1(h, s, f64, bsrc, Bs, Y64);
+      f64_contract2(h, s, f64, Y64, true, Bs, EPI_APPLY, bsrc, nullptr, nullptr, pT, nullptr);
     }
   };
   Timer tm(h);
@@ -767,8 +1025,8 @@ void run_lanczos(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts 
         LGW_TRY_CUDA(h, cudaMemcpy2DAsync(Y64, sizeof(double) * s.A, pv.d_M + (size_t)vec0 * s.n_aux,
                                           sizeof(double) * s.n_aux, sizeof(double) * s.n_aux, nvec,
                                           cudaMemcpyDeviceToDevice, st));
-        launch_gemm2_f64(s, Y64, Bs, EPI_START, nullptr, nullptr, nullptr, c.w, nullptr, st);
-        check_launch(h, "gemm2_f64(start)");
+        f64_contract2(h, s, f64, Y64, false, Bs, EPI_START, nullptr, nullptr, nullptr, c.w,
+                      nullptr);
         // padding rows of w (b >= nvec) hold L*0 = 0 already
         launch_norm_partials(c, c.w, c.norm_a, st);
         check_launch(h, "norm_partials");
@@ -865,21 +1123,15 @@ void run_lanczos(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts 
         } else if (dcgs) {
           // C w_{j-1} in FP64 with the partials of w . C w (alpha~ after
           // scaling by 1/beta_j^2)
-          launch_gemm1_f64(s, c.wv, Bs, Yp64, splits64, st);
-          check_launch(h, "gemm1_f64");
-          launch_reduce_y_f64(Yp64, splits64, Bs, s.A, Y64, st);
-          check_launch(h, "reduce_y_f64");
+          f64_contract1(h, s, f64, c.wv, Bs, Y64);
           tm.mark(C_GEMM2);
-          launch_gemm2_f64(s, Y64, Bs, EPI_APPLY, c.wv, nullptr, nullptr, c.w, c.alpha_part, st);
-          check_launch(h, "gemm2_f64");
+          f64_contract2(h, s, f64, Y64, true, Bs, EPI_APPLY, c.wv, nullptr, nullptr, c.w,
+                        c.alpha_part);
         } else {
-          launch_gemm1_f64(s, qj, Bs, Yp64, splits64, st);
-          check_launch(h, "gemm1_f64");
-          launch_reduce_y_f64(Yp64, splits64, Bs, s.A, Y64, st);
-          check_launch(h, "reduce_y_f64");
+          f64_contract1(h, s, f64, qj, Bs, Y64);
           tm.mark(C_GEMM2);
-          launch_gemm2_f64(s, Y64, Bs, EPI_LANCZOS, qj, qp, c.betaj, c.w, c.alpha_part, st);
-          check_launch(h, "gemm2_f64");
+          f64_contract2(h, s, f64, Y64, true, Bs, EPI_LANCZOS, qj, qp, c.betaj, c.w,
+                        c.alpha_part);
         }
         // ---- recurrence and reorthogonalisation ----
         tm.mark(C_DOTS);
@@ -964,7 +1216,8 @@ void run_lanczos(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts 
     rep->n_second_pass = n2;
     rep->n_sub_batches = nsub;
     rep->b_sub = Bs;
-    rep->gemm1_splits = tc ? splits_tc : splits64;
+    rep->gemm1_splits = tc ? splits_tc
+                           : (f64.x.d ? oz_splits(s.A, Bs, s.N / 64) : gemm1_f64_splits(s, Bs));
   }
 }
 
@@ -1075,8 +1328,8 @@ void run_band(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts &o,
   bc.xq = tc ? nullptr : wsT<double>(h, "band_xq", (size_t)Bs * N);
 
   double *Y64 = wsT<double>(h, "y64", (size_t)Bs * s.A);
-  const int splits64 = gemm1_f64_splits(s, Bs);
-  double *Yp64 = tc ? nullptr : wsT<double>(h, "yp64", (size_t)splits64 * Bs * s.A);
+  F64Work f64;
+  if (!tc) f64 = f64_work(h, s, Bs);
   float *ucd_buf = tc ? wsT<float>(h, "ucd", (size_t)Bs * N) : nullptr;
   TcPlan *plan = nullptr;
   float *Yp32 = nullptr;
@@ -1136,8 +1389,8 @@ void run_band(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts &o,
         LGW_TRY_CUDA(h, cudaMemcpy2DAsync(Y64, sizeof(double) * s.A, pv.d_M + row0 * s.n_aux,
                                           sizeof(double) * s.n_aux, sizeof(double) * s.n_aux,
                                           nvec, cudaMemcpyDeviceToDevice, st));
-        launch_gemm2_f64(s, Y64, Bs, EPI_START, nullptr, nullptr, nullptr, c.w, nullptr, st);
-        check_launch(h, "gemm2_f64(start)");
+        f64_contract2(h, s, f64, Y64, false, Bs, EPI_START, nullptr, nullptr, nullptr, c.w,
+                      nullptr);
       } else {
         launch_start_from_v(c, pv.d_V + row0 * s.n_vc, s.n_vc, s.n_vc, st);
         check_launch(h, "start_from_v");
@@ -1164,13 +1417,9 @@ void run_band(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts &o,
         launch_band_assemble(bc, j, ucd_buf, st);
         check_launch(h, "band_assemble");
       } else {
-        launch_gemm1_f64(s, bc.xq, Bs, Yp64, splits64, st);
-        check_launch(h, "gemm1_f64");
-        launch_reduce_y_f64(Yp64, splits64, Bs, s.A, Y64, st);
-        check_launch(h, "reduce_y_f64");
+        f64_contract1(h, s, f64, bc.xq, Bs, Y64);
         tm.mark(C_GEMM2);
-        launch_gemm2_f64(s, Y64, Bs, EPI_APPLY, bc.xq, nullptr, nullptr, c.w, nullptr, st);
-        check_launch(h, "gemm2_f64");
+        f64_contract2(h, s, f64, Y64, true, Bs, EPI_APPLY, bc.xq, nullptr, nullptr, c.w, nullptr);
       }
       tm.mark(C_DOTS);
       h->launches += launch_band_append(bc, 1, j, st);
@@ -1445,8 +1694,7 @@ void reverse_sweep(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opt
   double *useg = wsT<double>(h, "rev_useg", (size_t)cs * BN);
   double *yseg = wsT<double>(h, "rev_yseg", (size_t)cs * BA);
   double *ybseg = wsT<double>(h, "rev_ybseg", (size_t)cs * BA);
-  const int sp = gemm1_f64_splits(s, Bs);
-  double *yp = wsT<double>(h, "rev_yp", (size_t)sp * BA);
+  const F64Work f64 = f64_work(h, s, Bs);
   double *Y = wsT<double>(h, "adj_Y", BN);
   RevCtx r{};
   r.N = N;
@@ -1494,12 +1742,8 @@ void reverse_sweep(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opt
   }
   // T = C x with L^T D x into yout (FP64 contractions)
   auto apply_c = [&](const double *x, double *yout) {
-    launch_gemm1_f64(s, x, Bs, yp, sp, st);
-    check_launch(h, "gemm1_f64(reverse)");
-    launch_reduce_y_f64(yp, sp, Bs, A, yout, st);
-    check_launch(h, "reduce_y_f64(reverse)");
-    launch_gemm2_f64(s, yout, Bs, EPI_APPLY, x, nullptr, nullptr, T, nullptr, st);
-    check_launch(h, "gemm2_f64(reverse)");
+    f64_contract1(h, s, f64, x, Bs, yout);
+    f64_contract2(h, s, f64, yout, true, Bs, EPI_APPLY, x, nullptr, nullptr, T, nullptr);
   };
   auto fbk = [&](int k) { return fb + (size_t)(k - 1) * BN; };
   auto rbk = [&](int k) { return rb + (size_t)(k - 1) * BN; };
@@ -1556,12 +1800,8 @@ void reverse_sweep(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opt
         clenshaw(qj, qp, rc.betaj, rc.w, rc.alpha_part);
       } else {
         double *yj = yseg + (size_t)(j - s0) * BA;
-        launch_gemm1_f64(s, qj, Bs, yp, sp, st);
-        check_launch(h, "gemm1_f64(recompute)");
-        launch_reduce_y_f64(yp, sp, Bs, A, yj, st);
-        check_launch(h, "reduce_y_f64(recompute)");
-        launch_gemm2_f64(s, yj, Bs, EPI_LANCZOS, qj, qp, rc.betaj, rc.w, rc.alpha_part, st);
-        check_launch(h, "gemm2_f64(recompute)");
+        f64_contract1(h, s, f64, qj, Bs, yj);
+        f64_contract2(h, s, f64, yj, true, Bs, EPI_LANCZOS, qj, qp, rc.betaj, rc.w, rc.alpha_part);
       }
       launch_alpha_reduce(rc, j, st);
       check_launch(h, "alpha_reduce(recompute)");
@@ -1578,12 +1818,8 @@ void reverse_sweep(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opt
       const double *uj = useg + (size_t)(j - s0) * BN;
       if (!poly) {
         double *ybj = ybseg + (size_t)(j - s0) * BA;
-        launch_gemm1_f64(s, uj, Bs, yp, sp, st);
-        check_launch(h, "gemm1_f64(reverse)");
-        launch_reduce_y_f64(yp, sp, Bs, A, ybj, st);
-        check_launch(h, "reduce_y_f64(reverse)");
-        launch_gemm2_f64(s, ybj, Bs, EPI_APPLY, uj, nullptr, nullptr, cu, nullptr, st);
-        check_launch(h, "gemm2_f64(reverse)");
+        f64_contract1(h, s, f64, uj, Bs, ybj);
+        f64_contract2(h, s, f64, ybj, true, Bs, EPI_APPLY, uj, nullptr, nullptr, cu, nullptr);
         continue;
       }
       // Clenshaw vectors of q_j, then the reverse recurrence from u = ubar_j
@@ -1618,26 +1854,22 @@ void reverse_sweep(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opt
       launch_rev_gd(r.Gd, as, uj, fbk(1), BN, st);
       for (int kk = 1; kk < g; ++kk) launch_rev_gd(r.Gd, 2.0 * as, rbk(kk), fbk(kk + 1), BN, st);
       check_launch(h, "rev_gd");
-      launch_atb_f64(uj, N, fy, A, Bs, N, A, SC, st, as);
-      launch_atb_f64(fbk(1), N, ry, A, Bs, N, A, SC, st, as);
+      f64_atb(h, uj, N, fy, A, Bs, N, A, SC, as);
+      f64_atb(h, fbk(1), N, ry, A, Bs, N, A, SC, as);
       if (g > 1) {
-        launch_atb_f64(rbk(1), N, fy + BA, A, (g - 1) * Bs, N, A, SC, st, 2.0 * as);
-        launch_atb_f64(fbk(2), N, ry + BA, A, (g - 1) * Bs, N, A, SC, st, 2.0 * as);
+        f64_atb(h, rbk(1), N, fy + BA, A, (g - 1) * Bs, N, A, SC, 2.0 * as);
+        f64_atb(h, fbk(2), N, ry + BA, A, (g - 1) * Bs, N, A, SC, 2.0 * as);
       }
-      check_launch(h, "atb_f64(SC, poly pairs)");
     }
     if (poly) continue;
-    launch_atb_f64(useg, N, yseg, A, n * Bs, N, A, SC, st);
-    check_launch(h, "atb_f64(SC, ubar)");
-    launch_atb_f64(seg + BN, N, ybseg, A, n * Bs, N, A, SC, st);
-    check_launch(h, "atb_f64(SC, q)");
+    f64_atb(h, useg, N, yseg, A, n * Bs, N, A, SC);
+    f64_atb(h, seg + BN, N, ybseg, A, n * Bs, N, A, SC);
   }
   const double *q0 = ckpt + BN;
   launch_rev_finish(r, q0, Y, st);
   check_launch(h, "rev_finish");
   if (SB) {
-    launch_atb_f64(Y, N, pv.d_M + (size_t)c.vec0 * s.n_aux, s.n_aux, c.nvec, N, s.n_aux, SB, st);
-    check_launch(h, "atb_f64(SB)");
+    f64_atb(h, Y, N, pv.d_M + (size_t)c.vec0 * s.n_aux, s.n_aux, c.nvec, N, s.n_aux, SB);
   }
   launch_adj_accumulate(a, s.Delta, BasisRef{q0, nullptr, nullptr}, Y, r.Gd, dD, gdeps, st);
   check_launch(h, "adj_accumulate");
@@ -1870,6 +2102,11 @@ lgw_status lgw_release_system(lgw_system *sys) {
     if (p) cudaFree(p);
   if (sys->Ltb_lo) cudaFree(sys->Ltb_lo);
   if (sys->tda_buf) cudaFree(sys->tda_buf);
+  if (sys->oz_buf) {
+    free_digits(sys);
+    auto &v = sys->h->sliced;
+    v.erase(std::remove(v.begin(), v.end(), sys), v.end());
+  }
   if (s.L8) cudaFree(s.L8);
   if (s.L8t) cudaFree(s.L8t);
   if (s.sL) cudaFree(s.sL);
@@ -1970,14 +2207,9 @@ lgw_status lgw_apply_casida(lgw_handle *h, const lgw_system *sys, int32_t n_vec,
       LGW_TRY_CUDA(h, cudaStreamSynchronize(st));
       tc_plan_destroy(plan);
     } else {
-      const int splits = gemm1_f64_splits(s, Bs);
-      double *yp = wsT<double>(h, "yp64", (size_t)splits * Bs * s.A);
-      launch_gemm1_f64(s, xp, Bs, yp, splits, st);
-      check_launch(h, "gemm1_f64");
-      launch_reduce_y_f64(yp, splits, Bs, s.A, Y64, st);
-      check_launch(h, "reduce_y_f64");
-      launch_gemm2_f64(s, Y64, Bs, EPI_APPLY, xp, nullptr, nullptr, wp, nullptr, st);
-      check_launch(h, "gemm2_f64");
+      const F64Work f64 = f64_work(h, s, Bs);
+      f64_contract1(h, s, f64, xp, Bs, Y64);
+      f64_contract2(h, s, f64, Y64, true, Bs, EPI_APPLY, xp, nullptr, nullptr, wp, nullptr);
     }
     LGW_TRY_CUDA(h, cudaMemcpy2DAsync(Yo.dev, sizeof(double) * s.n_vc, wp, sizeof(double) * s.N,
                                       sizeof(double) * s.n_vc, n_vec, cudaMemcpyDeviceToDevice, st));
@@ -2664,24 +2896,14 @@ static lgw_status backward_impl(lgw_handle *h, const lgw_system *sys, const lgw_
         check_launch(h, "tc_gemm_f64out(SC)");
       } else {
         // P = Q^T D L over the k * Bs basis rows (FP64 GEMM1), R = Gam P
-        const int sp = gemm1_f64_splits(s, rows);
-        double *Pp = sp > 1 ? wsT<double>(h, "adj_Pp", (size_t)sp * rows * A) : P;
-        launch_gemm1_f64(s, c.basis, rows, Pp, sp, st);
-        check_launch(h, "gemm1_f64(adjoint)");
-        if (sp > 1) {
-          launch_reduce_y_f64(Pp, sp, rows, A, P, st);
-          check_launch(h, "reduce_y_f64(adjoint)");
-        }
+        f64_contract1(h, s, f64_work(h, s, rows), c.basis, rows, P);
         launch_gamma_p(a, P, A, R, st);
         check_launch(h, "gamma_p");
-        launch_atb_f64(c.basis, N, R, A, rows, N, A, SC, st);
-        check_launch(h, "atb_f64(SC)");
+        f64_atb(h, c.basis, N, R, A, rows, N, A, SC);
       }
       // SB += Y^T M
       if (SB) {
-        launch_atb_f64(Y, N, pv.d_M + (size_t)c.vec0 * s.n_aux, s.n_aux, c.nvec, N, s.n_aux, SB,
-                       st);
-        check_launch(h, "atb_f64(SB)");
+        f64_atb(h, Y, N, pv.d_M + (size_t)c.vec0 * s.n_aux, s.n_aux, c.nvec, N, s.n_aux, SB);
       }
       launch_adj_accumulate(a, s.Delta, qb, Y, Gd, dD, gdeps, st);
       check_launch(h, "adj_accumulate");
@@ -2781,8 +3003,7 @@ lgw_status lgw_fit_factors(lgw_handle *h, int32_t n_pairs, int32_t n_aux, const 
       const double *Cd = in_dev(h, "in_fitC", C, (size_t)n_pairs * n_aux);
       OutBuf<double> out;
       out.init(h, "out_fitB", B, (size_t)n_pairs * n_aux);
-      launch_gemm_nn_f64(Cd, R, n_pairs, n_aux, n_aux, out.dev, st);
-      check_launch(h, "gemm_nn_f64");
+      f64_fit(h, Cd, R, n_pairs, n_aux, out.dev);
       out.finish(h);
     }
     check_status(h);

@@ -32,6 +32,18 @@ enum : unsigned {
 inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 inline int64_t round_up64(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
+// Digits of one operand of an FP64 product on the tensor cores
+// (k_gemm_oz.cu): 8 BF16 planes [slice][K block of 64][rows][64] and each
+// row's largest exponent field.
+constexpr int OZ_SLICES = 8;
+constexpr int OZ_ROW_MAX = 24576;   // longest row sliced by one block (192 KB of shared memory)
+struct OzOperand {
+  uint16_t *d = nullptr;
+  int *e = nullptr;
+  int rows = 0, nkb = 0;
+  static size_t digits(size_t rows, size_t nkb) { return OZ_SLICES * rows * nkb * 64; }
+};
+
 // ---------------------------------------------------------------------------
 // Device-side system: padded copies owned by the system.
 // ---------------------------------------------------------------------------
@@ -58,6 +70,9 @@ struct SysDev {
   uint8_t *L8;      // [N][A]   e4m3(L / s_mu)
   uint8_t *L8t;     // [A][N]   its transpose, K-block-major (kblk_e4m3)
   float *sL;        // [A]      s_mu
+  // digits of L64, made on the first FP64 request: rows vc (contraction over
+  // mu) and rows mu (contraction over vc); absent where memory is short
+  OzOperand ozA, ozT;
 };
 
 // ---------------------------------------------------------------------------
@@ -227,6 +242,32 @@ enum { EPI_START = 0, EPI_LANCZOS = 1, EPI_APPLY = 2 };
 void launch_gemm2_f64(const SysDev &s, const double *Y, int Bs, int epi, const double *q,
                       const double *qprev, const double *betaj, double *w, double *alpha_part,
                       cudaStream_t st);
+
+// k_gemm_oz.cu : FP64 products on the tensor cores (error-free slicing)
+// out[col * ldo + row] from A's row `row` and B's row `col`:
+//   OZ_PART:  [split][Ncols][ldo] = product over the split's K range
+//   OZ_ADD:   += scale * product
+//   OZ_START, OZ_LANCZOS, OZ_APPLY: the epilogues EPI_* of k_gemm_f64.cu
+enum { OZ_START = EPI_START, OZ_LANCZOS = EPI_LANCZOS, OZ_APPLY = EPI_APPLY, OZ_PART, OZ_ADD };
+struct OzOut {
+  int mode = 0;
+  double *out = nullptr;
+  int ldo = 0;
+  double scale = 1.0;
+  const double *Delta2 = nullptr, *dsq = nullptr, *cd = nullptr, *q = nullptr, *qprev = nullptr,
+               *betaj = nullptr;
+  double *alpha_part = nullptr;   // [M / 64][Ncols]
+};
+int oz_splits(int M, int ncols, int nkb);
+// A.rows >= 128, B.rows >= min(Ncols, 64) (16 at least); false if a tensor
+// map cannot be made
+bool launch_oz_gemm(const OzOperand &A, const OzOperand &B, int M, int Ncols, int splits,
+                    const OzOut &o, unsigned *status, cudaStream_t st);
+void launch_oz_slice(const double *x, size_t ld, int nr, int nc, const double *scale, bool cols,
+                     const OzOperand &o, cudaStream_t st);
+void launch_oz_reduce(const double *part, int splits, int nr, int len, double *y,
+                      const OzOperand &o, cudaStream_t st);
+void launch_oz_check(const OzOperand &o, unsigned *bad, cudaStream_t st);
 
 // k_gemm_tc.cu : BF16 tcgen05 contractions
 struct TcPlan;
