@@ -13,6 +13,7 @@
 // warp owns 256 consecutive elements, each lane four double2 of them.  All
 // cross-block sums go through per-chunk partials reduced in a fixed order,
 // so results do not depend on scheduling.
+#include "fp_bits.cuh"
 #include "lgw_internal.cuh"
 
 namespace lgw {
@@ -63,8 +64,9 @@ __device__ __forceinline__ dfl df_add_f(dfl a, float b) {
   return df_fast(s.h, __fadd_rn(s.l, a.l));
 }
 __device__ __forceinline__ dfl df_from(double x) {
-  const float h = __double2float_rn(x);
-  return {h, __double2float_rn(x - (double)h)};
+  dfl r;
+  split_d(x, r.h, r.l);
+  return r;
 }
 // (sh, sl) += a . b, TwoProd with the cross terms and TwoSum
 __device__ __forceinline__ void df_dot_acc(float &sh, float &sl, dfl a, dfl b) {
@@ -184,8 +186,8 @@ __device__ __forceinline__ void assemble_w_chunk(const VecCtx &c, int j,
     const double2 q2 = *reinterpret_cast<const double2 *>(q + e);
     const float2 v2 = *reinterpret_cast<const float2 *>(ucd + kblk_f32(b, e, c.Bs));
     double2 w2;
-    w2.x = fma(c.Delta2[e], q2.x, (double)v2.x);
-    w2.y = fma(c.Delta2[e + 1], q2.y, (double)v2.y);
+    w2.x = fma(c.Delta2[e], q2.x, f2d(v2.x));
+    w2.y = fma(c.Delta2[e + 1], q2.y, f2d(v2.y));
     if (qp != nullptr) {
       const double2 p2 = *reinterpret_cast<const double2 *>(qp + e);
       w2.x = fma(-bj, p2.x, w2.x);
@@ -516,8 +518,8 @@ __device__ __forceinline__ void normalize_chunk(const VecCtx &c, int j, int is_s
       // the BF16 operand from the FP32 image of q (FP64 multiplies and
       // FP64 -> BF16 conversions would load GB300's narrow FP64 pipe)
       __nv_bfloat162 x2;
-      x2.x = __float2bfloat16_rn(c.dsqf[e] * __double2float_rn(q2.x));
-      x2.y = __float2bfloat16_rn(c.dsqf[e + 1] * __double2float_rn(q2.y));
+      x2.x = __float2bfloat16_rn(c.dsqf[e] * d2f(q2.x));
+      x2.y = __float2bfloat16_rn(c.dsqf[e + 1] * d2f(q2.y));
       *reinterpret_cast<__nv_bfloat162 *>(c.xh + kblk_bf16(b, e, c.Bs)) = x2;
     }
   }
@@ -569,8 +571,8 @@ __global__ void __launch_bounds__(VEC_THREADS) k_start_from_vf(VecCtx c, const f
     double x0 = 0.0, x1 = 0.0;
     if (b < c.nvec) {
       const float2 v2 = *reinterpret_cast<const float2 *>(vf + kblk_f32(b, e, c.Bs));
-      x0 = c.dsq[e] * (double)v2.x;
-      x1 = c.dsq[e + 1] * (double)v2.y;
+      x0 = c.dsq[e] * f2d(v2.x);
+      x1 = c.dsq[e + 1] * f2d(v2.y);
     }
     *reinterpret_cast<double2 *>(c.w + voff + e) = make_double2(x0, x1);
     nrm = fma(x0, x0, fma(x1, x1, nrm));
@@ -659,8 +661,8 @@ __global__ void __launch_bounds__(VEC_THREADS) k_band_operand(BandCtx bc, int j)
     if (bc.xq != nullptr) *reinterpret_cast<double2 *>(bc.xq + voff + e) = q2;
     if (c.xh != nullptr) {
       __nv_bfloat162 x2;
-      x2.x = __float2bfloat16_rn(c.dsqf[e] * __double2float_rn(q2.x));
-      x2.y = __float2bfloat16_rn(c.dsqf[e + 1] * __double2float_rn(q2.y));
+      x2.x = __float2bfloat16_rn(c.dsqf[e] * d2f(q2.x));
+      x2.y = __float2bfloat16_rn(c.dsqf[e + 1] * d2f(q2.y));
       *reinterpret_cast<__nv_bfloat162 *>(c.xh + kblk_bf16(b, e, c.Bs)) = x2;
     }
   }
@@ -682,8 +684,8 @@ __global__ void __launch_bounds__(VEC_THREADS) k_band_assemble(BandCtx bc, int j
     const double2 q2 = *reinterpret_cast<const double2 *>(q + e);
     const float2 v2 = *reinterpret_cast<const float2 *>(ucd + kblk_f32(b, e, c.Bs));
     double2 w2;
-    w2.x = fma(c.Delta2[e], q2.x, (double)v2.x);
-    w2.y = fma(c.Delta2[e + 1], q2.y, (double)v2.y);
+    w2.x = fma(c.Delta2[e], q2.x, f2d(v2.x));
+    w2.y = fma(c.Delta2[e + 1], q2.y, f2d(v2.y));
     *reinterpret_cast<double2 *>(c.w + voff + e) = w2;
   }
 }

@@ -11,6 +11,7 @@
 // Delta^1/2 b) or, from the tensor cores, as ucd = c_K Delta^1/2 (L y) in FP32
 // with Delta^2 b added here.  The continued fractions then use D's
 // tridiagonal directly (Eq. 14): Sigma_tm = (G(-eta z) - G(0)) / z.
+#include "fp_bits.cuh"
 #include "lgw_internal.cuh"
 
 namespace lgw {
@@ -20,46 +21,61 @@ __device__ __forceinline__ int poly_elem_base(int chunk) {
   return chunk * VEC_CHUNK + wid * 256 + 2 * lane;
 }
 
-// C b at element pair e of vector b (FP64 product T [Bs][N], or the FP32
-// coupling ucd (kblk_f32 over Bs = gridDim.y vectors) + Delta^2 b)
-__device__ __forceinline__ double2 cb_pair(const double *T, const float *ucd, const double *Delta2,
-                                           const double2 b1, int b, int e) {
-  if (T) return *reinterpret_cast<const double2 *>(T + e);   // T offset to vector b
-  const float2 u = *reinterpret_cast<const float2 *>(ucd + kblk_f32(b, e, gridDim.y));
-  return make_double2(fma(Delta2[e], b1.x, (double)u.x), fma(Delta2[e + 1], b1.y, (double)u.y));
-}
+// S b = a_s C b + b_s b at a pair element, C b = Delta^2 b + u or T itself:
+//   T given:  a_s T + b_s b;   u given:  (a_s Delta^2 + b_s) b + a_s u.
+// Two FP64 operations per element on top of `add` in either form; the factor
+// a_s Delta^2 + b_s is formed once for the vectors of a block.  (GB300's FP64
+// pipe bounds these passes: with seven operations, two of them conversions, a
+// pass of 256 vectors at N_vc 131072 took 408 us, 46% of the HBM rate; 244 us
+// with three, the conversions on the integer pipe.)
 
 // out = ck q + 2 (a_s C b1 + b_s b1) - b2   (b1, b2 may be NULL: zero);
 // xh = bf16(Delta^1/2 out) for the next tensor-core product (or NULL).
-__global__ void __launch_bounds__(VEC_THREADS) k_cheb_step(PolyStep p) {
-  const int chunk = blockIdx.x, b = blockIdx.y;
-  const size_t voff = (size_t)b * p.N;
+// CHEB_VECS vectors per block (the launch's Bs is a multiple of 16).
+constexpr int CHEB_VECS = 4;
+
+__global__ void __launch_bounds__(VEC_THREADS) k_cheb_step(PolyStep p, int Bs) {
+  const int chunk = blockIdx.x;
   const int e0 = poly_elem_base(chunk);
+  const double as2 = 2.0 * p.as, bs2 = 2.0 * p.bs;
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const int e = e0 + u * 64;
     if (e >= p.N) continue;
-    const size_t o = voff + e;
-    const double2 q = *reinterpret_cast<const double2 *>(p.q + o);
-    double2 r = make_double2(p.ck * q.x, p.ck * q.y);
-    if (p.b1) {
-      const double2 b1 = *reinterpret_cast<const double2 *>(p.b1 + o);
-      const double2 t = cb_pair(p.T ? p.T + voff : nullptr, p.ucd, p.Delta2, b1, b, e);
-      r.x = fma(2.0 * p.as, t.x, fma(2.0 * p.bs, b1.x, r.x));
-      r.y = fma(2.0 * p.as, t.y, fma(2.0 * p.bs, b1.y, r.y));
+    double2 cf = make_double2(bs2, bs2);
+    if (!p.T) {
+      const double2 d2 = *reinterpret_cast<const double2 *>(p.Delta2 + e);
+      cf = make_double2(fma(as2, d2.x, bs2), fma(as2, d2.y, bs2));
     }
-    if (p.b2) {
-      const double2 b2 = *reinterpret_cast<const double2 *>(p.b2 + o);
-      r.x -= b2.x;
-      r.y -= b2.y;
-    }
-    *reinterpret_cast<double2 *>(p.out + o) = r;
-    if (p.xh) {
-      __nv_bfloat162 x2;
-      x2.x = __float2bfloat16_rn(p.dsqf[e] * (float)r.x);
-      x2.y = __float2bfloat16_rn(p.dsqf[e + 1] * (float)r.y);
-      // K-block-major over the Bs = gridDim.y vectors of the launch
-      *reinterpret_cast<__nv_bfloat162 *>(p.xh + kblk_bf16(b, e, gridDim.y)) = x2;
+    const float2 ds = p.xh ? *reinterpret_cast<const float2 *>(p.dsqf + e) : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int vb = 0; vb < CHEB_VECS; ++vb) {
+      const int b = blockIdx.y * CHEB_VECS + vb;
+      const size_t o = (size_t)b * p.N + e;
+      const double2 q = *reinterpret_cast<const double2 *>(p.q + o);
+      double2 r = make_double2(0.0, 0.0);
+      if (p.b2) r = *reinterpret_cast<const double2 *>(p.b2 + o);
+      r.x = fma(p.ck, q.x, -r.x);
+      r.y = fma(p.ck, q.y, -r.y);
+      if (p.b1) {
+        const double2 b1 = *reinterpret_cast<const double2 *>(p.b1 + o);
+        double2 t;
+        if (p.T) {
+          t = *reinterpret_cast<const double2 *>(p.T + o);
+        } else {
+          const float2 uc = *reinterpret_cast<const float2 *>(p.ucd + kblk_f32(b, e, Bs));
+          t = make_double2(f2d(uc.x), f2d(uc.y));
+        }
+        r.x = fma(cf.x, b1.x, fma(as2, t.x, r.x));
+        r.y = fma(cf.y, b1.y, fma(as2, t.y, r.y));
+      }
+      *reinterpret_cast<double2 *>(p.out + o) = r;
+      if (p.xh) {
+        __nv_bfloat162 x2;
+        x2.x = __float2bfloat16_rn(ds.x * d2f(r.x));
+        x2.y = __float2bfloat16_rn(ds.y * d2f(r.y));
+        *reinterpret_cast<__nv_bfloat162 *>(p.xh + kblk_bf16(b, e, Bs)) = x2;
+      }
     }
   }
 }
@@ -82,24 +98,29 @@ __global__ void __launch_bounds__(VEC_THREADS) k_cheb_final(PolyStep p, const do
     const size_t o = voff + e;
     const double2 q = *reinterpret_cast<const double2 *>(p.q + o);
     const double2 b1 = *reinterpret_cast<const double2 *>(p.b1 + o);
-    const double2 t = cb_pair(p.T ? p.T + voff : nullptr, p.ucd, p.Delta2, b1, b, e);
-    double2 r;
-    r.x = fma(p.as, t.x, fma(p.bs, b1.x, p.ck * q.x));
-    r.y = fma(p.as, t.y, fma(p.bs, b1.y, p.ck * q.y));
-    if (p.b2) {
-      const double2 b2 = *reinterpret_cast<const double2 *>(p.b2 + o);
-      r.x -= b2.x;
-      r.y -= b2.y;
+    double2 r = make_double2(0.0, 0.0), cf = make_double2(p.bs, p.bs), t;
+    if (p.T) {
+      t = *reinterpret_cast<const double2 *>(p.T + o);
+    } else {
+      const float2 uc = *reinterpret_cast<const float2 *>(p.ucd + kblk_f32(b, e, Bs));
+      t = make_double2(f2d(uc.x), f2d(uc.y));
+      const double2 d2 = *reinterpret_cast<const double2 *>(p.Delta2 + e);
+      cf = make_double2(fma(p.as, d2.x, p.bs), fma(p.as, d2.y, p.bs));
     }
+    if (p.b2) r = *reinterpret_cast<const double2 *>(p.b2 + o);
+    r.x = fma(p.ck, q.x, -r.x);
+    r.y = fma(p.ck, q.y, -r.y);
     if (qprev) {
       const double2 qp = *reinterpret_cast<const double2 *>(qprev + o);
       r.x = fma(-bj, qp.x, r.x);
       r.y = fma(-bj, qp.y, r.y);
     }
+    r.x = fma(cf.x, b1.x, fma(p.as, t.x, r.x));
+    r.y = fma(cf.y, b1.y, fma(p.as, t.y, r.y));
     *reinterpret_cast<double2 *>(w + o) = r;
     ap = fma(q.x, r.x, fma(q.y, r.y, ap));
   }
-  ap = block_sum(ap, red);
+  ap = block_sum_to0(ap, red);
   if (threadIdx.x == 0) alpha_part[(size_t)chunk * Bs + b] = ap;
 }
 
@@ -134,7 +155,7 @@ __global__ void k_poly_prep(const double *__restrict__ alpha, const double *__re
 }
 
 void launch_cheb_step(const PolyStep &p, int nchunks, int Bs, cudaStream_t st) {
-  k_cheb_step<<<dim3(nchunks, Bs), VEC_THREADS, 0, st>>>(p);
+  k_cheb_step<<<dim3(nchunks, Bs / CHEB_VECS), VEC_THREADS, 0, st>>>(p, Bs);
 }
 void launch_cheb_final(const PolyStep &p, const double *qprev, const double *betaj, double *w,
                        double *alpha_part, int nchunks, int Bs, cudaStream_t st) {

@@ -29,6 +29,7 @@
 //
 // Block layout as in the FP64 kernels: one block per (chunk of VEC_CHUNK
 // elements, vector), eight elements per thread.
+#include "fp_bits.cuh"
 #include "lgw_internal.cuh"
 
 namespace lgw {
@@ -166,8 +167,8 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_dots_split(VecCtx c, int j) 
         if (ucd != nullptr) {
           // w = Delta^2 q_j + c_K Delta^1/2 (L y) - beta_j q_{j-1}   (Eq. 4, 13)
           const float2 u2 = *reinterpret_cast<const float2 *>(ucd + kblk_f32(b, e, c.Bs));
-          w2.x = fma(c.Delta2[e], q2.x, (double)u2.x);
-          w2.y = fma(c.Delta2[e + 1], q2.y, (double)u2.y);
+          w2.x = fma(c.Delta2[e], q2.x, f2d(u2.x));
+          w2.y = fma(c.Delta2[e + 1], q2.y, f2d(u2.y));
           if (qp != nullptr) {
             const double2 p2 = *reinterpret_cast<const double2 *>(qp + e);
             w2.x = fma(-bj, p2.x, w2.x);
@@ -184,12 +185,9 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_dots_split(VecCtx c, int j) 
       }
     }
     nrm = fma(w2.x, w2.x, fma(w2.y, w2.y, nrm));
-    const float hx = __double2float_rn(w2.x), hy = __double2float_rn(w2.y);
     const int le = e - cbase;
-    swh[le] = hx;
-    swh[le + 1] = hy;
-    swl[le] = __double2float_rn(w2.x - (double)hx);
-    swl[le + 1] = __double2float_rn(w2.y - (double)hy);
+    split_d(w2.x, swh[le], swl[le]);
+    split_d(w2.y, swh[le + 1], swl[le + 1]);
   }
   if (PASS == 1) {
     nrm = block_sum(nrm, red);   // contains a __syncthreads
@@ -332,8 +330,8 @@ __global__ void __launch_bounds__(VEC_THREADS) k_update_split(VecCtx c, int j) {
       const int e = e0 + u * 64;
       if (e >= c.N) continue;
       double2 w2 = *reinterpret_cast<const double2 *>(w + e);
-      w2.x -= (double)r[2 * u];
-      w2.y -= (double)r[2 * u + 1];
+      w2.x -= f2d(r[2 * u]);
+      w2.y -= f2d(r[2 * u + 1]);
       *reinterpret_cast<double2 *>(w + e) = w2;
       nrm = fma(w2.x, w2.x, fma(w2.y, w2.y, nrm));
     }
@@ -353,16 +351,16 @@ __global__ void __launch_bounds__(VEC_THREADS) k_update_split(VecCtx c, int j) {
     double2 q2 = make_double2(0.0, 0.0);
     if (work) {
       q2 = *reinterpret_cast<const double2 *>(w + e);
-      q2.x = (q2.x - (double)r[2 * u]) * inv;
-      q2.y = (q2.y - (double)r[2 * u + 1]) * inv;
+      q2.x = (q2.x - f2d(r[2 * u])) * inv;
+      q2.y = (q2.y - f2d(r[2 * u + 1])) * inv;
     }
     *reinterpret_cast<double2 *>(qn + e) = q2;
-    const float hx = __double2float_rn(q2.x), hy = __double2float_rn(q2.y);
+    float hx, hy, lx, ly;
+    split_d(q2.x, hx, lx);
+    split_d(q2.y, hy, ly);
     dq = fmaf(c.d2f[e] * hx, hx, fmaf(c.d2f[e + 1] * hy, hy, dq));
     *reinterpret_cast<float2 *>(hn + e) = make_float2(hx, hy);
-    if (ln != nullptr)
-      *reinterpret_cast<float2 *>(ln + e) = make_float2(__double2float_rn(q2.x - (double)hx),
-                                                        __double2float_rn(q2.y - (double)hy));
+    if (ln != nullptr) *reinterpret_cast<float2 *>(ln + e) = make_float2(lx, ly);
     if (c.xh != nullptr) {
       __nv_bfloat162 x2;
       x2.x = __float2bfloat16_rn(c.dsqf[e] * hx);
@@ -437,12 +435,12 @@ __global__ void __launch_bounds__(VEC_THREADS) k_start_split(VecCtx c) {
       q2.y *= inv;
     }
     *reinterpret_cast<double2 *>(qn + e) = q2;
-    const float hx = __double2float_rn(q2.x), hy = __double2float_rn(q2.y);
+    float hx, hy, lx, ly;
+    split_d(q2.x, hx, lx);
+    split_d(q2.y, hy, ly);
     dq = fmaf(c.d2f[e] * hx, hx, fmaf(c.d2f[e + 1] * hy, hy, dq));
     *reinterpret_cast<float2 *>(hn + e) = make_float2(hx, hy);
-    if (ln != nullptr)
-      *reinterpret_cast<float2 *>(ln + e) = make_float2(__double2float_rn(q2.x - (double)hx),
-                                                        __double2float_rn(q2.y - (double)hy));
+    if (ln != nullptr) *reinterpret_cast<float2 *>(ln + e) = make_float2(lx, ly);
     if (c.xh != nullptr) {
       __nv_bfloat162 x2;
       x2.x = __float2bfloat16_rn(c.dsqf[e] * hx);
@@ -497,6 +495,12 @@ __global__ void __launch_bounds__(VEC_THREADS) k_start_split(VecCtx c) {
 // takes Q_{j-1}^T w_j = d - g (Q orthonormal).  Bytes per element and step:
 // 8 per stored row (hi + lo) + 30, against 12 per row + 54 for the two
 // passes of k_dots_split and k_update_split.
+//
+// The FP64 pipe is what the short early launches wait for (2 lanes per SM
+// clock): of 28 operations per element before and after the row loop, 17 were
+// conversions between FP64 and the float pairs.  They run on the integer pipe
+// (fp_bits.cuh), bit for bit the same: 54.5 -> 49.7 us per launch at N_vc 4511,
+// 100 vectors, 442 -> 410 us at 32768, 128 vectors, k 120.
 //
 // Thread layout: one block per (2048-element chunk, vector); each thread
 // owns elements e = chunk*2048 + warp*256 + 4*lane + 128*u + {0..3},
@@ -851,7 +855,7 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_sweep_dcgs(VecCtx c, int j) 
       for (int t = 0; t < 4; ++t) {
         qt[t] = wq[t] * sinv;
         // C q~ = Delta^2 q~ + c_K Delta^1/2 L L^T Delta^1/2 q~   (Eq. 4)
-        uu[t] = fma(dd[t], qt[t], (double)ku[t]);
+        uu[t] = fma(dd[t], qt[t], f2d(ku[t]));
       }
     }
     double qp[4] = {0.0, 0.0, 0.0, 0.0};
@@ -859,17 +863,16 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_sweep_dcgs(VecCtx c, int j) 
       const float4 ph = *reinterpret_cast<const float4 *>(bhi_row(c, j - 1, b) + e);
       const float4 pl = LO ? *reinterpret_cast<const float4 *>(blo_row(c, j - 1, b) + e)
                            : make_float4(0.f, 0.f, 0.f, 0.f);
-      qp[0] = (double)ph.x + (double)pl.x;
-      qp[1] = (double)ph.y + (double)pl.y;
-      qp[2] = (double)ph.z + (double)pl.z;
-      qp[3] = (double)ph.w + (double)pl.w;
+      qp[0] = f2d(ph.x) + f2d(pl.x);
+      qp[1] = f2d(ph.y) + f2d(pl.y);
+      qp[2] = f2d(ph.z) + f2d(pl.z);
+      qp[3] = f2d(ph.w) + f2d(pl.w);
     }
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       const int m = 4 * u + t;
       const double vd = fma(-bj, qp[t], fma(-alpha, qt[t], uu[t]));
-      vh[m] = __double2float_rn(vd);
-      vl[m] = __double2float_rn(vd - (double)vh[m]);
+      split_d(vd, vh[m], vl[m]);
     }
   }
 
@@ -910,11 +913,10 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_sweep_dcgs(VecCtx c, int j) 
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       const int m = 4 * u + t;
-      vd[t] = ((double)vh[m] + (double)vl[m]) - (double)cv[m];   // w_j = v - Q_{j-1} g
-      vh[m] = __double2float_rn(vd[t]);
-      const double qj = wq[t] * sinv - (double)corr[m];
-      qh4[t] = __double2float_rn(qj);
-      ql4[t] = __double2float_rn(qj - (double)qh4[t]);
+      vd[t] = (f2d(vh[m]) + f2d(vl[m])) - f2d(cv[m]);   // w_j = v - Q_{j-1} g
+      vh[m] = d2f(vd[t]);
+      const double qj = fma(wq[t], sinv, -f2d(corr[m]));
+      split_d(qj, qh4[t], ql4[t]);
       hj = fma(qj, vd[t], hj);
       nrm = fma(vd[t], vd[t], nrm);
     }
