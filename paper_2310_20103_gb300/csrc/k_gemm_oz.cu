@@ -38,6 +38,7 @@
 #include <algorithm>
 #include <cstdio>
 
+#include "oz_digits.cuh"
 #include "tc_ptx.cuh"
 
 namespace lgw {
@@ -45,7 +46,6 @@ namespace oz {
 
 using namespace tc;
 
-constexpr int S = OZ_SLICES;
 constexpr int BM = 128;
 constexpr int KB = 64;          // K elements per block: one 128-byte swizzle row
 constexpr int CHUNK_KB = 16;    // 1024 terms per exact sum
@@ -352,34 +352,6 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 // ---------------------------------------------------------------------------
 // Digits of an operand
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
-
-// x on the grid 2^(f - 1022 - 55) of a row whose largest exponent field is f,
-// biased so that the base-128 digits come out as 64 + d_s.
-__device__ __forceinline__ unsigned long long fixed56(double x, int f) {
-  constexpr unsigned long long bias =
-      64ULL * ((1ULL << 49) + (1ULL << 42) + (1ULL << 35) + (1ULL << 28) + (1ULL << 21) +
-               (1ULL << 14) + (1ULL << 7) + 1ULL);
-  const long long b = __double_as_longlong(x);
-  const int ex = (int)((b >> 52) & 0x7ff);
-  long long m = b & 0xfffffffffffffLL;
-  if (ex != 0) m |= 1LL << 52;
-  const int sh = max(ex, 1) - f + 2;   // at most 2: |x| < 2^(f - 1022)
-  long long v = 0;
-  if (sh >= 0)
-    v = m << sh;
-  else if (sh > -56)
-    v = (m + (1LL << (-sh - 1))) >> -sh;
-  if (b < 0) v = -v;
-  return (unsigned long long)v + bias;
-}
-// BF16 bits of 2^(-7s) times digit s (an integer in [-64, 64]) of the biased
-// fixed point
-__device__ __forceinline__ uint32_t digit_bf16(unsigned long long u, int s) {
-  const uint32_t t = s == 0 ? (uint32_t)(u >> 49) : (uint32_t)(u >> (49 - 7 * s)) & 127u;
-  const float w = __uint_as_float((uint32_t)(127 - 7 * s) << 23);   // 2^(-7s)
-  return __float_as_uint((__uint_as_float(0x4B000000u | t) - 8388672.0f) * w) >> 16;
-}
 // 16 consecutive K elements of one operand row into its eight digit planes
 __device__ __forceinline__ void store_digits16(const unsigned long long (&u)[16], uint16_t *dst,
                                                size_t plane) {
@@ -625,9 +597,8 @@ bool launch_oz_gemm(const OzOperand &A, const OzOperand &B, int M, int Ncols, in
 void launch_oz_slice(const double *x, size_t ld, int nr, int nc, const double *scale, bool cols,
                      const OzOperand &o, cudaStream_t st) {
   const oz::Src src{x, scale, ld, nr, nc};
-  // short rows: one kernel, a block per row (4 us at 160 rows of 256); longer
-  // ones spread each row over many blocks (64 rows of 32768: 32 us in two
-  // kernels, where a block per row would take about 60)
+  // short rows: one kernel, a block per row (4.7 us at 160 rows of 256); longer
+  // ones spread each row over many blocks (64 rows of 32768: 12 + 20 us)
   if (!cols && o.nkb * 64 <= 4096) {
     oz::launch_rows(x, 1, 0, src, nullptr, o, st);
     return;

@@ -643,10 +643,19 @@ void oz_gemm(lgw_handle *h, const OzOperand &A, const OzOperand &B, int M, int N
   check_launch(h, what);
 }
 
+// Digits of the next step's vectors, for a producer of all of them at once.
+OzOperand f64_next_digits(const SysDev &s, const F64Work &f, int Bs) {
+  OzOperand x = f.x;
+  if (!s.ozT.d || Bs > F64_ROWS) return OzOperand{};
+  x.rows = Bs;
+  return x;
+}
+
 // Y [rows][A] = (Delta^1/2 q) L; with digits, those of Y too (of the last
-// F64_ROWS rows) for f64_contract2.
+// F64_ROWS rows) for f64_contract2.  ready: the digits of Delta^1/2 q are in
+// place (f64_next_digits).
 void f64_contract1(lgw_handle *h, const SysDev &s, const F64Work &f, const double *q, int rows,
-                   double *Y) {
+                   double *Y, bool ready = false) {
   cudaStream_t st = h->stream;
   if (!f.x.d || !s.ozT.d) {
     const int splits = gemm1_f64_splits(s, rows);
@@ -660,8 +669,10 @@ void f64_contract1(lgw_handle *h, const SysDev &s, const F64Work &f, const doubl
     const int nr = std::min(F64_ROWS, rows - r0);
     OzOperand x = f.x, y = f.y;
     x.rows = y.rows = nr;
-    launch_oz_slice(q + (size_t)r0 * s.N, (size_t)s.N, nr, s.N, s.dsq, false, x, st);
-    check_launch(h, "oz_slice(x)");
+    if (!ready) {
+      launch_oz_slice(q + (size_t)r0 * s.N, (size_t)s.N, nr, s.N, s.dsq, false, x, st);
+      check_launch(h, "oz_slice(x)");
+    }
     const int splits = oz_splits(s.A, nr, s.N / 64);
     OzOut o;
     o.mode = OZ_PART;
@@ -1040,6 +1051,7 @@ void run_lanczos(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts 
         launch_normalize(c, 0, 1, nullptr, st);
       check_launch(h, "normalize(start)");
       if (after_step) (*after_step)(c, -1);
+      bool x_ready = false;   // the digits of Delta^1/2 q_j are in place
 
       for (int j = 0; j < k; ++j) {
         const double *qj = slot_ptr(c, j);
@@ -1128,7 +1140,7 @@ void run_lanczos(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts 
           f64_contract2(h, s, f64, Y64, true, Bs, EPI_APPLY, c.wv, nullptr, nullptr, c.w,
                         c.alpha_part);
         } else {
-          f64_contract1(h, s, f64, qj, Bs, Y64);
+          f64_contract1(h, s, f64, qj, Bs, Y64, x_ready);
           tm.mark(C_GEMM2);
           f64_contract2(h, s, f64, Y64, true, Bs, EPI_LANCZOS, qj, qp, c.betaj, c.w,
                         c.alpha_part);
@@ -1165,6 +1177,15 @@ void run_lanczos(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts 
           launch_update_split(c, j, 2, st);
           check_launch(h, "update_split2");
           continue;
+        }
+        if (!tc) {
+          const OzOperand xd = poly || j + 1 == k ? OzOperand{} : f64_next_digits(s, f64, Bs);
+          if (launch_step_f64(c, j, xd, st)) {
+            check_launch(h, "step_f64");
+            x_ready = xd.d != nullptr;
+            if (after_step) (*after_step)(c, j);
+            continue;
+          }
         }
         launch_alpha_reduce(c, j, st);
         check_launch(h, "alpha_reduce");
@@ -1793,6 +1814,7 @@ void reverse_sweep(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opt
     r.s0 = s0;
     launch_rev_set_betaj(r, rc.betaj, st);
     check_launch(h, "rev_set_betaj");
+    bool x_ready = false;
     for (int j = s0; j < e; ++j) {
       const double *qj = slot_ptr(rc, j);
       const double *qp = j > 0 ? slot_ptr(rc, j - 1) : nullptr;
@@ -1800,8 +1822,14 @@ void reverse_sweep(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opt
         clenshaw(qj, qp, rc.betaj, rc.w, rc.alpha_part);
       } else {
         double *yj = yseg + (size_t)(j - s0) * BA;
-        f64_contract1(h, s, f64, qj, Bs, yj);
+        f64_contract1(h, s, f64, qj, Bs, yj, x_ready);
         f64_contract2(h, s, f64, yj, true, Bs, EPI_LANCZOS, qj, qp, rc.betaj, rc.w, rc.alpha_part);
+      }
+      const OzOperand xd = poly || j + 1 == e ? OzOperand{} : f64_next_digits(s, f64, Bs);
+      if (launch_step_f64(rc, j, xd, st)) {
+        check_launch(h, "step_f64(recompute)");
+        x_ready = xd.d != nullptr;
+        continue;
       }
       launch_alpha_reduce(rc, j, st);
       check_launch(h, "alpha_reduce(recompute)");

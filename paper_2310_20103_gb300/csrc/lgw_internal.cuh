@@ -374,6 +374,12 @@ void launch_band_small(const double *Tb, const double *R0, const int *keff, int 
 // x = a, pair (a, b) from (x+ - x-) / 4
 void launch_band_combine(const double *sig, int p, int F, double *out, cudaStream_t st);
 
+// k_step_f64.cu : alpha, axpy, Gram-Schmidt, beta and q_{j+1} of one FP64 step
+// in one kernel, one cluster per vector; with x.d also the digits of
+// Delta^1/2 q_{j+1}.  False (nothing launched) beyond its limits.
+constexpr int STEP_MAX_K1 = 4096;     // k + 1: three rows of coefficients in shared memory
+bool launch_step_f64(const VecCtx &c, int j, const OzOperand &x, cudaStream_t st);
+
 // k_reorth.cu : split-precision basis (double-float dots, FP32 small updates)
 void launch_dots_split(const VecCtx &c, int j, int pass, cudaStream_t st);
 void launch_reduce_dots_split(const VecCtx &c, int j, int pass, cudaStream_t st);
