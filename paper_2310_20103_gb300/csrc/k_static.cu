@@ -34,97 +34,135 @@ __global__ void k_sigma_x(const double *__restrict__ M, int n_m, int n_aux,
 // --------------------------------------------------------------------------
 constexpr int NB = 64;
 
-// factor the diagonal block at (j0, j0); one CTA of NB threads, row i per thread
-__global__ void __launch_bounds__(NB) k_potrf_diag(double *A, int n, int j0, unsigned *status) {
-  __shared__ double blk[NB][NB + 1];
-  const int i = threadIdx.x;
-  const int nb = min(NB, n - j0);
-  for (int c = 0; c < nb; ++c) blk[i][c] = (i < nb) ? A[(size_t)(j0 + i) * n + j0 + c] : 0.0;
-  __syncthreads();
-  for (int j = 0; j < nb; ++j) {
-    if (i == j) {
-      double d = blk[j][j];
-      for (int p = 0; p < j; ++p) d = fma(-blk[j][p], blk[j][p], d);
-      if (!(d > 0.0)) {
-        atomicOr(status, ST_NOT_SPD);
-        d = 1.0;
-      }
-      blk[j][j] = sqrt(d);
-    }
-    __syncthreads();
-    if (i > j && i < nb) {
-      double x = blk[i][j];
-      for (int p = 0; p < j; ++p) x = fma(-blk[i][p], blk[j][p], x);
-      blk[i][j] = x / blk[j][j];
-    }
-    __syncthreads();
-  }
-  if (i < nb)
-    for (int c = 0; c <= i; ++c) A[(size_t)(j0 + i) * n + j0 + c] = blk[i][c];
+// sqrt(d) and x / s to the last place or so from r ~ 1 / s: one Newton
+// correction each, instead of a square root and a division (a serial chain of
+// tens of FP64 operations) per column.
+__device__ __forceinline__ double sqrt_from(double d, double r) {
+  const double s = d * r;
+  return fma(fma(-s, s, d), 0.5 * r, s);
+}
+__device__ __forceinline__ double div_from(double x, double s, double r) {
+  const double q = x * r;
+  return fma(fma(-q, s, x), r, q);
 }
 
-// rows below the diagonal block: L_i = A_i L_jj^{-T} (forward substitution,
-// one row per thread)
-__global__ void k_trsm_panel(double *A, int n, int j0) {
-  __shared__ double Ljj[NB][NB + 1];
+// Factor the diagonal block at (j0, j0): one CTA, right-looking by columns,
+// the trailing columns dealt out to 128 threads (row i, columns 2 t, 2 t + 1
+// ...).  A serial chain of 64 columns: 216 us per block with one thread per
+// row and square root, division and row sums in sequence; 109 us now.
+constexpr int POTRF_THREADS = 128;
+
+__global__ void __launch_bounds__(POTRF_THREADS) k_potrf_diag(double *A, int n, int j0,
+                                                              unsigned *status) {
+  __shared__ double blk[NB][NB + 1];
+  const int t = threadIdx.x, i = t & (NB - 1), half = t / NB;
   const int nb = min(NB, n - j0);
-  for (int idx = threadIdx.x; idx < NB * NB; idx += blockDim.x) {
+  for (int idx = t; idx < NB * NB; idx += POTRF_THREADS) {
     const int r = idx / NB, c = idx % NB;
-    Ljj[r][c] = (r < nb && c <= r) ? A[(size_t)(j0 + r) * n + j0 + c] : 0.0;
+    blk[r][c] = r < nb && c <= r ? A[(size_t)(j0 + r) * n + j0 + c] : 0.0;
   }
   __syncthreads();
-  const int i = j0 + nb + blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  double *row = A + (size_t)i * n + j0;
-  for (int c = 0; c < nb; ++c) {
-    double v = row[c];
-    for (int p = 0; p < c; ++p) v = fma(-row[p], Ljj[c][p], v);
-    row[c] = v / Ljj[c][c];
+  for (int j = 0; j < nb; ++j) {
+    double d = blk[j][j];
+    if (!(d > 0.0)) {
+      if (t == 0) atomicOr(status, ST_NOT_SPD);
+      d = 1.0;
+    }
+    const bool plain = !(d > 1e-280 && d < 1e280);   // and infinities
+    const double r = rsqrt(d), s = plain ? sqrt(d) : sqrt_from(d, r);
+    const double x = i > j ? (plain ? blk[i][j] / s : div_from(blk[i][j], s, r)) : 0.0;
+    __syncthreads();   // every thread has read column j
+    if (half == 0 && i >= j) blk[i][j] = i == j ? s : x;
+    __syncthreads();
+    // row i, the columns c of this thread's parity
+    if (i > j)
+      for (int c = j + 1 + ((j + 1 + half) & 1); c <= i; c += 2)
+        blk[i][c] = fma(-x, blk[c][j], blk[i][c]);
+    __syncthreads();
   }
+  for (int idx = t; idx < NB * NB; idx += POTRF_THREADS) {
+    const int r = idx / NB, c = idx % NB;
+    if (r < nb && c <= r) A[(size_t)(j0 + r) * n + j0 + c] = blk[r][c];
+  }
+}
+
+// rows below the diagonal block: L_i = A_i L_jj^{-T} by forward substitution,
+// eight threads per row (thread l holds columns l, l + 8, ...), the row in
+// registers.  212 us per panel with a row per thread in global memory; 34 us now.
+constexpr int TRSM_ROWS = 16;
+
+__global__ void __launch_bounds__(8 * TRSM_ROWS) k_trsm_panel(double *A, int n, int j0) {
+  __shared__ double Ljj[NB][NB + 1];
+  __shared__ double rd[NB];
+  const int t = threadIdx.x, l = t & 7;
+  const int nb = min(NB, n - j0);   // a panel exists only below a full block
+  for (int idx = t; idx < NB * NB; idx += 8 * TRSM_ROWS) {
+    const int r = idx / NB, c = idx % NB;
+    Ljj[r][c] = (r < nb && c <= r) ? A[(size_t)(j0 + r) * n + j0 + c] : (r == c ? 1.0 : 0.0);
+  }
+  __syncthreads();
+  if (t < NB) rd[t] = 1.0 / Ljj[t][t];
+  __syncthreads();
+  const int i = j0 + nb + blockIdx.x * TRSM_ROWS + (t >> 3);
+  const bool ok = i < n;
+  double *row = A + (size_t)(ok ? i : 0) * n + j0;
+  double x[NB / 8];
+#pragma unroll
+  for (int k = 0; k < NB / 8; ++k) x[k] = ok && 8 * k + l < nb ? row[8 * k + l] : 0.0;
+#pragma unroll
+  for (int kb = 0; kb < NB / 8; ++kb) {
+#pragma unroll
+    for (int cc = 0; cc < 8; ++cc) {
+      const int c = 8 * kb + cc;
+      // a reciprocal outside the normal range (or of an infinity): divide
+      const bool plain = !(fabs(rd[c]) > 1e-150 && fabs(rd[c]) < 1e150);
+      const double q = plain ? x[kb] / Ljj[c][c] : div_from(x[kb], Ljj[c][c], rd[c]);
+      const double v = __shfl_sync(0xffffffffu, q, cc, 8);
+      if (l == cc) x[kb] = v;
+      if (l > cc) x[kb] = fma(-v, Ljj[8 * kb + l][c], x[kb]);
+#pragma unroll
+      for (int k = kb + 1; k < NB / 8; ++k) x[k] = fma(-v, Ljj[8 * k + l][c], x[k]);
+    }
+  }
+  if (!ok) return;
+#pragma unroll
+  for (int k = 0; k < NB / 8; ++k)
+    if (8 * k + l < nb) row[8 * k + l] = x[k];
 }
 
 // trailing update A[i][j] -= sum_p L[i][j0+p] L[j][j0+p] for i, j >= j0+nb,
-// lower triangle (64 x 64 output tiles, 4 x 4 per thread, the panel in
-// 16-column slices)
+// lower triangle.  32 x 32 output tiles, 2 x 2 per thread: FP64-bound, and
+// 64 x 64 tiles left most of the chip without one (86 us per update on average
+// at n 1024; 46 us now).
 __global__ void __launch_bounds__(256) k_syrk_update(double *A, int n, int j0, int nb) {
   const int t0 = j0 + nb;
   const int bi = blockIdx.y, bj = blockIdx.x;
   if (bj > bi) return;
-  __shared__ double Xs[16][65];
-  __shared__ double Ys[16][65];
-  const int i0 = t0 + bi * 64, jj0 = t0 + bj * 64;
+  __shared__ double Xs[NB][33];
+  __shared__ double Ys[NB][33];
+  const int i0 = t0 + bi * 32, jj0 = t0 + bj * 32;
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  double acc[4][4] = {};
-  for (int p0 = 0; p0 < nb; p0 += 16) {
-#pragma unroll
-    for (int rep = 0; rep < 4; ++rep) {
-      const int idx = t + 256 * rep;
-      const int p = idx & 15, r = idx >> 4;
-      const bool pk = p0 + p < nb;
-      Xs[p][r] = (i0 + r < n && pk) ? A[(size_t)(i0 + r) * n + j0 + p0 + p] : 0.0;
-      Ys[p][r] = (jj0 + r < n && pk) ? A[(size_t)(jj0 + r) * n + j0 + p0 + p] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int p = 0; p < 16; ++p) {
-      double xa[4], yb[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) xa[q] = Xs[p][ty + 16 * q];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) yb[q] = Ys[p][tx + 16 * q];
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int w = 0; w < 4; ++w) acc[q][w] = fma(xa[q], yb[w], acc[q][w]);
-    }
-    __syncthreads();
+  for (int idx = t; idx < 32 * NB; idx += 256) {
+    const int p = idx & (NB - 1), r = idx / NB;
+    Xs[p][r] = (i0 + r < n && p < nb) ? A[(size_t)(i0 + r) * n + j0 + p] : 0.0;
+    Ys[p][r] = (jj0 + r < n && p < nb) ? A[(size_t)(jj0 + r) * n + j0 + p] : 0.0;
+  }
+  __syncthreads();
+  double acc[2][2] = {};
+#pragma unroll 8
+  for (int p = 0; p < NB; ++p) {
+    const double x0 = Xs[p][ty], x1 = Xs[p][ty + 16], y0 = Ys[p][tx], y1 = Ys[p][tx + 16];
+    acc[0][0] = fma(x0, y0, acc[0][0]);
+    acc[0][1] = fma(x0, y1, acc[0][1]);
+    acc[1][0] = fma(x1, y0, acc[1][0]);
+    acc[1][1] = fma(x1, y1, acc[1][1]);
   }
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
+  for (int q = 0; q < 2; ++q) {
     const int i = i0 + ty + 16 * q;
     if (i >= n) continue;
 #pragma unroll
-    for (int w = 0; w < 4; ++w) {
+    for (int w = 0; w < 2; ++w) {
       const int j = jj0 + tx + 16 * w;
       if (j < n && j <= i) A[(size_t)i * n + j] -= acc[q][w];
     }
@@ -193,12 +231,12 @@ int launch_cholesky(double *A, int n, unsigned *status, cudaStream_t st) {
   int launches = 0;
   for (int j0 = 0; j0 < n; j0 += NB) {
     const int nb = std::min(NB, n - j0);
-    k_potrf_diag<<<1, NB, 0, st>>>(A, n, j0, status);
+    k_potrf_diag<<<1, POTRF_THREADS, 0, st>>>(A, n, j0, status);
     ++launches;
     const int rest = n - j0 - nb;
     if (rest > 0) {
-      k_trsm_panel<<<(rest + 127) / 128, 128, 0, st>>>(A, n, j0);
-      const int tiles = (rest + 63) / 64;
+      k_trsm_panel<<<(rest + TRSM_ROWS - 1) / TRSM_ROWS, 8 * TRSM_ROWS, 0, st>>>(A, n, j0);
+      const int tiles = (rest + 31) / 32;
       k_syrk_update<<<dim3(tiles, tiles), 256, 0, st>>>(A, n, j0, nb);
       launches += 2;
     }
