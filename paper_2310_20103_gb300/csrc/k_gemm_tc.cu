@@ -855,6 +855,12 @@ TcPlan *tc_plan_create(const SysDev &s, int Bs, const __nv_bfloat16 *xh, float *
   p->splits = choose_splits(tiles1, num_kb, nsm);
   p->kb_per_split = (num_kb + p->splits - 1) / p->splits;
   p->splits = (num_kb + p->kb_per_split - 1) / p->kb_per_split;
+  // GEMM2 runs persistent (its epilogue behind the next tile's MMAs) where the
+  // tiles make more than one round of the SMs: 123 against 176 us at N_vc
+  // 131072, N_aux 2048, 256 vectors, 623 against 1038 us in E4M3 at 400000,
+  // 4096, 512.  Below that a CTA has one tile and nothing to overlap
+  const int tiles2 = (s.N / tc::BM) * ((Bs + p->BN2 - 1) / p->BN2);
+  p->half2 = tiles2 > nsm ? 2 : 0;
   p->ypart = ypart;
   p->yh = yh;
   p->Delta2 = s.Delta2;
