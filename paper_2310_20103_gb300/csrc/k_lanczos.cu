@@ -85,43 +85,89 @@ __device__ __forceinline__ float *pair_lo(double *slot, const VecCtx &c) {
   return reinterpret_cast<float *>(slot) + (size_t)c.Bs * c.N;
 }
 
+// Four basis rows from row r0 on (the last one again past the end), all loads
+// before any use: one row at a time, a row costs a memory round trip per warp
+// and the FP64 pipe waits (band Lanczos, 64 groups of 32768: dots 172 -> 134,
+// update 126 -> 111 per pass of 26 rows on average).
+__device__ __forceinline__ void load_rows4(const VecCtx &c, int r0, int nrows, size_t voff, int e0,
+                                           double2 (&q)[4][4]) {
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const double *row = slot_ptr(c, min(r0 + r, nrows - 1)) + voff;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = e0 + u * 64;
+      q[r][u] = e < c.N ? *reinterpret_cast<const double2 *>(row + e) : make_double2(0.0, 0.0);
+    }
+  }
+}
+
 // Partial dot products of the thread's eight elements of w with basis rows
 // 0..nrows-1 of vector b; one partial per (row, chunk) after a warp
-// transposed reduction and a fixed-order sum over the eight warps.
+// transposed reduction of 16 rows and a fixed-order sum over the eight warps.
 __device__ void dots_rows(const VecCtx &c, int nrows, int b, int chunk, const double (&wr)[8],
-                          double (*sred)[32]) {
+                          double (*sred)[16]) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int e0 = elem_base(chunk);
   const size_t voff = (size_t)b * c.N;
-  for (int r0 = 0; r0 < nrows; r0 += 32) {
-    double acc[32];
+  for (int r0 = 0; r0 < nrows; r0 += 16) {
+    double acc[16];
 #pragma unroll
-    for (int r = 0; r < 32; ++r) {
-      acc[r] = 0.0;
-      if (r0 + r < nrows) {
-        const double *qrow = slot_ptr(c, r0 + r) + voff;
+    for (int r = 0; r < 16; ++r) acc[r] = 0.0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int e = e0 + u * 64;
-          if (e < c.N) {
-            const double2 q2 = *reinterpret_cast<const double2 *>(qrow + e);
-            acc[r] = fma(q2.x, wr[2 * u], acc[r]);
-            acc[r] = fma(q2.y, wr[2 * u + 1], acc[r]);
+    for (int rb = 0; rb < 16; rb += 4) {
+      if (r0 + rb < nrows) {
+        double2 q[4][4];
+        load_rows4(c, r0 + rb, nrows, voff, e0, q);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            acc[rb + r] = fma(q[r][u].x, wr[2 * u], acc[rb + r]);
+            acc[rb + r] = fma(q[r][u].y, wr[2 * u + 1], acc[rb + r]);
           }
-        }
       }
     }
-    warp_transpose_sum32(acc);
-    sred[wid][lane] = acc[0];
+    // transposed butterfly: lane l ends with row l % 16, then the two halves
+#pragma unroll
+    for (int off = 8; off >= 1; off >>= 1) {
+      const bool up = (lane & off) != 0;
+#pragma unroll
+      for (int i = 0; i < off; ++i) {
+        const double send = up ? acc[i] : acc[i + off];
+        const double keep = up ? acc[i + off] : acc[i];
+        acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+      }
+    }
+    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 16);
+    if (lane < 16) sred[wid][lane] = acc[0];
     __syncthreads();
-    if (wid == 0) {
+    if (threadIdx.x < 16 && r0 + (int)threadIdx.x < nrows) {
       double s = 0.0;
 #pragma unroll
-      for (int w8 = 0; w8 < VEC_THREADS / 32; ++w8) s += sred[w8][lane];
-      if (r0 + lane < nrows)
-        c.dot_part[((size_t)b * c.nchunks + chunk) * c.kmax1 + r0 + lane] = s;
+      for (int w8 = 0; w8 < VEC_THREADS / 32; ++w8) s += sred[w8][threadIdx.x];
+      c.dot_part[((size_t)b * c.nchunks + chunk) * c.kmax1 + r0 + threadIdx.x] = s;
     }
     __syncthreads();
+  }
+}
+
+// w <- w - sum_i h_i q_i over rows 0..nrows-1 (coefficients in shared memory).
+__device__ __forceinline__ void update_rows(const VecCtx &c, int nrows, size_t voff, int e0,
+                                            const double *hs, double2 (&wv)[4]) {
+  for (int i = 0; i < nrows; i += 4) {
+    double2 q[4][4];
+    load_rows4(c, i, nrows, voff, e0, q);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      if (i + r >= nrows) break;
+      const double hi = hs[i + r];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        wv[u].x = fma(-hi, q[r][u].x, wv[u].x);
+        wv[u].y = fma(-hi, q[r][u].y, wv[u].y);
+      }
+    }
   }
 }
 
@@ -238,7 +284,7 @@ __global__ void k_alpha_reduce(VecCtx c, int j) {
 template <bool DOTS>
 __device__ __forceinline__ void alpha_axpy_chunk(const VecCtx &c, int j, int chunk, int b) {
   __shared__ double red[VEC_THREADS / 32];
-  __shared__ double sred[DOTS ? VEC_THREADS / 32 : 1][32];
+  __shared__ double sred[DOTS ? VEC_THREADS / 32 : 1][16];
   if (!vec_live(c, b, j)) return;
   const double alpha = c.alpha[(size_t)(c.vec0 + b) * c.k + j];
   const size_t voff = (size_t)b * c.N;
@@ -302,7 +348,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_alpha_axpy(VecCtx c, int j) {
 
 // Second-pass dot products of the current w with rows 0..j.
 __global__ void __launch_bounds__(VEC_THREADS) k_dots(VecCtx c, int j) {
-  __shared__ double sred[VEC_THREADS / 32][32];
+  __shared__ double sred[VEC_THREADS / 32][16];
   const int chunk = blockIdx.x, b = blockIdx.y;
   if (!vec_live(c, b, j) || !c.flag2[b]) return;
   const double *w = c.w + (size_t)b * c.N;
@@ -350,19 +396,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_update(VecCtx c, int j, int pas
     const int e = e0 + u * 64;
     wv[u] = (e < c.N) ? *reinterpret_cast<const double2 *>(w + e) : make_double2(0.0, 0.0);
   }
-  for (int i = 0; i <= j; ++i) {
-    const double hi = hs[i];
-    const double *qrow = slot_ptr(c, i) + voff;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int e = e0 + u * 64;
-      if (e < c.N) {
-        const double2 q2 = *reinterpret_cast<const double2 *>(qrow + e);
-        wv[u].x = fma(-hi, q2.x, wv[u].x);
-        wv[u].y = fma(-hi, q2.y, wv[u].y);
-      }
-    }
-  }
+  update_rows(c, j + 1, voff, e0, hs, wv);
   double nrm = 0.0;
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
@@ -693,7 +727,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_band_assemble(BandCtx bc, int j
 // Dots of w with the group's basis vectors; pass 1 also ||w||^2 (norm_a).
 __global__ void __launch_bounds__(VEC_THREADS) k_band_dots(BandCtx bc, int pass) {
   __shared__ double red[VEC_THREADS / 32];
-  __shared__ double sred[VEC_THREADS / 32][32];
+  __shared__ double sred[VEC_THREADS / 32][16];
   const VecCtx &c = bc.c;
   const int chunk = blockIdx.x, b = blockIdx.y;
   if (!band_act(bc, b)) return;
@@ -753,19 +787,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_band_update(BandCtx bc, int pas
     const int e = e0 + u * 64;
     wv[u] = (e < c.N) ? *reinterpret_cast<const double2 *>(w + e) : make_double2(0.0, 0.0);
   }
-  for (int i = 0; i < n; ++i) {
-    const double hi = hs[i];
-    const double *qrow = slot_ptr(c, i) + voff;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int e = e0 + u * 64;
-      if (e < c.N) {
-        const double2 q2 = *reinterpret_cast<const double2 *>(qrow + e);
-        wv[u].x = fma(-hi, q2.x, wv[u].x);
-        wv[u].y = fma(-hi, q2.y, wv[u].y);
-      }
-    }
-  }
+  update_rows(c, n, voff, e0, hs, wv);
   double nrm = 0.0;
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
