@@ -25,40 +25,66 @@ namespace lgw {
 
 // --------------------------------------------------------------------------
 // Full eigen-decomposition of each T_k: implicit symmetric QR with Wilkinson
-// shifts (Golub & Van Loan, symmetric QR algorithm).  Lane 0 runs the scalar
-// chain and stages each sweep's rotations in shared memory; all 32 lanes then
-// rotate the rows of V = U^T (row s = eigenvector s, coalesced).  One warp
-// per vector.
+// shifts (the recurrences of Martin and Wilkinson's imtql2, Numer. Math. 12
+// (1968) 377, chasing downwards).  One block per vector: lane 0 of warp 0 runs
+// the scalar chain of a sweep and leaves its rotations in shared memory; the
+// other warps apply the previous sweep's to the rows of V = U^T (row s =
+// eigenvector s, coalesced) meanwhile.
+//
+// What bounds it: the scalar chain, about 1.7 n sweeps of rotations in
+// sequence, each FP64 instruction of which holds its unit for 64 clocks
+// however few lanes it has.  A rotation takes 20 of them (one reciprocal
+// square root from the hardware's estimate) where hypot, two divisions and the
+// plain update took about 60, and the row updates no longer wait in between:
+// 128 vectors, k 120: 45.3 ms -> 13.9.
 // --------------------------------------------------------------------------
-constexpr int EIG_WARPS = 4;
+constexpr int EIG_THREADS = 128;
 
-__global__ void __launch_bounds__(EIG_WARPS * 32) k_eig_full(AdjCtx a) {
+// (c, s, r) with c g + s f = r, c f - s g = 0; 1 / sqrt(g^2 + f^2) by one
+// third-order Newton step, y (1 + e/2 + 3/8 e^2), e = 1 - h y^2, on a
+// 20-bit estimate.  Where the squares leave the normal range: hypot.
+__device__ __forceinline__ void eig_rotation(double g, double f, double &c, double &s, double &r) {
+  const double h = fma(g, g, f * f);
+  if (h > 1e-270 && h < 1e270) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(h));
+    const double e = fma(-h * y, y, 1.0);
+    y = fma(y * e, fma(e, 0.375, 0.5), y);
+    c = g * y;
+    s = f * y;
+    r = h * y;
+    return;
+  }
+  r = hypot(g, f);
+  c = r > 0.0 ? g / r : 1.0;
+  s = r > 0.0 ? f / r : 0.0;
+}
+
+__global__ void __launch_bounds__(EIG_THREADS) k_eig_full(AdjCtx a) {
   extern __shared__ double sm[];
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b = blockIdx.x * EIG_WARPS + wid;
-  if (b >= a.Bs) return;
-  const int k = a.k;
-  double *d = sm + (size_t)wid * 4 * k;
-  double *e = d + k;
-  double *cs = e + k;      // c, s pairs of one sweep: cs[2*i], cs[2*i+1]
-  __shared__ int ctl[EIG_WARPS][3];
+  __shared__ int ctl[2][3];   // by sweep parity: first row, rotations, 1 = no convergence
+  const int tid = threadIdx.x;
+  const int b = blockIdx.x, k = a.k;
+  double *d = sm, *e = d + k;
+  double2 *rot = reinterpret_cast<double2 *>(e + k);   // [2][k]
   double *V = a.V + (size_t)b * k * k;
   const int v = a.vec0 + b;
   const int n = (b < a.nvec) ? a.k_eff[v] : 0;
-  for (int i = lane; i < k * k; i += 32) V[i] = ((i / k) == (i % k) && (i / k) < n) ? 1.0 : 0.0;
-  if (lane == 0) {
-    for (int i = 0; i < k; ++i) {
-      d[i] = (i < n) ? a.alpha[(size_t)v * k + i] : 0.0;
-      e[i] = (i + 1 < n) ? a.beta[(size_t)v * k + i] : 0.0;
-    }
+  for (int i = tid; i < k * k; i += EIG_THREADS)
+    V[i] = ((i / k) == (i % k) && (i / k) < n) ? 1.0 : 0.0;
+  for (int i = tid; i < k; i += EIG_THREADS) {
+    d[i] = (i < n) ? a.alpha[(size_t)v * k + i] : 0.0;
+    e[i] = (i + 1 < n) ? a.beta[(size_t)v * k + i] : 0.0;
   }
-  __syncwarp();
+  if (tid < 2) ctl[tid][0] = -1, ctl[tid][1] = ctl[tid][2] = 0;
+  __syncthreads();
   const double eps = 2.220446049250313e-16;
-  int hi = n - 1, iter = 0;
+  int hi = n - 1, iter = 0;   // warp 0, lane 0
   const int max_iter = 60 * n + 60;
-  while (true) {
-    if (lane == 0) {
-      int lo = -1, ncs = 0;
+  for (int sweep = 0;; ++sweep) {
+    const int cur = sweep & 1, prev = cur ^ 1;
+    if (tid == 0) {
+      int lo = -1, nr = 0;
       while (hi > 0 && fabs(e[hi - 1]) <= eps * (fabs(d[hi - 1]) + fabs(d[hi]))) {
         e[hi - 1] = 0.0;
         --hi;
@@ -72,61 +98,55 @@ __global__ void __launch_bounds__(EIG_WARPS * 32) k_eig_full(AdjCtx a) {
         const double bb = e[hi - 1];
         const double den = dl + copysign(sqrt(fma(dl, dl, bb * bb)), dl != 0.0 ? dl : 1.0);
         const double mu = d[hi] - bb * bb / den;
-        double x = d[lo] - mu, z = e[lo];
-        for (int kk = lo; kk < hi; ++kk) {
-          // R = [[c, s], [-s, c]] maps (x, z) to (r, 0); T <- R T R^T on rows kk, kk+1
-          const double r = hypot(x, z);
-          double c = 1.0, s = 0.0;
-          if (r > 0.0) {
-            c = x / r;
-            s = z / r;
-          }
-          if (kk > lo) e[kk - 1] = r;
-          const double a0 = d[kk], b0 = e[kk], c0 = d[kk + 1];
-          const double csn = c * s, c2 = c * c, s2 = s * s;
-          d[kk] = c2 * a0 + 2.0 * csn * b0 + s2 * c0;
-          d[kk + 1] = s2 * a0 - 2.0 * csn * b0 + c2 * c0;
-          e[kk] = csn * (c0 - a0) + (c2 - s2) * b0;
-          if (kk + 1 < hi) {
-            const double bulge = s * e[kk + 1];
-            e[kk + 1] *= c;
-            x = e[kk];
-            z = bulge;
-          }
-          cs[2 * ncs] = c;
-          cs[2 * ncs + 1] = s;
-          ++ncs;
+        double g = d[lo] - mu, c = 1.0, s = 1.0, p = 0.0;
+        double dk = d[lo];
+        for (int i = lo; i < hi; ++i) {
+          const double ei = e[i], dn = d[i + 1];
+          const double f = s * ei, bq = c * ei;
+          double r;
+          eig_rotation(g, f, c, s, r);
+          if (i > lo) e[i - 1] = r;
+          g = dk - p;
+          const double cb = c * bq;
+          r = fma(dn - g, s, cb) + cb;
+          p = s * r;
+          d[i] = g + p;
+          g = fma(c, r, -bq);
+          dk = dn;
+          rot[cur * k + nr++] = make_double2(c, s);
         }
+        d[hi] = dk - p;
+        e[hi - 1] = g;
       }
-      ctl[wid][0] = lo;
-      ctl[wid][1] = ncs;
-      ctl[wid][2] = (hi > 0 && iter > max_iter) ? 1 : 0;
+      ctl[cur][0] = lo;
+      ctl[cur][1] = nr;
+      ctl[cur][2] = (hi > 0 && iter > max_iter) ? 1 : 0;
+    } else if (tid >= 32 && ctl[prev][0] >= 0) {
+      // V <- R V of the previous sweep: each thread carries its columns
+      // through the whole sweep in a register
+      const int lo = ctl[prev][0], nr = ctl[prev][1];
+      const double2 *cs = rot + prev * k;
+      for (int i = tid - 32; i < n; i += EIG_THREADS - 32) {
+        double x = V[(size_t)lo * k + i];
+#pragma unroll 4
+        for (int r = 0; r < nr; ++r) {
+          const double2 q = cs[r];
+          const double y = V[(size_t)(lo + r + 1) * k + i];
+          V[(size_t)(lo + r) * k + i] = fma(q.x, x, q.y * y);
+          x = fma(q.x, y, -q.y * x);
+        }
+        V[(size_t)(lo + nr) * k + i] = x;
+      }
     }
-    __syncwarp();
-    const int lo = ctl[wid][0], ncs = ctl[wid][1];
-    if (ctl[wid][2]) {
-      if (lane == 0) atomicOr(a.status, ST_NO_CONV);
+    __syncthreads();
+    if (ctl[cur][2]) {
+      if (tid == 0) atomicOr(a.status, ST_NO_CONV);
       break;
     }
-    if (lo < 0) break;
-    // U <- U R^T: the sweep's rotations act on consecutive row pairs of
-    // V = U^T.  Each lane carries its columns through the whole sweep in a
-    // register (one load and one store per rotation, no reload of a row that
-    // the previous rotation wrote).
-    for (int i = lane; i < n; i += 32) {
-      double x = V[(size_t)lo * k + i];
-      for (int r = 0; r < ncs; ++r) {
-        const double c = cs[2 * r], s = cs[2 * r + 1];
-        const double y = V[(size_t)(lo + r + 1) * k + i];
-        V[(size_t)(lo + r) * k + i] = c * x + s * y;
-        x = -s * x + c * y;
-      }
-      V[(size_t)(lo + ncs) * k + i] = x;
-    }
-    __syncwarp();
+    // the sweep that found nothing left ran beside the last one's row updates
+    if (ctl[cur][0] < 0) break;
   }
-  __syncwarp();
-  for (int i = lane; i < k; i += 32) a.theta[(size_t)b * k + i] = (i < n) ? d[i] : 0.0;
+  for (int i = tid; i < k; i += EIG_THREADS) a.theta[(size_t)b * k + i] = (i < n) ? d[i] : 0.0;
 }
 
 // --------------------------------------------------------------------------
@@ -285,9 +305,79 @@ __global__ void __launch_bounds__(ROW_THREADS) k_adj_rows(AdjCtx a, BasisRef bas
 }
 
 // FP32 variant of k_adj_rows (BF16 mode: the gradient there is good to
-// ~1e-4, so y and diag(Q Gam Q^T) run on the FP32 pipe).
-__global__ void __launch_bounds__(ROW_THREADS) k_adj_rows_f32(AdjCtx a, BasisRef basis,
-                                                              double *Y, double *Gd) {
+// ~1e-4, so y and diag(Q Gam Q^T) run on the FP32 pipe).  Block = 128 elements
+// of one vector, its basis entries (the hi floats: hi + lo rounds to hi) in
+// shared memory; each warp takes four rows j at a time for all 128 elements
+// (4 per lane), so a basis entry is read once for four products; then one
+// thread per element adds the rows up in order.  Every sum keeps the order of
+// the row-by-row form.  That form (one element per thread, two loads per
+// product) took 13.6 ms at 128 vectors of 32768, k 120; 8.6 in this one.
+constexpr int RF_ELEMS = 128, RF_WARPS = 8;
+
+__global__ void __launch_bounds__(32 * RF_WARPS) k_adj_rows_f32(AdjCtx a, BasisRef basis,
+                                                                double *Y, double *Gd) {
+  extern __shared__ float qsf[];               // [k][RF_ELEMS] q, then [k][RF_ELEMS] row terms
+  const int b = blockIdx.y, k = a.k;
+  float *sf = qsf + (size_t)k * RF_ELEMS;
+  const int i0 = blockIdx.x * RF_ELEMS;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const float *Gm = a.Gamf + (size_t)b * k * k;
+  for (int idx = threadIdx.x; idx < k * RF_ELEMS; idx += 32 * RF_WARPS) {
+    const int j = idx / RF_ELEMS, i = i0 + idx % RF_ELEMS;
+    const size_t o = ((size_t)j * a.Bs + b) * a.N + i;
+    qsf[idx] = i < a.N ? (basis.d ? (float)basis.d[o] : basis.hi[o]) : 0.0f;
+  }
+  __syncthreads();
+  for (int j0 = wid * 4; j0 < k; j0 += 4 * RF_WARPS) {
+    float t[4][4];   // [row][element]
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) t[r][u] = 0.0f;
+    const int nr = min(4, k - j0);
+    auto column = [&](int l, bool inside) {
+      float q[4], g[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) q[u] = qsf[l * RF_ELEMS + 32 * u + lane];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) g[r] = __ldg(Gm + (size_t)(j0 + min(r, nr - 1)) * k + l);
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        if (!inside || l > j0 + r)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) t[r][u] = fmaf(g[r], q[u], t[r][u]);
+    };
+    for (int l = j0 + 1; l < min(j0 + 4, k); ++l) column(l, true);
+#pragma unroll 2
+    for (int l = j0 + 4; l < k; ++l) column(l, false);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      if (r >= nr) break;
+      const float gj = __ldg(Gm + (size_t)(j0 + r) * k + j0 + r);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int o = (j0 + r) * RF_ELEMS + 32 * u + lane;
+        sf[o] = fmaf(gj, qsf[o], 2.0f * t[r][u]);
+      }
+    }
+  }
+  __syncthreads();
+  const int i = i0 + threadIdx.x;
+  if (threadIdx.x >= RF_ELEMS || i >= a.N) return;
+  const double *Ay = a.ay + (size_t)b * k;
+  float y = 0.0f, g = 0.0f;
+  for (int j = 0; j < k; ++j) {
+    const float q = qsf[j * RF_ELEMS + threadIdx.x];
+    y = fmaf((float)Ay[j], q, y);
+    g = fmaf(q, sf[j * RF_ELEMS + threadIdx.x], g);
+  }
+  Y[(size_t)b * a.N + i] = (double)y;
+  Gd[(size_t)b * a.N + i] = (double)g;
+}
+
+// The row-by-row form, for depths whose two tables exceed shared memory.
+__global__ void __launch_bounds__(ROW_THREADS) k_adj_rows_f32_deep(AdjCtx a, BasisRef basis,
+                                                                   double *Y, double *Gd) {
   extern __shared__ float qsf[];   // [k][ROW_THREADS]
   const int b = blockIdx.y;
   const int i = blockIdx.x * ROW_THREADS + threadIdx.x;
@@ -332,9 +422,9 @@ __global__ void k_split_t(BasisRef src, int R, int C, int lds,
     const int c = c0 + cc, r = r0 + tx;
     if (r < R && c < C) {
       const double x = tile[tx][cc];
-      const __nv_bfloat16 h = __double2bfloat16(x);
+      const __nv_bfloat16 h = d2bf16(x);
       if (hi) hi[(size_t)c * R + r] = h;
-      if (lo) lo[(size_t)c * R + r] = __double2bfloat16(x - (double)__bfloat162float(h));
+      if (lo) lo[(size_t)c * R + r] = d2bf16(x - f2d(__bfloat162float(h)));
     }
   }
 }
@@ -348,9 +438,9 @@ __global__ void k_split_scaled(BasisRef src, int R, int C,
        idx += (size_t)gridDim.x * blockDim.x) {
     const int c = (int)(idx % C);
     const double x = scale[c] * src.at(idx);
-    const __nv_bfloat16 h = __double2bfloat16(x);
+    const __nv_bfloat16 h = d2bf16(x);
     hi[idx] = h;
-    lo[idx] = __double2bfloat16(x - (double)__bfloat162float(h));
+    lo[idx] = d2bf16(x - f2d(__bfloat162float(h)));
   }
 }
 
@@ -759,18 +849,18 @@ void launch_rev_finish(const RevCtx &r, const double *q0, double *Y, cudaStream_
 
 // ----------------------------------------------------------------------------
 int adj_max_k() {
-  // k_adj_rows stages k * ROW_THREADS doubles; k_eig_full 4 k per warp
+  // k_adj_rows stages k * ROW_THREADS doubles; k_eig_full 6 k
   return 768;
 }
 
 void launch_eig_full(const AdjCtx &a, cudaStream_t st) {
-  const size_t smem = (size_t)EIG_WARPS * 4 * a.k * sizeof(double);
+  const size_t smem = (size_t)6 * a.k * sizeof(double);
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(k_eig_full, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     attr = true;
   }
-  k_eig_full<<<(a.Bs + EIG_WARPS - 1) / EIG_WARPS, EIG_WARPS * 32, smem, st>>>(a);
+  k_eig_full<<<a.Bs, EIG_THREADS, smem, st>>>(a);
 }
 void launch_adj_coeffs(const AdjCtx &a, cudaStream_t st) {
   const size_t smem = (size_t)3 * a.k * sizeof(double);
@@ -788,14 +878,20 @@ void launch_adj_rows(const AdjCtx &a, BasisRef basis, double *Y, double *Gd, cud
 }
 void launch_adj_rows_f32(const AdjCtx &a, BasisRef basis, double *Y, double *Gd,
                          cudaStream_t st) {
-  const size_t smem = (size_t)a.k * ROW_THREADS * sizeof(float);
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(k_adj_rows_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaFuncSetAttribute(k_adj_rows_f32_deep, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         200 * 1024);
     attr = true;
   }
-  dim3 grid((a.N + ROW_THREADS - 1) / ROW_THREADS, a.Bs);
-  k_adj_rows_f32<<<grid, ROW_THREADS, smem, st>>>(a, basis, Y, Gd);
+  const size_t tables = (size_t)2 * a.k * RF_ELEMS * sizeof(float);
+  if (tables <= 200 * 1024)   // k up to 200
+    k_adj_rows_f32<<<dim3((a.N + RF_ELEMS - 1) / RF_ELEMS, a.Bs), 32 * RF_WARPS, tables, st>>>(
+        a, basis, Y, Gd);
+  else
+    k_adj_rows_f32_deep<<<dim3((a.N + ROW_THREADS - 1) / ROW_THREADS, a.Bs), ROW_THREADS,
+                          (size_t)a.k * ROW_THREADS * sizeof(float), st>>>(a, basis, Y, Gd);
 }
 void launch_split_t(BasisRef src, int R, int C, int lds, __nv_bfloat16 *hi, __nv_bfloat16 *lo,
                     cudaStream_t st) {

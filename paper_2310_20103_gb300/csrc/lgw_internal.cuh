@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fp_bits.cuh"
 #include "lgw.h"
 
 namespace lgw {
@@ -479,7 +480,7 @@ struct BasisRef {
   const float *hi, *lo;
   __device__ __forceinline__ double at(size_t i) const {
     if (d) return d[i];
-    return lo ? (double)hi[i] + (double)lo[i] : (double)hi[i];
+    return lo ? f2d(hi[i]) + f2d(lo[i]) : f2d(hi[i]);
   }
 };
 struct AdjCtx {
