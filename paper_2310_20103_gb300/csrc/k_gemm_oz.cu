@@ -117,6 +117,7 @@ struct Epi {
   double *out;             // OZ_PART: [split][Ncols][ldo]; else [Ncols][ldo]
   int ldo;
   double scale;            // OZ_ADD: out += scale * product
+  int lower;               // A's row i is zero before K index i: skip those K blocks
   const double *Delta2, *dsq, *cd, *q, *qprev, *betaj;
   double *alpha_part;      // [M / 64][Ncols] partials of q . w, or NULL
   unsigned *status;
@@ -146,7 +147,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // N tiles fastest: the CTAs that share A's tiles run together
   const int m_tile = blockIdx.y, n_tile = blockIdx.x, split = blockIdx.z;
-  const int kb0 = split * kb_per_split, kb1 = min(num_kb, kb0 + kb_per_split);
+  const int kb1 = min(num_kb, (split + 1) * kb_per_split);
+  const int kb0 = max(split * kb_per_split, e.lower ? m_tile * (BM / KB) : 0);
   const int nk = max(0, kb1 - kb0);
   const int chunks = (nk + CHUNK_KB - 1) / CHUNK_KB;
 
@@ -568,6 +570,7 @@ bool launch_oz_gemm(const OzOperand &A, const OzOperand &B, int M, int Ncols, in
   e.out = o.out;
   e.ldo = o.ldo;
   e.scale = o.scale;
+  e.lower = o.lower ? 1 : 0;
   e.Delta2 = o.Delta2;
   e.dsq = o.dsq;
   e.cd = o.cd;

@@ -780,6 +780,7 @@ void f64_fit(lgw_handle *h, const double *C, const double *R, int n_pairs, int n
     o.mode = OZ_PART;
     o.out = B + (size_t)p0 * n;
     o.ldo = n;
+    o.lower = true;   // column i of R starts in row i
     oz_gemm(h, a, b, n, np, 1, o, "oz_gemm(fit)");
   }
 }

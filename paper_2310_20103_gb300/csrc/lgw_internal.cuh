@@ -255,6 +255,7 @@ struct OzOut {
   double *out = nullptr;
   int ldo = 0;
   double scale = 1.0;
+  bool lower = false;   // A's row i is zero before K index i (one split only)
   const double *Delta2 = nullptr, *dsq = nullptr, *cd = nullptr, *q = nullptr, *qprev = nullptr,
                *betaj = nullptr;
   double *alpha_part = nullptr;   // [M / 64][Ncols]
