@@ -214,6 +214,13 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_dots_split(VecCtx c, int j) 
   }
 }
 
+// Sum of n values `stride` apart in order.
+__device__ __forceinline__ double chunk_sum(const double *p, size_t stride, int n) {
+  double s = 0.0;
+  for (int i = 0; i < n; ++i) s += p[(size_t)i * stride];
+  return s;
+}
+
 // h[b][i] = sum over chunks (fixed order), then the norm of the projected
 // vector without reading it back: with Q orthonormal,
 //   ||w - Q h||^2 = ||w||^2 - ||h||^2,
@@ -242,9 +249,8 @@ __global__ void __launch_bounds__(256) k_reduce_dots_split(VecCtx c, int j, int 
   if (pass == 2 && !c.flag2[b]) return;
   double hh = 0.0;
   for (int i = threadIdx.x; i <= j; i += blockDim.x) {
-    const double *p = c.dot_part + (size_t)b * c.nchunks * c.kmax1 + i;
-    double s = 0.0;
-    for (int ch = 0; ch < c.nchunks; ++ch) s += p[(size_t)ch * c.kmax1];
+    const double s = chunk_sum(c.dot_part + (size_t)b * c.nchunks * c.kmax1 + i, c.kmax1,
+                               c.nchunks);
     c.h[(size_t)b * c.kmax1 + i] = s;
     hh = fma(s, s, hh);
     if (pass == 1 && i == j) {
@@ -974,11 +980,10 @@ __global__ void __launch_bounds__(256) k_reduce_dcgs(VecCtx c, int j) {
   for (int i = threadIdx.x; i <= j; i += blockDim.x) {
     double s = 0.0;
     if (i < j) {
-      const double *p = c.dot_part + (size_t)b * c.nchunks * c.kmax1 + i;
-      for (int ch = 0; ch < c.nchunks; ++ch) s += p[(size_t)ch * c.kmax1];
+      s = chunk_sum(c.dot_part + (size_t)b * c.nchunks * c.kmax1 + i, c.kmax1, c.nchunks);
       s -= c.gq[(size_t)b * c.kmax1 + i];   // the sweep removed Q_{j-1} g
     } else {
-      for (int ch = 0; ch < c.nchunks; ++ch) s += c.hj_part[(size_t)b * c.nchunks + ch];
+      s = chunk_sum(c.hj_part + (size_t)b * c.nchunks, 1, c.nchunks);
       const size_t ai = (size_t)v * c.k + j;
       const double a = c.alpha[ai] + s - hprev;
       c.alpha[ai] = a;
@@ -998,6 +1003,7 @@ __global__ void __launch_bounds__(256) k_reduce_dcgs(VecCtx c, int j) {
   c.flag2[b] = f;
   if (f) {
     atomicAdd(c.n_second, 1);
+    c.p2_step[j] = 1;
     return;
   }
   const double beta = sqrt(fmax(rest, 0.0));
@@ -1009,16 +1015,23 @@ __global__ void __launch_bounds__(256) k_reduce_dcgs(VecCtx c, int j) {
 }
 
 // Second pass of the flagged vectors (rare: a large part of v lay in
-// span(Q_j)).  Blocks loop over the sub-batch and skip unflagged vectors.
+// span(Q_j)).  Blocks loop over the sub-batch and skip unflagged vectors; a
+// step without any (c.p2_step) ends at once.  A block's chunk of the dot
+// products needs only the block's chunk of the updated vector, so one kernel
+// does both:
 //  update: w' = v - Q_j h' in FP64 from the full float pair (h' need not be
 //          small here), with ||w'||^2 partials and the operand written anew;
 //  dots:   h'' = Q_j^T w' (double-float);
 //  reduce: beta_{j+1}^2 = ||w'||^2 - ||h''||^2, and h'' becomes the delayed
 //          update that the next sweep applies.
 template <bool LO>
-__global__ void __launch_bounds__(VEC_THREADS) k_p2_update_dcgs(VecCtx c, int j) {
-  extern __shared__ double hs[];   // [j + 1]
+__global__ void __launch_bounds__(VEC_THREADS) k_p2_dcgs(VecCtx c, int j) {
+  extern __shared__ float4 stg[];   // row staging ring, then [j + 1] coefficients
+  double *hs =
+      reinterpret_cast<double *>(reinterpret_cast<char *>(stg) + sweep_stage_bytes<LO>());
   __shared__ double red[VEC_THREADS / 32];
+  __shared__ float2 part[2][32][VEC_THREADS / 32];
+  if (!c.p2_step[j]) return;
   const int chunk = blockIdx.x;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int ebase = chunk * VEC_CHUNK + wid * 256 + 4 * lane;
@@ -1050,37 +1063,44 @@ __global__ void __launch_bounds__(VEC_THREADS) k_p2_update_dcgs(VecCtx c, int j)
     const size_t voff = (size_t)b * c.N;
     double nrm = 0.0;
     float dq = 0.0f;
+    float2 vh2[4], vl2[4], unused[4];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const int e = ebase + 128 * u;
-      if (e >= c.N) continue;
-      double w4[4];
-      const double2 w0 = *reinterpret_cast<const double2 *>(c.wv + voff + e);
-      const double2 w1 = *reinterpret_cast<const double2 *>(c.wv + voff + e + 2);
-      w4[0] = w0.x - r[4 * u];
-      w4[1] = w0.y - r[4 * u + 1];
-      w4[2] = w1.x - r[4 * u + 2];
-      w4[3] = w1.y - r[4 * u + 3];
-      *reinterpret_cast<double2 *>(c.wv + voff + e) = make_double2(w4[0], w4[1]);
-      *reinterpret_cast<double2 *>(c.wv + voff + e + 2) = make_double2(w4[2], w4[3]);
-      float f4[4];
+      float f4[4] = {0.f, 0.f, 0.f, 0.f}, l4[4] = {0.f, 0.f, 0.f, 0.f};
+      if (e < c.N) {
+        double w4[4];
+        const double2 w0 = *reinterpret_cast<const double2 *>(c.wv + voff + e);
+        const double2 w1 = *reinterpret_cast<const double2 *>(c.wv + voff + e + 2);
+        w4[0] = w0.x - r[4 * u];
+        w4[1] = w0.y - r[4 * u + 1];
+        w4[2] = w1.x - r[4 * u + 2];
+        w4[3] = w1.y - r[4 * u + 3];
+        *reinterpret_cast<double2 *>(c.wv + voff + e) = make_double2(w4[0], w4[1]);
+        *reinterpret_cast<double2 *>(c.wv + voff + e + 2) = make_double2(w4[2], w4[3]);
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        nrm = fma(w4[t], w4[t], nrm);
-        f4[t] = __double2float_rn(w4[t]);
-        if (c.dq2_part != nullptr) dq = fmaf(c.d2f[e + t] * f4[t], f4[t], dq);
+        for (int t = 0; t < 4; ++t) {
+          nrm = fma(w4[t], w4[t], nrm);
+          split_d(w4[t], f4[t], l4[t]);
+          if (c.dq2_part != nullptr) dq = fmaf(c.d2f[e + t] * f4[t], f4[t], dq);
+        }
+        if (c.xh != nullptr) {
+          __nv_bfloat162 x01, x23;
+          x01.x = __float2bfloat16_rn(c.dsqf[e] * f4[0]);
+          x01.y = __float2bfloat16_rn(c.dsqf[e + 1] * f4[1]);
+          x23.x = __float2bfloat16_rn(c.dsqf[e + 2] * f4[2]);
+          x23.y = __float2bfloat16_rn(c.dsqf[e + 3] * f4[3]);
+          uint2 pk;
+          pk.x = *reinterpret_cast<uint32_t *>(&x01);
+          pk.y = *reinterpret_cast<uint32_t *>(&x23);
+          *reinterpret_cast<uint2 *>(c.xh + kblk_bf16(b, e, c.Bs)) = pk;
+        }
       }
-      if (c.xh != nullptr) {
-        __nv_bfloat162 x01, x23;
-        x01.x = __float2bfloat16_rn(c.dsqf[e] * f4[0]);
-        x01.y = __float2bfloat16_rn(c.dsqf[e + 1] * f4[1]);
-        x23.x = __float2bfloat16_rn(c.dsqf[e + 2] * f4[2]);
-        x23.y = __float2bfloat16_rn(c.dsqf[e + 3] * f4[3]);
-        uint2 pk;
-        pk.x = *reinterpret_cast<uint32_t *>(&x01);
-        pk.y = *reinterpret_cast<uint32_t *>(&x23);
-        *reinterpret_cast<uint2 *>(c.xh + kblk_bf16(b, e, c.Bs)) = pk;
-      }
+      vh2[2 * u] = make_float2(f4[0], f4[1]);
+      vh2[2 * u + 1] = make_float2(f4[2], f4[3]);
+      vl2[2 * u] = make_float2(l4[0], l4[1]);
+      vl2[2 * u + 1] = make_float2(l4[2], l4[3]);
+      unused[2 * u] = unused[2 * u + 1] = make_float2(0.f, 0.f);
     }
     nrm = block_sum(nrm, red);
     if (c.dq2_part != nullptr) dq = block_sum_f(dq, red);
@@ -1088,40 +1108,6 @@ __global__ void __launch_bounds__(VEC_THREADS) k_p2_update_dcgs(VecCtx c, int j)
       c.norm_b[(size_t)b * c.nchunks + chunk] = nrm;
       if (c.dq2_part != nullptr)
         c.dq2_part[(size_t)((j + 1) & 1) * c.Bs * c.nchunks + (size_t)b * c.nchunks + chunk] = dq;
-    }
-  }
-}
-
-template <bool LO>
-__global__ void __launch_bounds__(VEC_THREADS) k_p2_dots_dcgs(VecCtx c, int j) {
-  extern __shared__ float4 stg[];   // row staging ring
-  __shared__ float2 part[2][32][VEC_THREADS / 32];
-  const int chunk = blockIdx.x;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int ebase = chunk * VEC_CHUNK + wid * 256 + 4 * lane;
-  for (int b = blockIdx.y; b < c.Bs; b += gridDim.y) {
-    if (!c.flag2[b]) continue;   // uniform over the block
-    const size_t voff = (size_t)b * c.N;
-    float vh[8], vl[8];
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int e = ebase + 128 * u;
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        vh[4 * u + t] = vl[4 * u + t] = 0.0f;
-        if (e < c.N) {
-          const double x = c.wv[voff + e + t];
-          vh[4 * u + t] = __double2float_rn(x);
-          vl[4 * u + t] = __double2float_rn(x - (double)vh[4 * u + t]);
-        }
-      }
-    }
-    float2 vh2[4], vl2[4], unused[4];
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      vh2[m] = make_float2(vh[2 * m], vh[2 * m + 1]);
-      vl2[m] = make_float2(vl[2 * m], vl[2 * m + 1]);
-      unused[m] = make_float2(0.f, 0.f);
     }
     double *dp = c.dot_part + ((size_t)b * c.nchunks + chunk) * c.kmax1;
     __syncthreads();   // the tile buffers of the previous vector are free
@@ -1134,12 +1120,11 @@ __global__ void __launch_bounds__(256) k_p2_reduce_dcgs(VecCtx c, int j) {
   __shared__ double red[256 / 32];
   const int b = blockIdx.x;
   const int v = c.vec0 + b;
-  if (!c.flag2[b]) return;
+  if (!c.p2_step[j] || !c.flag2[b]) return;
   double hh = 0.0;
   for (int i = threadIdx.x; i <= j; i += blockDim.x) {
-    const double *p = c.dot_part + (size_t)b * c.nchunks * c.kmax1 + i;
-    double s = 0.0;
-    for (int ch = 0; ch < c.nchunks; ++ch) s += p[(size_t)ch * c.kmax1];
+    const double s = chunk_sum(c.dot_part + (size_t)b * c.nchunks * c.kmax1 + i, c.kmax1,
+                               c.nchunks);
     c.h[(size_t)b * c.kmax1 + i] = s;
     hh = fma(s, s, hh);
   }
@@ -1189,22 +1174,22 @@ void launch_sweep_dcgs(const VecCtx &c, int j, cudaStream_t st) {
 void launch_reduce_dcgs(const VecCtx &c, int j, cudaStream_t st) {
   k_reduce_dcgs<<<c.Bs, 256, 0, st>>>(c, j);
 }
-void launch_pass2_dcgs(const VecCtx &c, int j, cudaStream_t st) {
-  const dim3 grid(c.nchunks, c.Bs < 16 ? c.Bs : 16);
-  const size_t sh = (size_t)(j + 1) * sizeof(double);
+template <bool LO>
+static void pass2_one(const VecCtx &c, int j, cudaStream_t st) {
   static bool attr = false;
   if (!attr) {
-    allow_smem(k_p2_dots_dcgs<true>, sweep_stage_bytes<true>());
-    allow_smem(k_p2_dots_dcgs<false>, sweep_stage_bytes<false>());
+    allow_smem(k_p2_dcgs<LO>, sweep_stage_bytes<LO>() + (size_t)4096 * sizeof(double));
     attr = true;
   }
-  if (c.blo != nullptr) {
-    k_p2_update_dcgs<true><<<grid, VEC_THREADS, sh, st>>>(c, j);
-    k_p2_dots_dcgs<true><<<grid, VEC_THREADS, sweep_stage_bytes<true>(), st>>>(c, j);
-  } else {
-    k_p2_update_dcgs<false><<<grid, VEC_THREADS, sh, st>>>(c, j);
-    k_p2_dots_dcgs<false><<<grid, VEC_THREADS, sweep_stage_bytes<false>(), st>>>(c, j);
-  }
+  const dim3 grid(c.nchunks, c.Bs < 16 ? c.Bs : 16);
+  k_p2_dcgs<LO><<<grid, VEC_THREADS, sweep_stage_bytes<LO>() + (size_t)(j + 1) * sizeof(double),
+                  st>>>(c, j);
+}
+void launch_pass2_dcgs(const VecCtx &c, int j, cudaStream_t st) {
+  if (c.blo != nullptr)
+    pass2_one<true>(c, j, st);
+  else
+    pass2_one<false>(c, j, st);
   k_p2_reduce_dcgs<<<c.Bs, 256, 0, st>>>(c, j);
 }
 

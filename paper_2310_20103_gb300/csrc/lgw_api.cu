@@ -898,6 +898,7 @@ void run_lanczos(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts 
     c.uC = tc ? nullptr : c.w;
     c.hj_part = wsT<double>(h, "hj_part", (size_t)Bs * nchunks);
     c.gq = wsT<double>(h, "gq", (size_t)Bs * kmax1);
+    c.p2_step = wsT<int>(h, "p2_step", (size_t)k);
   }
   LGW_TRY_CUDA(h, cudaMemsetAsync(c.n_second, 0, sizeof(int), st));
   LGW_TRY_CUDA(h, cudaMemsetAsync(c.flag2, 0, sizeof(int) * Bs, st));
@@ -1017,6 +1018,7 @@ void run_lanczos(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts 
     auto sub_body = [&]() {
       // ---- start vectors b = Delta^1/2 V, V = L M (text after Eq. 8) ----
       tm.mark(C_START);
+      if (dcgs) LGW_TRY_CUDA(h, cudaMemsetAsync(c.p2_step, 0, sizeof(int) * k, st));
       if (pv.d_M && tc && s.Lb) {
         // V = L M on the tensor cores in split BF16 (three products, FP32 sum)
         float *vf = ucd_buf;

@@ -132,6 +132,7 @@ struct VecCtx {
   double *wv;             // [Bs][N] the carried vector w_j (unnormalised q~_{j+1} = w_j / beta_{j+1})
   const double *uC;       // [Bs][N] C w_j from the FP64 contractions, or null (tensor cores)
   double *hj_part;        // [Bs][nchunks] partials of q_j . w_j
+  int *p2_step;           // [k] nonzero: step j flagged some vector for a second pass
   double *gq;             // [Bs][kmax1] g = (T_{j-1} - alpha~_j) h / beta_j, removed by the sweep
 };
 
