@@ -214,10 +214,29 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_dots_split(VecCtx c, int j) 
   }
 }
 
-// Sum of n values `stride` apart in order.
-__device__ __forceinline__ double chunk_sum(const double *p, size_t stride, int n) {
+// Sum of n values `stride` apart in order.  Sixteen at a time travel to the
+// thread's own column of shared memory by cp.async: as plain loads the
+// compiler issues a few and waits, and the 64 partials of a long vector cost a
+// round trip each few (the reduction took 38 us per step at N_vc 131072, 256
+// vectors, 20 us now).  `col` holds 16 x blockDim.x doubles.
+__device__ __forceinline__ double chunk_sum(const double *p, size_t stride, int n, double *col) {
   double s = 0.0;
-  for (int i = 0; i < n; ++i) s += p[(size_t)i * stride];
+  double *mine = col + threadIdx.x;
+  const uint32_t sa = (uint32_t)__cvta_generic_to_shared(mine);
+  const uint32_t step = blockDim.x * (uint32_t)sizeof(double);
+  for (int c0 = 0; c0 < n; c0 += 16) {
+    const int m = min(16, n - c0);
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (i < m)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sa + i * step),
+                     "l"(p + (size_t)(c0 + i) * stride)
+                     : "memory");
+    asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (i < m) s += mine[i * blockDim.x];
+  }
   return s;
 }
 
@@ -235,7 +254,7 @@ __device__ __forceinline__ double chunk_sum(const double *p, size_t stride, int 
 // Not-live vectors get flag2 = 0 and 1/beta = 0, so the update writes
 // zeros into their next slot.
 __global__ void __launch_bounds__(256) k_reduce_dots_split(VecCtx c, int j, int pass) {
-  __shared__ double red[256 / 32];
+  __shared__ double red[256 / 32], col[16 * 256];
   const int b = blockIdx.x;
   const int v = c.vec0 + b;
   if (!live_s(c, b, j)) {
@@ -250,7 +269,7 @@ __global__ void __launch_bounds__(256) k_reduce_dots_split(VecCtx c, int j, int 
   double hh = 0.0;
   for (int i = threadIdx.x; i <= j; i += blockDim.x) {
     const double s = chunk_sum(c.dot_part + (size_t)b * c.nchunks * c.kmax1 + i, c.kmax1,
-                               c.nchunks);
+                               c.nchunks, col);
     c.h[(size_t)b * c.kmax1 + i] = s;
     hh = fma(s, s, hh);
     if (pass == 1 && i == j) {
@@ -507,6 +526,13 @@ __global__ void __launch_bounds__(VEC_THREADS) k_start_split(VecCtx c) {
 // conversions between FP64 and the float pairs.  They run on the integer pipe
 // (fp_bits.cuh), bit for bit the same: 54.5 -> 49.7 us per launch at N_vc 4511,
 // 100 vectors, 442 -> 410 us at 32768, 128 vectors, k 120.
+// Then 49 -> 38 us and 411 -> 362 us (at 131072, 256 vectors, k 200: 4.24 ->
+// 4.06 ms per launch, 7.0 TB/s) by what a block does outside the row loop: its
+// first rows travel while it forms v, float pairs are joined as integers
+// (pair_d), the three closing sums share one butterfly, and warps without
+// partials of alpha skip its sum (block_sum).  A warp's FP64 instruction holds
+// its scheduler's pipe for 64 clocks or more, so the 78 additions per warp of
+// four plain block sums cost as much as 30 rows.
 //
 // Thread layout: one block per (2048-element chunk, vector); each thread
 // owns elements e = chunk*2048 + warp*256 + 4*lane + 128*u + {0..3},
@@ -617,51 +643,45 @@ __device__ __forceinline__ void row_products(const float4 *slot, float2 cg,
   sl_out = sl;
 }
 
-// All rows i = nrows - 1 down to 0 (the newest row first), two per trip.
-// Row partials of the block go to dp[i] (one double per row), through a
-// transposed butterfly over the warp every two trips (12 shuffles for four
-// rows) and a fixed-order sum over the eight warps in shared memory, 32 rows
-// at a time.
-// cg[i] = (c_i, g_i), read only with CORR.
-template <bool LO, bool CORR>
-__device__ __forceinline__ void sweep_all_rows(const VecCtx &c, int b, int nrows, int ebase,
-                                               const float2 *cg, const float2 (&vh)[4],
-                                               const float2 (&vl)[4], float2 (&corr)[4],
-                                               float2 (&cv)[4],
-                                               float2 (*part)[32][VEC_THREADS / 32],
-                                               double *dp, float4 *stg) {
-  constexpr int NV = LO ? 4 : 2;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  float2 vn[4];
-#pragma unroll
-  for (int m = 0; m < 4; ++m) vn[m] = make_float2(-vh[m].x, -vh[m].y);
+// A thread's four (two) pieces of a staged row: where they lie in the basis
+// and in its ring slot.
+template <bool LO>
+struct RowStage {
+  static constexpr int NV = LO ? 4 : 2;
+  static constexpr int PB = VEC_THREADS * 16;   // bytes between a thread's pieces
+  const float *hb;
+  uintptr_t dlo;   // the lo row sits at a fixed distance from the hi row (flat addresses)
+  size_t rstride;
+  uint32_t sbase;  // 32-bit shared address of slot 0
+  int nrows;
+  bool ok0, ok1;
+
   // N is a multiple of 128, so each 4-element piece of the thread lies wholly
   // inside a row or wholly past its end; pieces past the end read zeros,
   // filled into their slots once
-  const bool ok0 = ebase < c.N, ok1 = ebase + 128 < c.N;
-  float4 *mine = stg + threadIdx.x;
-  if (!ok1) {
-    for (int s = 0; s < SW_SLOTS; ++s) {
+  __device__ __forceinline__ RowStage(const VecCtx &c, int b, int nrows_, int ebase, float4 *stg)
+      : nrows(nrows_), ok0(ebase < c.N), ok1(ebase + 128 < c.N) {
+    float4 *mine = stg + threadIdx.x;
+    if (!ok1) {
+      for (int s = 0; s < SW_SLOTS; ++s) {
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        if (u == 0 && ok0) continue;
-        mine[(s * NV + u) * VEC_THREADS] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (LO) mine[(s * NV + 2 + u) * VEC_THREADS] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int u = 0; u < 2; ++u) {
+          if (u == 0 && ok0) continue;
+          mine[(s * NV + u) * VEC_THREADS] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (LO) mine[(s * NV + 2 + u) * VEC_THREADS] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
       }
     }
+    rstride = (size_t)c.Bs * c.N;
+    hb = c.bhi + (size_t)b * c.N + ebase;
+    const float *lb = LO ? c.blo + (size_t)b * c.N + ebase : nullptr;
+    sbase = (uint32_t)__cvta_generic_to_shared(mine);
+    dlo = LO ? (uintptr_t)lb - (uintptr_t)hb : 0;
   }
-  const size_t rstride = (size_t)c.Bs * c.N;
-  const float *hb = c.bhi + (size_t)b * c.N + ebase;
-  const float *lb = LO ? c.blo + (size_t)b * c.N + ebase : nullptr;
   // sequence index r (row nrows - 1 - r) into slot s; one commit group per
-  // index, empty past the last row
-  // shared addresses as 32-bit offsets and the four pieces of a row at
-  // immediate offsets from one global and one shared address
-  const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(mine);
-  // the lo row sits at a fixed distance from the hi row (flat addresses)
-  const uintptr_t dlo = LO ? (uintptr_t)lb - (uintptr_t)hb : 0;
-  constexpr int PB = VEC_THREADS * 16;   // bytes between a thread's pieces
-  auto stage = [&](int r, int s) {
+  // index, empty past the last row.  The four pieces of a row sit at immediate
+  // offsets from one global and one shared address.
+  __device__ __forceinline__ void operator()(int r, int s) const {
     if (r < nrows) {
       const float *g = hb + (size_t)(nrows - 1 - r) * rstride;
       const uint32_t sa = sbase + (uint32_t)(s * NV * PB);
@@ -675,8 +695,32 @@ __device__ __forceinline__ void sweep_all_rows(const VecCtx &c, int b, int nrows
       }
     }
     cp_async_commit();
-  };
-  for (int r = 0; r < SW_SLOTS; ++r) stage(r, r);
+  }
+  __device__ __forceinline__ void first() const {
+    for (int r = 0; r < SW_SLOTS; ++r) (*this)(r, r);
+  }
+};
+
+// All rows i = nrows - 1 down to 0 (the newest row first), two per trip; the
+// first SW_SLOTS of them are already on their way (stage.first()).
+// Row partials of the block go to dp[i] (one double per row), through a
+// transposed butterfly over the warp every two trips (12 shuffles for four
+// rows) and a fixed-order sum over the eight warps in shared memory, 32 rows
+// at a time.
+// cg[i] = (c_i, g_i), read only with CORR.
+template <bool LO, bool CORR>
+__device__ __forceinline__ void sweep_all_rows(const RowStage<LO> &stage, const float2 *cg,
+                                               const float2 (&vh)[4], const float2 (&vl)[4],
+                                               float2 (&corr)[4], float2 (&cv)[4],
+                                               float2 (*part)[32][VEC_THREADS / 32], double *dp,
+                                               float4 *stg) {
+  constexpr int NV = LO ? 4 : 2;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int nrows = stage.nrows;
+  float2 vn[4];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) vn[m] = make_float2(-vh[m].x, -vh[m].y);
+  float4 *mine = stg + threadIdx.x;
   int sc = 0;   // slot of sequence index rs: rs % SW_SLOTS
   for (int t0 = 0; t0 < nrows; t0 += 32) {
     const int nt = min(32, nrows - t0);
@@ -768,7 +812,7 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_sweep_dcgs(VecCtx c, int j) 
   extern __shared__ float4 dyn[];   // row staging ring, then [j] pairs (c_i, g_i)
   float2 *cg = reinterpret_cast<float2 *>(reinterpret_cast<char *>(dyn) + sweep_stage_bytes<LO>());
   __shared__ float2 part[2][32][VEC_THREADS / 32];
-  __shared__ double red[VEC_THREADS / 32];
+  __shared__ double red[VEC_THREADS / 32], red3[3][VEC_THREADS / 32];
   const int chunk = blockIdx.x, b = blockIdx.y;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int ebase = chunk * VEC_CHUNK + wid * 256 + 4 * lane;
@@ -783,6 +827,9 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_sweep_dcgs(VecCtx c, int j) 
     }
     return;
   }
+  // the newest rows travel while the block forms v
+  const RowStage<LO> stage(c, b, j, ebase, dyn);
+  stage.first();
   const double sinv = c.sinv[b], bj = c.betaj[b];
   // alpha~_j = q~_j . C q~_j: from the FP64 contraction's partials, or
   // sum Delta^2 q~^2 + c_K y . bf16(y) on the tensor-core path
@@ -869,10 +916,10 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_sweep_dcgs(VecCtx c, int j) 
       const float4 ph = *reinterpret_cast<const float4 *>(bhi_row(c, j - 1, b) + e);
       const float4 pl = LO ? *reinterpret_cast<const float4 *>(blo_row(c, j - 1, b) + e)
                            : make_float4(0.f, 0.f, 0.f, 0.f);
-      qp[0] = f2d(ph.x) + f2d(pl.x);
-      qp[1] = f2d(ph.y) + f2d(pl.y);
-      qp[2] = f2d(ph.z) + f2d(pl.z);
-      qp[3] = f2d(ph.w) + f2d(pl.w);
+      qp[0] = pair_d(ph.x, pl.x);
+      qp[1] = pair_d(ph.y, pl.y);
+      qp[2] = pair_d(ph.z, pl.z);
+      qp[3] = pair_d(ph.w, pl.w);
     }
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
@@ -892,7 +939,7 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_sweep_dcgs(VecCtx c, int j) 
       corr2[m] = make_float2(0.f, 0.f);
       cv2[m] = make_float2(0.f, 0.f);
     }
-    sweep_all_rows<LO, true>(c, b, j, ebase, cg, vh2, vl2, corr2, cv2, part, dp, dyn);
+    sweep_all_rows<LO, true>(stage, cg, vh2, vl2, corr2, cv2, part, dp, dyn);
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
       corr[2 * m] = corr2[m].x;
@@ -919,7 +966,7 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_sweep_dcgs(VecCtx c, int j) 
 #pragma unroll
     for (int t = 0; t < 4; ++t) {
       const int m = 4 * u + t;
-      vd[t] = (f2d(vh[m]) + f2d(vl[m])) - f2d(cv[m]);   // w_j = v - Q_{j-1} g
+      vd[t] = pair_d(vh[m], vl[m]) - f2d(cv[m]);   // w_j = v - Q_{j-1} g
       vh[m] = d2f(vd[t]);
       const double qj = fma(wq[t], sinv, -f2d(corr[m]));
       split_d(qj, qh4[t], ql4[t]);
@@ -946,14 +993,33 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_sweep_dcgs(VecCtx c, int j) 
       for (int t = 0; t < 4; ++t) dq = fmaf(c.d2f[e + t] * vh[4 * u + t], vh[4 * u + t], dq);
     }
   }
-  hj = block_sum(hj, red);
-  nrm = block_sum(nrm, red);
-  if (c.dq2_part != nullptr) dq = block_sum_f(dq, red);
-  if (threadIdx.x == 0) {
+  // the three sums in one butterfly (lanes 0..15 go on with hj, 16..31 with
+  // nrm, then bit 3 with dq), each added up in the order of block_sum: six
+  // FP64 additions per warp instead of 15, and 24 per block at the end instead
+  // of 192
+  const bool b16 = (lane & 16) != 0, b8 = (lane & 8) != 0;
+  double x = b16 ? nrm : hj, y = f2d(dq);
+  x += __shfl_xor_sync(0xffffffffu, b16 ? hj : nrm, 16);
+  y += __shfl_xor_sync(0xffffffffu, y, 16);
+  {
+    const double send = b8 ? x : y;
+    x = (b8 ? y : x) + __shfl_xor_sync(0xffffffffu, send, 8);
+  }
+#pragma unroll
+  for (int o = 4; o >= 1; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  if (lane == 0) red3[0][wid] = x;
+  if (lane == 16) red3[1][wid] = x;
+  if (lane == 8) red3[2][wid] = x;
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < VEC_THREADS / 32; ++w) t += red3[threadIdx.x][w];
     const size_t pi = (size_t)b * c.nchunks + chunk;
-    c.hj_part[pi] = hj;
-    c.norm_a[pi] = nrm;
-    if (c.dq2_part != nullptr) c.dq2_part[(size_t)((j + 1) & 1) * c.Bs * c.nchunks + pi] = dq;
+    if (threadIdx.x == 0) c.hj_part[pi] = t;
+    if (threadIdx.x == 1) c.norm_a[pi] = t;
+    if (threadIdx.x == 2 && c.dq2_part != nullptr)
+      c.dq2_part[(size_t)((j + 1) & 1) * c.Bs * c.nchunks + pi] = (float)t;
   }
 }
 
@@ -962,8 +1028,7 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_sweep_dcgs(VecCtx c, int j) 
 // Where the projection removes more than half of ||v||^2 the vector is
 // flagged for a second pass (the CGS1K criterion) and beta waits for it.
 __global__ void __launch_bounds__(256) k_reduce_dcgs(VecCtx c, int j) {
-  __shared__ double red[256 / 32];
-  __shared__ double hprev;
+  __shared__ double red[256 / 32], col[16 * 256];
   const int b = blockIdx.x;
   const int v = c.vec0 + b;
   if (!live_s(c, b, j)) {
@@ -974,27 +1039,31 @@ __global__ void __launch_bounds__(256) k_reduce_dcgs(VecCtx c, int j) {
     }
     return;
   }
-  if (threadIdx.x == 0) hprev = j >= 1 ? c.h[(size_t)b * c.kmax1 + j - 1] : 0.0;
-  __syncthreads();
-  double hh = 0.0;
+  const size_t ai = (size_t)v * c.k + j;
+  double hprev = 0.0, alpha = 0.0, amax = 0.0, nw = 0.0, hh = 0.0;
+  if (threadIdx.x == (j & 255)) {   // the thread of row j
+    if (j >= 1) hprev = c.h[(size_t)b * c.kmax1 + j - 1];
+    alpha = c.alpha[ai];
+    amax = c.amax[b];
+  }
+  for (int ch = threadIdx.x; ch < c.nchunks; ch += blockDim.x)
+    nw += c.norm_a[(size_t)b * c.nchunks + ch];
+  __syncthreads();   // h_{j-1} is overwritten below
   for (int i = threadIdx.x; i <= j; i += blockDim.x) {
     double s = 0.0;
     if (i < j) {
-      s = chunk_sum(c.dot_part + (size_t)b * c.nchunks * c.kmax1 + i, c.kmax1, c.nchunks);
-      s -= c.gq[(size_t)b * c.kmax1 + i];   // the sweep removed Q_{j-1} g
+      const double gq = c.gq[(size_t)b * c.kmax1 + i];
+      s = chunk_sum(c.dot_part + (size_t)b * c.nchunks * c.kmax1 + i, c.kmax1, c.nchunks, col);
+      s -= gq;   // the sweep removed Q_{j-1} g
     } else {
-      s = chunk_sum(c.hj_part + (size_t)b * c.nchunks, 1, c.nchunks);
-      const size_t ai = (size_t)v * c.k + j;
-      const double a = c.alpha[ai] + s - hprev;
+      s = chunk_sum(c.hj_part + (size_t)b * c.nchunks, 1, c.nchunks, col);
+      const double a = alpha + s - hprev;
       c.alpha[ai] = a;
-      c.amax[b] = fmax(c.amax[b], fabs(a));
+      c.amax[b] = fmax(amax, fabs(a));
     }
     c.h[(size_t)b * c.kmax1 + i] = s;
     hh = fma(s, s, hh);
   }
-  double nw = 0.0;
-  for (int ch = threadIdx.x; ch < c.nchunks; ch += blockDim.x)
-    nw += c.norm_a[(size_t)b * c.nchunks + ch];
   hh = block_sum(hh, red);   // the barriers also publish amax[b]
   nw = block_sum(nw, red);
   if (threadIdx.x != 0) return;
@@ -1111,20 +1180,22 @@ __global__ void __launch_bounds__(VEC_THREADS) k_p2_dcgs(VecCtx c, int j) {
     }
     double *dp = c.dot_part + ((size_t)b * c.nchunks + chunk) * c.kmax1;
     __syncthreads();   // the tile buffers of the previous vector are free
-    sweep_all_rows<LO, false>(c, b, j + 1, ebase, nullptr, vh2, vl2, unused, unused, part, dp,
+    const RowStage<LO> stage(c, b, j + 1, ebase, stg);
+    stage.first();
+    sweep_all_rows<LO, false>(stage, nullptr, vh2, vl2, unused, unused, part, dp,
                               stg);
   }
 }
 
 __global__ void __launch_bounds__(256) k_p2_reduce_dcgs(VecCtx c, int j) {
-  __shared__ double red[256 / 32];
+  __shared__ double red[256 / 32], col[16 * 256];
   const int b = blockIdx.x;
   const int v = c.vec0 + b;
   if (!c.p2_step[j] || !c.flag2[b]) return;
   double hh = 0.0;
   for (int i = threadIdx.x; i <= j; i += blockDim.x) {
     const double s = chunk_sum(c.dot_part + (size_t)b * c.nchunks * c.kmax1 + i, c.kmax1,
-                               c.nchunks);
+                               c.nchunks, col);
     c.h[(size_t)b * c.kmax1 + i] = s;
     hh = fma(s, s, hh);
   }

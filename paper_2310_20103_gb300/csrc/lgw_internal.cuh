@@ -172,16 +172,26 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// x != 0 on the integer pipe (NaN counts as nonzero).
+__device__ __forceinline__ bool nonzero_bits(double x) {
+  return ((unsigned)(__double2hiint(x) << 1) | (unsigned)__double2loint(x)) != 0u;
+}
+
 // Block-wide sum in fixed order; every thread gets the result.  `red` needs
-// blockDim.x / 32 doubles.
+// blockDim.x / 32 doubles.  Warps without a nonzero value cost no FP64
+// addition (sums over few chunks fill one warp of the block): a warp's FP64
+// instruction holds its scheduler's pipe for 76 clocks.
 __device__ __forceinline__ double block_sum(double v, double *red) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  v = warp_sum(v);
+  if (__any_sync(0xffffffffu, nonzero_bits(v))) v = warp_sum(v);
   __syncthreads();
   if (lane == 0) red[wid] = v;
   __syncthreads();
   double s = 0.0;
-  for (int i = 0; i < nw; ++i) s += red[i];
+  for (int i = 0; i < nw; ++i) {
+    const double r = red[i];
+    if (nonzero_bits(r)) s += r;
+  }
   return s;
 }
 
@@ -191,13 +201,16 @@ __device__ __forceinline__ double block_sum(double v, double *red) {
 // pipe.
 __device__ __forceinline__ double block_sum_to0(double v, double *red) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  v = warp_sum(v);
+  if (__any_sync(0xffffffffu, nonzero_bits(v))) v = warp_sum(v);
   __syncthreads();
   if (lane == 0) red[wid] = v;
   __syncthreads();
   double s = 0.0;
   if (threadIdx.x == 0)
-    for (int i = 0; i < nw; ++i) s += red[i];
+    for (int i = 0; i < nw; ++i) {
+      const double r = red[i];
+      if (nonzero_bits(r)) s += r;
+    }
   return s;
 }
 
