@@ -406,56 +406,123 @@ __global__ void __launch_bounds__(ROW_THREADS) k_adj_rows_f32_deep(AdjCtx a, Bas
 }
 
 // BF16 hi / lo split of a transposed FP64 matrix: src [R][C] (row stride
-// lds) -> hi, lo [C][R]; 32 x 32 shared-memory tiles so both sides coalesce.
-// Either output may be NULL.
-__global__ void k_split_t(BasisRef src, int R, int C, int lds,
-                          __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo) {
-  __shared__ double tile[32][33];
-  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8 threads
-  for (int rr = ty; rr < 32; rr += 8) {
-    const int r = r0 + rr, c = c0 + tx;
-    tile[rr][tx] = (r < R && c < C) ? src.at((size_t)r * lds + c) : 0.0;
+// lds) -> hi, lo [C][R].  Either output may be NULL.  Bound by DRAM (8 bytes
+// read, 4 written per element): 64 x 64 tiles, so that both sides move whole
+// 128-byte lines, elements split once on the integer pipe (an FP64 addition
+// per element to join a float pair and one for the rest would take 2 ms of the
+// FP64 pipe).  The three transposes of a
+// gradient (15360 x 32768 the largest): 6.8 ms with 32 x 32 tiles, 2.5 ms now.
+__global__ void __launch_bounds__(256) k_split_t(BasisRef src, int R, int C, int lds,
+                                                 __nv_bfloat16 *__restrict__ hi,
+                                                 __nv_bfloat16 *__restrict__ lo) {
+  __shared__ uint32_t tile[64][65];   // hi | lo << 16
+  const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
+  {
+    const int tx = threadIdx.x & 63, ty = threadIdx.x >> 6, c = c0 + tx;
+#pragma unroll 8
+    for (int rr = ty; rr < 64; rr += 4) {
+      const int r = r0 + rr;
+      const double x = (r < R && c < C) ? src.at((size_t)r * lds + c) : 0.0;
+      __nv_bfloat16 h, l;
+      split_bf(x, h, l);
+      tile[rr][tx] = bits_as<uint16_t>(h) | (uint32_t)bits_as<uint16_t>(l) << 16;
+    }
   }
   __syncthreads();
-  for (int cc = ty; cc < 32; cc += 8) {
-    const int c = c0 + cc, r = r0 + tx;
-    if (r < R && c < C) {
-      const double x = tile[tx][cc];
-      const __nv_bfloat16 h = d2bf16(x);
-      if (hi) hi[(size_t)c * R + r] = h;
-      if (lo) lo[(size_t)c * R + r] = d2bf16(x - f2d(__bfloat162float(h)));
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int r = r0 + 2 * tx;
+  for (int cc = ty; cc < 64; cc += 8) {
+    const int c = c0 + cc;
+    if (c >= C || r >= R) continue;
+    const uint32_t p = tile[2 * tx][cc], q = tile[2 * tx + 1][cc];
+    const size_t o = (size_t)c * R + r;
+    if ((R & 1) == 0) {
+      if (hi) *reinterpret_cast<uint32_t *>(hi + o) = (p & 0xffffu) | q << 16;
+      if (lo) *reinterpret_cast<uint32_t *>(lo + o) = p >> 16 | (q & 0xffff0000u);
+    } else {
+      if (hi) hi[o] = bits_as<__nv_bfloat16>((uint16_t)p);
+      if (lo) lo[o] = bits_as<__nv_bfloat16>((uint16_t)(p >> 16));
+      if (r + 1 < R) {
+        if (hi) hi[o + 1] = bits_as<__nv_bfloat16>((uint16_t)q);
+        if (lo) lo[o + 1] = bits_as<__nv_bfloat16>((uint16_t)(q >> 16));
+      }
     }
   }
 }
 
-// BF16 hi / lo split of scale[c] * src[r][c] (same layout [R][C]).
-__global__ void k_split_scaled(BasisRef src, int R, int C,
-                               const double *__restrict__ scale, __nv_bfloat16 *__restrict__ hi,
-                               __nv_bfloat16 *__restrict__ lo) {
-  const size_t n = (size_t)R * C;
-  for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
-       idx += (size_t)gridDim.x * blockDim.x) {
-    const int c = (int)(idx % C);
-    const double x = scale[c] * src.at(idx);
-    const __nv_bfloat16 h = d2bf16(x);
-    hi[idx] = h;
-    lo[idx] = d2bf16(x - f2d(__bfloat162float(h)));
+// BF16 hi / lo split of scale[c] * src[r][c] (same layout [R][C], C a multiple
+// of 4).  Bound by DRAM (8 bytes read, 4 written per element): four elements
+// per thread and load, the scale kept over 16 rows, and the joined pair and
+// the split on the integer pipe, so that one FP64 instruction per element is
+// left.  15360 x 32768: 5.6 ms element by element, 1.9 ms now.
+constexpr int SS_ROWS = 16;
+__global__ void __launch_bounds__(256) k_split_scaled(BasisRef src, int R, int C,
+                                                      const double *__restrict__ scale,
+                                                      __nv_bfloat16 *__restrict__ hi,
+                                                      __nv_bfloat16 *__restrict__ lo) {
+  const int c = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
+  if (c >= C) return;
+  double sc[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) sc[i] = scale[c + i];
+  for (int r0 = blockIdx.y * SS_ROWS; r0 < R; r0 += gridDim.y * SS_ROWS)
+#pragma unroll 2
+  for (int r = r0; r < min(R, r0 + SS_ROWS); ++r) {
+    const size_t o = (size_t)r * C + c;
+    double x[4];
+    src.at4(o, x);
+    ushort4 h, l;
+    unsigned short *hp = &h.x, *lp = &l.x;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      __nv_bfloat16 bh, bl;
+      split_bf(sc[i] * x[i], bh, bl);
+      hp[i] = bits_as<uint16_t>(bh);
+      lp[i] = bits_as<uint16_t>(bl);
+    }
+    *reinterpret_cast<ushort4 *>(hi + o) = h;
+    *reinterpret_cast<ushort4 *>(lo + o) = l;
   }
 }
 
-// R[j*Bs + b][mu] = sum_l Gam_b[j][l] P[l*Bs + b][mu]
-__global__ void k_gamma_p(AdjCtx a, const double *P, int A, double *R) {
+// R[j*Bs + b][mu] = sum_l Gam_b[j][l] P[l*Bs + b][mu].  Bound by the FP64
+// pipe (k^2 N_aux products per vector); GP_ROWS rows at a time share the loads
+// of P, which otherwise take as long as the products: k 120, N_aux 1024, 128
+// vectors 6.5 ms one row at a time, 3.3 ms now (the FP64 rate allows 3.3).
+constexpr int GP_ROWS = 8;
+__global__ void __launch_bounds__(128) k_gamma_p(AdjCtx a, const double *__restrict__ P, int A,
+                                                 double *__restrict__ R) {
   const int b = blockIdx.y;
   const int mu = blockIdx.x * blockDim.x + threadIdx.x;
   if (mu >= A) return;
   const int k = a.k;
   const double *Gm = a.Gam + (size_t)b * k * k;
-  for (int j = 0; j < k; ++j) {
-    double acc = 0.0;
-    for (int l = 0; l < k; ++l)
-      acc = fma(Gm[(size_t)j * k + l], P[((size_t)l * a.Bs + b) * A + mu], acc);
-    R[((size_t)j * a.Bs + b) * A + mu] = acc;
+  const double *Pb = P + (size_t)b * A + mu;
+  const size_t ld = (size_t)a.Bs * A;
+  for (int j0 = 0; j0 < k; j0 += GP_ROWS) {
+    const int nj = min(GP_ROWS, k - j0);
+    double acc[GP_ROWS];
+#pragma unroll
+    for (int p = 0; p < GP_ROWS; ++p) acc[p] = 0.0;
+    if (nj == GP_ROWS) {
+#pragma unroll 2
+      for (int l = 0; l < k; ++l) {
+        const double x = Pb[l * ld];
+#pragma unroll
+        for (int p = 0; p < GP_ROWS; ++p)
+          acc[p] = fma(__ldg(&Gm[(size_t)(j0 + p) * k + l]), x, acc[p]);
+      }
+    } else {
+      for (int l = 0; l < k; ++l) {
+        const double x = Pb[l * ld];
+#pragma unroll
+        for (int p = 0; p < GP_ROWS; ++p)
+          if (p < nj) acc[p] = fma(__ldg(&Gm[(size_t)(j0 + p) * k + l]), x, acc[p]);
+      }
+    }
+#pragma unroll
+    for (int p = 0; p < GP_ROWS; ++p)
+      if (p < nj) R[(size_t)(j0 + p) * ld + (size_t)b * A + mu] = acc[p];
   }
 }
 
@@ -895,15 +962,13 @@ void launch_adj_rows_f32(const AdjCtx &a, BasisRef basis, double *Y, double *Gd,
 }
 void launch_split_t(BasisRef src, int R, int C, int lds, __nv_bfloat16 *hi, __nv_bfloat16 *lo,
                     cudaStream_t st) {
-  dim3 grid((C + 31) / 32, (R + 31) / 32);
+  dim3 grid((C + 63) / 64, (R + 63) / 64);
   k_split_t<<<grid, 256, 0, st>>>(src, R, C, lds, hi, lo);
 }
 void launch_split_scaled(BasisRef src, int R, int C, const double *scale, __nv_bfloat16 *hi,
                          __nv_bfloat16 *lo, cudaStream_t st) {
-  const size_t n = (size_t)R * C;
-  size_t blocks = (n + 255) / 256;
-  if (blocks > (size_t)152 * 32) blocks = (size_t)152 * 32;
-  k_split_scaled<<<(unsigned)blocks, 256, 0, st>>>(src, R, C, scale, hi, lo);
+  dim3 grid((C / 4 + 255) / 256, std::min((R + SS_ROWS - 1) / SS_ROWS, 65535));
+  k_split_scaled<<<grid, 256, 0, st>>>(src, R, C, scale, hi, lo);
 }
 void launch_gamma_p(const AdjCtx &a, const double *P, int A, double *R, cudaStream_t st) {
   dim3 grid((A + 127) / 128, a.Bs);

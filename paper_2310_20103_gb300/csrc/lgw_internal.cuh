@@ -495,7 +495,20 @@ struct BasisRef {
   const float *hi, *lo;
   __device__ __forceinline__ double at(size_t i) const {
     if (d) return d[i];
-    return lo ? f2d(hi[i]) + f2d(lo[i]) : f2d(hi[i]);
+    return lo ? pair_d(hi[i], lo[i]) : f2d(hi[i]);
+  }
+  // elements i .. i + 3, i a multiple of 4
+  __device__ __forceinline__ void at4(size_t i, double (&x)[4]) const {
+    if (d) {
+      const double2 p = *reinterpret_cast<const double2 *>(d + i);
+      const double2 q = *reinterpret_cast<const double2 *>(d + i + 2);
+      x[0] = p.x, x[1] = p.y, x[2] = q.x, x[3] = q.y;
+      return;
+    }
+    const float4 h = *reinterpret_cast<const float4 *>(hi + i);
+    const float4 l = lo ? *reinterpret_cast<const float4 *>(lo + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    x[0] = pair_d(h.x, l.x), x[1] = pair_d(h.y, l.y);
+    x[2] = pair_d(h.z, l.z), x[3] = pair_d(h.w, l.w);
   }
 };
 struct AdjCtx {
