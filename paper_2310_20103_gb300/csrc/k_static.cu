@@ -46,39 +46,99 @@ __device__ __forceinline__ double div_from(double x, double s, double r) {
   return fma(fma(-q, s, x), r, q);
 }
 
-// Factor the diagonal block at (j0, j0): one CTA, right-looking by columns,
-// the trailing columns dealt out to 128 threads (row i, columns 2 t, 2 t + 1
-// ...).  A serial chain of 64 columns: 216 us per block with one thread per
-// row and square root, division and row sums in sequence; 109 us now.
-constexpr int POTRF_THREADS = 128;
+// 1 / sqrt(d), 1e-280 < d < 1e280: the hardware's approximation and one cubic
+// Newton step.
+__device__ __forceinline__ double rsqrt_newton(double d) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+  const double e = fma(-d * y, y, 1.0);
+  return fma(y * e, fma(e, 0.375, 0.5), y);
+}
+
+// Factor the diagonal block at (j0, j0): one CTA, columns in panels of eight.
+// A warp's FP64 instruction holds its scheduler's pipe for 76 clocks whatever
+// the lanes do, so the count of instructions per warp is what bounds the serial
+// chain of 64 columns.  Every warp factors the panel's eight diagonal rows
+// (lanes 0..7) along with a quarter of the rows below (lanes 8..), by shuffles
+// and without barriers; then the panel updates the rest of the block, row i and
+// row 63 - i dealt together to the same threads.  216 us per block with one
+// thread per row and square root, division and row sums in sequence, 109 us
+// column by column with three barriers each, 75 us now.
+constexpr int POTRF_THREADS = 128, PW = 8;
 
 __global__ void __launch_bounds__(POTRF_THREADS) k_potrf_diag(double *A, int n, int j0,
                                                               unsigned *status) {
   __shared__ double blk[NB][NB + 1];
-  const int t = threadIdx.x, i = t & (NB - 1), half = t / NB;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int nb = min(NB, n - j0);
   for (int idx = t; idx < NB * NB; idx += POTRF_THREADS) {
     const int r = idx / NB, c = idx % NB;
-    blk[r][c] = r < nb && c <= r ? A[(size_t)(j0 + r) * n + j0 + c] : 0.0;
+    // past the matrix: the identity, which leaves the rest as it is
+    blk[r][c] = r < nb ? (c <= r ? A[(size_t)(j0 + r) * n + j0 + c] : 0.0) : (r == c ? 1.0 : 0.0);
   }
   __syncthreads();
-  for (int j = 0; j < nb; ++j) {
-    double d = blk[j][j];
-    if (!(d > 0.0)) {
-      if (t == 0) atomicOr(status, ST_NOT_SPD);
-      d = 1.0;
+#pragma unroll 1
+  for (int p0 = 0; p0 < nb; p0 += PW) {
+    const int below = NB - p0 - PW, quarter = (below + 3) / 4;   // rows under the panel, per warp
+    const int row = lane < PW ? p0 + lane : p0 + PW + w * quarter + lane - PW;
+    const bool mine = lane < PW || (lane - PW < quarter && row < NB);
+    double v[PW];
+#pragma unroll
+    for (int c = 0; c < PW; ++c) v[c] = mine ? blk[row][p0 + c] : 0.0;
+#pragma unroll
+    for (int j = 0; j < PW; ++j) {
+      double d = __shfl_sync(0xffffffffu, v[j], j);
+      if (!(d > 0.0)) {
+        if (t == 0) atomicOr(status, ST_NOT_SPD);
+        d = 1.0;
+      }
+      double x, s;
+      if (d > 1e-280 && d < 1e280) {
+        const double r = rsqrt_newton(d);
+        s = sqrt_from(d, r);
+        x = div_from(v[j], s, r);
+      } else {   // infinities too
+        s = sqrt(d);
+        x = v[j] / s;
+      }
+      v[j] = lane == j ? s : x;
+#pragma unroll
+      for (int c = j + 1; c < PW; ++c) {
+        const double l = __shfl_sync(0xffffffffu, v[j], c);
+        v[c] = fma(-v[j], l, v[c]);
+      }
     }
-    const bool plain = !(d > 1e-280 && d < 1e280);   // and infinities
-    const double r = rsqrt(d), s = plain ? sqrt(d) : sqrt_from(d, r);
-    const double x = i > j ? (plain ? blk[i][j] / s : div_from(blk[i][j], s, r)) : 0.0;
-    __syncthreads();   // every thread has read column j
-    if (half == 0 && i >= j) blk[i][j] = i == j ? s : x;
+    __syncthreads();   // every warp has read the diagonal rows
+    if (mine && (w == 0 || lane >= PW)) {
+#pragma unroll
+      for (int c = 0; c < PW; ++c)
+        if (p0 + c <= row) blk[row][p0 + c] = v[c];
+    }
     __syncthreads();
-    // row i, the columns c of this thread's parity
-    if (i > j)
-      for (int c = j + 1 + ((j + 1 + half) & 1); c <= i; c += 2)
-        blk[i][c] = fma(-x, blk[c][j], blk[i][c]);
-    __syncthreads();
+    if (below > 0) {
+      // rows p0 + 8 + m and 63 - m, each up to its diagonal: together below + 1
+      // elements, dealt to `per` threads
+      int per = 4;
+      while (2 * per * (below / 2) <= POTRF_THREADS) per *= 2;
+      const int m = t / per, l = t % per;
+      if (m < below / 2) {
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          const int i = hf ? NB - 1 - m : p0 + PW + m;
+          double li[PW];
+#pragma unroll
+          for (int p = 0; p < PW; ++p) li[p] = blk[i][p0 + p];
+#pragma unroll 1
+          for (int c = p0 + PW + l; c <= i; c += per) {
+            double x = blk[i][c];
+#pragma unroll
+            for (int p = 0; p < PW; ++p) x = fma(-li[p], blk[c][p0 + p], x);
+            blk[i][c] = x;
+          }
+        }
+      }
+      __syncthreads();
+    }
   }
   for (int idx = t; idx < NB * NB; idx += POTRF_THREADS) {
     const int r = idx / NB, c = idx % NB;
