@@ -17,11 +17,15 @@
 // (tests/test_gpu_f64_products.py; against exact sums, B = C R with 1024 terms
 // errs by 2.6e-16 of its norm, the FP64 FMA chain by 1.08e-15).
 //
-// N_vc 32768, N_aux 1024, 64 vectors: L^T x 207 us and L y 272 us, against 3.6
-// and 4.1 ms on the FP64 pipe (2 x 32768 x 1024 x 64 flops: 20 TFLOP/s in FP64
-// terms).  The tensor pipe is 37% busy there, DRAM at 2.6 TB/s: an MMA of few
-// columns costs more than its share, and a tile's sums are joined with the
-// tensor pipe idle (TMEM holds one tile).
+// N_vc 32768, N_aux 1024, 64 vectors: 180 us per product on average (C x with
+// its digits 474 us), against 3.6 and 4.1 ms on the FP64 pipe (24 TFLOP/s in
+// FP64 terms).  Where a tile of L y spends its time: 73 us in the products
+// (43 per K block, 19 MMAs of 64 to 256 columns per 16 terms, 63% of the BF16
+// rate: an MMA of few columns costs more than its share) and then the joined
+// sums with the tensor pipe idle (TMEM holds one tile).  These took 60 us with
+// four warps, a memory round trip per column and the conversions on the FP64
+// pipe (244 us per product); now eight warps issue all loads of eight columns
+// first and convert on the integer pipe.
 //
 // Layout: digits as BF16, [slice][K block of 64][row][64], so a TMA box (64
 // elements by rows) is one contiguous run, as for the other contractions.  A
@@ -38,6 +42,7 @@
 #include <algorithm>
 #include <cstdio>
 
+#include "fp_bits.cuh"
 #include "oz_digits.cuh"
 #include "tc_ptx.cuh"
 
@@ -49,7 +54,8 @@ using namespace tc;
 constexpr int BM = 128;
 constexpr int KB = 64;          // K elements per block: one 128-byte swizzle row
 constexpr int CHUNK_KB = 16;    // 1024 terms per exact sum
-constexpr int NTHREADS = 192;
+constexpr int EPI_WARPS = 8;    // two per TMEM lane quarter, each half of the columns
+constexpr int NTHREADS = 64 + 32 * EPI_WARPS;
 
 template <int NT>
 struct Cfg {
@@ -82,31 +88,23 @@ __device__ __forceinline__ void tmem_ld_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-__device__ __forceinline__ int hi_abs(double p) { return __double2hiint(p) & 0x7fffffff; }
-
-// d * 2^sh for a finite d: on the exponent field while argument and result
-// are normal (FP64 multiplications load the narrow FP64 pipe).
-__device__ __forceinline__ double scale_pow2(double d, int sh) {
-  const int hi = __double2hiint(d), f = ((hi >> 20) & 0x7ff) + sh;
-  if (d == 0.0) return 0.0;
-  if (f >= 1 && f <= 2046 && (hi & 0x7ff00000) != 0) return __hiloint2double(hi + (sh << 20), __double2loint(d));
-  return scalbn(d, sh);
-}
-
-// sum_t 2^(40 - 7t) S_t from the weighted sums s[t] = 2^(-7t) S_t: a 64-bit
-// integer below 2^62.3 in magnitude, and what is left below its unit where the
-// double has room for it.
-__device__ __forceinline__ double join_sums(const float (&s)[8]) {
+// 2^sh sum_t 2^(40 - 7t) S_t from the weighted sums s[t] = 2^(-7t) S_t: a 64-bit
+// integer below 2^62.3 in magnitude, seven more bits of what lies below its
+// unit where a double has room for them, one rounding.  On the integer pipe
+// throughout (the FP64 pipe's conversions run at 2 lanes per SM clock).
+__device__ __forceinline__ double join_sums(const float (&s)[8], int sh) {
   const int h = __float2int_rn(s[0]) * 128 + __float2int_rn(s[1] * 0x1p+7f);
   const int g = __float2int_rn(s[2] * 0x1p+14f) * 128 + __float2int_rn(s[3] * 0x1p+21f);
   const float low = (s[6] + s[7]) * 0x1p+40f;
   const int il = __float2int_rn(low);
   const int f = __float2int_rn(s[5] * 0x1p+35f) * 32 + il;
-  const long long t = ((long long)h << 33) + (long long)g * (1 << 19) +
-                      (long long)__float2int_rn(s[4] * 0x1p+28f) * 4096 + f;
-  double d = __ll2double_rn(t);
-  if (hi_abs(d) < ((1023 + 55) << 20)) d += (double)(low - (float)il);
-  return d;
+  long long t = ((long long)h << 33) + (long long)g * (1 << 19) +
+                (long long)__float2int_rn(s[4] * 0x1p+28f) * 4096 + f;
+  if (t + (1LL << 55) >= 0 && t < (1LL << 55)) {
+    t = t * 128 + __float2int_rn((low - (float)il) * 128.0f);
+    sh -= 7;
+  }
+  return ll2d_scaled(t, sh);
 }
 
 // out[col * ldo + row] of the tile's products; the epilogues of the FP64
@@ -162,7 +160,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       mbar_init(&bempty[s], 1);
     }
     mbar_init(tfull, 1);
-    mbar_init(tempty, 4);   // one arrival per epilogue warp
+    mbar_init(tempty, EPI_WARPS);
     mbar_init(mdone, 1);
     fence_barrier_init();
   }
@@ -251,12 +249,15 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     }
   } else {
     // ------------------------------ epilogue ------------------------------
-    const int qd = warp & 3;
+    // warp & 3 is the TMEM lane quarter a warp can read
+    const int qd = warp & 3, half = (warp - 2) >> 2;
     const int row = m_tile * BM + qd * 32 + lane;
     const bool rok = row < M;
     const int fa = rok ? e.ea[row] : 1;
+    const bool with_q = e.mode == OZ_LANCZOS || e.mode == OZ_APPLY;
+    const bool with_prev = e.mode == OZ_LANCZOS && e.qprev != nullptr;
     double d2 = 0.0, cdr = 0.0;
-    if (rok && (e.mode == OZ_LANCZOS || e.mode == OZ_APPLY)) {
+    if (rok && with_q) {
       d2 = e.Delta2[row];
       cdr = e.cd[row];
     } else if (rok && e.mode == OZ_START) {
@@ -267,50 +268,68 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       if (!mbar_wait(tfull, c & 1, e.status)) break;
       tc_fence_after();
       const bool last = c + 1 == chunks;
+      const bool add_old = c > 0 || e.mode == OZ_ADD;
 #pragma unroll 1
-      for (int c8 = 0; c8 < NT; c8 += 8) {
+      for (int c8 = half * (NT / 2); c8 < (half + 1) * (NT / 2); c8 += 8) {
         const int col0 = n_tile * NT + c8;
-        const uint32_t tc0 = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)c8;
         if (col0 >= Ncols) break;
+        const uint32_t tc0 = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)c8;
         float s[S][8];
 #pragma unroll
         for (int t = 0; t < S; ++t)
           tmem_ld8(tc0 + (uint32_t)(t * NT), s[t]);
-        tmem_ld_wait();
-        double part[8];
+        // everything the eight columns need from memory, before the first use
+        double old[8], qv[8], qp[8];
+        int fb[8];
+        double *o = out + (size_t)col0 * e.ldo + row;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          const int col = col0 + i;
-          part[i] = 0.0;
-          if (!rok || col >= Ncols) continue;
-          const int fb = e.eb[col];
+          const bool ok = rok && col0 + i < Ncols;
+          const size_t oi = (size_t)(col0 + i) * e.ldo + row;
+          fb[i] = ok ? e.eb[col0 + i] : 1;
+          old[i] = ok && add_old ? o[(size_t)i * e.ldo] : 0.0;
+          qv[i] = ok && last && with_q ? e.q[oi] : 0.0;
+          qp[i] = ok && last && with_prev ? e.qprev[oi] : 0.0;
+        }
+        tmem_ld_wait();
+#pragma unroll
+        for (int t = 0; t < S; ++t)
+#pragma unroll
+          for (int i = 0; i < 8; ++i) asm volatile("" : "+f"(s[t][i]));   // no use before the wait
+        double v[8], part[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
           float v8[S];
 #pragma unroll
           for (int t = 0; t < S; ++t) v8[t] = s[t][i];
           // row scales 2^(field - 1022); a non-finite row gives NaN
-          double v = (fa >= 2047 || fb >= 2047)
-                         ? __longlong_as_double(0x7ff8000000000000LL)
-                         : scale_pow2(join_sums(v8), max(fa, 1) + max(fb, 1) - 2044 - 52);
-          double *o = out + (size_t)col * e.ldo + row;
-          if (e.mode == OZ_ADD) {
-            *o = fma(e.scale, v, *o);
-            continue;
+          v[i] = join_sums(v8, max(fa, 1) + max(fb[i], 1) - 2044 - 52);
+          if (fa >= 2047 || fb[i] >= 2047) v[i] = __longlong_as_double(0x7ff8000000000000LL);
+          part[i] = 0.0;
+        }
+        if (e.mode == OZ_ADD) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) v[i] = fma(e.scale, v[i], old[i]);
+        } else {
+          if (c > 0) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] += old[i];
           }
-          if (c > 0) v += *o;
-          if (!last || e.mode == OZ_PART) {
-            *o = v;
-          } else if (e.mode == OZ_START) {
-            *o = cdr * v;
-          } else {
-            const size_t oi = (size_t)col * e.ldo + row;
-            const double qv = e.q[oi];
-            double w = fma(d2, qv, cdr * v);
-            if (e.mode == OZ_LANCZOS && e.qprev != nullptr)
-              w = fma(-e.betaj[col], e.qprev[oi], w);
-            *o = w;
-            part[i] = qv * w;
+          if (last && e.mode == OZ_START) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = cdr * v[i];
+          } else if (last && with_q) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              v[i] = fma(d2, qv[i], cdr * v[i]);
+              if (with_prev) v[i] = fma(-(col0 + i < Ncols ? e.betaj[col0 + i] : 0.0), qp[i], v[i]);
+              part[i] = rok ? qv[i] * v[i] : 0.0;
+            }
           }
         }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (rok && col0 + i < Ncols) o[(size_t)i * e.ldo] = v[i];
         if (e.alpha_part != nullptr && last) {
           // the eight columns' sums over the warp's rows: a transposed
           // butterfly (lane bits 2..0 pick the column), then bits 3 and 4
@@ -334,12 +353,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       if (lane == 0) mbar_arrive(tempty);
     }
     if (e.alpha_part != nullptr && chunks > 0) {
-      asm volatile("bar.sync 1, 128;" ::: "memory");
-      for (int i = threadIdx.x - 64; i < 2 * NT; i += 128) {
-        const int half = i / NT, col = i % NT, b = n_tile * NT + col;
-        if (b < Ncols && m_tile * BM + 64 * half < M)
-          e.alpha_part[(size_t)(2 * m_tile + half) * Ncols + b] =
-              red[2 * half][col] + red[2 * half + 1][col];
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      for (int i = threadIdx.x - 64; i < 2 * NT; i += 32 * EPI_WARPS) {
+        const int hf = i / NT, col = i % NT, b = n_tile * NT + col;
+        if (b < Ncols && m_tile * BM + 64 * hf < M)
+          e.alpha_part[(size_t)(2 * m_tile + hf) * Ncols + b] =
+              red[2 * hf][col] + red[2 * hf + 1][col];
       }
     }
   }
