@@ -11,8 +11,7 @@
 //
 // Why: as ten kernels of this step, w went through memory at each, a vector
 // of one or two chunks kept one warp of a block busy (elements were dealt out
-// 256 to a warp), and launches cost as much as the work: N_vc 256, 160
-// vectors, k 64, CGS2: STEP_TINY per step.  Elements are dealt out 512 to
+// 256 to a warp), and launches cost as much as the work.  Elements are dealt out 512 to
 // the block, so a short vector spreads over all four FP64 units of an SM.
 // What bounds it now: the FP64 pipe (2 operations per element, row and pass).
 #include <cooperative_groups.h>
@@ -29,18 +28,27 @@ constexpr int SE = 4;   // element pairs per thread
 __device__ __forceinline__ int pair_elem(int chunk, int u) {
   return chunk * VEC_CHUNK + u * (2 * VEC_THREADS) + 2 * (int)threadIdx.x;
 }
+// How many of a warp's SE pairs per thread lie inside the vector.  Operations
+// on the zeros past its end would take their share of the FP64 pipe: N_vc 256
+// leaves four of a block's eight warps empty (160 vectors, k 64, CGS2: 65 us
+// per step with them at work, 42 us without).
+__device__ __forceinline__ int warp_pairs(int N, int chunk, int warp) {
+  const int left = N - chunk * VEC_CHUNK - 64 * warp;
+  return max(0, min(SE, (left + 2 * VEC_THREADS - 1) / (2 * VEC_THREADS)));
+}
 
 // RB rows from row r0 on (the last one again past the end), NU pairs per
 // thread, loaded before any of them is used: the loads of a batch overlap
 // (one row at a time a row costs an L2 round trip).
 template <int NU, int RB>
 __device__ __forceinline__ void load_rows(const VecCtx &c, int r0, int nrows, size_t voff,
-                                          int chunk, double2 (&q)[RB][NU]) {
+                                          int chunk, int nu, double2 (&q)[RB][NU]) {
 #pragma unroll
   for (int r = 0; r < RB; ++r) {
     const double *row = slot_ptr(c, min(r0 + r, nrows - 1)) + voff;
 #pragma unroll
     for (int u = 0; u < NU; ++u) {
+      if (u >= nu) break;
       const int e = pair_elem(chunk, u);
       q[r][u] = e < c.N ? *reinterpret_cast<const double2 *>(row + e) : make_double2(0.0, 0.0);
     }
@@ -50,47 +58,52 @@ __device__ __forceinline__ void load_rows(const VecCtx &c, int r0, int nrows, si
 // Dots of the block's chunk of w with rows 0..nrows-1 into part[0..nrows),
 // 16 rows per reduction.
 template <int NU>
-__device__ void step_dots(const VecCtx &c, int nrows, int b, int chunk, const double2 (&w)[SE],
-                          double (*sred)[16], double *part) {
+__device__ void step_dots(const VecCtx &c, int nrows, int b, int chunk, int nu,
+                          const double2 (&w)[SE], double (*sred)[16], double *part) {
   constexpr int RB = NU == 1 ? 8 : 4;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  // the warps of the chunk that hold elements
+  const int nw = min(VEC_THREADS / 32, (c.N - chunk * VEC_CHUNK + 63) / 64);
   const size_t voff = (size_t)b * c.N;
   for (int r0 = 0; r0 < nrows; r0 += 16) {
-    double acc[16];
+    if (nu > 0) {
+      double acc[16];
 #pragma unroll
-    for (int r = 0; r < 16; ++r) acc[r] = 0.0;
+      for (int r = 0; r < 16; ++r) acc[r] = 0.0;
 #pragma unroll
-    for (int rb = 0; rb < 16; rb += RB) {
-      if (r0 + rb < nrows) {
-        double2 q[RB][NU];
-        load_rows<NU, RB>(c, r0 + rb, nrows, voff, chunk, q);
-#pragma unroll
-        for (int r = 0; r < RB; ++r)
+      for (int rb = 0; rb < 16; rb += RB) {
+        if (r0 + rb < nrows) {
+          double2 q[RB][NU];
+          load_rows<NU, RB>(c, r0 + rb, nrows, voff, chunk, nu, q);
 #pragma unroll
           for (int u = 0; u < NU; ++u) {
-            acc[rb + r] = fma(q[r][u].x, w[u].x, acc[rb + r]);
-            acc[rb + r] = fma(q[r][u].y, w[u].y, acc[rb + r]);
+            if (u >= nu) break;
+#pragma unroll
+            for (int r = 0; r < RB; ++r) {
+              acc[rb + r] = fma(q[r][u].x, w[u].x, acc[rb + r]);
+              acc[rb + r] = fma(q[r][u].y, w[u].y, acc[rb + r]);
+            }
           }
+        }
       }
-    }
-    // transposed butterfly: lane l ends with row l % 16, then the two halves
+      // transposed butterfly: lane l ends with row l % 16, then the two halves
 #pragma unroll
-    for (int off = 8; off >= 1; off >>= 1) {
-      const bool up = (lane & off) != 0;
+      for (int off = 8; off >= 1; off >>= 1) {
+        const bool up = (lane & off) != 0;
 #pragma unroll
-      for (int i = 0; i < off; ++i) {
-        const double send = up ? acc[i] : acc[i + off];
-        const double keep = up ? acc[i + off] : acc[i];
-        acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        for (int i = 0; i < off; ++i) {
+          const double send = up ? acc[i] : acc[i + off];
+          const double keep = up ? acc[i + off] : acc[i];
+          acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
       }
+      acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 16);
+      if (lane < 16) sred[wid][lane] = acc[0];
     }
-    acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 16);
-    if (lane < 16) sred[wid][lane] = acc[0];
     __syncthreads();
     if (threadIdx.x < 16 && r0 + (int)threadIdx.x < nrows) {
       double s = 0.0;
-#pragma unroll
-      for (int w8 = 0; w8 < VEC_THREADS / 32; ++w8) s += sred[w8][threadIdx.x];
+      for (int w8 = 0; w8 < nw; ++w8) s += sred[w8][threadIdx.x];
       part[r0 + threadIdx.x] = s;
     }
     __syncthreads();
@@ -99,19 +112,21 @@ __device__ void step_dots(const VecCtx &c, int nrows, int b, int chunk, const do
 
 // w <- w - sum_i h_i q_i; returns this thread's share of ||w||^2.
 template <int NU>
-__device__ double step_update(const VecCtx &c, int nrows, int b, int chunk, double2 (&w)[SE],
-                              const double *h) {
+__device__ double step_update(const VecCtx &c, int nrows, int b, int chunk, int nu,
+                              double2 (&w)[SE], const double *h) {
   constexpr int RB = NU == 1 ? 8 : 4;
   const size_t voff = (size_t)b * c.N;
+  if (nu == 0) return 0.0;
   for (int i = 0; i < nrows; i += RB) {
     double2 q[RB][NU];
-    load_rows<NU, RB>(c, i, nrows, voff, chunk, q);
+    load_rows<NU, RB>(c, i, nrows, voff, chunk, nu, q);
 #pragma unroll
-    for (int r = 0; r < RB; ++r) {
-      if (i + r >= nrows) break;
-      const double hi = h[i + r];
+    for (int u = 0; u < NU; ++u) {
+      if (u >= nu) break;
 #pragma unroll
-      for (int u = 0; u < NU; ++u) {
+      for (int r = 0; r < RB; ++r) {
+        if (i + r >= nrows) break;
+        const double hi = h[i + r];
         w[u].x = fma(-hi, q[r][u].x, w[u].x);
         w[u].y = fma(-hi, q[r][u].y, w[u].y);
       }
@@ -119,7 +134,8 @@ __device__ double step_update(const VecCtx &c, int nrows, int b, int chunk, doub
   }
   double nrm = 0.0;
 #pragma unroll
-  for (int u = 0; u < NU; ++u) nrm = fma(w[u].x, w[u].x, fma(w[u].y, w[u].y, nrm));
+  for (int u = 0; u < NU; ++u)
+    if (u < nu) nrm = fma(w[u].x, w[u].x, fma(w[u].y, w[u].y, nrm));
   return nrm;
 }
 
@@ -153,18 +169,19 @@ __global__ void __launch_bounds__(VEC_THREADS, GS ? 2 : 4)
     return;
   }
   const int nrows = j + 1;
+  const int nu = warp_pairs(c.N, chunk, threadIdx.x >> 5);
   // at most 512 elements: one pair per thread (the others' operations would
   // each take their share of the FP64 pipe)
   const bool one = c.N <= 2 * VEC_THREADS;
   auto dots = [&](const double2 (&x)[SE], double *out) {
     if (one)
-      step_dots<1>(c, nrows, b, chunk, x, sred, out);
+      step_dots<1>(c, nrows, b, chunk, nu, x, sred, out);
     else
-      step_dots<SE>(c, nrows, b, chunk, x, sred, out);
+      step_dots<SE>(c, nrows, b, chunk, nu, x, sred, out);
   };
   auto update = [&](double2 (&x)[SE], const double *co) {
-    return one ? step_update<1>(c, nrows, b, chunk, x, co)
-               : step_update<SE>(c, nrows, b, chunk, x, co);
+    return one ? step_update<1>(c, nrows, b, chunk, nu, x, co)
+               : step_update<SE>(c, nrows, b, chunk, nu, x, co);
   };
   double *h1 = dyn, *h2 = dyn + c.kmax1, *h = dyn + 2 * c.kmax1;
   // ||w||^2 over the cluster from part[i] of every block
@@ -189,6 +206,7 @@ __global__ void __launch_bounds__(VEC_THREADS, GS ? 2 : 4)
   for (int u = 0; u < SE; ++u) {
     const int e = pair_elem(chunk, u);
     w[u] = make_double2(0.0, 0.0);
+    if (u >= nu) continue;
     if (e < c.N) {
       const double2 q2 = *reinterpret_cast<const double2 *>(qj + e);
       w[u] = *reinterpret_cast<const double2 *>(c.w + voff + e);
