@@ -335,7 +335,7 @@ __device__ __forceinline__ void alpha_axpy_chunk(const VecCtx &c, int j, int chu
     wr[2 * u + 1] = w2.y;
     nrm = fma(w2.x, w2.x, fma(w2.y, w2.y, nrm));
   }
-  nrm = block_sum(nrm, red);
+  nrm = block_sum_to0(nrm, red);
   if (threadIdx.x == 0) c.norm_a[(size_t)b * c.nchunks + chunk] = nrm;
   if constexpr (DOTS) dots_rows(c, j + 1, b, chunk, wr, sred);
 }
@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_update(VecCtx c, int j, int pas
     if (e < c.N) *reinterpret_cast<double2 *>(w + e) = wv[u];
     nrm = fma(wv[u].x, wv[u].x, fma(wv[u].y, wv[u].y, nrm));
   }
-  nrm = block_sum(nrm, red);
+  nrm = block_sum_to0(nrm, red);
   if (threadIdx.x == 0) (pass == 1 ? c.norm_b : c.norm_c)[(size_t)b * c.nchunks + chunk] = nrm;
 }
 
@@ -586,7 +586,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_start_from_v(VecCtx c, const do
     c.w[voff + e + 1] = x1;
     nrm = fma(x0, x0, fma(x1, x1, nrm));
   }
-  nrm = block_sum(nrm, red);
+  nrm = block_sum_to0(nrm, red);
   if (threadIdx.x == 0) c.norm_a[(size_t)b * c.nchunks + chunk] = nrm;
 }
 
@@ -611,7 +611,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_start_from_vf(VecCtx c, const f
     *reinterpret_cast<double2 *>(c.w + voff + e) = make_double2(x0, x1);
     nrm = fma(x0, x0, fma(x1, x1, nrm));
   }
-  nrm = block_sum(nrm, red);
+  nrm = block_sum_to0(nrm, red);
   if (threadIdx.x == 0) c.norm_a[(size_t)b * c.nchunks + chunk] = nrm;
 }
 
@@ -629,7 +629,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_norm_partials(VecCtx c, const d
     const double2 x2 = *reinterpret_cast<const double2 *>(x + voff + e);
     nrm = fma(x2.x, x2.x, fma(x2.y, x2.y, nrm));
   }
-  nrm = block_sum(nrm, red);
+  nrm = block_sum_to0(nrm, red);
   if (threadIdx.x == 0) out[(size_t)b * c.nchunks + chunk] = nrm;
 }
 
@@ -745,7 +745,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_band_dots(BandCtx bc, int pass)
     nrm = fma(w2.x, w2.x, fma(w2.y, w2.y, nrm));
   }
   if (pass == 1) {
-    nrm = block_sum(nrm, red);
+    nrm = block_sum_to0(nrm, red);
     if (threadIdx.x == 0) c.norm_a[(size_t)b * c.nchunks + chunk] = nrm;
   }
   dots_rows(c, bc.nv[b], b, chunk, wr, sred);
@@ -795,7 +795,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_band_update(BandCtx bc, int pas
     if (e < c.N) *reinterpret_cast<double2 *>(w + e) = wv[u];
     nrm = fma(wv[u].x, wv[u].x, fma(wv[u].y, wv[u].y, nrm));
   }
-  nrm = block_sum(nrm, red);
+  nrm = block_sum_to0(nrm, red);
   if (threadIdx.x == 0) (pass == 1 ? c.norm_b : c.norm_c)[(size_t)b * c.nchunks + chunk] = nrm;
 }
 

@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_dots_split(VecCtx c, int j) 
     split_d(w2.y, swh[le + 1], swl[le + 1]);
   }
   if (PASS == 1) {
-    nrm = block_sum(nrm, red);   // contains a __syncthreads
+    nrm = block_sum_to0(nrm, red);   // contains a __syncthreads
     if (threadIdx.x == 0) c.norm_a[(size_t)b * c.nchunks + chunk] = nrm;
   } else {
     __syncthreads();
@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_update_split(VecCtx c, int j) {
       *reinterpret_cast<double2 *>(w + e) = w2;
       nrm = fma(w2.x, w2.x, fma(w2.y, w2.y, nrm));
     }
-    nrm = block_sum(nrm, red);
+    nrm = block_sum_to0(nrm, red);
     if (threadIdx.x == 0) c.norm_b[(size_t)b * c.nchunks + chunk] = nrm;
     return;
   }
