@@ -96,6 +96,19 @@ __global__ void k_quantize_L8(const double *__restrict__ src, int ld, int nr, in
   }
 }
 
+// Eight BF16 values times inv in E4M3.
+__device__ __forceinline__ uint2 quant8(const uint4 &v, float inv) {
+  const __nv_bfloat162 *p2 = reinterpret_cast<const __nv_bfloat162 *>(&v);
+  uint32_t wq[2] = {0u, 0u};
+#pragma unroll
+  for (int t = 0; t < 4; ++t) {
+    const float2 f = __bfloat1622float2(p2[t]);
+    const uint32_t lo = to_e4m3(f.x * inv), hi = to_e4m3(f.y * inv);
+    wq[t >> 1] |= (lo | (hi << 8)) << (16 * (t & 1));
+  }
+  return make_uint2(wq[0], wq[1]);
+}
+
 // x8[b] = e4m3(xh[b] / s_b), s_b from max |xh[b]|; one block per vector.
 // Both operands are K-block-major over Bs rows.
 __global__ void __launch_bounds__(256) k_quant_x8(const __nv_bfloat16 *__restrict__ xh, int Bs,
@@ -135,16 +148,24 @@ __global__ void __launch_bounds__(256) k_quant_x8(const __nv_bfloat16 *__restric
   const float inv = 1.0f / sc;   // a power of two: exact
   for (int g = threadIdx.x; g < N / 8; g += 256) {
     const uint4 v = *reinterpret_cast<const uint4 *>(xh + kblk_bf16(b, 8 * g, Bs));
-    const __nv_bfloat162 *p2 = reinterpret_cast<const __nv_bfloat162 *>(&v);
-    uint32_t wq[2] = {0u, 0u};
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const float2 f = __bfloat1622float2(p2[t]);
-      const uint32_t lo = to_e4m3(f.x * inv), hi = to_e4m3(f.y * inv);
-      wq[t >> 1] |= (lo | (hi << 8)) << (16 * (t & 1));
-    }
-    *reinterpret_cast<uint2 *>(x8 + kblk_e4m3(b, 8 * g, Bs)) = make_uint2(wq[0], wq[1]);
+    *reinterpret_cast<uint2 *>(x8 + kblk_e4m3(b, 8 * g, Bs)) = quant8(v, inv);
   }
+}
+
+
+// The same where the pass that made xh has left its maximum: one read of xh,
+// spread over the chip (N_vc 400000, 512 vectors: 180 us with a block per
+// vector and two reads, 129 us).
+__global__ void __launch_bounds__(256) k_quant_x8_max(const __nv_bfloat16 *__restrict__ xh, int Bs,
+                                                      int N, const unsigned *__restrict__ xmax,
+                                                      uint8_t *__restrict__ x8,
+                                                      float *__restrict__ sx) {
+  const int b = blockIdx.x, g = blockIdx.y * 256 + threadIdx.x;
+  const float sc = pow2_scale(__uint_as_float(xmax[b])), inv = 1.0f / sc;
+  if (g == 0) sx[b] = sc;
+  if (g >= N / 8) return;
+  const uint4 v = *reinterpret_cast<const uint4 *>(xh + kblk_bf16(b, 8 * g, Bs));
+  *reinterpret_cast<uint2 *>(x8 + kblk_e4m3(b, 8 * g, Bs)) = quant8(v, inv);
 }
 
 // From the split-K partials of gemm1: y_mu = s_b s_mu sum_p Ypart, then
@@ -319,6 +340,11 @@ void launch_prepare_fp8(const double *src, int ld, int nr, int nc, const SysDev 
   k_col_scales<<<(s.A + 255) / 256, 256, 0, st>>>(colmax, s.A, sL);
   k_quantize_L8<<<dim3((s.A + 31) / 32, (s.N + 31) / 32), 256, 0, st>>>(src, ld, nr, nc, s.N, s.A,
                                                                         sL, L8, L8t);
+}
+
+void launch_quant_x8_max(const __nv_bfloat16 *xh, int Bs, int N, const unsigned *xmax, uint8_t *x8,
+                         float *sx, cudaStream_t st) {
+  k_quant_x8_max<<<dim3(Bs, (N / 8 + 255) / 256), 256, 0, st>>>(xh, Bs, N, xmax, x8, sx);
 }
 
 void launch_quant_x8(const __nv_bfloat16 *xh, int Bs, int N, uint8_t *x8, float *sx,

@@ -23,6 +23,11 @@ __device__ __forceinline__ int elem_base(int chunk) {
   return chunk * VEC_CHUNK + wid * 256 + 2 * lane;
 }
 
+// the same with four consecutive elements per lane, twice (128 apart)
+__device__ __forceinline__ int elem_base4(int chunk) {
+  return chunk * VEC_CHUNK + (threadIdx.x >> 5) * 256 + 4 * (threadIdx.x & 31);
+}
+
 __device__ __forceinline__ bool vec_live(const VecCtx &c, int b, int j) {
   return b < c.nvec && c.k_eff[c.vec0 + b] > j;
 }
@@ -83,6 +88,18 @@ __device__ __forceinline__ float *pair_hi(double *slot, const VecCtx &c) {
 }
 __device__ __forceinline__ float *pair_lo(double *slot, const VecCtx &c) {
   return reinterpret_cast<float *>(slot) + (size_t)c.Bs * c.N;
+}
+// A slot holds its vector unnormalised: 1 / beta_j, which normalises slot j of
+// vector b, is applied by each pass that reads it (a double-float product per
+// element), so that the normalisation writes the contractions' operand only.
+// The passes are bound by DRAM: 28 + 24 + 10 bytes per element and step against
+// 28 + 24 + 18.  N_vc 400000, 512 vectors: assembly 795 -> 826 us, axpy 730 ->
+// 719, normalisation 612 -> 428.  (Forming w twice instead of storing it, 20 +
+// 28 + 10 bytes, gave 699 + 1029 + 427; one cluster per vector with w in shared
+// memory 4100 us in all.)
+__device__ __forceinline__ dfl pair_scale(const VecCtx &c, int j, int b) {
+  const float2 t = c.qscale[(size_t)(j % 3) * c.Bs + b];
+  return {t.x, t.y};
 }
 
 // Four basis rows from row r0 on (the last one again past the end), all loads
@@ -188,7 +205,8 @@ __device__ __forceinline__ void assemble_w_chunk(const VecCtx &c, int j,
     const float *qh = pair_hi(slot_ptr(c, j), c) + voff, *ql = pair_lo(slot_ptr(c, j), c) + voff;
     const float *ph = j > 0 ? pair_hi(slot_ptr(c, j - 1), c) + voff : nullptr;
     const float *pl = j > 0 ? pair_lo(slot_ptr(c, j - 1), c) + voff : nullptr;
-    float *wh = pair_hi(c.w, c) + voff, *wl = pair_lo(c.w, c) + voff;
+    float *wh = pair_hi(slot_ptr(c, j + 1), c) + voff, *wl = pair_lo(slot_ptr(c, j + 1), c) + voff;
+    const dfl sq = pair_scale(c, j, b), sp = j > 0 ? pair_scale(c, j - 1, b) : dfl{0.f, 0.f};
     const dfl nbj = (j > 0 && c.nbeta_f) ? dfl{c.nbeta_f[b].x, c.nbeta_f[b].y} : df_from(-bj);
     float sh = 0.f, sl = 0.f;
 #pragma unroll
@@ -205,12 +223,12 @@ __device__ __forceinline__ void assemble_w_chunk(const VecCtx &c, int j,
         p2 = *reinterpret_cast<const float2 *>(ph + e);
         r2 = *reinterpret_cast<const float2 *>(pl + e);
       }
-      const dfl q0{a2.x, b2.x}, q1{a2.y, b2.y};
+      const dfl q0 = df_mul({a2.x, b2.x}, sq), q1 = df_mul({a2.y, b2.y}, sq);
       dfl w0 = df_add_f(df_mul({dh.x, dl.x}, q0), v2.x);
       dfl w1 = df_add_f(df_mul({dh.y, dl.y}, q1), v2.y);
       if (ph != nullptr) {
-        w0 = df_add(w0, df_mul(nbj, {p2.x, r2.x}));
-        w1 = df_add(w1, df_mul(nbj, {p2.y, r2.y}));
+        w0 = df_add(w0, df_mul(nbj, df_mul({p2.x, r2.x}, sp)));
+        w1 = df_add(w1, df_mul(nbj, df_mul({p2.y, r2.y}, sp)));
       }
       *reinterpret_cast<float2 *>(wh + e) = make_float2(w0.h, w1.h);
       *reinterpret_cast<float2 *>(wl + e) = make_float2(w0.l, w1.l);
@@ -293,7 +311,8 @@ __device__ __forceinline__ void alpha_axpy_chunk(const VecCtx &c, int j, int chu
     if (c.pair) {
       const float *qh = pair_hi(slot_ptr(c, j), c) + voff;
       const float *ql = pair_lo(slot_ptr(c, j), c) + voff;
-      float *wh = pair_hi(c.w, c) + voff, *wl = pair_lo(c.w, c) + voff;
+      float *wh = pair_hi(slot_ptr(c, j + 1), c) + voff, *wl = pair_lo(slot_ptr(c, j + 1), c) + voff;
+      const dfl sq = pair_scale(c, j, b);
       const dfl nal = c.nalpha_f ? dfl{c.nalpha_f[b].x, c.nalpha_f[b].y} : df_from(-alpha);
       float sh = 0.f, sl = 0.f;
 #pragma unroll
@@ -304,8 +323,8 @@ __device__ __forceinline__ void alpha_axpy_chunk(const VecCtx &c, int j, int chu
         const float2 b2 = *reinterpret_cast<const float2 *>(ql + e);
         const float2 x2 = *reinterpret_cast<const float2 *>(wh + e);
         const float2 y2 = *reinterpret_cast<const float2 *>(wl + e);
-        const dfl w0 = df_add({x2.x, y2.x}, df_mul(nal, {a2.x, b2.x}));
-        const dfl w1 = df_add({x2.y, y2.y}, df_mul(nal, {a2.y, b2.y}));
+        const dfl w0 = df_add({x2.x, y2.x}, df_mul(nal, df_mul({a2.x, b2.x}, sq)));
+        const dfl w1 = df_add({x2.y, y2.y}, df_mul(nal, df_mul({a2.y, b2.y}, sq)));
         *reinterpret_cast<float2 *>(wh + e) = make_float2(w0.h, w1.h);
         *reinterpret_cast<float2 *>(wl + e) = make_float2(w0.l, w1.l);
         df_dot_acc(sh, sl, w0, w0);
@@ -459,11 +478,21 @@ __global__ void k_beta_vec(VecCtx c, int j) {
     c.betaj[b] = 0.0;
     if (c.nbeta_f) c.nbeta_f[b] = make_float2(-0.0f, 0.0f);
   }
-  if (lane == 0) c.sinv[b] = inv;
+  if (lane == 0) {
+    c.sinv[b] = inv;
+    if (c.pair) {
+      const dfl t = df_from(inv);
+      c.qscale[(size_t)((j + 1) % 3) * c.Bs + b] = make_float2(t.h, t.l);
+      c.xmax[b] = 0u;
+    }
+  }
 }
 
 // q_next = w / beta into the next basis slot and xh = bf16(Delta^1/2 q_next)
-// (beta, the breakdown test and 1/beta from k_beta_vec).  is_start: w
+// (beta, the breakdown test and 1/beta from k_beta_vec); pair mode: xh only,
+// from the unnormalised vector.  Vectors run fastest over the grid: the rows of
+// xh's K blocks lie next to one another, so blocks that run together write runs
+// of DRAM pages (pair mode 678 us with chunks fastest, 428 us).  is_start: w
 // holds b_tm; ||b|| from the partials here, beta0, and q_0 into slot 0.
 __device__ __forceinline__ void normalize_chunk(const VecCtx &c, int j, int is_start, int chunk,
                                                 int b) {
@@ -504,35 +533,63 @@ __device__ __forceinline__ void normalize_chunk(const VecCtx &c, int j, int is_s
   const size_t voff = (size_t)b * c.N;
   const int e0 = elem_base(chunk);
   if (c.pair) {
-    // float-pair slots: the start reads the FP64 b of the start kernels,
-    // a step the float-pair w of the axpy pass
+    // float-pair slots: the start normalises the FP64 b of the start kernels
+    // into slot 0; a step finds w in its slot and 1 / beta in qscale, and only
+    // the operand is formed.  The largest |xh| goes to c.xmax (the scale of the
+    // 8-bit operand).
     float *qh = pair_hi(slot_ptr(c, next), c) + voff, *ql = pair_lo(slot_ptr(c, next), c) + voff;
-    const float *wh = pair_hi(c.w, c) + voff, *wl = pair_lo(c.w, c) + voff;
+    if (is_start && chunk == 0 && threadIdx.x == 0)
+      c.qscale[b] = make_float2(live ? 1.f : 0.f, 0.f);
     const dfl si = df_from(inv);
+    float m = 0.f;
+    const int e4 = elem_base4(chunk);
+    float4 xh[2], xl[2], ds[2];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int e = e0 + u * 64;
-      if (e >= c.N) continue;
-      dfl q0{0.f, 0.f}, q1{0.f, 0.f};
-      if (live && is_start) {
-        const double2 w2 = *reinterpret_cast<const double2 *>(c.w + voff + e);
-        q0 = df_from(w2.x * inv);
-        q1 = df_from(w2.y * inv);
-      } else if (live) {
-        const float2 x2 = *reinterpret_cast<const float2 *>(wh + e);
-        const float2 y2 = *reinterpret_cast<const float2 *>(wl + e);
-        q0 = df_mul({x2.x, y2.x}, si);
-        q1 = df_mul({x2.y, y2.y}, si);
+    for (int u = 0; u < 2; ++u) {
+      const int e = e4 + 128 * u;
+      xh[u] = xl[u] = ds[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (e >= c.N || !live) continue;
+      if (!is_start) {
+        xh[u] = *reinterpret_cast<const float4 *>(qh + e);
+        xl[u] = *reinterpret_cast<const float4 *>(ql + e);
       }
-      *reinterpret_cast<float2 *>(qh + e) = make_float2(q0.h, q1.h);
-      *reinterpret_cast<float2 *>(ql + e) = make_float2(q0.l, q1.l);
-      if (c.xh != nullptr) {
-        __nv_bfloat162 x2;
-        x2.x = __float2bfloat16_rn(c.dsqf[e] * q0.h);
-        x2.y = __float2bfloat16_rn(c.dsqf[e + 1] * q1.h);
-        *reinterpret_cast<__nv_bfloat162 *>(c.xh + kblk_bf16(b, e, c.Bs)) = x2;
-      }
+      ds[u] = *reinterpret_cast<const float4 *>(c.dsqf + e);
     }
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int e = e4 + 128 * u;
+      if (e >= c.N) continue;
+      float qv[4] = {0.f, 0.f, 0.f, 0.f};
+      if (is_start) {
+        float lo[4] = {0.f, 0.f, 0.f, 0.f};
+        if (live) {
+          const double2 w0 = *reinterpret_cast<const double2 *>(c.w + voff + e);
+          const double2 w1 = *reinterpret_cast<const double2 *>(c.w + voff + e + 2);
+          split_d(w0.x * inv, qv[0], lo[0]);
+          split_d(w0.y * inv, qv[1], lo[1]);
+          split_d(w1.x * inv, qv[2], lo[2]);
+          split_d(w1.y * inv, qv[3], lo[3]);
+        }
+        *reinterpret_cast<float4 *>(qh + e) = make_float4(qv[0], qv[1], qv[2], qv[3]);
+        *reinterpret_cast<float4 *>(ql + e) = make_float4(lo[0], lo[1], lo[2], lo[3]);
+      } else if (live) {
+        qv[0] = df_mul(dfl{xh[u].x, xl[u].x}, si).h;
+        qv[1] = df_mul(dfl{xh[u].y, xl[u].y}, si).h;
+        qv[2] = df_mul(dfl{xh[u].z, xl[u].z}, si).h;
+        qv[3] = df_mul(dfl{xh[u].w, xl[u].w}, si).h;
+      }
+      __nv_bfloat162 x01, x23;
+      x01.x = __float2bfloat16_rn(ds[u].x * qv[0]);
+      x01.y = __float2bfloat16_rn(ds[u].y * qv[1]);
+      x23.x = __float2bfloat16_rn(ds[u].z * qv[2]);
+      x23.y = __float2bfloat16_rn(ds[u].w * qv[3]);
+      *reinterpret_cast<uint2 *>(c.xh + kblk_bf16(b, e, c.Bs)) =
+          make_uint2(bits_as<uint32_t>(x01), bits_as<uint32_t>(x23));
+      const float2 f0 = __bfloat1622float2(x01), f1 = __bfloat1622float2(x23);
+      m = fmaxf(m, fmaxf(fmaxf(fabsf(f0.x), fabsf(f0.y)), fmaxf(fabsf(f1.x), fabsf(f1.y))));
+    }
+    const unsigned mw = __reduce_max_sync(0xffffffffu, __float_as_uint(m));   // m >= 0
+    if ((threadIdx.x & 31) == 0 && mw != 0u) atomicMax(&c.xmax[b], mw);
     return;
   }
   double *qn = slot_ptr(c, next) + voff;
@@ -560,8 +617,8 @@ __device__ __forceinline__ void normalize_chunk(const VecCtx &c, int j, int is_s
 }
 
 __global__ void __launch_bounds__(VEC_THREADS) k_normalize(VecCtx c, int j, int is_start) {
-  const int n = cpb_of(c), c0 = blockIdx.x * n, c1 = min(c.nchunks, c0 + n);
-  for (int chunk = c0; chunk < c1; ++chunk) normalize_chunk(c, j, is_start, chunk, blockIdx.y);
+  const int n = cpb_of(c), c0 = blockIdx.y * n, c1 = min(c.nchunks, c0 + n);
+  for (int chunk = c0; chunk < c1; ++chunk) normalize_chunk(c, j, is_start, chunk, blockIdx.x);
 }
 
 // w = Delta^1/2 V for the rows of a given coupling block (V row stride ldv,
@@ -1062,7 +1119,8 @@ static dim3 vec_grid_cpb(const VecCtx &c) {
   return dim3((c.nchunks + n - 1) / n, c.Bs);
 }
 void launch_normalize(const VecCtx &c, int j, int is_start, const double *, cudaStream_t st) {
-  k_normalize<<<vec_grid_cpb(c), VEC_THREADS, 0, st>>>(c, j, is_start);
+  const dim3 g = vec_grid_cpb(c);
+  k_normalize<<<dim3(g.y, g.x), VEC_THREADS, 0, st>>>(c, j, is_start);
 }
 void launch_assemble_w(const VecCtx &c, int j, const float *ucd, cudaStream_t st) {
   k_assemble_w<<<vec_grid_cpb(c), VEC_THREADS, 0, st>>>(c, j, ucd);

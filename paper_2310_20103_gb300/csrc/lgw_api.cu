@@ -853,6 +853,9 @@ void run_lanczos(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts 
   // the start of each sub-batch, the tensor-core coupling vectors V = L M
   float *ucd_buf = tc ? wsT<float>(h, "ucd", (size_t)Bs * N) : nullptr;
   c.ucd = split ? ucd_buf : nullptr;
+  c.ucd_pair = c.pair ? ucd_buf : nullptr;
+  c.qscale = c.pair ? wsT<float2>(h, "qscale", (size_t)3 * Bs) : nullptr;
+  c.xmax = c.pair ? wsT<unsigned>(h, "xmax", (size_t)Bs) : nullptr;
   c.d2f = s.d2f;
   c.kf = s.kf;
   c.n_yb = (s.A + 255) / 256;
@@ -1048,6 +1051,7 @@ void run_lanczos(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts 
         launch_start_from_v(c, pv.d_V + (size_t)vec0 * s.n_vc, s.n_vc, s.n_vc, st);
         check_launch(h, "start_from_v");
       }
+      if (c.pair) LGW_TRY_CUDA(h, cudaMemsetAsync(c.xmax, 0, sizeof(unsigned) * Bs, st));
       if (split)
         launch_start_split(c, st);
       else
@@ -1105,7 +1109,10 @@ void run_lanczos(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opts 
           // vector; 1/beta_j is applied to each column of the reduction
           const double *vscale = dcgs ? c.sinv : nullptr;
           if (fp8) {
-            launch_quant_x8(c.xh, Bs, N, x8, sx, st, vscale);
+            if (c.pair)
+              launch_quant_x8_max(c.xh, Bs, N, c.xmax, x8, sx, st);
+            else
+              launch_quant_x8(c.xh, Bs, N, x8, sx, st, vscale);
             check_launch(h, "quant_x8");
           } else if (deq) {
             launch_quant_x16(c.xh, Bs, N, x16, sx, st, vscale);

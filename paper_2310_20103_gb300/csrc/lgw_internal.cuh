@@ -100,11 +100,14 @@ struct VecCtx {
   const float *dsqf;      // [N]
   const float *d2f;       // [N] Delta^2 (float)
   const float *d2lo;      // [N] second float of Delta^2
-  // pair: the ring slots and w hold float pairs (hi = the first Bs*N floats
-  // of the slot, lo = the next Bs*N) and the vector passes run in double-
-  // float arithmetic on the FP32 pipe (tensor-core path without
-  // reorthogonalisation, ring mode)
+  // pair: the ring slots hold float pairs (hi = the first Bs*N floats of the
+  // slot, lo = the next Bs*N), unnormalised, with their 1 / beta in qscale, and
+  // the vector passes run in double-float arithmetic on the FP32 pipe
+  // (tensor-core path without reorthogonalisation, ring mode)
   int pair;
+  float2 *qscale;         // [3][Bs] 1 / beta of the vector in each slot as a float pair
+  unsigned *xmax;         // [Bs] bits of max |xh| (pair mode)
+  const float *ucd_pair;  // ucd in pair mode
   float2 *nalpha_f;       // [Bs] -alpha_j as a float pair (pair mode; written by the
                           // alpha reduction, so the passes convert no FP64 per thread)
   float2 *nbeta_f;        // [Bs] -beta_{j+1} as a float pair (pair mode; k_beta_vec)
@@ -294,6 +297,9 @@ void launch_prepare_fp8(const double *src, int ld, int nr, int nc, const SysDev 
                         unsigned *colmax, uint8_t *L8, uint8_t *L8t, float *sL, cudaStream_t st);
 // vscale (optional, [Bs]): normalisation factor of an unnormalised operand,
 // folded into sx
+// with max |xh| known (bits in xmax[b])
+void launch_quant_x8_max(const __nv_bfloat16 *xh, int Bs, int N, const unsigned *xmax, uint8_t *x8,
+                         float *sx, cudaStream_t st);
 void launch_quant_x8(const __nv_bfloat16 *xh, int Bs, int N, uint8_t *x8, float *sx,
                      cudaStream_t st, const double *vscale = nullptr);
 void launch_reduce_y_fp8(const float *Ypart, int splits, int Bs, int A, const float *sx,
