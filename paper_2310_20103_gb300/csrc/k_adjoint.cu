@@ -61,6 +61,7 @@ __device__ __forceinline__ void eig_rotation(double g, double f, double &c, doub
 }
 
 __global__ void __launch_bounds__(EIG_THREADS) k_eig_full(AdjCtx a) {
+  pdl_wait();
   extern __shared__ double sm[];
   __shared__ int ctl[2][3];   // by sweep parity: first row, rotations, 1 = no convergence
   const int tid = threadIdx.x;
@@ -157,6 +158,7 @@ __global__ void __launch_bounds__(EIG_THREADS) k_eig_full(AdjCtx a) {
 constexpr int COEF_THREADS = 128;
 
 __global__ void __launch_bounds__(COEF_THREADS) k_adj_coeffs(AdjCtx a) {
+  pdl_wait();
   extern __shared__ double sm[];   // Om[k], u1[k], fu[k]
   __shared__ double red[COEF_THREADS / 32];
   const int b = blockIdx.x;
@@ -277,6 +279,7 @@ constexpr int ROW_THREADS = 32;
 
 __global__ void __launch_bounds__(ROW_THREADS) k_adj_rows(AdjCtx a, BasisRef basis,
                                                           double *Y, double *Gd) {
+  pdl_wait();
   extern __shared__ double qs[];   // [k][ROW_THREADS]
   const int b = blockIdx.y;
   const int i = blockIdx.x * ROW_THREADS + threadIdx.x;
@@ -316,6 +319,7 @@ constexpr int RF_ELEMS = 128, RF_WARPS = 8;
 
 __global__ void __launch_bounds__(32 * RF_WARPS) k_adj_rows_f32(AdjCtx a, BasisRef basis,
                                                                 double *Y, double *Gd) {
+  pdl_wait();
   extern __shared__ float qsf[];               // [k][RF_ELEMS] q, then [k][RF_ELEMS] row terms
   const int b = blockIdx.y, k = a.k;
   float *sf = qsf + (size_t)k * RF_ELEMS;
@@ -378,6 +382,7 @@ __global__ void __launch_bounds__(32 * RF_WARPS) k_adj_rows_f32(AdjCtx a, BasisR
 // The row-by-row form, for depths whose two tables exceed shared memory.
 __global__ void __launch_bounds__(ROW_THREADS) k_adj_rows_f32_deep(AdjCtx a, BasisRef basis,
                                                                    double *Y, double *Gd) {
+  pdl_wait();
   extern __shared__ float qsf[];   // [k][ROW_THREADS]
   const int b = blockIdx.y;
   const int i = blockIdx.x * ROW_THREADS + threadIdx.x;
@@ -415,6 +420,7 @@ __global__ void __launch_bounds__(ROW_THREADS) k_adj_rows_f32_deep(AdjCtx a, Bas
 __global__ void __launch_bounds__(256) k_split_t(BasisRef src, int R, int C, int lds,
                                                  __nv_bfloat16 *__restrict__ hi,
                                                  __nv_bfloat16 *__restrict__ lo) {
+  pdl_wait();
   __shared__ uint32_t tile[64][65];   // hi | lo << 16
   const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
   {
@@ -460,6 +466,7 @@ __global__ void __launch_bounds__(256) k_split_scaled(BasisRef src, int R, int C
                                                       const double *__restrict__ scale,
                                                       __nv_bfloat16 *__restrict__ hi,
                                                       __nv_bfloat16 *__restrict__ lo) {
+  pdl_wait();
   const int c = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
   if (c >= C) return;
   double sc[4];
@@ -492,6 +499,7 @@ __global__ void __launch_bounds__(256) k_split_scaled(BasisRef src, int R, int C
 constexpr int GP_ROWS = 8;
 __global__ void __launch_bounds__(128) k_gamma_p(AdjCtx a, const double *__restrict__ P, int A,
                                                  double *__restrict__ R) {
+  pdl_wait();
   const int b = blockIdx.y;
   const int mu = blockIdx.x * blockDim.x + threadIdx.x;
   if (mu >= A) return;
@@ -531,6 +539,7 @@ __global__ void __launch_bounds__(256) k_atb_f64(const double *__restrict__ X, i
                                                  const double *__restrict__ Yr, int ldy, int R,
                                                  int Ni, int Nmu, double *__restrict__ S,
                                                  double scale) {
+  pdl_wait();
   __shared__ double Xs[16][65];
   __shared__ double Ys[16][65];
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
@@ -581,6 +590,7 @@ __global__ void __launch_bounds__(256) k_atb_f64(const double *__restrict__ X, i
 __global__ void k_adj_accumulate(AdjCtx a, const double *Delta, BasisRef basis,
                                  const double *Y, const double *Gd, double *dDelta,
                                  double *deps) {
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < a.N && Delta[i] > 0.0) {
     double s = 0.0;
@@ -611,6 +621,7 @@ __global__ void k_adj_accumulate(AdjCtx a, const double *Delta, BasisRef basis,
 __global__ void k_adj_dL(const double *L64, const double *dsq, const double *SC,
                          const double *SB, int A, int n_vc, int n_aux, double kf, double *dL,
                          double *dDelta, int tda) {
+  pdl_wait();
   const int i = blockIdx.x;
   if (i >= n_vc) return;
   __shared__ double red[8];
@@ -630,6 +641,7 @@ __global__ void k_adj_dL(const double *L64, const double *dsq, const double *SC,
 // deps from dDelta (Delta_vc = eps_c - eps_v) plus the direct dE_t Z_t term.
 __global__ void k_adj_deps(const double *dDelta, int n_v, int n_c, const int *targets, int n_t,
                            const double *Z, const double *dE, double *deps) {
+  pdl_wait();
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= n_v + n_c) return;
   double s = 0.0;
@@ -660,6 +672,7 @@ __global__ void k_adj_deps(const double *dDelta, int n_v, int n_c, const int *ta
 // elementwise pass per step, besides the matvec.  dF/dC = sum_j ubar_j q_j^T.
 // --------------------------------------------------------------------------
 __global__ void k_rev_init(RevCtx r) {
+  pdl_wait();
   const int b = blockIdx.x;
   const int k = r.k;
   for (int j = threadIdx.x; j < k; j += blockDim.x)
@@ -668,6 +681,7 @@ __global__ void k_rev_init(RevCtx r) {
 }
 
 __global__ void k_rev_set_betaj(RevCtx r, double *betaj) {
+  pdl_wait();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= r.Bs) return;
   double v = 0.0;
@@ -685,6 +699,7 @@ __device__ __forceinline__ int rev_elem_base(int chunk) {
 // qbar_{j+1}.q_{j+1}, qbar_{j+1}.q_j, q_{j+1}.q_j, qbar_{j+1}.q_{j-1},
 // q_{j+1}.q_{j-1}, q_j.q_{j-1}.
 __global__ void __launch_bounds__(VEC_THREADS) k_rev_dots(RevCtx r, int j) {
+  pdl_wait();
   __shared__ double red[VEC_THREADS / 32];
   const int chunk = blockIdx.x, b = blockIdx.y;
   const size_t BN = (size_t)r.Bs * r.N, voff = (size_t)b * r.N;
@@ -725,6 +740,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_rev_dots(RevCtx r, int j) {
 // coefficients: ubar = a1 qbar_{j+1} + a2 q_{j+1} + ab q_j,
 // qbar_j += cA qbar_{j+1} + cB q_{j+1} + cC q_j, qbar_{j-1} = mb ubar.
 __global__ void k_rev_scalars(RevCtx r, int j) {
+  pdl_wait();
   const int b = blockIdx.x, lane = threadIdx.x;
   double d[6];
 #pragma unroll
@@ -766,6 +782,7 @@ __global__ void k_rev_scalars(RevCtx r, int j) {
 }
 
 __global__ void __launch_bounds__(VEC_THREADS) k_rev_elem(RevCtx r, int j) {
+  pdl_wait();
   const int chunk = blockIdx.x, b = blockIdx.y;
   const size_t BN = (size_t)r.Bs * r.N, voff = (size_t)b * r.N;
   const double *cf = r.coef + (size_t)b * 8;
@@ -806,6 +823,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_rev_elem(RevCtx r, int j) {
 
 // qbar_0 += C ubar_0 (written back) and per-chunk partials of qbar_0 . q_0.
 __global__ void __launch_bounds__(VEC_THREADS) k_rev_final_dot(RevCtx r, const double *q0v) {
+  pdl_wait();
   __shared__ double red[VEC_THREADS / 32];
   const int chunk = blockIdx.x, b = blockIdx.y;
   const size_t voff = (size_t)b * r.N;
@@ -833,6 +851,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_rev_final_dot(RevCtx r, const d
 // y = dF/db = (dF/dbeta0) q_0 + (qbar_0 - (qbar_0 . q_0) q_0) / beta0.
 __global__ void __launch_bounds__(VEC_THREADS) k_rev_final(RevCtx r, const double *q0v,
                                                            double *Y) {
+  pdl_wait();
   __shared__ double sdot;
   const int chunk = blockIdx.x, b = blockIdx.y;
   const int v = r.vec0 + b;
@@ -870,6 +889,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_rev_final(RevCtx r, const doubl
 // out = a x + b out (b = 0: out is not read), over [Bs][N]
 __global__ void k_rev_axpby(double *out, double a, const double *__restrict__ x, double b,
                             size_t n) {
+  pdl_wait();
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (size_t)gridDim.x * blockDim.x)
     out[i] = (b == 0.0) ? a * x[i] : fma(a, x[i], b * out[i]);
@@ -878,6 +898,7 @@ __global__ void k_rev_axpby(double *out, double a, const double *__restrict__ x,
 // Gd += coef x o y over [Bs][N]
 __global__ void k_rev_gd(double *Gd, double coef, const double *__restrict__ x,
                          const double *__restrict__ y, size_t n) {
+  pdl_wait();
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (size_t)gridDim.x * blockDim.x)
     Gd[i] = fma(coef * x[i], y[i], Gd[i]);
@@ -889,29 +910,29 @@ static unsigned flat_blocks(size_t n) {
 }
 void launch_rev_axpby(double *out, double a, const double *x, double b, size_t n,
                       cudaStream_t st) {
-  k_rev_axpby<<<flat_blocks(n), 256, 0, st>>>(out, a, x, b, n);
+  launch_pdl(k_rev_axpby, dim3(flat_blocks(n)), dim3(256), 0, st, out, a, x, b, n);
 }
 void launch_rev_gd(double *Gd, double coef, const double *x, const double *y, size_t n,
                    cudaStream_t st) {
-  k_rev_gd<<<flat_blocks(n), 256, 0, st>>>(Gd, coef, x, y, n);
+  launch_pdl(k_rev_gd, dim3(flat_blocks(n)), dim3(256), 0, st, Gd, coef, x, y, n);
 }
 
 void launch_rev_init(const RevCtx &r, cudaStream_t st) {
-  k_rev_init<<<r.Bs, 128, 0, st>>>(r);
+  launch_pdl(k_rev_init, dim3(r.Bs), dim3(128), 0, st, r);
 }
 void launch_rev_set_betaj(const RevCtx &r, double *betaj, cudaStream_t st) {
-  k_rev_set_betaj<<<(r.Bs + 127) / 128, 128, 0, st>>>(r, betaj);
+  launch_pdl(k_rev_set_betaj, dim3((r.Bs + 127) / 128), dim3(128), 0, st, r, betaj);
 }
 void launch_rev_step(const RevCtx &r, int j, cudaStream_t st) {
   dim3 grid(r.nchunks, r.Bs);
-  k_rev_dots<<<grid, VEC_THREADS, 0, st>>>(r, j);
-  k_rev_scalars<<<r.Bs, 32, 0, st>>>(r, j);
-  k_rev_elem<<<grid, VEC_THREADS, 0, st>>>(r, j);
+  launch_pdl(k_rev_dots, grid, dim3(VEC_THREADS), 0, st, r, j);
+  launch_pdl(k_rev_scalars, dim3(r.Bs), dim3(32), 0, st, r, j);
+  launch_pdl(k_rev_elem, grid, dim3(VEC_THREADS), 0, st, r, j);
 }
 void launch_rev_finish(const RevCtx &r, const double *q0, double *Y, cudaStream_t st) {
   dim3 grid(r.nchunks, r.Bs);
-  k_rev_final_dot<<<grid, VEC_THREADS, 0, st>>>(r, q0);
-  k_rev_final<<<grid, VEC_THREADS, 0, st>>>(r, q0, Y);
+  launch_pdl(k_rev_final_dot, grid, dim3(VEC_THREADS), 0, st, r, q0);
+  launch_pdl(k_rev_final, grid, dim3(VEC_THREADS), 0, st, r, q0, Y);
 }
 
 // ----------------------------------------------------------------------------
@@ -927,11 +948,11 @@ void launch_eig_full(const AdjCtx &a, cudaStream_t st) {
     cudaFuncSetAttribute(k_eig_full, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     attr = true;
   }
-  k_eig_full<<<a.Bs, EIG_THREADS, smem, st>>>(a);
+  launch_pdl(k_eig_full, dim3(a.Bs), dim3(EIG_THREADS), smem, st, a);
 }
 void launch_adj_coeffs(const AdjCtx &a, cudaStream_t st) {
   const size_t smem = (size_t)3 * a.k * sizeof(double);
-  k_adj_coeffs<<<a.Bs, COEF_THREADS, smem, st>>>(a);
+  launch_pdl(k_adj_coeffs, dim3(a.Bs), dim3(COEF_THREADS), smem, st, a);
 }
 void launch_adj_rows(const AdjCtx &a, BasisRef basis, double *Y, double *Gd, cudaStream_t st) {
   const size_t smem = (size_t)a.k * ROW_THREADS * sizeof(double);
@@ -941,7 +962,7 @@ void launch_adj_rows(const AdjCtx &a, BasisRef basis, double *Y, double *Gd, cud
     attr = true;
   }
   dim3 grid((a.N + ROW_THREADS - 1) / ROW_THREADS, a.Bs);
-  k_adj_rows<<<grid, ROW_THREADS, smem, st>>>(a, basis, Y, Gd);
+  launch_pdl(k_adj_rows, grid, dim3(ROW_THREADS), smem, st, a, basis, Y, Gd);
 }
 void launch_adj_rows_f32(const AdjCtx &a, BasisRef basis, double *Y, double *Gd,
                          cudaStream_t st) {
@@ -954,45 +975,48 @@ void launch_adj_rows_f32(const AdjCtx &a, BasisRef basis, double *Y, double *Gd,
   }
   const size_t tables = (size_t)2 * a.k * RF_ELEMS * sizeof(float);
   if (tables <= 200 * 1024)   // k up to 200
-    k_adj_rows_f32<<<dim3((a.N + RF_ELEMS - 1) / RF_ELEMS, a.Bs), 32 * RF_WARPS, tables, st>>>(
-        a, basis, Y, Gd);
+    launch_pdl(k_adj_rows_f32, dim3((a.N + RF_ELEMS - 1) / RF_ELEMS, a.Bs), dim3(32 * RF_WARPS),
+               tables, st, a, basis, Y, Gd);
   else
-    k_adj_rows_f32_deep<<<dim3((a.N + ROW_THREADS - 1) / ROW_THREADS, a.Bs), ROW_THREADS,
-                          (size_t)a.k * ROW_THREADS * sizeof(float), st>>>(a, basis, Y, Gd);
+    launch_pdl(k_adj_rows_f32_deep, dim3((a.N + ROW_THREADS - 1) / ROW_THREADS, a.Bs),
+               dim3(ROW_THREADS), (size_t)a.k * ROW_THREADS * sizeof(float), st, a, basis, Y, Gd);
 }
 void launch_split_t(BasisRef src, int R, int C, int lds, __nv_bfloat16 *hi, __nv_bfloat16 *lo,
                     cudaStream_t st) {
   dim3 grid((C + 63) / 64, (R + 63) / 64);
-  k_split_t<<<grid, 256, 0, st>>>(src, R, C, lds, hi, lo);
+  launch_pdl(k_split_t, grid, dim3(256), 0, st, src, R, C, lds, hi, lo);
 }
 void launch_split_scaled(BasisRef src, int R, int C, const double *scale, __nv_bfloat16 *hi,
                          __nv_bfloat16 *lo, cudaStream_t st) {
   dim3 grid((C / 4 + 255) / 256, std::min((R + SS_ROWS - 1) / SS_ROWS, 65535));
-  k_split_scaled<<<grid, 256, 0, st>>>(src, R, C, scale, hi, lo);
+  launch_pdl(k_split_scaled, grid, dim3(256), 0, st, src, R, C, scale, hi, lo);
 }
 void launch_gamma_p(const AdjCtx &a, const double *P, int A, double *R, cudaStream_t st) {
   dim3 grid((A + 127) / 128, a.Bs);
-  k_gamma_p<<<grid, 128, 0, st>>>(a, P, A, R);
+  launch_pdl(k_gamma_p, grid, dim3(128), 0, st, a, P, A, R);
 }
 void launch_atb_f64(const double *X, int ldx, const double *Yr, int ldy, int R, int Ni, int Nmu,
                     double *S, cudaStream_t st, double scale) {
   dim3 grid((Nmu + 63) / 64, (Ni + 63) / 64);
-  k_atb_f64<<<grid, 256, 0, st>>>(X, ldx, Yr, ldy, R, Ni, Nmu, S, scale);
+  launch_pdl(k_atb_f64, grid, dim3(256), 0, st, X, ldx, Yr, ldy, R, Ni, Nmu, S, scale);
 }
 void launch_adj_accumulate(const AdjCtx &a, const double *Delta, BasisRef basis,
                            const double *Y, const double *Gd, double *dDelta, double *deps,
                            cudaStream_t st) {
-  k_adj_accumulate<<<(a.N + 255) / 256, 256, 0, st>>>(a, Delta, basis, Y, Gd, dDelta, deps);
+  launch_pdl(k_adj_accumulate, dim3((a.N + 255) / 256), dim3(256), 0, st, a, Delta, basis, Y, Gd,
+             dDelta, deps);
 }
 void launch_adj_dL(const double *L64, const double *dsq, const double *SC, const double *SB,
                    int A, int n_vc, int n_aux, double kf, double *dL, double *dDelta, int tda,
                    cudaStream_t st) {
-  k_adj_dL<<<n_vc, 256, 0, st>>>(L64, dsq, SC, SB, A, n_vc, n_aux, kf, dL, dDelta, tda);
+  launch_pdl(k_adj_dL, dim3(n_vc), dim3(256), 0, st, L64, dsq, SC, SB, A, n_vc, n_aux, kf, dL,
+             dDelta, tda);
 }
 void launch_adj_deps(const double *dDelta, int n_v, int n_c, const int *targets, int n_t,
                      const double *Z, const double *dE, double *deps, cudaStream_t st) {
   const int n = n_v + n_c;
-  k_adj_deps<<<(n + 127) / 128, 128, 0, st>>>(dDelta, n_v, n_c, targets, n_t, Z, dE, deps);
+  launch_pdl(k_adj_deps, dim3((n + 127) / 128), dim3(128), 0, st, dDelta, n_v, n_c, targets, n_t,
+             Z, dE, deps);
 }
 
 }  // namespace lgw

@@ -73,6 +73,7 @@ __device__ __forceinline__ double pole_rcp(double d) {
 // pipe: 8 operations per pole, against about 18 per level of the fraction
 // (2 targets x 1000 frequencies x 256 orbitals x 200: 2.13 -> 1.57 ms).
 __global__ void k_cf_poles(CfProblem p, JacobiBufs jb, double *__restrict__ out, int mchunk) {
+  pdl_wait();
   const int f = blockIdx.x * blockDim.x + threadIdx.x;
   const int ti = blockIdx.y, sl = blockIdx.z;
   if (f >= p.n_freq) return;
@@ -108,6 +109,7 @@ __global__ void k_cf_poles(CfProblem p, JacobiBufs jb, double *__restrict__ out,
 // thread writes Sigma_t(omega_f) itself; otherwise its partial sum goes to
 // part[slice] and k_cf_reduce adds the slices in a fixed order.
 __global__ void k_cf_grid(CfProblem p, JacobiBufs jb, double *__restrict__ out, int mchunk) {
+  pdl_wait();
   const int f = blockIdx.x * blockDim.x + threadIdx.x;
   const int ti = blockIdx.y, sl = blockIdx.z;
   if (f >= p.n_freq) return;
@@ -143,6 +145,7 @@ __global__ void k_cf_grid(CfProblem p, JacobiBufs jb, double *__restrict__ out, 
 
 __global__ void k_cf_reduce(const double *__restrict__ part, int S, size_t n,
                             double *__restrict__ sigma) {
+  pdl_wait();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   double s = 0.0;
@@ -252,6 +255,7 @@ __device__ void sigma_at(const CfProblem &p, const JacobiBufs &jb, int ti, doubl
 __global__ void __cluster_dims__(QP_CTAS, 1, 1) __launch_bounds__(QP_THREADS)
     k_qp(CfProblem p, JacobiBufs jb, const double *__restrict__ sigma, int max_iter, double tol,
          double *e_qp, double *z_qp, unsigned *status) {
+  pdl_wait();
   namespace cg = cooperative_groups;
   __shared__ QpShared sh;
   const int ti = blockIdx.x / QP_CTAS;
@@ -351,12 +355,13 @@ int launch_cf_grid(const CfProblem &p, JacobiBufs jb, double *sigma, double *par
   dim3 grid((p.n_freq + 127) / 128, p.n_t, S);
   double *out = S == 1 ? sigma : part;
   if (jb.poles)
-    k_cf_poles<<<grid, 128, 0, st>>>(p, jb, out, std::max(1, mchunk));
+    launch_pdl(k_cf_poles, grid, dim3(128), 0, st, p, jb, out, std::max(1, mchunk));
   else
-    k_cf_grid<<<grid, 128, 0, st>>>(p, jb, out, std::max(1, mchunk));
+    launch_pdl(k_cf_grid, grid, dim3(128), 0, st, p, jb, out, std::max(1, mchunk));
   if (S > 1) {
     const size_t n = (size_t)p.n_t * p.n_freq * 2;
-    k_cf_reduce<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(part, S, n, sigma);
+    launch_pdl(k_cf_reduce, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, part, S, n,
+               sigma);
     return 2;
   }
   return 1;
@@ -365,7 +370,8 @@ int launch_cf_grid(const CfProblem &p, JacobiBufs jb, double *sigma, double *par
 void launch_qp(const CfProblem &p, JacobiBufs jb, const double *sigma, int max_iter, double tol,
                double *e_qp, double *z_qp, unsigned *status, cudaStream_t st) {
   if (p.n_t <= 0) return;
-  k_qp<<<p.n_t * QP_CTAS, QP_THREADS, 0, st>>>(p, jb, sigma, max_iter, tol, e_qp, z_qp, status);
+  launch_pdl(k_qp, dim3(p.n_t * QP_CTAS), dim3(QP_THREADS), 0, st, p, jb, sigma, max_iter, tol,
+             e_qp, z_qp, status);
 }
 
 }  // namespace lgw

@@ -50,6 +50,7 @@ __device__ __forceinline__ float from_e4m3(uint8_t v) {
 // order like their bit patterns
 __global__ void k_col_absmax(const double *__restrict__ src, int ld, int nr, int nc,
                              unsigned *__restrict__ colmax) {
+  pdl_wait();
   __shared__ float red[8][32];
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int mu = blockIdx.x * 32 + tx;
@@ -67,6 +68,7 @@ __global__ void k_col_absmax(const double *__restrict__ src, int ld, int nr, int
 }
 
 __global__ void k_col_scales(const unsigned *__restrict__ colmax, int A, float *__restrict__ sL) {
+  pdl_wait();
   const int mu = blockIdx.x * blockDim.x + threadIdx.x;
   if (mu < A) sL[mu] = pow2_scale(__uint_as_float(colmax[mu]));
 }
@@ -76,6 +78,7 @@ __global__ void k_col_scales(const unsigned *__restrict__ colmax, int A, float *
 __global__ void k_quantize_L8(const double *__restrict__ src, int ld, int nr, int nc, int N, int A,
                               const float *__restrict__ sL, uint8_t *__restrict__ L8,
                               uint8_t *__restrict__ L8t) {
+  pdl_wait();
   __shared__ uint8_t tile[32][33];
   const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -115,6 +118,7 @@ __global__ void __launch_bounds__(256) k_quant_x8(const __nv_bfloat16 *__restric
                                                   int N, uint8_t *__restrict__ x8,
                                                   float *__restrict__ sx,
                                                   const double *__restrict__ vscale) {
+  pdl_wait();
   __shared__ float red[8];
   __shared__ float sc;
   const int b = blockIdx.x;
@@ -160,6 +164,7 @@ __global__ void __launch_bounds__(256) k_quant_x8_max(const __nv_bfloat16 *__res
                                                       int N, const unsigned *__restrict__ xmax,
                                                       uint8_t *__restrict__ x8,
                                                       float *__restrict__ sx) {
+  pdl_wait();
   const int b = blockIdx.x, g = blockIdx.y * 256 + threadIdx.x;
   const float sc = pow2_scale(__uint_as_float(xmax[b])), inv = 1.0f / sc;
   if (g == 0) sx[b] = sc;
@@ -179,6 +184,7 @@ __global__ void __launch_bounds__(256) k_reduce_y_fp8(const float *__restrict__ 
                                                       uint8_t *__restrict__ y8,
                                                       float *__restrict__ ty,
                                                       float *__restrict__ yy, int n_yb) {
+  pdl_wait();
   extern __shared__ float yp[];   // [A]: s_mu y_mu
   __shared__ float red[8];
   __shared__ float sc;
@@ -233,6 +239,7 @@ __global__ void __launch_bounds__(256) k_quant_x16(const __nv_bfloat16 *__restri
                                                    int N, uint16_t *__restrict__ x16,
                                                    float *__restrict__ sx,
                                                    const double *__restrict__ vscale) {
+  pdl_wait();
   __shared__ float red[8];
   __shared__ float sc;
   const int b = blockIdx.x;
@@ -284,6 +291,7 @@ __global__ void __launch_bounds__(256) k_reduce_y_f16(const float *__restrict__ 
                                                       uint16_t *__restrict__ y16,
                                                       float *__restrict__ ty,
                                                       float *__restrict__ yy, int n_yb) {
+  pdl_wait();
   extern __shared__ float yp[];   // [A]: s_mu y_mu
   __shared__ float red[8];
   __shared__ float sc;
@@ -335,40 +343,41 @@ __global__ void __launch_bounds__(256) k_reduce_y_f16(const float *__restrict__ 
 void launch_prepare_fp8(const double *src, int ld, int nr, int nc, const SysDev &s,
                         unsigned *colmax, uint8_t *L8, uint8_t *L8t, float *sL, cudaStream_t st) {
   cudaMemsetAsync(colmax, 0, sizeof(unsigned) * s.A, st);
-  k_col_absmax<<<dim3((s.A + 31) / 32, (nr + 1023) / 1024), 256, 0, st>>>(src, ld, nr, nc,
-                                                                         colmax);
-  k_col_scales<<<(s.A + 255) / 256, 256, 0, st>>>(colmax, s.A, sL);
-  k_quantize_L8<<<dim3((s.A + 31) / 32, (s.N + 31) / 32), 256, 0, st>>>(src, ld, nr, nc, s.N, s.A,
-                                                                        sL, L8, L8t);
+  launch_pdl(k_col_absmax, dim3((s.A + 31) / 32, (nr + 1023) / 1024), dim3(256), 0, st, src, ld,
+             nr, nc, colmax);
+  launch_pdl(k_col_scales, dim3((s.A + 255) / 256), dim3(256), 0, st, colmax, s.A, sL);
+  launch_pdl(k_quantize_L8, dim3((s.A + 31) / 32, (s.N + 31) / 32), dim3(256), 0, st, src, ld, nr,
+             nc, s.N, s.A, sL, L8, L8t);
 }
 
 void launch_quant_x8_max(const __nv_bfloat16 *xh, int Bs, int N, const unsigned *xmax, uint8_t *x8,
                          float *sx, cudaStream_t st) {
-  k_quant_x8_max<<<dim3(Bs, (N / 8 + 255) / 256), 256, 0, st>>>(xh, Bs, N, xmax, x8, sx);
+  launch_pdl(k_quant_x8_max, dim3(Bs, (N / 8 + 255) / 256), dim3(256), 0, st, xh, Bs, N, xmax, x8,
+             sx);
 }
 
 void launch_quant_x8(const __nv_bfloat16 *xh, int Bs, int N, uint8_t *x8, float *sx,
                      cudaStream_t st, const double *vscale) {
-  k_quant_x8<<<Bs, 256, 0, st>>>(xh, Bs, N, x8, sx, vscale);
+  launch_pdl(k_quant_x8, dim3(Bs), dim3(256), 0, st, xh, Bs, N, x8, sx, vscale);
 }
 
 void launch_reduce_y_fp8(const float *Ypart, int splits, int Bs, int A, const float *sx,
                          const float *sL, uint8_t *y8, float *ty, float *yy, int n_yb,
                          cudaStream_t st) {
-  k_reduce_y_fp8<<<Bs, 256, (size_t)A * sizeof(float), st>>>(Ypart, splits, Bs, A, sx, sL, y8, ty,
-                                                             yy, n_yb);
+  launch_pdl(k_reduce_y_fp8, dim3(Bs), dim3(256), (size_t)A * sizeof(float), st, Ypart, splits,
+             Bs, A, sx, sL, y8, ty, yy, n_yb);
 }
 
 void launch_quant_x16(const __nv_bfloat16 *xh, int Bs, int N, uint16_t *x16, float *sx,
                       cudaStream_t st, const double *vscale) {
-  k_quant_x16<<<Bs, 256, 0, st>>>(xh, Bs, N, x16, sx, vscale);
+  launch_pdl(k_quant_x16, dim3(Bs), dim3(256), 0, st, xh, Bs, N, x16, sx, vscale);
 }
 
 void launch_reduce_y_f16(const float *Ypart, int splits, int Bs, int A, const float *sx,
                          const float *sL, uint16_t *y16, float *ty, float *yy, int n_yb,
                          cudaStream_t st) {
-  k_reduce_y_f16<<<Bs, 256, (size_t)A * sizeof(float), st>>>(Ypart, splits, Bs, A, sx, sL, y16,
-                                                             ty, yy, n_yb);
+  launch_pdl(k_reduce_y_f16, dim3(Bs), dim3(256), (size_t)A * sizeof(float), st, Ypart, splits,
+             Bs, A, sx, sL, y16, ty, yy, n_yb);
 }
 
 }  // namespace lgw

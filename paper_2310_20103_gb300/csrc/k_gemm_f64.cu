@@ -21,6 +21,7 @@ __global__ void __launch_bounds__(256) k_gemm1_f64(const double *__restrict__ L6
                                                    const double *__restrict__ q, int N, int A,
                                                    int Bs, int kb_per_split,
                                                    double *__restrict__ Ypart) {
+  pdl_wait();
   __shared__ double As[BK][TB + 1];
   __shared__ double Bt[BK][TB + 1];
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
@@ -71,6 +72,7 @@ __global__ void __launch_bounds__(256) k_gemm1_f64(const double *__restrict__ L6
 
 __global__ void k_reduce_y_f64(const double *__restrict__ Ypart, int splits, int n,
                                double *__restrict__ Y) {
+  pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   double s = 0.0;
@@ -89,6 +91,7 @@ __global__ void __launch_bounds__(256) k_gemm2_f64(const double *__restrict__ L6
                                                    const double *__restrict__ betaj,
                                                    double *__restrict__ w,
                                                    double *__restrict__ alpha_part) {
+  pdl_wait();
   __shared__ double As[BK][TB + 1];
   __shared__ double Bt[BK][TB + 1];
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
@@ -168,21 +171,21 @@ void launch_gemm1_f64(const SysDev &s, const double *q, int Bs, double *Ypart, i
   int nkb = s.N / BK;
   int per = (nkb + splits - 1) / splits;
   dim3 grid(s.A / TB, (Bs + TB - 1) / TB, splits);
-  k_gemm1_f64<<<grid, 256, 0, st>>>(s.L64, s.dsq, q, s.N, s.A, Bs, per, Ypart);
+  launch_pdl(k_gemm1_f64, grid, dim3(256), 0, st, s.L64, s.dsq, q, s.N, s.A, Bs, per, Ypart);
 }
 
 void launch_reduce_y_f64(const double *Ypart, int splits, int Bs, int A, double *Y,
                          cudaStream_t st) {
   int n = Bs * A, th = 256;
-  k_reduce_y_f64<<<(n + th - 1) / th, th, 0, st>>>(Ypart, splits, n, Y);
+  launch_pdl(k_reduce_y_f64, dim3((n + th - 1) / th), dim3(th), 0, st, Ypart, splits, n, Y);
 }
 
 void launch_gemm2_f64(const SysDev &s, const double *Y, int Bs, int epi, const double *q,
                       const double *qprev, const double *betaj, double *w, double *alpha_part,
                       cudaStream_t st) {
   dim3 grid(s.N / TB, (Bs + TB - 1) / TB);
-  k_gemm2_f64<<<grid, 256, 0, st>>>(s.L64, Y, s.N, s.A, Bs, epi, s.Delta2, s.dsq, s.cd, q, qprev,
-                                    betaj, w, alpha_part);
+  launch_pdl(k_gemm2_f64, grid, dim3(256), 0, st, s.L64, Y, s.N, s.A, Bs, epi, s.Delta2, s.dsq,
+             s.cd, q, qprev, betaj, w, alpha_part);
 }
 
 }  // namespace lgw

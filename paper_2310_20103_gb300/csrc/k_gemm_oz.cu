@@ -169,6 +169,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
+  pdl_wait();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -405,6 +406,7 @@ struct Src {
 // matrix's rows (COLS = false, contraction along c) or its columns.
 template <bool COLS>
 __global__ void __launch_bounds__(256) k_oz_max(Src src, int *__restrict__ e) {
+  pdl_wait();
   const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
   if (COLS) {
     const int c = c0 + (threadIdx.x & 63);
@@ -426,6 +428,7 @@ __global__ void __launch_bounds__(256) k_oz_max(Src src, int *__restrict__ e) {
 template <bool COLS>
 __global__ void __launch_bounds__(256) k_oz_slice(Src src, const int *__restrict__ e,
                                                   uint16_t *__restrict__ out, int rows, int nkb) {
+  pdl_wait();
   __shared__ double tile[COLS ? 64 : 1][65];
   const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
   const int i = threadIdx.x >> 2, k0 = (threadIdx.x & 3) * 16;   // row and K offset in the tile
@@ -452,6 +455,7 @@ __global__ void __launch_bounds__(256) k_oz_rows(const double *__restrict__ x, i
                                                  int rows, int nkb) {
   extern __shared__ double v[];
   __shared__ int wmax[8];
+  pdl_wait();
   const int r = blockIdx.x;
   int m = 0;
   for (int i = threadIdx.x; i < nkb * 64; i += 256) {
@@ -483,6 +487,7 @@ __global__ void __launch_bounds__(256) k_oz_rows(const double *__restrict__ x, i
 
 // *bad != 0 if an exponent field says Inf or NaN
 __global__ void k_oz_check(const int *__restrict__ e, int n, unsigned *bad) {
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n && e[i] >= 2047) atomicOr(bad, 1u);
 }
@@ -523,7 +528,7 @@ static void launch(const CUtensorMap &A, const CUtensorMap &B, int M, int Ncols,
     attr = true;
   }
   const dim3 grid((Ncols + NT - 1) / NT, (M + BM - 1) / BM, splits);
-  k_oz_gemm<NT><<<grid, NTHREADS, Cfg<NT>::SMEM, st>>>(A, B, M, Ncols, nkb, per, e);
+  launch_pdl(k_oz_gemm<NT>, grid, dim3(NTHREADS), Cfg<NT>::SMEM, st, A, B, M, Ncols, nkb, per, e);
 }
 
 static void launch_rows(const double *x, int splits, size_t part, const Src &src, double *y,
@@ -534,8 +539,9 @@ static void launch_rows(const double *x, int splits, size_t part, const Src &src
                          OZ_ROW_MAX * (int)sizeof(double));
     attr = true;
   }
-  k_oz_rows<<<o.rows, 256, (size_t)o.nkb * 64 * sizeof(double), st>>>(x, splits, part, src, y, o.e,
-                                                                      o.d, o.rows, o.nkb);
+  launch_pdl(k_oz_rows, dim3(o.rows), dim3(256), (size_t)o.nkb * 64 * sizeof(double), st, x,
+             splits,
+             part, src, y, o.e, o.d, o.rows, o.nkb);
 }
 
 static int sm_count() {
@@ -629,11 +635,11 @@ void launch_oz_slice(const double *x, size_t ld, int nr, int nc, const double *s
   const int kr = cols ? o.nkb : (o.rows + 63) / 64, kc = cols ? (o.rows + 63) / 64 : o.nkb;
   const dim3 grid(kc, kr), data((nc + 63) / 64, (nr + 63) / 64);
   if (cols) {
-    oz::k_oz_max<true><<<data, 256, 0, st>>>(src, o.e);
-    oz::k_oz_slice<true><<<grid, 256, 0, st>>>(src, o.e, o.d, o.rows, o.nkb);
+    launch_pdl(oz::k_oz_max<true>, data, dim3(256), 0, st, src, o.e);
+    launch_pdl(oz::k_oz_slice<true>, grid, dim3(256), 0, st, src, o.e, o.d, o.rows, o.nkb);
   } else {
-    oz::k_oz_max<false><<<data, 256, 0, st>>>(src, o.e);
-    oz::k_oz_slice<false><<<grid, 256, 0, st>>>(src, o.e, o.d, o.rows, o.nkb);
+    launch_pdl(oz::k_oz_max<false>, data, dim3(256), 0, st, src, o.e);
+    launch_pdl(oz::k_oz_slice<false>, grid, dim3(256), 0, st, src, o.e, o.d, o.rows, o.nkb);
   }
 }
 
@@ -645,7 +651,7 @@ void launch_oz_reduce(const double *part, int splits, int nr, int len, double *y
 }
 
 void launch_oz_check(const OzOperand &o, unsigned *bad, cudaStream_t st) {
-  oz::k_oz_check<<<(o.rows + 255) / 256, 256, 0, st>>>(o.e, o.rows, bad);
+  launch_pdl(oz::k_oz_check, dim3((o.rows + 255) / 256), dim3(256), 0, st, o.e, o.rows, bad);
 }
 
 }  // namespace lgw

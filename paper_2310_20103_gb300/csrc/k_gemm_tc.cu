@@ -161,6 +161,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
+  pdl_wait();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -402,6 +403,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tslot;
+  pdl_wait();
   auto tile_of = [&](int t, int &m_tile, int &n_tile) {
     if (ea.mfast) {
       m_tile = t % m_tiles;
@@ -534,6 +536,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                     const __grid_constant__ CUtensorMap tmBhi,
                     const __grid_constant__ CUtensorMap tmBlo, int M, int Ncols, int nk,
                     float *__restrict__ vf, unsigned *status) {
+  pdl_wait();
   using C = CplCfg<BN>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>(
@@ -634,6 +637,7 @@ __global__ void k_reduce_y_bf16(const float *__restrict__ Ypart, int splits, int
                                 __nv_bfloat16 *__restrict__ Yh, float *__restrict__ yy,
                                 const double *__restrict__ vscale) {
   __shared__ float red[8];
+  pdl_wait();
   const int b = blockIdx.y;
   const int mu = blockIdx.x * 256 + threadIdx.x;
   const size_t n = (size_t)Bs * A;
@@ -899,7 +903,8 @@ static void launch_tc(const CUtensorMap &A, const CUtensorMap &B, int M, int Nco
     attr_done = true;
   }
   dim3 grid((M + tc::BM - 1) / tc::BM, (Ncols + BN - 1) / BN, splits);
-  tc::k_gemm_tc<BN, EPI, EB, HALF><<<grid, tc::NTHREADS, C::SMEM, st>>>(A, B, M, Ncols, num_kb,
+  launch_pdl(tc::k_gemm_tc<BN, EPI, EB, HALF>, grid, dim3(tc::NTHREADS), C::SMEM, st, A, B, M,
+             Ncols, num_kb,
                                                                         kb_per_split, ea);
 }
 
@@ -919,7 +924,8 @@ static void launch_persist(const CUtensorMap &A, const CUtensorMap &B, int M, in
   }
   const int total = ((M + tc::BM - 1) / tc::BM) * ((Ncols + BN - 1) / BN);
   const int grid = std::max(1, std::min(total, nsm > 0 ? nsm : 148));
-  tc::k_gemm_persist<BN, EB><<<grid, tc::NTHREADS, C::SMEM, st>>>(A, B, M, Ncols, num_kb, ea);
+  launch_pdl(tc::k_gemm_persist<BN, EB>, dim3(grid), dim3(tc::NTHREADS), C::SMEM, st, A, B, M,
+             Ncols, num_kb, ea);
 }
 
 // half: 1 = the half-depth pipeline (two CTAs per SM), 2 = the persistent
@@ -985,7 +991,7 @@ void launch_gemm1_tc(const TcPlan *p, unsigned *status, cudaStream_t st) {
 void launch_reduce_y_bf16(const float *Ypart, int splits, int Bs, int A, __nv_bfloat16 *Yh,
                           float *yy, cudaStream_t st, const double *vscale) {
   dim3 grid((A + 255) / 256, Bs);
-  tc::k_reduce_y_bf16<<<grid, 256, 0, st>>>(Ypart, splits, Bs, A, Yh, yy, vscale);
+  launch_pdl(tc::k_reduce_y_bf16, grid, dim3(256), 0, st, Ypart, splits, Bs, A, Yh, yy, vscale);
 }
 
 void launch_gemm2_tc(const TcPlan *p, int epi, const double *q, const double *qprev,
@@ -1038,6 +1044,7 @@ namespace tc {
 // bf16 hi and lo halves of M rows into zero-padded [Bs][A] operands.
 __global__ void k_split_m(const double *__restrict__ M, int nvec, int n_aux, int Bs, int A,
                           __nv_bfloat16 *__restrict__ hi, __nv_bfloat16 *__restrict__ lo) {
+  pdl_wait();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (size_t)Bs * A) return;
   const int b = (int)(i / A), mu = (int)(i - (size_t)b * A);
@@ -1063,8 +1070,8 @@ static void launch_coupling(const TcPlan *p, const CUtensorMap &bhi, const CUten
     attr_done = true;
   }
   const dim3 grid((p->Bs + BN - 1) / BN, (p->N + tc::BM - 1) / tc::BM);
-  tc::k_gemm_coupling<BN><<<grid, tc::NTHREADS, C::SMEM, st>>>(
-      p->g2A, p->g2Alo, bhi, blo, p->N, p->Bs, p->A / tc::BK, vf, status);
+  launch_pdl(tc::k_gemm_coupling<BN>, grid, dim3(tc::NTHREADS), C::SMEM, st, p->g2A, p->g2Alo,
+             bhi, blo, p->N, p->Bs, p->A / tc::BK, vf, status);
 }
 
 bool launch_coupling_tc(const TcPlan *p, const SysDev &s, const double *M, int nvec,
@@ -1078,8 +1085,8 @@ bool launch_coupling_tc(const TcPlan *p, const SysDev &s, const double *M, int n
   if (!encode_2d(&bhi, p->yh, (uint64_t)p->A, (uint64_t)p->Bs, (uint32_t)bn) ||
       !encode_2d(&blo, lo, (uint64_t)p->A, (uint64_t)p->Bs, (uint32_t)bn))
     return false;
-  tc::k_split_m<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(M, nvec, s.n_aux, p->Bs, p->A, p->yh,
-                                                             lo);
+  launch_pdl(tc::k_split_m, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, M, nvec, s.n_aux,
+             p->Bs, p->A, p->yh, lo);
   if (bn == 128)
     launch_coupling<128>(p, bhi, blo, vf, status, st);
   else

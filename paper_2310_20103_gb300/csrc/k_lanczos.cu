@@ -272,6 +272,7 @@ __device__ __forceinline__ int cpb_of(const VecCtx &c) { return c.cpb > 1 ? c.cp
 
 __global__ void __launch_bounds__(VEC_THREADS, 8) k_assemble_w(VecCtx c, int j,
                                                            const float *__restrict__ ucd) {
+  pdl_wait();
   const int n = cpb_of(c), c0 = blockIdx.x * n, c1 = min(c.nchunks, c0 + n);
   for (int chunk = c0; chunk < c1; ++chunk) assemble_w_chunk(c, j, ucd, chunk, blockIdx.y);
 }
@@ -281,6 +282,7 @@ __global__ void __launch_bounds__(VEC_THREADS, 8) k_assemble_w(VecCtx c, int j,
 // back by every block of the axpy pass (which would otherwise each repeat
 // the n_mt strided loads: 12500 of them per block at N_vc 1.6M).
 __global__ void k_alpha_reduce(VecCtx c, int j) {
+  pdl_wait();
   const int b = blockIdx.x, lane = threadIdx.x;
   if (!vec_live(c, b, j)) return;
   double s = 0.0;
@@ -361,12 +363,14 @@ __device__ __forceinline__ void alpha_axpy_chunk(const VecCtx &c, int j, int chu
 
 template <bool DOTS>
 __global__ void __launch_bounds__(VEC_THREADS) k_alpha_axpy(VecCtx c, int j) {
+  pdl_wait();
   const int n = cpb_of(c), c0 = blockIdx.x * n, c1 = min(c.nchunks, c0 + n);
   for (int chunk = c0; chunk < c1; ++chunk) alpha_axpy_chunk<DOTS>(c, j, chunk, blockIdx.y);
 }
 
 // Second-pass dot products of the current w with rows 0..j.
 __global__ void __launch_bounds__(VEC_THREADS) k_dots(VecCtx c, int j) {
+  pdl_wait();
   __shared__ double sred[VEC_THREADS / 32][16];
   const int chunk = blockIdx.x, b = blockIdx.y;
   if (!vec_live(c, b, j) || !c.flag2[b]) return;
@@ -386,6 +390,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_dots(VecCtx c, int j) {
 
 // h[b][i] = sum over chunks of the dot partials, fixed order.
 __global__ void k_reduce_dots(VecCtx c, int j, int pass) {
+  pdl_wait();
   const int b = blockIdx.x;
   if (!vec_live(c, b, j)) return;
   if (pass == 2 && !c.flag2[b]) return;
@@ -399,6 +404,7 @@ __global__ void k_reduce_dots(VecCtx c, int j, int pass) {
 
 // w <- w - sum_i h_i q_i over rows 0..j and ||w||^2 partials.
 __global__ void __launch_bounds__(VEC_THREADS) k_update(VecCtx c, int j, int pass) {
+  pdl_wait();
   extern __shared__ double hs[];
   __shared__ double red[VEC_THREADS / 32];
   const int chunk = blockIdx.x, b = blockIdx.y;
@@ -430,6 +436,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_update(VecCtx c, int j, int pas
 // Second Gram-Schmidt pass: always (CGS2), or where the first pass removed
 // more than half of ||w||^2 (the 1/sqrt(2) norm criterion).
 __global__ void k_second_pass_decide(VecCtx c, int j) {
+  pdl_wait();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= c.Bs) return;
   int f = 0;
@@ -453,6 +460,7 @@ __global__ void k_second_pass_decide(VecCtx c, int j) {
 // vector, fixed order), the breakdown test, and 1/beta (0 when the vector
 // stops or is not live) for k_normalize.
 __global__ void k_beta_vec(VecCtx c, int j) {
+  pdl_wait();
   const int b = blockIdx.x, lane = threadIdx.x;
   const int v = c.vec0 + b;
   double inv = 0.0;
@@ -617,6 +625,7 @@ __device__ __forceinline__ void normalize_chunk(const VecCtx &c, int j, int is_s
 }
 
 __global__ void __launch_bounds__(VEC_THREADS) k_normalize(VecCtx c, int j, int is_start) {
+  pdl_wait();
   const int n = cpb_of(c), c0 = blockIdx.y * n, c1 = min(c.nchunks, c0 + n);
   for (int chunk = c0; chunk < c1; ++chunk) normalize_chunk(c, j, is_start, chunk, blockIdx.x);
 }
@@ -625,6 +634,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_normalize(VecCtx c, int j, int 
 // n_valid real pair elements per row), zero elsewhere; ||w||^2 partials.
 __global__ void __launch_bounds__(VEC_THREADS) k_start_from_v(VecCtx c, const double *V, int ldv,
                                                               int n_valid) {
+  pdl_wait();
   __shared__ double red[VEC_THREADS / 32];
   const int chunk = blockIdx.x, b = blockIdx.y;
   const size_t voff = (size_t)b * c.N;
@@ -650,6 +660,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_start_from_v(VecCtx c, const do
 // w = Delta^1/2 * vf (float coupling vectors from the tensor cores) and
 // ||w||^2 partials; padding vectors get zeros.
 __global__ void __launch_bounds__(VEC_THREADS) k_start_from_vf(VecCtx c, const float *vf) {
+  pdl_wait();
   __shared__ double red[VEC_THREADS / 32];
   const int chunk = blockIdx.x, b = blockIdx.y;
   const size_t voff = (size_t)b * c.N;
@@ -674,6 +685,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_start_from_vf(VecCtx c, const f
 
 __global__ void __launch_bounds__(VEC_THREADS) k_norm_partials(VecCtx c, const double *x,
                                                                double *out) {
+  pdl_wait();
   __shared__ double red[VEC_THREADS / 32];
   const int chunk = blockIdx.x, b = blockIdx.y;
   const size_t voff = (size_t)b * c.N;
@@ -694,6 +706,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_norm_partials(VecCtx c, const d
 // operand layout)
 __global__ void k_scale_rows_to_bf16(const double *__restrict__ x, const double *__restrict__ dsq,
                                      int Bs, int N, __nv_bfloat16 *__restrict__ out) {
+  pdl_wait();
   size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   size_t n = (size_t)Bs * N;
   if (i >= n) return;
@@ -717,6 +730,7 @@ __device__ __forceinline__ bool band_act(const BandCtx &bc, int b) {
 }
 
 __global__ void k_band_init(BandCtx bc) {
+  pdl_wait();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= bc.c.Bs) return;
   bc.nv[b] = 0;
@@ -730,6 +744,7 @@ __global__ void k_band_init(BandCtx bc) {
 // mode 0 (a start vector): every real group; mode 1 (step j): the groups
 // whose basis vector j exists.
 __global__ void k_band_activate(BandCtx bc, int mode, int j) {
+  pdl_wait();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= bc.c.Bs) return;
   bc.act[b] = (b < bc.c.nvec && (mode == 0 || j < bc.nv[b])) ? 1 : 0;
@@ -738,6 +753,7 @@ __global__ void k_band_activate(BandCtx bc, int mode, int j) {
 // The contraction operand of q_j: FP64 copy (FP64 contractions) or
 // bf16(Delta^1/2 q_j); zeros for groups without vector j.
 __global__ void __launch_bounds__(VEC_THREADS) k_band_operand(BandCtx bc, int j) {
+  pdl_wait();
   const VecCtx &c = bc.c;
   const int chunk = blockIdx.x, b = blockIdx.y;
   const bool act = band_act(bc, b);
@@ -762,6 +778,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_band_operand(BandCtx bc, int j)
 // w = Delta^2 q_j + c_K Delta^1/2 L y   (Eq. 4; the contraction in FP32)
 __global__ void __launch_bounds__(VEC_THREADS) k_band_assemble(BandCtx bc, int j,
                                                               const float *__restrict__ ucd) {
+  pdl_wait();
   const VecCtx &c = bc.c;
   const int chunk = blockIdx.x, b = blockIdx.y;
   if (!band_act(bc, b)) return;
@@ -783,6 +800,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_band_assemble(BandCtx bc, int j
 
 // Dots of w with the group's basis vectors; pass 1 also ||w||^2 (norm_a).
 __global__ void __launch_bounds__(VEC_THREADS) k_band_dots(BandCtx bc, int pass) {
+  pdl_wait();
   __shared__ double red[VEC_THREADS / 32];
   __shared__ double sred[VEC_THREADS / 32][16];
   const VecCtx &c = bc.c;
@@ -810,6 +828,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_band_dots(BandCtx bc, int pass)
 
 // h = sum over chunks (fixed order); hsum accumulates the two passes.
 __global__ void k_band_reduce(BandCtx bc, int pass) {
+  pdl_wait();
   const VecCtx &c = bc.c;
   const int b = blockIdx.x;
   if (!band_act(bc, b)) return;
@@ -827,6 +846,7 @@ __global__ void k_band_reduce(BandCtx bc, int pass) {
 // w <- w - sum_i h_i q_i over the group's vectors; ||w||^2 partials
 // (pass 1: norm_b, pass 2: norm_c).
 __global__ void __launch_bounds__(VEC_THREADS) k_band_update(BandCtx bc, int pass) {
+  pdl_wait();
   extern __shared__ double hs[];
   __shared__ double red[VEC_THREADS / 32];
   const VecCtx &c = bc.c;
@@ -859,6 +879,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_band_update(BandCtx bc, int pas
 // One warp per group: beta = ||w|| after both passes, the coefficient
 // record and the breakdown test; sets the row to append (or -1).
 __global__ void k_band_beta(BandCtx bc, int mode, int idx) {
+  pdl_wait();
   const VecCtx &c = bc.c;
   const int b = blockIdx.x, lane = threadIdx.x;
   if (!band_act(bc, b)) {
@@ -912,6 +933,7 @@ __global__ void k_band_beta(BandCtx bc, int mode, int idx) {
 
 // q_new = w / beta into the appended row.
 __global__ void __launch_bounds__(VEC_THREADS) k_band_normalize(BandCtx bc) {
+  pdl_wait();
   const VecCtx &c = bc.c;
   const int chunk = blockIdx.x, b = blockIdx.y;
   if (b >= c.nvec) return;
@@ -934,6 +956,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_band_normalize(BandCtx bc) {
 }
 
 __global__ void k_band_finish(BandCtx bc) {
+  pdl_wait();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= bc.c.nvec) return;
   bc.keff[bc.c.vec0 + b] = min(bc.c.k, bc.nv[b]);
@@ -957,6 +980,7 @@ __global__ void k_band_small(const double *__restrict__ Tb, const double *__rest
                              double *__restrict__ scratch, double *__restrict__ alpha,
                              double *__restrict__ beta, double *__restrict__ beta0,
                              int *__restrict__ keff_out) {
+  pdl_wait();
   const int warps = blockDim.x >> 5;
   const int wv = blockIdx.x * warps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (wv >= nx * G) return;
@@ -1042,6 +1066,7 @@ __global__ void k_band_small(const double *__restrict__ Tb, const double *__rest
 
 __global__ void k_band_combine(const double *__restrict__ sig, int p, int F,
                                double *__restrict__ out) {
+  pdl_wait();
   const int f = blockIdx.x * blockDim.x + threadIdx.x;
   const int ab = blockIdx.y;
   if (f >= F) return;
@@ -1066,52 +1091,52 @@ __global__ void k_band_combine(const double *__restrict__ sig, int p, int F,
 static dim3 vec_grid(const VecCtx &c) { return dim3(c.nchunks, c.Bs); }
 
 void launch_band_init(const BandCtx &bc, cudaStream_t st) {
-  k_band_init<<<(bc.c.Bs + 255) / 256, 256, 0, st>>>(bc);
+  launch_pdl(k_band_init, dim3((bc.c.Bs + 255) / 256), dim3(256), 0, st, bc);
 }
 void launch_band_activate(const BandCtx &bc, int mode, int j, cudaStream_t st) {
-  k_band_activate<<<(bc.c.Bs + 255) / 256, 256, 0, st>>>(bc, mode, j);
+  launch_pdl(k_band_activate, dim3((bc.c.Bs + 255) / 256), dim3(256), 0, st, bc, mode, j);
 }
 void launch_band_operand(const BandCtx &bc, int j, cudaStream_t st) {
-  k_band_operand<<<vec_grid(bc.c), VEC_THREADS, 0, st>>>(bc, j);
+  launch_pdl(k_band_operand, vec_grid(bc.c), dim3(VEC_THREADS), 0, st, bc, j);
 }
 void launch_band_assemble(const BandCtx &bc, int j, const float *ucd, cudaStream_t st) {
-  k_band_assemble<<<vec_grid(bc.c), VEC_THREADS, 0, st>>>(bc, j, ucd);
+  launch_pdl(k_band_assemble, vec_grid(bc.c), dim3(VEC_THREADS), 0, st, bc, j, ucd);
 }
 int launch_band_append(const BandCtx &bc, int mode, int idx, cudaStream_t st) {
   const size_t sh = (size_t)bc.c.kmax1 * sizeof(double);
   for (int pass = 1; pass <= 2; ++pass) {
-    k_band_dots<<<vec_grid(bc.c), VEC_THREADS, 0, st>>>(bc, pass);
-    k_band_reduce<<<bc.c.Bs, 256, 0, st>>>(bc, pass);
-    k_band_update<<<vec_grid(bc.c), VEC_THREADS, sh, st>>>(bc, pass);
+    launch_pdl(k_band_dots, vec_grid(bc.c), dim3(VEC_THREADS), 0, st, bc, pass);
+    launch_pdl(k_band_reduce, dim3(bc.c.Bs), dim3(256), 0, st, bc, pass);
+    launch_pdl(k_band_update, vec_grid(bc.c), dim3(VEC_THREADS), sh, st, bc, pass);
   }
-  k_band_beta<<<bc.c.Bs, 32, 0, st>>>(bc, mode, idx);
-  k_band_normalize<<<vec_grid(bc.c), VEC_THREADS, 0, st>>>(bc);
+  launch_pdl(k_band_beta, dim3(bc.c.Bs), dim3(32), 0, st, bc, mode, idx);
+  launch_pdl(k_band_normalize, vec_grid(bc.c), dim3(VEC_THREADS), 0, st, bc);
   return 8;
 }
 void launch_band_finish(const BandCtx &bc, cudaStream_t st) {
-  k_band_finish<<<(bc.c.Bs + 255) / 256, 256, 0, st>>>(bc);
+  launch_pdl(k_band_finish, dim3((bc.c.Bs + 255) / 256), dim3(256), 0, st, bc);
 }
 void launch_band_small(const double *Tb, const double *R0, const int *keff, int G, int k, int p,
                        const double *xs, int nx, double tol, double *scratch, double *alpha,
                        double *beta, double *beta0, int *keff_out, cudaStream_t st) {
   const int warps = 4;
   const int n = nx * G;
-  k_band_small<<<(n + warps - 1) / warps, 32 * warps, 0, st>>>(
-      Tb, R0, keff, G, k, p, xs, nx, tol, scratch, alpha, beta, beta0, keff_out);
+  launch_pdl(k_band_small, dim3((n + warps - 1) / warps), dim3(32 * warps), 0, st, Tb, R0, keff,
+             G, k, p, xs, nx, tol, scratch, alpha, beta, beta0, keff_out);
 }
 void launch_band_combine(const double *sig, int p, int F, double *out, cudaStream_t st) {
   dim3 grid((F + 127) / 128, p * p);
-  k_band_combine<<<grid, 128, 0, st>>>(sig, p, F, out);
+  launch_pdl(k_band_combine, grid, dim3(128), 0, st, sig, p, F, out);
 }
 
 void launch_start_from_v(const VecCtx &c, const double *V, int ldv, int n_valid, cudaStream_t st) {
-  k_start_from_v<<<vec_grid(c), VEC_THREADS, 0, st>>>(c, V, ldv, n_valid);
+  launch_pdl(k_start_from_v, vec_grid(c), dim3(VEC_THREADS), 0, st, c, V, ldv, n_valid);
 }
 void launch_start_from_vf(const VecCtx &c, const float *vf, cudaStream_t st) {
-  k_start_from_vf<<<vec_grid(c), VEC_THREADS, 0, st>>>(c, vf);
+  launch_pdl(k_start_from_vf, vec_grid(c), dim3(VEC_THREADS), 0, st, c, vf);
 }
 void launch_norm_partials(const VecCtx &c, const double *x, double *out, cudaStream_t st) {
-  k_norm_partials<<<vec_grid(c), VEC_THREADS, 0, st>>>(c, x, out);
+  launch_pdl(k_norm_partials, vec_grid(c), dim3(VEC_THREADS), 0, st, c, x, out);
 }
 // grid of the kernels that take c.cpb chunks per block
 static dim3 vec_grid_cpb(const VecCtx &c) {
@@ -1120,40 +1145,41 @@ static dim3 vec_grid_cpb(const VecCtx &c) {
 }
 void launch_normalize(const VecCtx &c, int j, int is_start, const double *, cudaStream_t st) {
   const dim3 g = vec_grid_cpb(c);
-  k_normalize<<<dim3(g.y, g.x), VEC_THREADS, 0, st>>>(c, j, is_start);
+  launch_pdl(k_normalize, dim3(g.y, g.x), dim3(VEC_THREADS), 0, st, c, j, is_start);
 }
 void launch_assemble_w(const VecCtx &c, int j, const float *ucd, cudaStream_t st) {
-  k_assemble_w<<<vec_grid_cpb(c), VEC_THREADS, 0, st>>>(c, j, ucd);
+  launch_pdl(k_assemble_w, vec_grid_cpb(c), dim3(VEC_THREADS), 0, st, c, j, ucd);
 }
 void launch_alpha_reduce(const VecCtx &c, int j, cudaStream_t st) {
-  k_alpha_reduce<<<c.Bs, 32, 0, st>>>(c, j);
+  launch_pdl(k_alpha_reduce, dim3(c.Bs), dim3(32), 0, st, c, j);
 }
 void launch_alpha_axpy(const VecCtx &c, int j, cudaStream_t st) {
   if (c.reorth != LGW_REORTH_NONE)
-    k_alpha_axpy<true><<<vec_grid_cpb(c), VEC_THREADS, 0, st>>>(c, j);
+    launch_pdl(k_alpha_axpy<true>, vec_grid_cpb(c), dim3(VEC_THREADS), 0, st, c, j);
   else
-    k_alpha_axpy<false><<<vec_grid_cpb(c), VEC_THREADS, 0, st>>>(c, j);
+    launch_pdl(k_alpha_axpy<false>, vec_grid_cpb(c), dim3(VEC_THREADS), 0, st, c, j);
 }
 void launch_beta_vec(const VecCtx &c, int j, cudaStream_t st) {
-  k_beta_vec<<<c.Bs, 32, 0, st>>>(c, j);
+  launch_pdl(k_beta_vec, dim3(c.Bs), dim3(32), 0, st, c, j);
 }
 void launch_reduce_dots(const VecCtx &c, int j, int pass, cudaStream_t st) {
-  k_reduce_dots<<<c.Bs, 256, 0, st>>>(c, j, pass);
+  launch_pdl(k_reduce_dots, dim3(c.Bs), dim3(256), 0, st, c, j, pass);
 }
 void launch_update(const VecCtx &c, int j, int pass, cudaStream_t st) {
   size_t sh = (size_t)c.kmax1 * sizeof(double);
-  k_update<<<vec_grid(c), VEC_THREADS, sh, st>>>(c, j, pass);
+  launch_pdl(k_update, vec_grid(c), dim3(VEC_THREADS), sh, st, c, j, pass);
 }
 void launch_dots(const VecCtx &c, int j, int, cudaStream_t st) {
-  k_dots<<<vec_grid(c), VEC_THREADS, 0, st>>>(c, j);
+  launch_pdl(k_dots, vec_grid(c), dim3(VEC_THREADS), 0, st, c, j);
 }
 void launch_second_pass_decide_j(const VecCtx &c, int j, cudaStream_t st) {
-  k_second_pass_decide<<<(c.Bs + 255) / 256, 256, 0, st>>>(c, j);
+  launch_pdl(k_second_pass_decide, dim3((c.Bs + 255) / 256), dim3(256), 0, st, c, j);
 }
 void launch_scale_rows_to_bf16(const double *x, const double *dsq, int Bs, int N,
                                __nv_bfloat16 *out, cudaStream_t st) {
   size_t n = (size_t)Bs * N;
-  k_scale_rows_to_bf16<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(x, dsq, Bs, N, out);
+  launch_pdl(k_scale_rows_to_bf16, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, x, dsq,
+             Bs, N, out);
 }
 
 }  // namespace lgw

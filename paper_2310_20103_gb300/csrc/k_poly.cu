@@ -35,6 +35,7 @@ __device__ __forceinline__ int poly_elem_base(int chunk) {
 constexpr int CHEB_VECS = 4;
 
 __global__ void __launch_bounds__(VEC_THREADS) k_cheb_step(PolyStep p, int Bs) {
+  pdl_wait();
   const int chunk = blockIdx.x;
   const int e0 = poly_elem_base(chunk);
   const double as2 = 2.0 * p.as, bs2 = 2.0 * p.bs;
@@ -85,6 +86,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_cheb_step(PolyStep p, int Bs) {
 __global__ void __launch_bounds__(VEC_THREADS) k_cheb_final(PolyStep p, const double *qprev,
                                                             const double *betaj, double *w,
                                                             double *alpha_part, int Bs) {
+  pdl_wait();
   __shared__ double red[VEC_THREADS / 32];
   const int chunk = blockIdx.x, b = blockIdx.y;
   const size_t voff = (size_t)b * p.N;
@@ -130,6 +132,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_cheb_final(PolyStep p, const do
 __global__ void k_poly_prep(const double *__restrict__ alpha, const double *__restrict__ beta,
                             const double *__restrict__ beta0, const int *__restrict__ k_eff,
                             int B, int k, JacobiBufs jb, unsigned *status) {
+  pdl_wait();
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= B) return;
   const int n = k_eff[v];
@@ -155,16 +158,18 @@ __global__ void k_poly_prep(const double *__restrict__ alpha, const double *__re
 }
 
 void launch_cheb_step(const PolyStep &p, int nchunks, int Bs, cudaStream_t st) {
-  k_cheb_step<<<dim3(nchunks, Bs / CHEB_VECS), VEC_THREADS, 0, st>>>(p, Bs);
+  launch_pdl(k_cheb_step, dim3(nchunks, Bs / CHEB_VECS), dim3(VEC_THREADS), 0, st, p, Bs);
 }
 void launch_cheb_final(const PolyStep &p, const double *qprev, const double *betaj, double *w,
                        double *alpha_part, int nchunks, int Bs, cudaStream_t st) {
-  k_cheb_final<<<dim3(nchunks, Bs), VEC_THREADS, 0, st>>>(p, qprev, betaj, w, alpha_part, Bs);
+  launch_pdl(k_cheb_final, dim3(nchunks, Bs), dim3(VEC_THREADS), 0, st, p, qprev, betaj, w,
+             alpha_part, Bs);
 }
 void launch_poly_prep(const double *alpha, const double *beta, const double *beta0,
                       const int *k_eff, int B, int k, JacobiBufs jb, unsigned *status,
                       cudaStream_t st) {
-  k_poly_prep<<<(B + 127) / 128, 128, 0, st>>>(alpha, beta, beta0, k_eff, B, k, jb, status);
+  launch_pdl(k_poly_prep, dim3((B + 127) / 128), dim3(128), 0, st, alpha, beta, beta0, k_eff, B,
+             k, jb, status);
 }
 
 // Tamm-Dancoff view of a system: the Casida arrays of A = Delta + c L L^T
@@ -173,6 +178,7 @@ void launch_poly_prep(const double *alpha, const double *beta, const double *bet
 __global__ void k_tda_view(const double *__restrict__ Delta, int n_vc, int N, double c,
                            double *ones, double *cd, float *onesf, float *d2f, float *d2lo,
                            float *cdf) {
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   const bool real = i < n_vc;
@@ -188,6 +194,7 @@ __global__ void k_tda_view(const double *__restrict__ Delta, int n_vc, int N, do
 // 2i and 2i+1 of pair i carry the rows of t + t' and t - t'.
 __global__ void k_pol_rows(const double *__restrict__ src, int n_m, int len,
                            const int *__restrict__ pairs, int n_pairs, double *__restrict__ dst) {
+  pdl_wait();
   const size_t row_len = (size_t)n_m * len;
   const size_t n = (size_t)n_pairs * 2 * row_len;
   for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
@@ -202,6 +209,7 @@ __global__ void k_pol_rows(const double *__restrict__ src, int n_m, int len,
 
 __global__ void k_pol_combine(const double *__restrict__ sig2, int n_pairs, int n_freq,
                               double *__restrict__ out) {
+  pdl_wait();
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   const size_t per = (size_t)n_freq * 2;
   if (idx >= (size_t)n_pairs * per) return;
@@ -211,20 +219,22 @@ __global__ void k_pol_combine(const double *__restrict__ sig2, int n_pairs, int 
 
 void launch_tda_view(const double *Delta, int n_vc, int N, double c, double *ones, double *cd,
                      float *onesf, float *d2f, float *d2lo, float *cdf, cudaStream_t st) {
-  k_tda_view<<<(N + 255) / 256, 256, 0, st>>>(Delta, n_vc, N, c, ones, cd, onesf, d2f, d2lo,
-                                               cdf);
+  launch_pdl(k_tda_view, dim3((N + 255) / 256), dim3(256), 0, st, Delta, n_vc, N, c, ones, cd,
+             onesf, d2f, d2lo, cdf);
 }
 void launch_pol_rows(const double *src, int n_m, int len, const int *pairs, int n_pairs,
                      double *dst, cudaStream_t st) {
   const size_t n = (size_t)n_pairs * 2 * n_m * len;
   size_t blocks = (n + 255) / 256;
   if (blocks > 152 * 64) blocks = 152 * 64;
-  if (n) k_pol_rows<<<(unsigned)blocks, 256, 0, st>>>(src, n_m, len, pairs, n_pairs, dst);
+  if (n) launch_pdl(k_pol_rows, dim3((unsigned)blocks), dim3(256), 0, st, src, n_m, len, pairs,
+                    n_pairs, dst);
 }
 void launch_pol_combine(const double *sig2, int n_pairs, int n_freq, double *out,
                         cudaStream_t st) {
   const size_t n = (size_t)n_pairs * n_freq * 2;
-  if (n) k_pol_combine<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(sig2, n_pairs, n_freq, out);
+  if (n) launch_pdl(k_pol_combine, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, sig2,
+                    n_pairs, n_freq, out);
 }
 
 }  // namespace lgw

@@ -9,6 +9,7 @@ namespace lgw {
 __global__ void k_pair_energies(const double *__restrict__ eps, int n_v, int n_c, int n_vc, int N,
                                 double kf, double *Delta, double *dsq, double *Delta2,
                                 double *cd, float *dsqf, float *d2f, float *d2lo, float *cdf) {
+  pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   double D = 0.0;
@@ -28,6 +29,7 @@ __global__ void k_pair_energies(const double *__restrict__ eps, int n_v, int n_c
 }
 
 __global__ void k_check_delta(const double *__restrict__ Delta, int n_vc, unsigned *status) {
+  pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n_vc && !(Delta[i] > 0.0)) atomicOr(status, ST_NOT_SPD);
 }
@@ -35,6 +37,7 @@ __global__ void k_check_delta(const double *__restrict__ Delta, int n_vc, unsign
 // L [n_vc][n_aux] -> L64 [N][A], zero padded.
 __global__ void k_pad_L(const double *__restrict__ L, int n_vc, int n_aux, int N, int A,
                         double *__restrict__ L64) {
+  pdl_wait();
   int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int64_t total = (int64_t)N * A;
   for (; idx < total; idx += (int64_t)gridDim.x * blockDim.x) {
@@ -49,6 +52,7 @@ __global__ void k_pad_L(const double *__restrict__ L, int n_vc, int n_aux, int N
 __global__ void k_quantize_L(const double *__restrict__ src, int ld, int nr, int nc, int N, int A,
                              __nv_bfloat16 *__restrict__ Lb, __nv_bfloat16 *__restrict__ Ltb,
                              __nv_bfloat16 *__restrict__ Lb_lo) {
+  pdl_wait();
   __shared__ __nv_bfloat16 tile[32][33];
   int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
   int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 32 x 8 threads
@@ -72,13 +76,13 @@ __global__ void k_quantize_L(const double *__restrict__ src, int ld, int nr, int
 
 void launch_pair_energies(const SysDev &s, cudaStream_t st) {
   int th = 256, bl = (s.N + th - 1) / th;
-  k_pair_energies<<<bl, th, 0, st>>>(s.eps, s.n_v, s.n_c, s.n_vc, s.N, s.kf, s.Delta, s.dsq,
-                                     s.Delta2, s.cd, s.dsqf, s.d2f, s.d2lo, s.cdf);
+  launch_pdl(k_pair_energies, dim3(bl), dim3(th), 0, st, s.eps, s.n_v, s.n_c, s.n_vc, s.N, s.kf,
+             s.Delta, s.dsq, s.Delta2, s.cd, s.dsqf, s.d2f, s.d2lo, s.cdf);
 }
 
 void launch_check_delta(const SysDev &s, unsigned *status, cudaStream_t st) {
   int th = 256, bl = (s.n_vc + th - 1) / th;
-  k_check_delta<<<bl, th, 0, st>>>(s.Delta, s.n_vc, status);
+  launch_pdl(k_check_delta, dim3(bl), dim3(th), 0, st, s.Delta, s.n_vc, status);
 }
 
 void launch_pad_L(const double *L, const SysDev &s, cudaStream_t st) {
@@ -86,13 +90,14 @@ void launch_pad_L(const double *L, const SysDev &s, cudaStream_t st) {
   int th = 256;
   int64_t bl = (total + th - 1) / th;
   if (bl > 152 * 64) bl = 152 * 64;
-  k_pad_L<<<(int)bl, th, 0, st>>>(L, s.n_vc, s.n_aux, s.N, s.A, s.L64);
+  launch_pdl(k_pad_L, dim3((int)bl), dim3(th), 0, st, L, s.n_vc, s.n_aux, s.N, s.A, s.L64);
 }
 
 void launch_quantize_L(const double *src, int ld, int nr, int nc, const SysDev &s,
                        cudaStream_t st) {
   dim3 grid((s.A + 31) / 32, (s.N + 31) / 32);
-  k_quantize_L<<<grid, 256, 0, st>>>(src, ld, nr, nc, s.N, s.A, s.Lb, s.Ltb, s.Lb_lo);
+  launch_pdl(k_quantize_L, grid, dim3(256), 0, st, src, ld, nr, nc, s.N, s.A, s.Lb, s.Ltb,
+             s.Lb_lo);
 }
 
 }  // namespace lgw

@@ -123,6 +123,7 @@ __device__ __forceinline__ void dot_row_df(const float *__restrict__ qh,
 // partial.  No block barrier inside the row loop.
 template <int PASS>
 __global__ void __launch_bounds__(VEC_THREADS, 2) k_dots_split(VecCtx c, int j) {
+  pdl_wait();
   __shared__ __align__(16) float swh[VEC_CHUNK];
   __shared__ __align__(16) float swl[VEC_CHUNK];
   __shared__ double red[VEC_THREADS / 32];
@@ -254,6 +255,7 @@ __device__ __forceinline__ double chunk_sum(const double *p, size_t stride, int 
 // Not-live vectors get flag2 = 0 and 1/beta = 0, so the update writes
 // zeros into their next slot.
 __global__ void __launch_bounds__(256) k_reduce_dots_split(VecCtx c, int j, int pass) {
+  pdl_wait();
   __shared__ double red[256 / 32], col[16 * 256];
   const int b = blockIdx.x;
   const int v = c.vec0 + b;
@@ -311,6 +313,7 @@ __global__ void __launch_bounds__(256) k_reduce_dots_split(VecCtx c, int j, int 
 // next slot.
 template <int PASS>
 __global__ void __launch_bounds__(VEC_THREADS) k_update_split(VecCtx c, int j) {
+  pdl_wait();
   extern __shared__ float hsf[];
   __shared__ double red[VEC_THREADS / 32];
   __shared__ float sdq[VEC_THREADS / 32];
@@ -410,6 +413,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_update_split(VecCtx c, int j) {
 // into ring slot 0, the split basis slot 0 and the bf16 contraction
 // operand; beta0, k_eff and the per-vector state of the recurrence.
 __global__ void __launch_bounds__(VEC_THREADS) k_start_split(VecCtx c) {
+  pdl_wait();
   const int chunk = blockIdx.x, b = blockIdx.y;
   const int v = c.vec0 + b;
   __shared__ double sbeta, sinv;
@@ -816,6 +820,7 @@ __global__ void __launch_bounds__(VEC_THREADS, 2) k_sweep_dcgs(VecCtx c, int j) 
   const int chunk = blockIdx.x, b = blockIdx.y;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int ebase = chunk * VEC_CHUNK + wid * 256 + 4 * lane;
+  pdl_wait();
   if (!live_s(c, b, j)) {
     // stopped or padding vector: the contractions see zeros
     if (c.xh != nullptr) {
@@ -1031,6 +1036,7 @@ __global__ void __launch_bounds__(256) k_reduce_dcgs(VecCtx c, int j) {
   __shared__ double red[256 / 32], col[16 * 256];
   const int b = blockIdx.x;
   const int v = c.vec0 + b;
+  pdl_wait();
   if (!live_s(c, b, j)) {
     if (threadIdx.x == 0) {
       c.flag2[b] = 0;
@@ -1100,6 +1106,7 @@ __global__ void __launch_bounds__(VEC_THREADS) k_p2_dcgs(VecCtx c, int j) {
       reinterpret_cast<double *>(reinterpret_cast<char *>(stg) + sweep_stage_bytes<LO>());
   __shared__ double red[VEC_THREADS / 32];
   __shared__ float2 part[2][32][VEC_THREADS / 32];
+  pdl_wait();
   if (!c.p2_step[j]) return;
   const int chunk = blockIdx.x;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1191,6 +1198,7 @@ __global__ void __launch_bounds__(256) k_p2_reduce_dcgs(VecCtx c, int j) {
   __shared__ double red[256 / 32], col[16 * 256];
   const int b = blockIdx.x;
   const int v = c.vec0 + b;
+  pdl_wait();
   if (!c.p2_step[j] || !c.flag2[b]) return;
   double hh = 0.0;
   for (int i = threadIdx.x; i <= j; i += blockDim.x) {
@@ -1228,7 +1236,7 @@ static void sweep_one(const VecCtx &c, int j, cudaStream_t st) {
     attr = true;
   }
   const size_t sh = sweep_stage_bytes<LO>() + (size_t)(j > 0 ? j : 1) * sizeof(float2);
-  k_sweep_dcgs<LO, F64U><<<dim3(c.nchunks, c.Bs), VEC_THREADS, sh, st>>>(c, j);
+  launch_pdl(k_sweep_dcgs<LO, F64U>, dim3(c.nchunks, c.Bs), dim3(VEC_THREADS), sh, st, c, j);
 }
 
 void launch_sweep_dcgs(const VecCtx &c, int j, cudaStream_t st) {
@@ -1243,7 +1251,7 @@ void launch_sweep_dcgs(const VecCtx &c, int j, cudaStream_t st) {
     sweep_one<false, false>(c, j, st);
 }
 void launch_reduce_dcgs(const VecCtx &c, int j, cudaStream_t st) {
-  k_reduce_dcgs<<<c.Bs, 256, 0, st>>>(c, j);
+  launch_pdl(k_reduce_dcgs, dim3(c.Bs), dim3(256), 0, st, c, j);
 }
 template <bool LO>
 static void pass2_one(const VecCtx &c, int j, cudaStream_t st) {
@@ -1253,37 +1261,37 @@ static void pass2_one(const VecCtx &c, int j, cudaStream_t st) {
     attr = true;
   }
   const dim3 grid(c.nchunks, c.Bs < 16 ? c.Bs : 16);
-  k_p2_dcgs<LO><<<grid, VEC_THREADS, sweep_stage_bytes<LO>() + (size_t)(j + 1) * sizeof(double),
-                  st>>>(c, j);
+  launch_pdl(k_p2_dcgs<LO>, grid, dim3(VEC_THREADS),
+             sweep_stage_bytes<LO>() + (size_t)(j + 1) * sizeof(double), st, c, j);
 }
 void launch_pass2_dcgs(const VecCtx &c, int j, cudaStream_t st) {
   if (c.blo != nullptr)
     pass2_one<true>(c, j, st);
   else
     pass2_one<false>(c, j, st);
-  k_p2_reduce_dcgs<<<c.Bs, 256, 0, st>>>(c, j);
+  launch_pdl(k_p2_reduce_dcgs, dim3(c.Bs), dim3(256), 0, st, c, j);
 }
 
 static dim3 grid_s(const VecCtx &c) { return dim3(c.nchunks, c.Bs); }
 
 void launch_dots_split(const VecCtx &c, int j, int pass, cudaStream_t st) {
   if (pass == 1)
-    k_dots_split<1><<<grid_s(c), VEC_THREADS, 0, st>>>(c, j);
+    launch_pdl(k_dots_split<1>, grid_s(c), dim3(VEC_THREADS), 0, st, c, j);
   else
-    k_dots_split<2><<<grid_s(c), VEC_THREADS, 0, st>>>(c, j);
+    launch_pdl(k_dots_split<2>, grid_s(c), dim3(VEC_THREADS), 0, st, c, j);
 }
 void launch_reduce_dots_split(const VecCtx &c, int j, int pass, cudaStream_t st) {
-  k_reduce_dots_split<<<c.Bs, 256, 0, st>>>(c, j, pass);
+  launch_pdl(k_reduce_dots_split, dim3(c.Bs), dim3(256), 0, st, c, j, pass);
 }
 void launch_update_split(const VecCtx &c, int j, int pass, cudaStream_t st) {
   const size_t sh = (size_t)c.kmax1 * sizeof(float);
   if (pass == 1)
-    k_update_split<1><<<grid_s(c), VEC_THREADS, sh, st>>>(c, j);
+    launch_pdl(k_update_split<1>, grid_s(c), dim3(VEC_THREADS), sh, st, c, j);
   else
-    k_update_split<2><<<grid_s(c), VEC_THREADS, sh, st>>>(c, j);
+    launch_pdl(k_update_split<2>, grid_s(c), dim3(VEC_THREADS), sh, st, c, j);
 }
 void launch_start_split(const VecCtx &c, cudaStream_t st) {
-  k_start_split<<<grid_s(c), VEC_THREADS, 0, st>>>(c);
+  launch_pdl(k_start_split, grid_s(c), dim3(VEC_THREADS), 0, st, c);
 }
 
 }  // namespace lgw

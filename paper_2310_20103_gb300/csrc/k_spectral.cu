@@ -192,6 +192,7 @@ __global__ void __launch_bounds__(SPEC_THREADS) k_spectral(
     const double *__restrict__ alpha, const double *__restrict__ beta,
     const double *__restrict__ beta0, const int *__restrict__ k_eff, int k, JacobiBufs jb,
     unsigned long long *min_theta_bits, unsigned *status) {
+  pdl_wait();
   extern __shared__ double2 ab[];                       // [k] scaled (a, b^2)
   float2 *abf = reinterpret_cast<float2 *>(ab + k);     // [k] the same about the middle, FP32
   double *ths = reinterpret_cast<double *>(abf + k);    // [k] scaled nodes
@@ -327,7 +328,8 @@ void launch_spectral_impl(const double *alpha, const double *beta, const double 
   }
   const int threads = std::min(SPEC_THREADS, (k + 31) / 32 * 32);
   const size_t sh = (size_t)k * (sizeof(double2) + sizeof(float2) + 2 * sizeof(double));
-  k_spectral<<<B, threads, sh, st>>>(alpha, beta, beta0, k_eff, k, jb, min_theta_bits, status);
+  launch_pdl(k_spectral, dim3(B), dim3(threads), sh, st, alpha, beta, beta0, k_eff, k, jb,
+             min_theta_bits, status);
 }
 
 // ---------------------------------------------------------------------------
@@ -337,6 +339,7 @@ void launch_spectral_impl(const double *alpha, const double *beta, const double 
 // Start vector with entries uniform in [-1, 1) from a counter-based hash
 // (splitmix64 of seed + index), zero in the padding.
 __global__ void k_hash_vector(double *v, int n_vc, int N, unsigned long long seed) {
+  pdl_wait();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= N) return;
   if (e >= n_vc) {
@@ -371,6 +374,7 @@ __device__ int sturm_below(const double *a, const double *b, int n, double x, do
 // can lie from an eigenvalue.
 __global__ void k_interval(const double *__restrict__ Delta2, int n_vc, const double *a,
                            const double *b, const int *k_eff, double *out) {
+  pdl_wait();
   __shared__ double red[256];
   double m = 1e300;
   for (int e = threadIdx.x; e < n_vc; e += blockDim.x) m = fmin(m, Delta2[e]);
@@ -407,8 +411,8 @@ void launch_interval(const double *Delta2, int n_vc, int N, const double *a, con
                      const int *k_eff, double *out, double *vec, unsigned long long seed,
                      bool make_vector, cudaStream_t st) {
   if (make_vector)
-    k_hash_vector<<<(N + 255) / 256, 256, 0, st>>>(vec, n_vc, N, seed);
+    launch_pdl(k_hash_vector, dim3((N + 255) / 256), dim3(256), 0, st, vec, n_vc, N, seed);
   else
-    k_interval<<<1, 256, 0, st>>>(Delta2, n_vc, a, b, k_eff, out);
+    launch_pdl(k_interval, dim3(1), dim3(256), 0, st, Delta2, n_vc, a, b, k_eff, out);
 }
 }  // namespace lgw

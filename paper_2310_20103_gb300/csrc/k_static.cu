@@ -16,6 +16,7 @@ namespace lgw {
 
 __global__ void k_sigma_x(const double *__restrict__ M, int n_m, int n_aux,
                           const int *__restrict__ m_idx, int n_v, double *__restrict__ out) {
+  pdl_wait();
   __shared__ double red[8];
   const int t = blockIdx.x;
   double s = 0.0;
@@ -68,6 +69,7 @@ constexpr int POTRF_THREADS = 128, PW = 8;
 
 __global__ void __launch_bounds__(POTRF_THREADS) k_potrf_diag(double *A, int n, int j0,
                                                               unsigned *status) {
+  pdl_wait();
   __shared__ double blk[NB][NB + 1];
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int nb = min(NB, n - j0);
@@ -152,6 +154,7 @@ __global__ void __launch_bounds__(POTRF_THREADS) k_potrf_diag(double *A, int n, 
 constexpr int TRSM_ROWS = 16;
 
 __global__ void __launch_bounds__(8 * TRSM_ROWS) k_trsm_panel(double *A, int n, int j0) {
+  pdl_wait();
   __shared__ double Ljj[NB][NB + 1];
   __shared__ double rd[NB];
   const int t = threadIdx.x, l = t & 7;
@@ -195,6 +198,7 @@ __global__ void __launch_bounds__(8 * TRSM_ROWS) k_trsm_panel(double *A, int n, 
 // 64 x 64 tiles left most of the chip without one (86 us per update on average
 // at n 1024; 46 us now).
 __global__ void __launch_bounds__(256) k_syrk_update(double *A, int n, int j0, int nb) {
+  pdl_wait();
   const int t0 = j0 + nb;
   const int bi = blockIdx.y, bj = blockIdx.x;
   if (bj > bi) return;
@@ -230,6 +234,7 @@ __global__ void __launch_bounds__(256) k_syrk_update(double *A, int n, int j0, i
 }
 
 __global__ void k_zero_upper(double *A, int n) {
+  pdl_wait();
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (size_t)n * n) return;
   const int i = (int)(idx / n), j = (int)(idx % n);
@@ -240,6 +245,7 @@ __global__ void k_zero_upper(double *A, int n) {
 __global__ void __launch_bounds__(256) k_gemm_nn_f64(const double *__restrict__ Am,
                                                      const double *__restrict__ Bm, int M, int N,
                                                      int K, double *__restrict__ Cm) {
+  pdl_wait();
   __shared__ double As[16][65];
   __shared__ double Bs[16][65];
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
@@ -284,31 +290,32 @@ __global__ void __launch_bounds__(256) k_gemm_nn_f64(const double *__restrict__ 
 // ----------------------------------------------------------------------------
 void launch_sigma_x(const double *M, int n_t, int n_m, int n_aux, const int *m_idx, int n_v,
                     double *out, cudaStream_t st) {
-  if (n_t > 0) k_sigma_x<<<n_t, 256, 0, st>>>(M, n_m, n_aux, m_idx, n_v, out);
+  if (n_t > 0) launch_pdl(k_sigma_x, dim3(n_t), dim3(256), 0, st, M, n_m, n_aux, m_idx, n_v, out);
 }
 
 int launch_cholesky(double *A, int n, unsigned *status, cudaStream_t st) {
   int launches = 0;
   for (int j0 = 0; j0 < n; j0 += NB) {
     const int nb = std::min(NB, n - j0);
-    k_potrf_diag<<<1, POTRF_THREADS, 0, st>>>(A, n, j0, status);
+    launch_pdl(k_potrf_diag, dim3(1), dim3(POTRF_THREADS), 0, st, A, n, j0, status);
     ++launches;
     const int rest = n - j0 - nb;
     if (rest > 0) {
-      k_trsm_panel<<<(rest + TRSM_ROWS - 1) / TRSM_ROWS, 8 * TRSM_ROWS, 0, st>>>(A, n, j0);
+      launch_pdl(k_trsm_panel, dim3((rest + TRSM_ROWS - 1) / TRSM_ROWS), dim3(8 * TRSM_ROWS), 0,
+                 st, A, n, j0);
       const int tiles = (rest + 31) / 32;
-      k_syrk_update<<<dim3(tiles, tiles), 256, 0, st>>>(A, n, j0, nb);
+      launch_pdl(k_syrk_update, dim3(tiles, tiles), dim3(256), 0, st, A, n, j0, nb);
       launches += 2;
     }
   }
-  k_zero_upper<<<(unsigned)(((size_t)n * n + 255) / 256), 256, 0, st>>>(A, n);
+  launch_pdl(k_zero_upper, dim3((unsigned)(((size_t)n * n + 255) / 256)), dim3(256), 0, st, A, n);
   return launches + 1;
 }
 
 void launch_gemm_nn_f64(const double *A, const double *B, int M, int N, int K, double *C,
                         cudaStream_t st) {
   dim3 grid((N + 63) / 64, (M + 63) / 64);
-  k_gemm_nn_f64<<<grid, 256, 0, st>>>(A, B, M, N, K, C);
+  launch_pdl(k_gemm_nn_f64, grid, dim3(256), 0, st, A, B, M, N, K, C);
 }
 
 }  // namespace lgw

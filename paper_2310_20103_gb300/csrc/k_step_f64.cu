@@ -147,6 +147,7 @@ __global__ void __launch_bounds__(VEC_THREADS, GS ? 2 : 4)
   __shared__ double sred[GS ? VEC_THREADS / 32 : 1][16];
   __shared__ double part[3];        // the block's ||w||^2 before, between and after the passes
   __shared__ int xmax;
+  pdl_wait();
   cg::cluster_group cl = cg::this_cluster();
   const int nb = gridDim.x, chunk = blockIdx.x, b = blockIdx.y, v = c.vec0 + b;
   const bool lead = chunk == 0 && threadIdx.x == 0;
@@ -307,12 +308,14 @@ void launch_one(const VecCtx &c, int j, const OzOperand &x, cudaStream_t st) {
   cfg.blockDim = dim3(VEC_THREADS);
   cfg.dynamicSmemBytes = GS ? (size_t)3 * c.kmax1 * sizeof(double) : 0;
   cfg.stream = st;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = c.nchunks;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute at[2] = {};
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = c.nchunks;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
   cudaLaunchKernelEx(&cfg, k_step_f64<GS>, c, j, x);
 }
 }  // namespace

@@ -3084,6 +3084,7 @@ double *g_noalloc_addr[kMaxDevices] = {nullptr};
 __global__ void k_noalloc_prologue(unsigned long long *min_theta_bits, const int *targets, int n_t,
                                    const int *m_idx, int n_m, int norb, const int *k_eff, int B,
                                    int k, unsigned *status) {
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i == 0) *min_theta_bits = 0x7FEFFFFFFFFFFFFFull;   // largest finite double
   if (i < n_t && (targets[i] < 0 || targets[i] >= norb)) atomicOr(status, ST_BAD_INPUT);
@@ -3176,8 +3177,8 @@ extern "C" lgw_status lgw_sigma_from_coeffs_noalloc(lgw_handle *h, const lgw_sys
   // Index check first, and its verdict read back before any kernel that
   // dereferences an index (eps[m], eps[t], the k_eff-deep rows) is queued.
   const size_t nmax = std::max<size_t>(std::max(n_t, n_m), B);
-  k_noalloc_prologue<<<(unsigned)((nmax + 255) / 256), 256, 0, st>>>(
-      mt, p->targets, n_t, p->m_idx, n_m, s.n_v + s.n_c, k_eff, (int)B, k, h->d_status);
+  launch_pdl(k_noalloc_prologue, dim3((unsigned)((nmax + 255) / 256)), dim3(256), 0, st, mt,
+             p->targets, n_t, p->m_idx, n_m, s.n_v + s.n_c, k_eff, (int)B, k, h->d_status);
   {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess)
