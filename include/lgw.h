@@ -297,7 +297,10 @@ lgw_status lgw_selftest_bounded_wait(lgw_handle *h, int32_t arrive, double secon
  * LGW_ERR_ARG for unknown flags or LGW_SYS_NO_FP64 | LGW_SYS_NO_BF16. */
 lgw_status lgw_prepare_system(lgw_handle *h, const lgw_system_desc *desc, lgw_system **out);
 
-/* Free a system's device memory.  NULL is accepted. */
+/* Free a system's device memory.  NULL is accepted.  Up to 2 GiB of it stay
+ * with the handle for its next system, unless the handle has a workspace
+ * limit; lgw_release_workspace, lgw_set_workspace_limit and lgw_destroy free
+ * them, and so does an allocation of the handle that would fail. */
 lgw_status lgw_release_system(lgw_system *s);
 
 /* Apply C to n_vec vectors: Y[i] = C X[i], X and Y [n_vec][n_v*n_c] FP64,

@@ -1,6 +1,7 @@
 // C ABI of the lgw library: argument checks, host/device staging, workspace
 // management and the per-sub-batch schedule of the hot path.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -47,6 +48,12 @@ struct lgw_handle {
   std::vector<cudaStream_t> lanes;
   std::string ws_prefix;
   std::vector<lgw_system *> sliced;   // systems that hold digits of L (k_gemm_oz.cu)
+  // device memory of systems: the size of every block, and the blocks of
+  // released systems that the next one may take (SPARE_MAX bytes at most)
+  std::mutex mem_mu;
+  std::map<void *, size_t> sys_mem;
+  std::multimap<size_t, void *> spare;
+  size_t spare_bytes = 0;
   void drop_graphs() {
     for (auto &kv : graphs)
       if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
@@ -111,23 +118,91 @@ void check_launch(lgw_handle *h, const char *what) {
   }
 }
 
+// Memory of systems.  A gradient prepares and releases a system in each of its
+// two passes, and the driver maps and unmaps its memory every time: 3.1 ms of
+// cudaMalloc and cudaFree in the 19.2 ms of an exact gradient at N_vc 32768,
+// N_aux 1024 (1.5 GB).  A handle therefore keeps up to 2 GiB of released
+// blocks for its next system (all handles of the process together: less than
+// 1% of the device); they go back with lgw_release_workspace, lgw_destroy, when
+// a byte limit is set, and before any allocation of the handle is refused.
+constexpr size_t SPARE_MAX = (size_t)2 << 30;
+std::atomic<size_t> spare_total{0};
+
+void spare_free(lgw_handle *h) {
+  std::lock_guard<std::mutex> lock(h->mem_mu);
+  for (auto &kv : h->spare) {
+    cudaFree(kv.second);
+    h->sys_mem.erase(kv.second);
+  }
+  h->spare.clear();
+  spare_total -= h->spare_bytes;
+  h->spare_bytes = 0;
+}
+
+// NULL (and no sticky error) where the device has no room.
+void *sys_alloc(lgw_handle *h, size_t bytes) {
+  {
+    // the smallest spare block that fits and wastes at most a quarter
+    std::lock_guard<std::mutex> lock(h->mem_mu);
+    auto it = h->spare.lower_bound(bytes);
+    if (it != h->spare.end() && it->first <= bytes + bytes / 4) {
+      void *p = it->second;
+      h->spare_bytes -= it->first;
+      spare_total -= it->first;
+      h->spare.erase(it);
+      return p;
+    }
+  }
+  void *p = nullptr;
+  if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    spare_free(h);
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+  }
+  std::lock_guard<std::mutex> lock(h->mem_mu);
+  h->sys_mem[p] = bytes;
+  return p;
+}
+
+// The caller has waited for the work that uses the block.
+void sys_free(lgw_handle *h, void *p) {
+  if (!p) return;
+  std::lock_guard<std::mutex> lock(h->mem_mu);
+  const auto it = h->sys_mem.find(p);
+  const size_t n = it->second;
+  if (h->ws_limit == 0) {
+    if (spare_total.fetch_add(n) + n <= SPARE_MAX) {
+      h->spare.emplace(n, p);
+      h->spare_bytes += n;
+      return;
+    }
+    spare_total -= n;
+  }
+  h->sys_mem.erase(it);
+  cudaFree(p);
+}
+
 void free_digits(lgw_system *sys) {
-  if (sys->oz_buf) cudaFree(sys->oz_buf);
+  sys_free(sys->h, sys->oz_buf);
   sys->oz_buf = nullptr;
   sys->s.ozA = sys->s.ozT = sys->tda.ozA = sys->tda.ozT = OzOperand{};
   sys->oz_state = -1;
 }
 
-// Gives back every system's digits of L and the workspace of the digits
-// (oz_* buffers); the FP64 products then run on the CUDA cores.  False if
+// Gives back every system's digits of L, the workspace of the digits (oz_*
+// buffers) and the spare blocks; the FP64 products then run on the CUDA cores.  False if
 // there was nothing to give back.
 bool drop_digits(lgw_handle *h) {
-  bool any = !h->sliced.empty();
+  bool any = !h->sliced.empty() || h->spare_bytes != 0;
   for (auto &kv : h->bufs) any = any || (kv.first.find("oz_") != std::string::npos && kv.second.p);
   if (!any) return false;
   cudaDeviceSynchronize();
   for (lgw_system *sys : h->sliced) free_digits(sys);
   h->sliced.clear();
+  spare_free(h);
   for (auto &kv : h->bufs)
     if (kv.first.find("oz_") != std::string::npos && kv.second.p) {
       cudaFree(kv.second.p);
@@ -164,6 +239,11 @@ void *ws(lgw_handle *h, const std::string &name, size_t bytes, bool optional = f
     }
     void *p = nullptr;
     cudaError_t e = cudaMalloc(&p, bytes);
+    if (e == cudaErrorMemoryAllocation && h->spare_bytes != 0) {
+      cudaGetLastError();
+      spare_free(h);
+      e = cudaMalloc(&p, bytes);
+    }
     if (e == cudaErrorMemoryAllocation && !optional && drop_digits(h)) {
       cudaGetLastError();
       e = cudaMalloc(&p, bytes);
@@ -424,14 +504,12 @@ Opts resolve_opts(lgw_handle *h, const lgw_options *o, const SysDev &s) {
 // E4M3 copies of L from src [nr][nc] (row stride ld) into s.
 void make_fp8(lgw_handle *h, SysDev &s, const double *src, int ld, int nr, int nc) {
   const size_t n = (size_t)s.N * s.A;
-  uint8_t *a = nullptr, *b = nullptr;
-  float *sc = nullptr;
-  if (cudaMalloc(&a, n) != cudaSuccess || cudaMalloc(&b, n) != cudaSuccess ||
-      cudaMalloc(&sc, sizeof(float) * s.A) != cudaSuccess) {
-    cudaGetLastError();
-    if (a) cudaFree(a);
-    if (b) cudaFree(b);
-    if (sc) cudaFree(sc);
+  uint8_t *a = static_cast<uint8_t *>(sys_alloc(h, n));
+  uint8_t *b = a ? static_cast<uint8_t *>(sys_alloc(h, n)) : nullptr;
+  float *sc = b ? static_cast<float *>(sys_alloc(h, sizeof(float) * s.A)) : nullptr;
+  if (!sc) {
+    sys_free(h, a);
+    sys_free(h, b);
     set_err(h, LGW_ERR_OOM, "device allocation for the E4M3 copies of L failed");
     throw Fail{LGW_ERR_OOM};
   }
@@ -456,12 +534,9 @@ void ensure_digits(lgw_handle *h, lgw_system *sys) {
   const size_t ints = ((size_t)s.N + s.A + 64) * sizeof(int);
   size_t fr = 0, tot = 0;
   LGW_TRY_CUDA(h, cudaMemGetInfo(&fr, &tot));
-  if (2 * plane + ints > fr / 3) return;
-  void *p = nullptr;
-  if (cudaMalloc(&p, 2 * plane + ints) != cudaSuccess) {
-    cudaGetLastError();
-    return;
-  }
+  if (2 * plane + ints > (fr + h->spare_bytes) / 3) return;
+  void *p = sys_alloc(h, 2 * plane + ints);
+  if (!p) return;
   sys->oz_buf = p;
   uint16_t *d = static_cast<uint16_t *>(p);
   int *e = reinterpret_cast<int *>(static_cast<uint8_t *>(p) + 2 * plane);
@@ -1608,8 +1683,11 @@ const SysDev &tda_view(lgw_handle *h, const lgw_system *csys) {
   const SysDev &s = sys->s;
   if (!sys->tda_buf) {
     const size_t N = (size_t)s.N;
-    void *buf = nullptr;
-    LGW_TRY_CUDA(h, cudaMalloc(&buf, N * (2 * sizeof(double) + 4 * sizeof(float))));
+    void *buf = sys_alloc(h, N * (2 * sizeof(double) + 4 * sizeof(float)));
+    if (!buf) {
+      set_err(h, LGW_ERR_OOM, "device allocation for the Tamm-Dancoff view failed");
+      throw Fail{LGW_ERR_OOM};
+    }
     sys->tda_buf = buf;
     double *ones = static_cast<double *>(buf), *cd = ones + N;
     float *onesf = reinterpret_cast<float *>(cd + N), *d2f = onesf + N, *cdf = d2f + N;
@@ -1962,6 +2040,7 @@ lgw_status lgw_destroy(lgw_handle *h) {
   for (auto l : h->lanes) cudaStreamDestroy(l);
   for (auto &kv : h->bufs)
     if (kv.second.p) cudaFree(kv.second.p);
+  spare_free(h);
   for (auto e : h->ev_pool) cudaEventDestroy(e);
   if (h->d_status) cudaFree(h->d_status);
   delete h;
@@ -1972,6 +2051,7 @@ lgw_status lgw_set_workspace_limit(lgw_handle *h, size_t bytes) {
   lgw_status g = guard_handle(h);
   if (g != LGW_OK) return g;
   h->ws_limit = bytes;
+  if (bytes) spare_free(h);
   return LGW_OK;
 }
 
@@ -1994,6 +2074,7 @@ lgw_status lgw_release_workspace(lgw_handle *h) {
   h->bufs.clear();
   h->ws_bytes = 0;
   h->ws_gen++;
+  spare_free(h);
   return LGW_OK;
 }
 
@@ -2055,12 +2136,8 @@ lgw_status lgw_prepare_system(lgw_handle *h, const lgw_system_desc *d, lgw_syste
   s.kf = d->kernel_factor;
   std::vector<void *> allocs;
   auto alloc = [&](size_t bytes) -> void * {
-    void *p = nullptr;
-    if (cudaMalloc(&p, bytes) != cudaSuccess) {
-      cudaGetLastError();
-      return nullptr;
-    }
-    allocs.push_back(p);
+    void *p = sys_alloc(h, bytes);
+    if (p) allocs.push_back(p);
     return p;
   };
   const int flags = d->flags;
@@ -2089,7 +2166,7 @@ lgw_status lgw_prepare_system(lgw_handle *h, const lgw_system_desc *d, lgw_syste
     ok = s.Lb && s.Ltb && s.Lb_lo;
   }
   if (!ok) {
-    for (void *p : allocs) cudaFree(p);
+    for (void *p : allocs) sys_free(h, p);
     delete sys;
     return set_err(h, LGW_ERR_OOM, "device allocation for the system failed");
   }
@@ -2116,10 +2193,11 @@ lgw_status lgw_prepare_system(lgw_handle *h, const lgw_system_desc *d, lgw_syste
     if (!keep64 || (flags & LGW_SYS_FP8)) make_fp8(h, s, Lsrc, s.n_aux, s.n_vc, s.n_aux);
     check_status(h);
   } catch (Fail &f) {
-    for (void *p : allocs) cudaFree(p);
-    if (s.L8) cudaFree(s.L8);
-    if (s.L8t) cudaFree(s.L8t);
-    if (s.sL) cudaFree(s.sL);
+    cudaStreamSynchronize(h->stream);
+    for (void *p : allocs) sys_free(h, p);
+    sys_free(h, s.L8);
+    sys_free(h, s.L8t);
+    sys_free(h, s.sL);
     delete sys;
     return f.st;
   }
@@ -2136,18 +2214,17 @@ lgw_status lgw_release_system(lgw_system *sys) {
   SysDev &s = sys->s;
   void *ps[] = {s.eps,  s.Delta, s.dsq, s.Delta2, s.cd,  s.dsqf,
                 s.d2f, s.cdf,   s.L64, s.Lb,     s.Ltb, s.Lb_lo};
-  for (void *p : ps)
-    if (p) cudaFree(p);
-  if (sys->Ltb_lo) cudaFree(sys->Ltb_lo);
-  if (sys->tda_buf) cudaFree(sys->tda_buf);
+  for (void *p : ps) sys_free(sys->h, p);
+  sys_free(sys->h, sys->Ltb_lo);
+  sys_free(sys->h, sys->tda_buf);
   if (sys->oz_buf) {
     free_digits(sys);
     auto &v = sys->h->sliced;
     v.erase(std::remove(v.begin(), v.end(), sys), v.end());
   }
-  if (s.L8) cudaFree(s.L8);
-  if (s.L8t) cudaFree(s.L8t);
-  if (s.sL) cudaFree(s.sL);
+  sys_free(sys->h, s.L8);
+  sys_free(sys->h, s.L8t);
+  sys_free(sys->h, s.sL);
   delete sys;
   return LGW_OK;
 }
@@ -2800,7 +2877,12 @@ static lgw_status backward_impl(lgw_handle *h, const lgw_system *sys, const lgw_
     const bool one_pass = bsub >= B;
     if (tc && !sys->Ltb_lo) {
       lgw_system *ms = const_cast<lgw_system *>(sys);
-      LGW_TRY_CUDA(h, cudaMalloc(&ms->Ltb_lo, sizeof(__nv_bfloat16) * (size_t)N * A));
+      ms->Ltb_lo = static_cast<__nv_bfloat16 *>(
+          sys_alloc(h, sizeof(__nv_bfloat16) * (size_t)N * A));
+      if (!ms->Ltb_lo) {
+        set_err(h, LGW_ERR_OOM, "device allocation for the low half of L^T failed");
+        throw Fail{LGW_ERR_OOM};
+      }
       launch_split_t(BasisRef{s.L64, nullptr, nullptr}, N, A, A, nullptr, ms->Ltb_lo, st);
       check_launch(h, "split_t(L lo)");
     }
