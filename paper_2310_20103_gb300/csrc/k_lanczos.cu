@@ -498,9 +498,11 @@ __global__ void k_beta_vec(VecCtx c, int j) {
 
 // q_next = w / beta into the next basis slot and xh = bf16(Delta^1/2 q_next)
 // (beta, the breakdown test and 1/beta from k_beta_vec); pair mode: xh only,
-// from the unnormalised vector.  Vectors run fastest over the grid: the rows of
-// xh's K blocks lie next to one another, so blocks that run together write runs
-// of DRAM pages (pair mode 678 us with chunks fastest, 428 us).  is_start: w
+// from the unnormalised vector, and vectors run fastest over the grid: the rows
+// of xh's K blocks lie next to one another, so blocks that run together write
+// runs of DRAM pages (678 us with chunks fastest, 428 us; where FP64 vectors are
+// written too, chunks fastest is better: 104 against 127 us at N_vc 131072, 256
+// vectors).  is_start: w
 // holds b_tm; ||b|| from the partials here, beta0, and q_0 into slot 0.
 __device__ __forceinline__ void normalize_chunk(const VecCtx &c, int j, int is_start, int chunk,
                                                 int b) {
@@ -626,8 +628,9 @@ __device__ __forceinline__ void normalize_chunk(const VecCtx &c, int j, int is_s
 
 __global__ void __launch_bounds__(VEC_THREADS) k_normalize(VecCtx c, int j, int is_start) {
   pdl_wait();
-  const int n = cpb_of(c), c0 = blockIdx.y * n, c1 = min(c.nchunks, c0 + n);
-  for (int chunk = c0; chunk < c1; ++chunk) normalize_chunk(c, j, is_start, chunk, blockIdx.x);
+  const int n = cpb_of(c), b = c.pair ? blockIdx.x : blockIdx.y;
+  const int c0 = (c.pair ? blockIdx.y : blockIdx.x) * n, c1 = min(c.nchunks, c0 + n);
+  for (int chunk = c0; chunk < c1; ++chunk) normalize_chunk(c, j, is_start, chunk, b);
 }
 
 // w = Delta^1/2 V for the rows of a given coupling block (V row stride ldv,
@@ -1145,7 +1148,7 @@ static dim3 vec_grid_cpb(const VecCtx &c) {
 }
 void launch_normalize(const VecCtx &c, int j, int is_start, const double *, cudaStream_t st) {
   const dim3 g = vec_grid_cpb(c);
-  launch_pdl(k_normalize, dim3(g.y, g.x), dim3(VEC_THREADS), 0, st, c, j, is_start);
+  launch_pdl(k_normalize, c.pair ? dim3(g.y, g.x) : g, dim3(VEC_THREADS), 0, st, c, j, is_start);
 }
 void launch_assemble_w(const VecCtx &c, int j, const float *ucd, cudaStream_t st) {
   launch_pdl(k_assemble_w, vec_grid_cpb(c), dim3(VEC_THREADS), 0, st, c, j, ucd);

@@ -82,48 +82,74 @@ __global__ void __launch_bounds__(VEC_THREADS) k_cheb_step(PolyStep p, int Bs) {
 }
 
 // w = c_0 q + a_s C b1 + b_s b1 - b2 - beta_j q_{j-1}, and the per-chunk
-// partials of alpha_j = q . w into alpha_part[chunk][b].
+// partials of alpha_j = q . w into alpha_part[chunk][b].  Bound by the FP64
+// pipe; CHEB_VECS vectors per block share a_s Delta^2 + b_s and one butterfly
+// for their sums (each added up in the order of block_sum).  N_vc 131072, 256
+// vectors: 480 us with a block per vector, 386 us now.
 __global__ void __launch_bounds__(VEC_THREADS) k_cheb_final(PolyStep p, const double *qprev,
                                                             const double *betaj, double *w,
                                                             double *alpha_part, int Bs) {
   pdl_wait();
-  __shared__ double red[VEC_THREADS / 32];
-  const int chunk = blockIdx.x, b = blockIdx.y;
-  const size_t voff = (size_t)b * p.N;
+  static_assert(CHEB_VECS == 4, "the sums' butterfly takes four");
+  __shared__ double red[4][VEC_THREADS / 32];
+  const int chunk = blockIdx.x, b0 = blockIdx.y * CHEB_VECS;
   const int e0 = poly_elem_base(chunk);
-  const double bj = betaj[b];
-  double ap = 0.0;
-#pragma unroll
+  double ap[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
   for (int u = 0; u < 4; ++u) {
     const int e = e0 + u * 64;
     if (e >= p.N) continue;
-    const size_t o = voff + e;
-    const double2 q = *reinterpret_cast<const double2 *>(p.q + o);
-    const double2 b1 = *reinterpret_cast<const double2 *>(p.b1 + o);
-    double2 r = make_double2(0.0, 0.0), cf = make_double2(p.bs, p.bs), t;
-    if (p.T) {
-      t = *reinterpret_cast<const double2 *>(p.T + o);
-    } else {
-      const float2 uc = *reinterpret_cast<const float2 *>(p.ucd + kblk_f32(b, e, Bs));
-      t = make_double2(f2d(uc.x), f2d(uc.y));
+    double2 cf = make_double2(p.bs, p.bs);
+    if (!p.T) {
       const double2 d2 = *reinterpret_cast<const double2 *>(p.Delta2 + e);
       cf = make_double2(fma(p.as, d2.x, p.bs), fma(p.as, d2.y, p.bs));
     }
-    if (p.b2) r = *reinterpret_cast<const double2 *>(p.b2 + o);
-    r.x = fma(p.ck, q.x, -r.x);
-    r.y = fma(p.ck, q.y, -r.y);
-    if (qprev) {
-      const double2 qp = *reinterpret_cast<const double2 *>(qprev + o);
-      r.x = fma(-bj, qp.x, r.x);
-      r.y = fma(-bj, qp.y, r.y);
+#pragma unroll
+    for (int i = 0; i < CHEB_VECS; ++i) {
+      const int b = b0 + i;
+      const size_t o = (size_t)b * p.N + e;
+      const double2 q = *reinterpret_cast<const double2 *>(p.q + o);
+      const double2 b1 = *reinterpret_cast<const double2 *>(p.b1 + o);
+      double2 r = make_double2(0.0, 0.0), t;
+      if (p.T) {
+        t = *reinterpret_cast<const double2 *>(p.T + o);
+      } else {
+        const float2 uc = *reinterpret_cast<const float2 *>(p.ucd + kblk_f32(b, e, Bs));
+        t = make_double2(f2d(uc.x), f2d(uc.y));
+      }
+      if (p.b2) r = *reinterpret_cast<const double2 *>(p.b2 + o);
+      r.x = fma(p.ck, q.x, -r.x);
+      r.y = fma(p.ck, q.y, -r.y);
+      if (qprev) {
+        const double2 qp = *reinterpret_cast<const double2 *>(qprev + o);
+        const double bj = betaj[b];
+        r.x = fma(-bj, qp.x, r.x);
+        r.y = fma(-bj, qp.y, r.y);
+      }
+      r.x = fma(cf.x, b1.x, fma(p.as, t.x, r.x));
+      r.y = fma(cf.y, b1.y, fma(p.as, t.y, r.y));
+      *reinterpret_cast<double2 *>(w + o) = r;
+      ap[i] = fma(q.x, r.x, fma(q.y, r.y, ap[i]));
     }
-    r.x = fma(cf.x, b1.x, fma(p.as, t.x, r.x));
-    r.y = fma(cf.y, b1.y, fma(p.as, t.y, r.y));
-    *reinterpret_cast<double2 *>(w + o) = r;
-    ap = fma(q.x, r.x, fma(q.y, r.y, ap));
   }
-  ap = block_sum_to0(ap, red);
-  if (threadIdx.x == 0) alpha_part[(size_t)chunk * Bs + b] = ap;
+  // lane bits 4 and 3 pick the vector, then the other three bits
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const bool b16 = (lane & 16) != 0, b8 = (lane & 8) != 0;
+  double x = b16 ? ap[2] : ap[0], y = b16 ? ap[3] : ap[1];
+  x += __shfl_xor_sync(0xffffffffu, b16 ? ap[0] : ap[2], 16);
+  y += __shfl_xor_sync(0xffffffffu, b16 ? ap[1] : ap[3], 16);
+  const double send = b8 ? x : y;
+  x = (b8 ? y : x) + __shfl_xor_sync(0xffffffffu, send, 8);
+#pragma unroll
+  for (int o = 4; o >= 1; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  if ((lane & 7) == 0) red[2 * b16 + b8][wid] = x;
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    double t = 0.0;
+#pragma unroll
+    for (int k = 0; k < VEC_THREADS / 32; ++k) t += red[threadIdx.x][k];
+    alpha_part[(size_t)chunk * Bs + b0 + threadIdx.x] = t;
+  }
 }
 
 // Haydock coefficients of D's tridiagonal for the continued fractions:
@@ -162,7 +188,7 @@ void launch_cheb_step(const PolyStep &p, int nchunks, int Bs, cudaStream_t st) {
 }
 void launch_cheb_final(const PolyStep &p, const double *qprev, const double *betaj, double *w,
                        double *alpha_part, int nchunks, int Bs, cudaStream_t st) {
-  launch_pdl(k_cheb_final, dim3(nchunks, Bs), dim3(VEC_THREADS), 0, st, p, qprev, betaj, w,
+  launch_pdl(k_cheb_final, dim3(nchunks, Bs / CHEB_VECS), dim3(VEC_THREADS), 0, st, p, qprev, betaj, w,
              alpha_part, Bs);
 }
 void launch_poly_prep(const double *alpha, const double *beta, const double *beta0,
