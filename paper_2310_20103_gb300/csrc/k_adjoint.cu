@@ -45,7 +45,9 @@ constexpr int EIG_THREADS = 128;
 // 20-bit estimate.  Where the squares leave the normal range: hypot.
 __device__ __forceinline__ void eig_rotation(double g, double f, double &c, double &s, double &r) {
   const double h = fma(g, g, f * f);
-  if (h > 1e-270 && h < 1e270) {
+  // 2^-900 <= h < 2^900, on the exponent field (an FP64 comparison would take
+  // its turn on the chain)
+  if ((((unsigned)__double2hiint(h) >> 20) - 123u) < 1800u) {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(h));
     const double e = fma(-h * y, y, 1.0);
@@ -946,6 +948,10 @@ void launch_eig_full(const AdjCtx &a, cudaStream_t st) {
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(k_eig_full, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    // the GEMM that runs beside it needs an SM's shared memory, which is split
+    // from the L1 when the first block arrives
+    cudaFuncSetAttribute(k_eig_full, cudaFuncAttributePreferredSharedMemoryCarveout,
+                         cudaSharedmemCarveoutMaxShared);
     attr = true;
   }
   launch_pdl(k_eig_full, dim3(a.Bs), dim3(EIG_THREADS), smem, st, a);

@@ -1675,6 +1675,41 @@ const PolyOp *poly_arg(lgw_handle *h, const lgw_system *sys, const lgw_poly *pp,
   return &store;
 }
 
+// A stretch of work beside the handle's stream, on the first lane: it starts
+// after what the stream holds so far, and the stream goes on after it from
+// join() (or the destructor: also when an exception passes).  Off: the stream.
+struct SideStream {
+  lgw_handle *h;
+  cudaStream_t st;
+  cudaEvent_t ev = nullptr;
+  SideStream(lgw_handle *h_, bool on) : h(h_), st(h_->stream) {
+    if (!on) return;
+    if (h->lanes.empty()) {
+      cudaStream_t l;
+      LGW_TRY_CUDA(h, cudaStreamCreateWithFlags(&l, cudaStreamNonBlocking));
+      h->lanes.push_back(l);
+    }
+    LGW_TRY_CUDA(h, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+    if (cudaEventRecord(ev, h->stream) != cudaSuccess ||
+        cudaStreamWaitEvent(h->lanes[0], ev, 0) != cudaSuccess) {
+      cudaEventDestroy(ev);
+      ev = nullptr;
+      cudaGetLastError();
+      return;   // on the stream itself
+    }
+    st = h->lanes[0];
+  }
+  SideStream(const SideStream &) = delete;
+  void join() {
+    if (!ev) return;
+    if (cudaEventRecord(ev, st) != cudaSuccess || cudaStreamWaitEvent(h->stream, ev, 0) != cudaSuccess)
+      cudaStreamSynchronize(st);
+    cudaEventDestroy(ev);
+    ev = nullptr;
+  }
+  ~SideStream() { join(); }
+};
+
 // Tamm-Dancoff view of a system: the same copies of L with Delta^1/2 -> 1,
 // Delta^2 -> Delta, c_K Delta^1/2 -> c_K / 2 (refreshed on every use, so
 // copies made later, such as the E4M3 ones, are seen).
@@ -2962,8 +2997,53 @@ static lgw_status backward_impl(lgw_handle *h, const lgw_system *sys, const lgw_
       a.status = h->d_status;
       a.tda = tda ? 1 : 0;
       a.poly = poly ? 1 : 0;
-      launch_eig_full(a, st);
-      check_launch(h, "eig_full");
+      // The eigenvectors take one block per vector and a serial chain (13.9 ms at
+      // 128 vectors, k 120) that leaves the chip idle: on the tensor-core path
+      // what does not need them runs beside them, P = Q^T D L and the transposed
+      // split of Q (7.5 ms), where a block still fits beside a tile of the GEMM
+      // (24 KB; the gradient of one bf16 state 146.3 ->
+      // 139.1).
+      const int rows = k * Bs;
+      const bool beside = tc && !exact && (size_t)6 * k * sizeof(double) <= (size_t)20 * 1024;
+      double *P = nullptr, *R = nullptr;
+      __nv_bfloat16 *Shi = nullptr, *Slo = nullptr, *Rhi = nullptr, *Rlo = nullptr;
+      auto products_of_q = [&](cudaStream_t ss) {
+        // P = Q^T D L: three split-BF16 products, FP64 sums of 16384-long chunks;
+        // then the transposed split of Q in the same buffers
+        char err[256];
+        launch_split_scaled(qb, rows, N, s.dsq, Shi, Slo, ss);
+        check_launch(h, "split_scaled(D Q)");
+        // Ltb is K-block-major; the adjoint's own Ltb_lo is row-major
+        const __nv_bfloat16 *pa[3] = {s.Ltb, s.Ltb, sys->Ltb_lo};
+        const int pk[3] = {1, 1, 0};
+        const __nv_bfloat16 *pb[3] = {Shi, Slo, Shi};
+        if (!tc_gemm_f64out(3, pa, pk, pb, A, rows, N, 16384, P, A, 0, h->d_status, ss, err,
+                            sizeof err)) {
+          set_err(h, LGW_ERR_CUDA, "%s", err);
+          throw Fail{LGW_ERR_CUDA};
+        }
+        check_launch(h, "tc_gemm_f64out(P)");
+        launch_split_t(qb, rows, N, N, Shi, Slo, ss);
+        check_launch(h, "split_t(Q)");
+      };
+      if (!exact) {
+        P = wsT<double>(h, "adj_P", (size_t)rows * A);
+        R = wsT<double>(h, "adj_R", (size_t)rows * A);
+        if (tc) {
+          Shi = wsT<__nv_bfloat16>(h, "adj_Shi", (size_t)rows * N);
+          Slo = wsT<__nv_bfloat16>(h, "adj_Slo", (size_t)rows * N);
+          Rhi = wsT<__nv_bfloat16>(h, "adj_Rhi", (size_t)rows * A);
+          Rlo = wsT<__nv_bfloat16>(h, "adj_Rlo", (size_t)rows * A);
+        }
+      }
+      {
+        // the eigenvectors stay on the stream and so start first, a block per SM
+        SideStream side(h, beside);
+        launch_eig_full(a, st);
+        check_launch(h, "eig_full");
+        if (tc && !exact) products_of_q(side.st);
+        side.join();
+      }
       launch_adj_coeffs(a, st);
       check_launch(h, "adj_coeffs");
       if (exact) {
@@ -2977,35 +3057,13 @@ static lgw_status backward_impl(lgw_handle *h, const lgw_system *sys, const lgw_
       else
         launch_adj_rows(a, qb, Y, Gd, st);
       check_launch(h, "adj_rows");
-      const int rows = k * Bs;
-      double *P = wsT<double>(h, "adj_P", (size_t)rows * A);
-      double *R = wsT<double>(h, "adj_R", (size_t)rows * A);
       if (tc) {
-        // P = Q^T D L: three split-BF16 products, FP64 sums of 16384-long chunks
-        __nv_bfloat16 *Shi = wsT<__nv_bfloat16>(h, "adj_Shi", (size_t)rows * N);
-        __nv_bfloat16 *Slo = wsT<__nv_bfloat16>(h, "adj_Slo", (size_t)rows * N);
-        __nv_bfloat16 *Rhi = wsT<__nv_bfloat16>(h, "adj_Rhi", (size_t)rows * A);
-        __nv_bfloat16 *Rlo = wsT<__nv_bfloat16>(h, "adj_Rlo", (size_t)rows * A);
         char err[256];
-        launch_split_scaled(qb, rows, N, s.dsq, Shi, Slo, st);
-        check_launch(h, "split_scaled(D Q)");
-        // Ltb is K-block-major; the adjoint's own Ltb_lo is row-major
-        const __nv_bfloat16 *pa[3] = {s.Ltb, s.Ltb, sys->Ltb_lo};
-        const int pk[3] = {1, 1, 0};
-        const __nv_bfloat16 *pb[3] = {Shi, Slo, Shi};
-        if (!tc_gemm_f64out(3, pa, pk, pb, A, rows, N, 16384, P, A, 0, h->d_status, st, err,
-                            sizeof err)) {
-          set_err(h, LGW_ERR_CUDA, "%s", err);
-          throw Fail{LGW_ERR_CUDA};
-        }
-        check_launch(h, "tc_gemm_f64out(P)");
         launch_gamma_p(a, P, A, R, st);
         check_launch(h, "gamma_p");
         // SC += Q R  (M = N_aux, N = N_vc, K = k Bs, transposed split operands)
         launch_split_t(BasisRef{R, nullptr, nullptr}, rows, A, A, Rhi, Rlo, st);
         check_launch(h, "split_t(R)");
-        launch_split_t(qb, rows, N, N, Shi, Slo, st);
-        check_launch(h, "split_t(Q)");
         const __nv_bfloat16 *qa[3] = {Rhi, Rhi, Rlo};
         const __nv_bfloat16 *qb[3] = {Shi, Slo, Shi};
         if (!tc_gemm_f64out(3, qa, nullptr, qb, A, N, rows, 16384, SC, A, 1, h->d_status, st, err,
