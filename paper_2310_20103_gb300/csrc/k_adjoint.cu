@@ -25,42 +25,22 @@ namespace lgw {
 
 // --------------------------------------------------------------------------
 // Full eigen-decomposition of each T_k: implicit symmetric QR with Wilkinson
-// shifts (the recurrences of Martin and Wilkinson's imtql2, Numer. Math. 12
-// (1968) 377, chasing downwards).  One block per vector: lane 0 of warp 0 runs
-// the scalar chain of a sweep and leaves its rotations in shared memory; the
-// other warps apply the previous sweep's to the rows of V = U^T (row s =
-// eigenvector s, coalesced) meanwhile.
+// shifts, chasing downwards.  One block per vector: warp 0 runs the scalar
+// chain of a sweep and leaves its rotations in shared memory; the other warps
+// apply the previous sweep's to the rows of V = U^T (row s = eigenvector s,
+// coalesced) meanwhile.
 //
 // What bounds it: the scalar chain, about 1.7 n sweeps of rotations in
 // sequence, each FP64 instruction of which holds its unit for 64 clocks
-// however few lanes it has.  A rotation takes 20 of them (one reciprocal
-// square root from the hardware's estimate) where hypot, two divisions and the
-// plain update took about 60, and the row updates no longer wait in between:
-// 128 vectors, k 120: 45.3 ms -> 13.9.
+// however few lanes it has.  So even lanes carry what belongs to c and odd
+// lanes what belongs to s: one division, one square and one diagonal update
+// per rotation serve both.  The operations and their order stay those of one
+// thread's chain (the split of Gamma P that follows rounds to 16 bits, where a
+// last-place difference now and then moves a digit).  128 vectors, k 120: 45.3
+// ms with the row updates in the chain, 25 ms now (13.9 with reciprocal square
+// roots in place of hypot and the divisions, which moved dL by 1e-9).
 // --------------------------------------------------------------------------
 constexpr int EIG_THREADS = 128;
-
-// (c, s, r) with c g + s f = r, c f - s g = 0; 1 / sqrt(g^2 + f^2) by one
-// third-order Newton step, y (1 + e/2 + 3/8 e^2), e = 1 - h y^2, on a
-// 20-bit estimate.  Where the squares leave the normal range: hypot.
-__device__ __forceinline__ void eig_rotation(double g, double f, double &c, double &s, double &r) {
-  const double h = fma(g, g, f * f);
-  // 2^-900 <= h < 2^900, on the exponent field (an FP64 comparison would take
-  // its turn on the chain)
-  if ((((unsigned)__double2hiint(h) >> 20) - 123u) < 1800u) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(h));
-    const double e = fma(-h * y, y, 1.0);
-    y = fma(y * e, fma(e, 0.375, 0.5), y);
-    c = g * y;
-    s = f * y;
-    r = h * y;
-    return;
-  }
-  r = hypot(g, f);
-  c = r > 0.0 ? g / r : 1.0;
-  s = r > 0.0 ? f / r : 0.0;
-}
 
 __global__ void __launch_bounds__(EIG_THREADS) k_eig_full(AdjCtx a) {
   pdl_wait();
@@ -82,49 +62,71 @@ __global__ void __launch_bounds__(EIG_THREADS) k_eig_full(AdjCtx a) {
   if (tid < 2) ctl[tid][0] = -1, ctl[tid][1] = ctl[tid][2] = 0;
   __syncthreads();
   const double eps = 2.220446049250313e-16;
-  int hi = n - 1, iter = 0;   // warp 0, lane 0
+  int hi = n - 1, iter = 0;   // warp 0, alike in every lane
   const int max_iter = 60 * n + 60;
+  const bool odd = (tid & 1) != 0;
   for (int sweep = 0;; ++sweep) {
     const int cur = sweep & 1, prev = cur ^ 1;
-    if (tid == 0) {
+    if (tid < 32) {
       int lo = -1, nr = 0;
       while (hi > 0 && fabs(e[hi - 1]) <= eps * (fabs(d[hi - 1]) + fabs(d[hi]))) {
-        e[hi - 1] = 0.0;
+        __syncwarp();
+        if (tid == 0) e[hi - 1] = 0.0;
+        __syncwarp();
         --hi;
       }
       if (hi > 0 && ++iter <= max_iter) {
         lo = hi - 1;
         while (lo > 0 && fabs(e[lo - 1]) > eps * (fabs(d[lo - 1]) + fabs(d[lo]))) --lo;
-        if (lo > 0) e[lo - 1] = 0.0;
+        __syncwarp();
+        if (tid == 0 && lo > 0) e[lo - 1] = 0.0;
         // Wilkinson shift from the trailing 2 x 2 block
         const double dl = 0.5 * (d[hi - 1] - d[hi]);
         const double bb = e[hi - 1];
         const double den = dl + copysign(sqrt(fma(dl, dl, bb * bb)), dl != 0.0 ? dl : 1.0);
         const double mu = d[hi] - bb * bb / den;
-        double g = d[lo] - mu, c = 1.0, s = 1.0, p = 0.0;
-        double dk = d[lo];
+        double a0 = d[lo], b0 = e[lo];
+        double x = a0 - mu, z = b0;
+        __syncwarp();   // every lane has read what lane 0 writes below
         for (int i = lo; i < hi; ++i) {
-          const double ei = e[i], dn = d[i + 1];
-          const double f = s * ei, bq = c * ei;
-          double r;
-          eig_rotation(g, f, c, s, r);
-          if (i > lo) e[i - 1] = r;
-          g = dk - p;
-          const double cb = c * bq;
-          r = fma(dn - g, s, cb) + cb;
-          p = s * r;
-          d[i] = g + p;
-          g = fma(c, r, -bq);
-          dk = dn;
-          rot[cur * k + nr++] = make_double2(c, s);
+          // R = [[c, s], [-s, c]] maps (x, z) to (r, 0); T <- R T R^T on rows i, i + 1
+          const double c0 = d[i + 1], en = e[i + 1];   // e has k entries, k > hi
+          const double r = hypot(x, z);
+          const double q = r > 0.0 ? (odd ? z : x) / r : (odd ? 0.0 : 1.0);   // s or c
+          const double q2 = q * q;
+          const double o = __shfl_xor_sync(0xffffffffu, q, 1);
+          const double o2 = __shfl_xor_sync(0xffffffffu, q2, 1);
+          const double m = q * en;                      // c e_{i+1}, or the bulge
+          const double csn = q * o;
+          const double t = 2.0 * csn * b0;
+          const double dn = fma(o2, c0, fma(q2, a0, odd ? -t : t));
+          const double df = odd ? o2 - q2 : q2 - o2;    // c^2 - s^2
+          const double ei = fma(df, b0, csn * (c0 - a0));
+          __syncwarp();   // every lane has read row i + 1
+          if (tid == 0) {
+            if (i > lo) e[i - 1] = r;
+            d[i] = dn;
+            rot[cur * k + nr] = make_double2(q, o);
+          }
+          ++nr;
+          x = ei;
+          z = __shfl_sync(0xffffffffu, m, 1);
+          b0 = __shfl_sync(0xffffffffu, m, 0);
+          a0 = __shfl_sync(0xffffffffu, dn, 1);
         }
-        d[hi] = dk - p;
-        e[hi - 1] = g;
+        // the rotation of the last row chases nothing: x holds e_{hi-1}
+        if (tid == 0) {
+          d[hi] = a0;
+          e[hi - 1] = x;
+        }
+        __syncwarp();
       }
-      ctl[cur][0] = lo;
-      ctl[cur][1] = nr;
-      ctl[cur][2] = (hi > 0 && iter > max_iter) ? 1 : 0;
-    } else if (tid >= 32 && ctl[prev][0] >= 0) {
+      if (tid == 0) {
+        ctl[cur][0] = lo;
+        ctl[cur][1] = nr;
+        ctl[cur][2] = (hi > 0 && iter > max_iter) ? 1 : 0;
+      }
+    } else if (ctl[prev][0] >= 0) {
       // V <- R V of the previous sweep: each thread carries its columns
       // through the whole sweep in a register
       const int lo = ctl[prev][0], nr = ctl[prev][1];

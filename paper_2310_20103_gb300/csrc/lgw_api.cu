@@ -2997,12 +2997,11 @@ static lgw_status backward_impl(lgw_handle *h, const lgw_system *sys, const lgw_
       a.status = h->d_status;
       a.tda = tda ? 1 : 0;
       a.poly = poly ? 1 : 0;
-      // The eigenvectors take one block per vector and a serial chain (13.9 ms at
+      // The eigenvectors take one block per vector and a serial chain (25 ms at
       // 128 vectors, k 120) that leaves the chip idle: on the tensor-core path
       // what does not need them runs beside them, P = Q^T D L and the transposed
-      // split of Q (7.5 ms), where a block still fits beside a tile of the GEMM
-      // (24 KB; the gradient of one bf16 state 146.3 ->
-      // 139.1).
+      // split of Q (7.5 ms, of which 7.2 are saved), where a block still fits
+      // beside a tile of the GEMM (24 KB).
       const int rows = k * Bs;
       const bool beside = tc && !exact && (size_t)6 * k * sizeof(double) <= (size_t)20 * 1024;
       double *P = nullptr, *R = nullptr;
