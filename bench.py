@@ -633,9 +633,10 @@ def fp64_legs(args, L, wl, eps_d, L_d, prob, e_head, sig_head, value_head, dev, 
     in a fresh handle so that no other Krylov basis shares the device:
       cgs2_fp64_basis_step  BF16 contractions, CGS2 against an FP64 basis
                             (every product and sum on the FP64 pipe);
-      fp64_path             the plain FP64 GPU path: FP64 CUDA-core
-                            contractions, FP64 basis, CGS1K; its QP energies
-                            against the headline's (the 1 meV criterion).
+      fp64_path             the plain FP64 GPU path: FP64 contractions (tensor
+                            cores by error-free slicing), FP64 basis, CGS1K;
+                            its QP energies against the headline's (the 1 meV
+                            criterion).
     mixed_over_fp64 = headline states/s over the FP64 path's states/s."""
     import torch
     tps = args.tps
@@ -647,7 +648,7 @@ def fp64_legs(args, L, wl, eps_d, L_d, prob, e_head, sig_head, value_head, dev, 
     runs = [("cgs2_fp64_basis_step", "bf16", "cgs2", args.k, 1,
              "BF16 contractions, CGS2 against an FP64 Krylov basis (FP64 dots and updates)"),
             ("fp64_path", "fp64", "cgs1k", args.fp64_k, 0,
-             "plain FP64 path: FP64 CUDA-core contractions, FP64 basis, CGS1K")]
+             "plain FP64 path: FP64 contractions by error-free slicing, FP64 basis, CGS1K")]
     for name, prec, reorth, kk, warm, note in runs:
         o = L.Options(k=kk, precision=prec, reorth=reorth, b_sub=tps * M_PER_TARGET,
                       reorth_arith="fp64")

@@ -65,7 +65,9 @@ typedef enum {
  * continued fractions, QP) is FP64 in every mode.  Start vectors V = L M
  * are FP64 in the FP64 mode and split BF16 (three products) otherwise. */
 typedef enum {
-  LGW_FP64 = 0,   /* FP64 CUDA-core GEMMs: the plain FP64 path            */
+  LGW_FP64 = 0,   /* FP64 products: the plain FP64 path (on the tensor cores
+                     by error-free slicing where the digits of L fit the
+                     device's memory, else on the CUDA cores)              */
   LGW_BF16 = 1,   /* BF16 tcgen05 tensor-core GEMMs, FP32 accumulate      */
   LGW_FP8 = 3,    /* E4M3 tcgen05 GEMMs (kind::f8f6f4), FP32 accumulate:
                      L with one power-of-two scale per column (max -> (224,
