@@ -44,6 +44,7 @@
 
 #include "fp_bits.cuh"
 #include "oz_digits.cuh"
+#include "oz_plan.cuh"
 #include "tc_ptx.cuh"
 
 namespace lgw {
@@ -51,9 +52,6 @@ namespace oz {
 
 using namespace tc;
 
-constexpr int BM = 128;
-constexpr int KB = 64;          // K elements per block: one 128-byte swizzle row
-constexpr int CHUNK_KB = 16;    // 1024 terms per exact sum
 constexpr int EPI_WARPS = 8;    // two per TMEM lane quarter, each half of the columns
 constexpr int NTHREADS = 64 + 32 * EPI_WARPS;
 
@@ -554,36 +552,12 @@ static int sm_count() {
   return n;
 }
 
-// Columns of B per tile: as many as fill the chip with up to `splits` K splits
-// (an A tile is loaded once per column tile, so wide tiles load less), no
-// wider than B.
-static int tile_cols(int m_tiles, int ncols, int splits) {
-  int nt = ncols >= 64 ? 64 : (ncols >= 32 ? 32 : 16);
-  while (nt > 16 && m_tiles * ((ncols + nt - 1) / nt) * splits * 2 <= sm_count()) nt /= 2;
-  return nt;
-}
-
 }  // namespace oz
 
-// K splits of A's M rows by ncols columns over nkb K blocks: the count with
-// the fewest K blocks in sequence, a CTA's fixed cost (pipeline fill, eight
-// sums joined and stored) standing for four of them.
-int oz_splits(int M, int ncols, int nkb) {
-  const int m_tiles = (M + oz::BM - 1) / oz::BM;
-  const int nt = oz::tile_cols(m_tiles, ncols, std::min(64, nkb));
-  const int tiles = m_tiles * ((ncols + nt - 1) / nt), nsm = oz::sm_count();
-  int best = 1;
-  long long best_cost = 1LL << 60;
-  for (int s = 1; s <= std::min(64, nkb); ++s) {
-    const int per = (nkb + s - 1) / s, real = (nkb + per - 1) / per;
-    const long long waves = ((long long)tiles * real + nsm - 1) / nsm;
-    const long long cost = waves * (per + 4 * ((per + oz::CHUNK_KB - 1) / oz::CHUNK_KB));
-    if (cost < best_cost) {
-      best_cost = cost;
-      best = real;
-    }
-  }
-  return best;
+int oz_splits(int M, int ncols, int nkb) { return oz::k_splits(M, ncols, nkb, oz::sm_count()); }
+
+size_t oz_part_rows(int M, int rows, int slice, int nkb) {
+  return oz::part_rows(M, rows, slice, nkb, oz::sm_count());
 }
 
 bool launch_oz_gemm(const OzOperand &A, const OzOperand &B, int M, int Ncols, int splits,
@@ -606,7 +580,8 @@ bool launch_oz_gemm(const OzOperand &A, const OzOperand &B, int M, int Ncols, in
   e.status = status;
   const int nkb = A.nkb, per = (nkb + splits - 1) / splits;
   const int m_tiles = (M + oz::BM - 1) / oz::BM;
-  const int nt = oz::tile_cols(m_tiles, Ncols, o.mode == OZ_PART ? std::min(64, nkb) : 1);
+  const int nt =
+      oz::tile_cols(m_tiles, Ncols, o.mode == OZ_PART ? std::min(64, nkb) : 1, oz::sm_count());
   CUtensorMap ta, tb;
   if (A.rows < oz::BM || B.rows < nt || A.nkb != B.nkb || !oz::encode(&ta, A, oz::BM, 1) ||
       !oz::encode(&tb, B, nt, nt == 64 ? oz::Cfg<64>::BOX : OZ_SLICES))

@@ -683,30 +683,38 @@ constexpr int F64_ROWS = 1024;   // vectors sliced at a time
 struct F64Work {
   OzOperand x, y;        // digits of the vectors and of y = L^T (Delta^1/2 x); d NULL: none
   double *part = nullptr;
-  int rows = 0;
+  size_t part_n = 0;     // doubles that `part` holds
 };
 
 F64Work f64_work(lgw_handle *h, const SysDev &s, int rows) {
   F64Work f;
-  f.rows = rows;
-  size_t part = (size_t)gemm1_f64_splits(s, rows) * rows * s.A;
+  const size_t part = (size_t)gemm1_f64_splits(s, rows) * rows * s.A;
   if (s.ozA.d) {
     const int r = std::min(rows, F64_ROWS);
     const size_t nx = OzOperand::digits(r, s.N / 64), ny = OzOperand::digits(r, s.A / 64);
     uint16_t *d = static_cast<uint16_t *>(ws(h, "oz_xy", (nx + ny) * sizeof(uint16_t), true));
     int *e = d ? static_cast<int *>(ws(h, "oz_e", 2 * (size_t)r * sizeof(int), true)) : nullptr;
-    const size_t op = (size_t)oz_splits(s.A, r, s.N / 64) * r * s.A;
-    double *pp = e ? static_cast<double *>(ws(h, "yp64", std::max(part, op) * sizeof(double), true))
-                   : nullptr;
+    const size_t op = std::max(part, oz_part_rows(s.A, rows, F64_ROWS, s.N / 64) * s.A);
+    double *pp = e ? static_cast<double *>(ws(h, "yp64", op * sizeof(double), true)) : nullptr;
     if (pp) {
       f.x = OzOperand{d, e, r, s.N / 64};
       f.y = OzOperand{d + nx, e + r, r, s.A / 64};
       f.part = pp;
+      f.part_n = op;
       return f;
     }
   }
   f.part = wsT<double>(h, "yp64", part);
+  f.part_n = part;
   return f;
+}
+
+// No contraction writes more split partials than its work holds.
+void check_part(lgw_handle *h, const F64Work &f, int splits, int rows, int A) {
+  if ((size_t)splits * rows * A <= f.part_n) return;
+  set_err(h, LGW_ERR_SHAPE, "%d splits of %d x %d partials exceed the %zu that were planned",
+          splits, rows, A, f.part_n);
+  throw Fail{LGW_ERR_SHAPE};
 }
 
 void oz_gemm(lgw_handle *h, const OzOperand &A, const OzOperand &B, int M, int Ncols, int splits,
@@ -734,6 +742,7 @@ void f64_contract1(lgw_handle *h, const SysDev &s, const F64Work &f, const doubl
   cudaStream_t st = h->stream;
   if (!f.x.d || !s.ozT.d) {
     const int splits = gemm1_f64_splits(s, rows);
+    check_part(h, f, splits, rows, s.A);
     launch_gemm1_f64(s, q, rows, f.part, splits, st);
     check_launch(h, "gemm1_f64");
     launch_reduce_y_f64(f.part, splits, rows, s.A, Y, st);
@@ -749,6 +758,7 @@ void f64_contract1(lgw_handle *h, const SysDev &s, const F64Work &f, const doubl
       check_launch(h, "oz_slice(x)");
     }
     const int splits = oz_splits(s.A, nr, s.N / 64);
+    check_part(h, f, splits, nr, s.A);
     OzOut o;
     o.mode = OZ_PART;
     o.out = f.part;

@@ -306,6 +306,8 @@ struct OzOut {
   double *alpha_part = nullptr;   // [M / 64][Ncols]
 };
 int oz_splits(int M, int ncols, int nkb);
+// rows of partials of OZ_PART products of `rows` columns, `slice` at a time
+size_t oz_part_rows(int M, int rows, int slice, int nkb);
 // A.rows >= 128, B.rows >= min(Ncols, 64) (16 at least); false if a tensor
 // map cannot be made
 bool launch_oz_gemm(const OzOperand &A, const OzOperand &B, int M, int Ncols, int splits,
