@@ -686,16 +686,19 @@ struct F64Work {
   size_t part_n = 0;     // doubles that `part` holds
 };
 
-F64Work f64_work(lgw_handle *h, const SysDev &s, int rows) {
+// own: prefix of the buffers' names.  A recurrence takes its buffers once, so
+// work of another width that runs between its sub-batches has names of its own
+// (ws frees a buffer that has to grow).
+F64Work f64_work(lgw_handle *h, const SysDev &s, int rows, const std::string &own = "") {
   F64Work f;
   const size_t part = (size_t)gemm1_f64_splits(s, rows) * rows * s.A;
   if (s.ozA.d) {
     const int r = std::min(rows, F64_ROWS);
     const size_t nx = OzOperand::digits(r, s.N / 64), ny = OzOperand::digits(r, s.A / 64);
-    uint16_t *d = static_cast<uint16_t *>(ws(h, "oz_xy", (nx + ny) * sizeof(uint16_t), true));
-    int *e = d ? static_cast<int *>(ws(h, "oz_e", 2 * (size_t)r * sizeof(int), true)) : nullptr;
+    uint16_t *d = static_cast<uint16_t *>(ws(h, own + "oz_xy", (nx + ny) * sizeof(uint16_t), true));
+    int *e = d ? static_cast<int *>(ws(h, own + "oz_e", 2 * (size_t)r * sizeof(int), true)) : nullptr;
     const size_t op = std::max(part, oz_part_rows(s.A, rows, F64_ROWS, s.N / 64) * s.A);
-    double *pp = e ? static_cast<double *>(ws(h, "yp64", op * sizeof(double), true)) : nullptr;
+    double *pp = e ? static_cast<double *>(ws(h, own + "yp64", op * sizeof(double), true)) : nullptr;
     if (pp) {
       f.x = OzOperand{d, e, r, s.N / 64};
       f.y = OzOperand{d + nx, e + r, r, s.A / 64};
@@ -704,7 +707,7 @@ F64Work f64_work(lgw_handle *h, const SysDev &s, int rows) {
       return f;
     }
   }
-  f.part = wsT<double>(h, "yp64", part);
+  f.part = wsT<double>(h, own + "yp64", part);
   f.part_n = part;
   return f;
 }
@@ -1848,7 +1851,7 @@ void reverse_sweep(lgw_handle *h, const SysDev &s, const ProbView &pv, const Opt
   double *useg = wsT<double>(h, "rev_useg", (size_t)cs * BN);
   double *yseg = wsT<double>(h, "rev_yseg", (size_t)cs * BA);
   double *ybseg = wsT<double>(h, "rev_ybseg", (size_t)cs * BA);
-  const F64Work f64 = f64_work(h, s, Bs);
+  const F64Work f64 = f64_work(h, s, Bs);   // the recurrence's own: same width
   double *Y = wsT<double>(h, "adj_Y", BN);
   RevCtx r{};
   r.N = N;
@@ -3083,7 +3086,7 @@ static lgw_status backward_impl(lgw_handle *h, const lgw_system *sys, const lgw_
         check_launch(h, "tc_gemm_f64out(SC)");
       } else {
         // P = Q^T D L over the k * Bs basis rows (FP64 GEMM1), R = Gam P
-        f64_contract1(h, s, f64_work(h, s, rows), c.basis, rows, P);
+        f64_contract1(h, s, f64_work(h, s, rows, "adj_"), c.basis, rows, P);
         launch_gamma_p(a, P, A, R, st);
         check_launch(h, "gamma_p");
         f64_atb(h, c.basis, N, R, A, rows, N, A, SC);

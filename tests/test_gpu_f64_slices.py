@@ -84,3 +84,30 @@ def test_gradient_with_a_short_last_slice(L, n_v, n_c, A, n_m, k):
             L.lgw_destroy(h)
     for a, b in zip(out[0], out[1 << 40]):
         assert float((a - b).abs().max()) <= 1e-8 * float(b.abs().max())
+
+
+@pytest.mark.parametrize("reorth", ["cgs2", "cgs1k"])
+def test_sub_batches_on_a_fresh_handle(L, reorth):
+    """A gradient in sub-batches on a handle whose buffers have not grown yet: the adjoint of
+    one sub-batch contracts k times as many rows as the recurrence of the next, which must
+    still find its own buffers.  Against the single pass, on a handle of its own."""
+    wl = gi.tiny(k=40)
+    dE = _t(np.random.default_rng(3).normal(size=wl.n_t))
+    prob = L.Problem(targets=_t(wl.targets), m_idx=_t(wl.m_idx), omega=_t(wl.omega),
+                     delta=wl.delta, M=_t(wl.M))
+    out = []
+    for b_sub in (48, 0):
+        h = L.lgw_create(0)
+        try:
+            s = L.lgw_prepare_system(h, wl.n_v, wl.n_c, wl.n_aux, _t(wl.eps), _t(wl.L), 4.0)
+            dL = torch.zeros(wl.n_vc, wl.n_aux, dtype=torch.float64, device=DEV)
+            de = torch.zeros(wl.n_v + wl.n_c, dtype=torch.float64, device=DEV)
+            opt = L.Options(k=40, precision="fp64", reorth=reorth, b_sub=b_sub)
+            L.lgw_sigma_c_backward(h, s, prob, opt, dE, dL, de)
+            torch.cuda.synchronize()
+            out.append((dL, de))
+            L.lgw_release_system(s)
+        finally:
+            L.lgw_destroy(h)
+    for a, b in zip(*out):
+        assert float((a - b).abs().max()) <= 1e-12 * float(b.abs().max())
