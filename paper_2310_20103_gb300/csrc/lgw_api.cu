@@ -691,7 +691,9 @@ struct F64Work {
 // (ws frees a buffer that has to grow).
 F64Work f64_work(lgw_handle *h, const SysDev &s, int rows, const std::string &own = "") {
   F64Work f;
-  const size_t part = (size_t)gemm1_f64_splits(s, rows) * rows * s.A;
+  // a contraction of one split writes its result, not partials
+  const int splits = gemm1_f64_splits(s, rows);
+  const size_t part = splits > 1 ? (size_t)splits * rows * s.A : 0;
   if (s.ozA.d) {
     const int r = std::min(rows, F64_ROWS);
     const size_t nx = OzOperand::digits(r, s.N / 64), ny = OzOperand::digits(r, s.A / 64);
@@ -707,7 +709,7 @@ F64Work f64_work(lgw_handle *h, const SysDev &s, int rows, const std::string &ow
       return f;
     }
   }
-  f.part = wsT<double>(h, own + "yp64", part);
+  if (part > 0) f.part = wsT<double>(h, own + "yp64", part);
   f.part_n = part;
   return f;
 }
@@ -745,9 +747,10 @@ void f64_contract1(lgw_handle *h, const SysDev &s, const F64Work &f, const doubl
   cudaStream_t st = h->stream;
   if (!f.x.d || !s.ozT.d) {
     const int splits = gemm1_f64_splits(s, rows);
-    check_part(h, f, splits, rows, s.A);
-    launch_gemm1_f64(s, q, rows, f.part, splits, st);
+    if (splits > 1) check_part(h, f, splits, rows, s.A);
+    launch_gemm1_f64(s, q, rows, splits > 1 ? f.part : Y, splits, st);
     check_launch(h, "gemm1_f64");
+    if (splits == 1) return;
     launch_reduce_y_f64(f.part, splits, rows, s.A, Y, st);
     check_launch(h, "reduce_y_f64");
     return;

@@ -111,3 +111,26 @@ def test_sub_batches_on_a_fresh_handle(L, reorth):
             L.lgw_destroy(h)
     for a, b in zip(*out):
         assert float((a - b).abs().max()) <= 1e-12 * float(b.abs().max())
+
+
+def test_one_split_needs_no_partials(L):
+    """On a handle with a byte limit (CUDA-core products) a contraction of one split writes
+    its result directly: vectors, results and y are all that a wide product holds."""
+    n_v, n_c, A, n_vec = 8, 32, 1024, 1216       # 16 x 19 tiles: one split
+    wl = gi.make_workload("p", n_v, n_c, A, [0], [0], 1, 3, aux_scaled=True)
+    X = torch.randn(n_vec, n_v * n_c, dtype=torch.float64, device=DEV,
+                    generator=torch.Generator(device=DEV).manual_seed(5))
+    out = []
+    for limit in (0, 8 * n_vec * (2 * n_v * n_c + A)):
+        h = L.lgw_create(0)
+        try:
+            s = L.lgw_prepare_system(h, n_v, n_c, A, _t(wl.eps), _t(wl.L), 4.0)
+            L.lgw_set_workspace_limit(h, limit)
+            Y = torch.zeros_like(X)
+            L.lgw_apply_casida(h, s, X, Y, "fp64")
+            torch.cuda.synchronize()
+            out.append(Y)
+            L.lgw_release_system(s)
+        finally:
+            L.lgw_destroy(h)
+    assert float((out[0] - out[1]).norm() / out[0].norm()) <= 1e-14
