@@ -47,6 +47,9 @@ constexpr int SPEC_THREADS = 256;
 constexpr int SPEC_FP32_ITS = 22;
 constexpr int SPEC_MAX_ITS = 160;
 
+__device__ __forceinline__ bool finite_bits(double x) {
+  return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
+}
 __device__ __forceinline__ int hi_abs(double p) { return __double2hiint(p) & 0x7fffffff; }
 
 // The trailing minors r_i = det(T_{i:n} - x) from the last row up: p = r_0,
@@ -212,8 +215,10 @@ __global__ void __launch_bounds__(SPEC_THREADS) k_spectral(
   const double *al = alpha + (size_t)v * k, *be = beta + (size_t)v * k;
   // Gershgorin interval
   double glo = 1e300, ghi = -1e300;
+  bool nan = !finite_bits(beta0[v]);
   for (int i = tid; i < n; i += blockDim.x) {
     const double a = al[i];
+    nan |= !finite_bits(a) || (i + 1 < n && !finite_bits(be[i]));
     const double r = (i > 0 ? fabs(be[i - 1]) : 0.0) + (i + 1 < n ? fabs(be[i]) : 0.0);
     glo = fmin(glo, a - r);
     ghi = fmax(ghi, a + r);
@@ -227,7 +232,16 @@ __global__ void __launch_bounds__(SPEC_THREADS) k_spectral(
     slo[wid] = glo;
     shi[wid] = ghi;
   }
-  __syncthreads();
+  // A coefficient that is not a number: the counts below would still close in
+  // on some node, and weights formed from the nodes alone would be finite.  The
+  // vector's weights are NaN instead, and with them all that is summed from it.
+  if (__syncthreads_or(nan)) {
+    for (int j = tid; j < n; j += blockDim.x) {
+      jb.a[(size_t)v * k + j] = 1.0;
+      jb.b2[(size_t)v * k + j] = __longlong_as_double(0x7ff8000000000000LL);
+    }
+    return;
+  }
   glo = slo[0];
   ghi = shi[0];
   for (int w = 1; w < nw; ++w) {
