@@ -280,6 +280,9 @@ __global__ void __launch_bounds__(SPEC_THREADS) k_spectral(
   // nodes errs by eps ||T|| / gap, and their sum with it.  The product formula
   // over the computed nodes and the computed eigenvalues without row 0 gives
   // the weights of a nearby tridiagonal, whose sums over a cluster are right.
+  // Nodes that coincide to the last bit have the eigenvalues between them there
+  // too; their factors are 0 / 0, and the group's weight, which the other
+  // factors give, is shared equally.
   bool close = false;
   for (int j = tid; j + 1 < n; j += blockDim.x) close |= ths[j + 1] - ths[j] < 0x1p-16 * w;
   if (__syncthreads_or(close)) {
@@ -296,12 +299,17 @@ __global__ void __launch_bounds__(SPEC_THREADS) k_spectral(
     for (int j = tid; j < n; j += blockDim.x) {
       const double th = ths[j];
       double wt = 1.0;
+      int same = 1;   // nodes that coincide with this one, itself included
       for (int i = 0; i < n; ++i) {
         if (i == j) continue;
         // mu between theta_i and theta_j: a factor within [0, 1]
         const double den = th - ths[i];
-        wt *= den != 0.0 ? (th - mus[i < j ? i : i - 1]) / den : 0.5;
+        if (den != 0.0)
+          wt *= (th - mus[i < j ? i : i - 1]) / den;
+        else
+          ++same;
       }
+      if (same > 1) wt /= same;
       weight[j] = wt;
     }
   }

@@ -86,3 +86,44 @@ def test_the_unused_last_beta_is_not_read(L):
     b[:, -1] = np.nan
     got = _run(L, a, b, b0)
     assert np.array_equal(got[0], clean[0]) and np.array_equal(got[1], clean[1])
+
+
+def _reference(a, b, b0, wl):
+    out = np.zeros((2, wl.omega.size), dtype=complex)
+    for v in range(6):
+        k = a.shape[1]
+        th, U = np.linalg.eigh(np.diag(a[v]) + np.diag(b[v, :k - 1], 1) + np.diag(b[v, :k - 1], -1))
+        m = M_IDX[v % 3]
+        eta = 1.0 if m < wl.n_v else -1.0
+        z = wl.omega - wl.eps[m] - 1j * eta * wl.delta
+        Om = np.sqrt(th)
+        out[v // 3] += (b0[v] ** 2 * U[0] ** 2 / Om / (z[:, None] + eta * Om)).sum(1)
+    return out
+
+
+@pytest.mark.parametrize("kind", ["constant", "copies 1e-7", "copies 1e-30", "copies 0",
+                                  "one in the middle"])
+@pytest.mark.parametrize("m,n", [(2, 9), (3, 11), (4, 25), (7, 36)])
+def test_coincident_nodes_share_their_weight(L, kind, m, n):
+    """m weakly coupled copies of one n-row tridiagonal: every node m times."""
+    wl = gw_inputs.tiny(k=64)
+    rng = np.random.default_rng(10 * m + n)
+    k = m * n
+    a, b, b0 = np.zeros((6, k)), np.zeros((6, k)), rng.uniform(0.1, 0.2, 6)
+    for v in range(6):
+        if kind == "constant":
+            a[v] = 500.0
+            continue
+        x, y = 500 + 20 * rng.uniform(-1, 1, n), 200 * rng.uniform(0.9, 1.0, n)
+        for c in range(m):
+            # every second copy upside down, so that the first row meets its image
+            a[v, c * n:(c + 1) * n] = x if c % 2 == 0 else x[::-1]
+            b[v, c * n:c * n + n - 1] = y[:n - 1] if c % 2 == 0 else y[:n - 1][::-1]
+            b[v, (c + 1) * n - 1] = 0.0 if kind == "one in the middle" else float(kind.split()[1])
+        if kind == "one in the middle":      # an isolated row at an eigenvalue of the first copy
+            a[v, k // 2] = np.linalg.eigvalsh(np.diag(x) + np.diag(y[:n - 1], 1)
+                                              + np.diag(y[:n - 1], -1))[n // 2]
+            b[v, k // 2 - 1] = b[v, k // 2] = 0.0
+    sig, _ = _run(L, a, b, b0)
+    ref = _reference(a, b, b0, wl)
+    assert np.abs(sig[..., 0] + 1j * sig[..., 1] - ref).max() <= 1e-10 * np.abs(ref).max()
