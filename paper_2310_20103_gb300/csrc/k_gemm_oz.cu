@@ -12,10 +12,16 @@
 // largest product).  Products are at most 2^12, so over 1024 terms S_0..S_3
 // are exact multiples of their unit below 2^24 of it; the others carry weights
 // of 2^-28 and less and may round.  Every 1024 terms the sums are joined in
-// 64-bit integers and rounded once to FP64.  The digits of a product thus lose
-// less than an FP64 dot product's own roundings do
-// (tests/test_gpu_f64_products.py; against exact sums, B = C R with 1024 terms
-// errs by 2.6e-16 of its norm, the FP64 FMA chain by 1.08e-15).
+// 64-bit integers and rounded once to FP64.
+//
+// What the digits lose is relative to the two rows' largest elements, max |x_k|
+// max |y_k|, where the roundings of an FMA chain are relative to the terms x_k
+// y_k.  For rows whose large elements meet (normal matrices, Krylov vectors)
+// that is less than FP64's own roundings: against exact sums, B = C R with 1024
+// terms errs by 2.6e-16 of its norm, the FMA chain by 1.08e-15
+// (tests/test_gpu_f64_products.py).  Rows graded along the contraction, one
+// rising where the other falls, would lose digits: density fitting balances
+// their scales first, by exact powers of two (tests/test_gpu_f64_graded.py).
 //
 // N_vc 32768, N_aux 1024, 64 vectors: 180 us per product on average (C x with
 // its digits 474 us), against 3.6 and 4.1 ms on the FP64 pipe (24 TFLOP/s in
@@ -387,45 +393,63 @@ __device__ __forceinline__ void store_digits16(const unsigned long long (&u)[16]
   }
 }
 
-// A matrix in memory: element (r, c) = x[r * ld + c] * (scale ? scale[c] : 1)
-// inside [nr][nc], zero outside.
+// A matrix in memory: element (r, c) = x[r * ld + c], times scale[c],
+// rscale[r] and 2^shift[c] where given, inside [nr][nc], zero outside.
 struct Src {
-  const double *x, *scale;
+  const double *x, *scale, *rscale;
+  const int *shift;
   size_t ld;
   int nr, nc;
   __device__ __forceinline__ double at(int r, int c) const {
     if (r >= nr || c >= nc) return 0.0;
-    const double v = x[(size_t)r * ld + c];
-    return scale ? scale[c] * v : v;
+    double v = x[(size_t)r * ld + c];
+    if (scale) v *= scale[c];
+    if (shift) v *= __hiloint2double((1023 + shift[c]) << 20, 0);
+    return rscale ? rscale[r] * v : v;
   }
 };
 
 // Largest exponent field of each operand row: the operand's rows are the
-// matrix's rows (COLS = false, contraction along c) or its columns.
+// matrix's rows (COLS = false, contraction along c) or its columns.  finite:
+// Inf and NaN do not count.
 template <bool COLS>
-__global__ void __launch_bounds__(256) k_oz_max(Src src, int *__restrict__ e) {
+__global__ void __launch_bounds__(256) k_oz_max(Src src, int *__restrict__ e, bool finite) {
   pdl_wait();
+  auto field = [&](int r, int c) {
+    const int f = exp_field(src.at(r, c));
+    return finite && f == 2047 ? 0 : f;
+  };
   const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
   if (COLS) {
     const int c = c0 + (threadIdx.x & 63);
     int m = 0;
-    for (int r = r0 + (threadIdx.x >> 6); r < r0 + 64; r += 4) m = max(m, exp_field(src.at(r, c)));
+    for (int r = r0 + (threadIdx.x >> 6); r < r0 + 64; r += 4) m = max(m, field(r, c));
     if (m > 0) atomicMax(&e[c], m);
   } else {
     const int r = r0 + (threadIdx.x >> 2), cc = c0 + (threadIdx.x & 3) * 16;
     int m = 0;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) m = max(m, exp_field(src.at(r, cc + i)));
+    for (int i = 0; i < 16; ++i) m = max(m, field(r, cc + i));
     m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
     m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
     if ((threadIdx.x & 3) == 0 && m > 0) atomicMax(&e[r], m);
   }
 }
 
+// blk[kb] of an operand row from the four threads that hold its 64 elements
+// (subnormals count as zeros)
+__device__ __forceinline__ void store_block_exp(int m, int part, short *blk) {
+  const unsigned quad = 0xfu << (threadIdx.x & 28);
+  m = max(m, __shfl_xor_sync(quad, m, 1));
+  m = max(m, __shfl_xor_sync(quad, m, 2));
+  if (part == 0) *blk = (short)(m > 0 ? m : OZ_ZERO);
+}
+
 // Digits of a 64 x 64 tile; the operand has `rows` rows and nkb K blocks.
 template <bool COLS>
 __global__ void __launch_bounds__(256) k_oz_slice(Src src, const int *__restrict__ e,
-                                                  uint16_t *__restrict__ out, int rows, int nkb) {
+                                                  uint16_t *__restrict__ out, int rows, int nkb,
+                                                  short *__restrict__ blk) {
   pdl_wait();
   __shared__ double tile[COLS ? 64 : 1][65];
   const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
@@ -439,18 +463,26 @@ __global__ void __launch_bounds__(256) k_oz_slice(Src src, const int *__restrict
   if (row >= rows || kb >= nkb) return;
   const int f = max(e[row], 1);
   unsigned long long u[16];
+  int m = 0;
 #pragma unroll
-  for (int k = 0; k < 16; ++k)
-    u[k] = fixed56(COLS ? tile[k0 + k][i] : src.at(row, c0 + k0 + k), f);
+  for (int k = 0; k < 16; ++k) {
+    const double x = COLS ? tile[k0 + k][i] : src.at(row, c0 + k0 + k);
+    u[k] = fixed56(x, f);
+    m = max(m, exp_field(x));
+  }
+  if (blk) store_block_exp(m, threadIdx.x & 3, blk + (size_t)row * nkb + kb);
   store_digits16(u, out + ((size_t)kb * rows + row) * 64 + k0, (size_t)nkb * rows * 64);
 }
 
 // One operand row per block, up to OZ_ROW_MAX elements: the sum of `splits`
 // partials (fixed order, optionally stored to y), its exponent and its digits.
+// Sixteen elements lie 17 doubles apart in shared memory: their readers meet
+// different banks (8192 rows of 1024 with shifts and block exponents: 93 us,
+// 101 without the gap).
 __global__ void __launch_bounds__(256) k_oz_rows(const double *__restrict__ x, int splits,
                                                  size_t part, Src src, double *__restrict__ y,
                                                  int *__restrict__ e, uint16_t *__restrict__ out,
-                                                 int rows, int nkb) {
+                                                 int rows, int nkb, short *__restrict__ blk) {
   extern __shared__ double v[];
   __shared__ int wmax[8];
   pdl_wait();
@@ -464,8 +496,12 @@ __global__ void __launch_bounds__(256) k_oz_rows(const double *__restrict__ x, i
       if (src.scale) s *= src.scale[i];
       if (y) y[o] = s;
     }
-    v[i] = s;
-    m = max(m, exp_field(s));
+    v[i + (i >> 4)] = s;
+    int f = exp_field(s);
+    // the power of two is added to the exponents (a multiplication would take
+    // the FP64 pipe, which the factorisation beside this kernel needs)
+    if (src.shift && i < src.nc && nonzero_bits(s)) f = max(f, 1) + src.shift[i];
+    m = max(m, f);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -476,11 +512,133 @@ __global__ void __launch_bounds__(256) k_oz_rows(const double *__restrict__ x, i
   m = max(m, 1);
   for (int g = threadIdx.x; g < nkb * 4; g += 256) {
     unsigned long long u[16];
+    int mb = 0;
 #pragma unroll
-    for (int k = 0; k < 16; ++k) u[k] = fixed56(v[g * 16 + k], m);
+    for (int k = 0; k < 16; ++k) {
+      const double s = v[g * 17 + k];
+      const int sh = src.shift && g * 16 + k < src.nc ? src.shift[g * 16 + k] : 0;
+      u[k] = fixed56(s, m - sh);
+      if (nonzero_bits(s)) mb = max(mb, max(exp_field(s), 1) + sh);
+    }
+    if (blk) {
+      store_block_exp(mb, g & 3, blk + (size_t)r * nkb + (g >> 2));
+    }
     store_digits16(u, out + ((size_t)(g >> 2) * rows + r) * 64 + (g & 3) * 16,
                    (size_t)nkb * rows * 64);
   }
+}
+
+// Scales of n contraction indices from their largest exponent fields e_k: the
+// factors 2^-s_k (down), s_k = max e - e_k, for one operand and the shifts s_k
+// (up) for the other, kept within 400, past which *unbalanced is set.
+__global__ void __launch_bounds__(256) k_oz_balance(const int *__restrict__ e, int n,
+                                                    double *__restrict__ down,
+                                                    int *__restrict__ up,
+                                                    unsigned *unbalanced) {
+  pdl_wait();
+  __shared__ int top;
+  if (threadIdx.x == 0) top = 0;
+  __syncthreads();
+  int m = 0;
+  for (int k = threadIdx.x; k < n; k += 256) m = max(m, e[k]);
+  atomicMax(&top, m);
+  __syncthreads();
+  for (int k = threadIdx.x; k < n; k += 256) {
+    const int d = e[k] > 0 ? top - e[k] : 0, s = min(d, 400);
+    down[k] = __hiloint2double((1023 - s) << 20, 0);
+    up[k] = s;
+    if (d != s) *unbalanced = 1u;
+  }
+}
+
+// Whether eight digits are enough for the products of operands a (its row i
+// zero before K index i) and b.  What they lose is relative to max |a_i| max
+// |b_j|, so an output (i, j) is as good as FP64's while some K block's largest
+// |a| times its largest |b| comes near that.  *poor is set where, in some 64 x
+// 64 tile of outputs, more than an eighth miss it by more than 2^6: a chance
+// small element in a short last block is not counted, operands graded against
+// one another are.  (8192 x 1024 outputs: 14 us.)  Where in some K block no row of the tile falls far below
+// its own largest element, as usual, the outputs need not be looked at one by
+// one.
+constexpr int LOSS_BITS = 6;
+
+__global__ void __launch_bounds__(256) k_oz_loss(const short *__restrict__ a,
+                                                 const short *__restrict__ b,
+                                                 const int *__restrict__ ea,
+                                                 const int *__restrict__ eb, int na, int nb,
+                                                 int nkb, unsigned *poor) {
+  pdl_wait();
+  __shared__ short sa[64][33], sb[64][33];
+  __shared__ int da[32], db[32];   // by K block: the rows' largest distance from their maxima
+  __shared__ int nbad, nall;
+  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+  const int a0 = blockIdx.x * 64, b0 = blockIdx.y * 64, kfirst = a0 / 64;
+  auto load = [&](int k0) {
+    for (int idx = t; idx < 64 * 32; idx += 256) {
+      const int r = idx >> 5, k = idx & 31;
+      const bool in = k0 + k < nkb;
+      sa[r][k] = in && a0 + r < na ? a[(size_t)(a0 + r) * nkb + k0 + k] : OZ_ZERO;
+      sb[r][k] = in && b0 + r < nb ? b[(size_t)(b0 + r) * nkb + k0 + k] : OZ_ZERO;
+    }
+  };
+  if (t == 0) nbad = nall = 0;
+  for (int k0 = kfirst; k0 < nkb; k0 += 32) {
+    __syncthreads();
+    if (t < 32) da[t] = db[t] = 0;
+    load(k0);
+    __syncthreads();
+    const int k = t & 31, r0 = (t >> 5) * 8;
+    int xa = 0, xb = 0;
+#pragma unroll
+    for (int r = r0; r < r0 + 8; ++r) {   // rows of zeros have no say
+      const int ma = a0 + r < na ? ea[a0 + r] : 0, mb = b0 + r < nb ? eb[b0 + r] : 0;
+      if (ma > 0) xa = max(xa, ma - sa[r][k]);
+      if (mb > 0) xb = max(xb, mb - sb[r][k]);
+    }
+    atomicMax(&da[k], xa);
+    atomicMax(&db[k], xb);
+    __syncthreads();
+    if (__syncthreads_or(t < 32 && k0 + t < nkb && da[t & 31] + db[t & 31] <= LOSS_BITS)) return;
+  }
+  int best[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) best[i][j] = 2 * OZ_ZERO;
+  for (int k0 = kfirst; k0 < nkb; k0 += 32) {
+    __syncthreads();
+    load(k0);
+    __syncthreads();
+    for (int k = 0; k < min(32, nkb - k0); ++k) {
+      int x[4], y[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[i] = sa[ty + 16 * i][k], y[i] = sb[tx + 16 * i][k];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) best[i][j] = max(best[i][j], x[i] + y[j]);
+    }
+  }
+  int bad = 0, all = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int r = a0 + ty + 16 * i, ma = r < na ? ea[r] : 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int c = b0 + tx + 16 * j, mb = c < nb ? eb[c] : 0;
+      if (best[i][j] <= 0) continue;   // no product at all: exactly zero
+      ++all;
+      bad += ma + mb - best[i][j] > LOSS_BITS ? 1 : 0;
+    }
+  }
+  bad = __reduce_add_sync(0xffffffffu, bad);
+  all = __reduce_add_sync(0xffffffffu, all);
+  if ((t & 31) == 0) {
+    atomicAdd(&nbad, bad);
+    atomicAdd(&nall, all);
+  }
+  __syncthreads();
+  if (t == 0 && 8 * nbad > nall) *poor = 1u;
 }
 
 // *bad != 0 if an exponent field says Inf or NaN
@@ -534,12 +692,11 @@ static void launch_rows(const double *x, int splits, size_t part, const Src &src
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(k_oz_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         OZ_ROW_MAX * (int)sizeof(double));
+                         OZ_ROW_MAX / 16 * 17 * (int)sizeof(double));
     attr = true;
   }
-  launch_pdl(k_oz_rows, dim3(o.rows), dim3(256), (size_t)o.nkb * 64 * sizeof(double), st, x,
-             splits,
-             part, src, y, o.e, o.d, o.rows, o.nkb);
+  launch_pdl(k_oz_rows, dim3(o.rows), dim3(256), (size_t)o.nkb * 68 * sizeof(double), st, x,
+             splits, part, src, y, o.e, o.d, o.rows, o.nkb, o.blk);
 }
 
 static int sm_count() {
@@ -598,11 +755,12 @@ bool launch_oz_gemm(const OzOperand &A, const OzOperand &B, int M, int Ncols, in
 // Digits of x [nr][nc] (row stride ld, optional column scale): operand rows
 // are x's rows, or its columns.  o.rows covers them (more rows become zeros).
 void launch_oz_slice(const double *x, size_t ld, int nr, int nc, const double *scale, bool cols,
-                     const OzOperand &o, cudaStream_t st) {
-  const oz::Src src{x, scale, ld, nr, nc};
+                     const OzOperand &o, cudaStream_t st, const double *rscale,
+                     const int *shift) {
+  const oz::Src src{x, scale, rscale, shift, ld, nr, nc};
   // short rows: one kernel, a block per row (4.7 us at 160 rows of 256); longer
   // ones spread each row over many blocks (64 rows of 32768: 12 + 20 us)
-  if (!cols && o.nkb * 64 <= 4096) {
+  if (!cols && !rscale && o.nkb * 64 <= 4096) {
     oz::launch_rows(x, 1, 0, src, nullptr, o, st);
     return;
   }
@@ -610,19 +768,43 @@ void launch_oz_slice(const double *x, size_t ld, int nr, int nc, const double *s
   const int kr = cols ? o.nkb : (o.rows + 63) / 64, kc = cols ? (o.rows + 63) / 64 : o.nkb;
   const dim3 grid(kc, kr), data((nc + 63) / 64, (nr + 63) / 64);
   if (cols) {
-    launch_pdl(oz::k_oz_max<true>, data, dim3(256), 0, st, src, o.e);
-    launch_pdl(oz::k_oz_slice<true>, grid, dim3(256), 0, st, src, o.e, o.d, o.rows, o.nkb);
+    launch_pdl(oz::k_oz_max<true>, data, dim3(256), 0, st, src, o.e, false);
+    launch_pdl(oz::k_oz_slice<true>, grid, dim3(256), 0, st, src, o.e, o.d, o.rows, o.nkb,
+               o.blk);
   } else {
-    launch_pdl(oz::k_oz_max<false>, data, dim3(256), 0, st, src, o.e);
-    launch_pdl(oz::k_oz_slice<false>, grid, dim3(256), 0, st, src, o.e, o.d, o.rows, o.nkb);
+    launch_pdl(oz::k_oz_max<false>, data, dim3(256), 0, st, src, o.e, false);
+    launch_pdl(oz::k_oz_slice<false>, grid, dim3(256), 0, st, src, o.e, o.d, o.rows, o.nkb,
+               o.blk);
   }
 }
 
 // y [rows][len] = sum of the split partials, and its digits (len <= OZ_ROW_MAX)
 void launch_oz_reduce(const double *part, int splits, int nr, int len, double *y,
                       const OzOperand &o, cudaStream_t st) {
-  const oz::Src src{part, nullptr, (size_t)len, nr, len};
+  const oz::Src src{part, nullptr, nullptr, nullptr, (size_t)len, nr, len};
   oz::launch_rows(part, splits, (size_t)nr * len, src, y, o, st);
+}
+
+void launch_oz_col_max(const double *x, size_t ld, int nr, int nc, int *e, cudaStream_t st) {
+  cudaMemsetAsync(e, 0, sizeof(int) * round_up(nc, 64), st);
+  constexpr int ROWS = 1 << 21;   // a grid's second dimension ends at 65535 tiles
+  for (int r0 = 0; r0 < nr; r0 += ROWS) {
+    const int n = std::min(ROWS, nr - r0);
+    const oz::Src src{x + (size_t)r0 * ld, nullptr, nullptr, nullptr, ld, n, nc};
+    launch_pdl(oz::k_oz_max<true>, dim3((nc + 63) / 64, (n + 63) / 64), dim3(256), 0, st, src, e,
+               true);
+  }
+}
+
+void launch_oz_balance(const int *e, int n, double *down, int *up, unsigned *unbalanced,
+                       cudaStream_t st) {
+  launch_pdl(oz::k_oz_balance, dim3(1), dim3(256), 0, st, e, n, down, up, unbalanced);
+}
+
+void launch_oz_loss(const OzOperand &a, const OzOperand &b, int na, int nb, unsigned *poor,
+                    cudaStream_t st) {
+  launch_pdl(oz::k_oz_loss, dim3((na + 63) / 64, (nb + 63) / 64), dim3(256), 0, st, a.blk, b.blk,
+             a.e, b.e, na, nb, a.nkb, poor);
 }
 
 void launch_oz_check(const OzOperand &o, unsigned *bad, cudaStream_t st) {

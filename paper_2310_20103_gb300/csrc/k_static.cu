@@ -244,8 +244,10 @@ __global__ void k_zero_upper(double *A, int n) {
 // Cm[M][N] = Am[M][K] Bm[K][N], row-major, FP64 (64 x 64 tiles)
 __global__ void __launch_bounds__(256) k_gemm_nn_f64(const double *__restrict__ Am,
                                                      const double *__restrict__ Bm, int M, int N,
-                                                     int K, double *__restrict__ Cm) {
+                                                     int K, double *__restrict__ Cm,
+                                                     const unsigned *only) {
   pdl_wait();
+  if (only != nullptr && *only == 0u) return;
   __shared__ double As[16][65];
   __shared__ double Bs[16][65];
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
@@ -313,9 +315,9 @@ int launch_cholesky(double *A, int n, unsigned *status, cudaStream_t st) {
 }
 
 void launch_gemm_nn_f64(const double *A, const double *B, int M, int N, int K, double *C,
-                        cudaStream_t st) {
+                        cudaStream_t st, const unsigned *only) {
   dim3 grid((N + 63) / 64, (M + 63) / 64);
-  launch_pdl(k_gemm_nn_f64, grid, dim3(256), 0, st, A, B, M, N, K, C);
+  launch_pdl(k_gemm_nn_f64, grid, dim3(256), 0, st, A, B, M, N, K, C, only);
 }
 
 }  // namespace lgw

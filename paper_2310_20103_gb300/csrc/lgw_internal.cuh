@@ -37,11 +37,13 @@ inline int64_t round_up64(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 // (k_gemm_oz.cu): 8 BF16 planes [slice][K block of 64][rows][64] and each
 // row's largest exponent field.
 constexpr int OZ_SLICES = 8;
-constexpr int OZ_ROW_MAX = 24576;   // longest row sliced by one block (192 KB of shared memory)
+constexpr int OZ_ROW_MAX = 24576;   // longest row sliced by one block (204 KB of shared memory)
+constexpr int OZ_ZERO = -8000;       // stands for the exponent field of zero
 struct OzOperand {
   uint16_t *d = nullptr;
   int *e = nullptr;
   int rows = 0, nkb = 0;
+  short *blk = nullptr;   // [rows][nkb] largest exponent field of each K block (optional)
   static size_t digits(size_t rows, size_t nkb) { return OZ_SLICES * rows * nkb * 64; }
 };
 
@@ -313,7 +315,14 @@ size_t oz_part_rows(int M, int rows, int slice, int nkb);
 bool launch_oz_gemm(const OzOperand &A, const OzOperand &B, int M, int Ncols, int splits,
                     const OzOut &o, unsigned *status, cudaStream_t st);
 void launch_oz_slice(const double *x, size_t ld, int nr, int nc, const double *scale, bool cols,
-                     const OzOperand &o, cudaStream_t st);
+                     const OzOperand &o, cudaStream_t st, const double *rscale = nullptr,
+                     const int *shift = nullptr);
+// largest finite exponent field of each column of x [nr][nc] (e: nc rounded up to 64)
+void launch_oz_col_max(const double *x, size_t ld, int nr, int nc, int *e, cudaStream_t st);
+void launch_oz_balance(const int *e, int n, double *down, int *up, unsigned *unbalanced,
+                       cudaStream_t st);
+void launch_oz_loss(const OzOperand &a, const OzOperand &b, int na, int nb, unsigned *poor,
+                    cudaStream_t st);
 void launch_oz_reduce(const double *part, int splits, int nr, int len, double *y,
                       const OzOperand &o, cudaStream_t st);
 void launch_oz_check(const OzOperand &o, unsigned *bad, cudaStream_t st);
@@ -521,8 +530,9 @@ void launch_pol_combine(const double *sig2, int n_pairs, int n_freq, double *out
 void launch_sigma_x(const double *M, int n_t, int n_m, int n_aux, const int *m_idx, int n_v,
                     double *out, cudaStream_t st);
 int launch_cholesky(double *A, int n, unsigned *status, cudaStream_t st);
+// only: nothing is done unless *only is nonzero
 void launch_gemm_nn_f64(const double *A, const double *B, int M, int N, int K, double *C,
-                        cudaStream_t st);
+                        cudaStream_t st, const unsigned *only = nullptr);
 
 // k_adjoint.cu : gradient of the QP energies (implicit function + Daleckii-Krein)
 // A stored Krylov basis [slot][Bs][N]: FP64, or the float pair hi (+ lo).

@@ -1,0 +1,103 @@
+"""FP64 products of graded operands: auxiliary functions and pairs of very different scales.
+
+The digits of a sliced product are a fixed point relative to a row's largest element, so what
+is graded along the contraction has to be balanced first.  Yardstick: numpy's own FP64
+evaluation against extended precision; over all outputs, each relative to the typical
+magnitude of the terms it sums, the largest error may be 4 times numpy's (plus 2^-50: digits
+of 2^-56 of the largest of a few hundred terms)."""
+import numpy as np
+import pytest
+
+import gw_inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+LD = np.longdouble
+
+
+@pytest.fixture(scope="module")
+def L():
+    from paper_2310_20103_gb300.build import build
+    build()
+    from paper_2310_20103_gb300 import lgw
+    return lgw
+
+
+def _factor(n, rng):
+    """A lower triangular factor of small integers with 16 on its diagonal: R R^T and every
+    step of its Cholesky factorisation are exact in FP64, so that what a fit errs by is the
+    product's own."""
+    R = np.tril(rng.integers(-3, 4, (n, n)), -1).astype(np.float64)
+    np.fill_diagonal(R, 16.0)
+    return R
+
+
+def _fit(L, C, metric):
+    B = np.zeros_like(C)
+    h = L.lgw_create(0)
+    try:
+        L.lgw_fit_factors(h, C, metric, B)
+    finally:
+        L.lgw_destroy(h)
+    return B
+
+
+@pytest.mark.parametrize("order", ["random", "falling", "rising"])
+@pytest.mark.parametrize("coeffs", ["inverse", "flat", "same"])
+@pytest.mark.parametrize("decades", [0, 8, 12, 16, 24])
+@pytest.mark.parametrize("n_pairs,n", [(200, 64), (150, 200)])
+def test_fit_factors_of_a_graded_metric(L, n_pairs, n, decades, coeffs, order):
+    """metric = D R R^T D, R exact, with `decades` between the diagonal's ends, C as 1 / D (auxiliary
+    functions of any normalisation), without, or as D."""
+    rng = np.random.default_rng(n + decades)
+    u = np.linspace(0, 1, n)
+    u = {"random": rng.permutation(u), "falling": u[::-1], "rising": u}[order]
+    d = 2.0 ** np.round(0.5 * decades * np.log2(10) * (u - 0.5))
+    R = d[:, None] * _factor(n, rng)
+    metric = R @ R.T
+    C = rng.standard_normal((n_pairs, n)) * {"inverse": 1 / d, "flat": np.ones(n), "same": d}[coeffs]
+    B = _fit(L, C, metric)
+    ref = C.astype(LD) @ R.astype(LD)
+    typical = np.abs(C).mean(0) @ np.abs(R)      # per column of B
+    own = np.abs(C @ R - ref) / typical
+    err = np.abs(B - ref) / typical
+    assert np.isfinite(B).all()
+    assert err.max() <= 4 * own.max() + 2.0 ** -50
+
+
+def test_fit_factors_of_rows_with_gradings_of_their_own(L):
+    """No scale per auxiliary function helps where every pair has its own: pairs on fragment
+    a see a's functions at 1 and b's at 1e-12, pairs on b the other way round, and B's columns
+    of b's functions come from the small ones."""
+    rng = np.random.default_rng(1)
+    n, n_pairs = 256, 120
+    R = _factor(n, rng)
+    R[128:, :128] *= 2.0 ** -20
+    C = rng.standard_normal((n_pairs, n))
+    C[:60, 128:] *= 1e-12
+    C[60:, :128] *= 1e-12
+    B = _fit(L, C, R @ R.T)
+    ref = C.astype(LD) @ R.astype(LD)
+    typical = np.empty_like(C)
+    for rows in (slice(0, 60), slice(60, n_pairs)):
+        typical[rows] = np.abs(C[rows]).mean(0) @ np.abs(R)
+    own = np.abs(C @ R - ref) / typical
+    err = np.abs(B - ref) / typical
+    assert err.max() <= 4 * own.max() + 2.0 ** -50
+
+
+def test_fit_factors_of_infinities(L):
+    """A row of C with an infinity is not finite where it was not, the other rows are as
+    without it."""
+    rng = np.random.default_rng(2)
+    C = rng.standard_normal((70, 96))
+    W = rng.standard_normal((96, 96))
+    metric = W @ W.T / 96 + np.eye(96)
+    metric = 0.5 * (metric + metric.T)
+    clean = _fit(L, C, metric)
+    C[5, 95] = np.inf          # meets every column's last row of R
+    B = _fit(L, C, metric)
+    others = np.arange(70) != 5
+    assert np.abs(B[others] - clean[others]).max() <= 1e-13 * np.abs(clean).max()
+    assert not np.isfinite(B[5]).any()
