@@ -20,8 +20,10 @@
 // that is less than FP64's own roundings: against exact sums, B = C R with 1024
 // terms errs by 2.6e-16 of its norm, the FMA chain by 1.08e-15
 // (tests/test_gpu_f64_products.py).  Rows graded along the contraction, one
-// rising where the other falls, would lose digits: density fitting balances
-// their scales first, by exact powers of two (tests/test_gpu_f64_graded.py).
+// rising where the other falls, would lose digits: what is graded by index is
+// balanced first, by exact powers of two, for L and the vectors by L's rows and
+// columns (ensure_digits), for density fitting by the auxiliary functions
+// (tests/test_gpu_f64_graded.py).
 //
 // N_vc 32768, N_aux 1024, 64 vectors: 180 us per product on average (C x with
 // its digits 474 us), against 3.6 and 4.1 ms on the FP64 pipe (24 TFLOP/s in
@@ -393,21 +395,30 @@ __device__ __forceinline__ void store_digits16(const unsigned long long (&u)[16]
   }
 }
 
-// A matrix in memory: element (r, c) = x[r * ld + c], times scale[c],
-// rscale[r] and 2^shift[c] where given, inside [nr][nc], zero outside.
+// A matrix in memory: element (r, c) = x[r * ld + c], times scale[c] and
+// rscale[r] where given, inside [nr][nc], zero outside; times 2^lift(r, c),
+// which is added to the exponents (a multiplication would take the FP64 pipe).
 struct Src {
   const double *x, *scale, *rscale;
-  const int *shift;
+  const int *shift, *rshift;   // by column, by row
   size_t ld;
   int nr, nc;
   __device__ __forceinline__ double at(int r, int c) const {
     if (r >= nr || c >= nc) return 0.0;
     double v = x[(size_t)r * ld + c];
     if (scale) v *= scale[c];
-    if (shift) v *= __hiloint2double((1023 + shift[c]) << 20, 0);
     return rscale ? rscale[r] * v : v;
   }
+  __device__ __forceinline__ int lift(int r, int c) const {
+    return (shift && c < nc ? shift[c] : 0) + (rshift && r < nr ? rshift[r] : 0);
+  }
 };
+
+// Exponent field of x 2^sh, 0 for zero; subnormals count as the smallest
+// normal numbers.
+__device__ __forceinline__ int lifted_field(double x, int sh) {
+  return nonzero_bits(x) ? max(exp_field(x), 1) + sh : 0;
+}
 
 // Largest exponent field of each operand row: the operand's rows are the
 // matrix's rows (COLS = false, contraction along c) or its columns.  finite:
@@ -416,8 +427,8 @@ template <bool COLS>
 __global__ void __launch_bounds__(256) k_oz_max(Src src, int *__restrict__ e, bool finite) {
   pdl_wait();
   auto field = [&](int r, int c) {
-    const int f = exp_field(src.at(r, c));
-    return finite && f == 2047 ? 0 : f;
+    const double v = src.at(r, c);
+    return finite && exp_field(v) == 2047 ? 0 : lifted_field(v, src.lift(r, c));
   };
   const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
   if (COLS) {
@@ -467,8 +478,9 @@ __global__ void __launch_bounds__(256) k_oz_slice(Src src, const int *__restrict
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
     const double x = COLS ? tile[k0 + k][i] : src.at(row, c0 + k0 + k);
-    u[k] = fixed56(x, f);
-    m = max(m, exp_field(x));
+    const int sh = COLS ? src.lift(r0 + k0 + k, row) : src.lift(row, c0 + k0 + k);
+    u[k] = fixed56(x, f - sh);
+    if (blk) m = max(m, lifted_field(x, sh));
   }
   if (blk) store_block_exp(m, threadIdx.x & 3, blk + (size_t)row * nkb + kb);
   store_digits16(u, out + ((size_t)kb * rows + row) * 64 + k0, (size_t)nkb * rows * 64);
@@ -478,7 +490,8 @@ __global__ void __launch_bounds__(256) k_oz_slice(Src src, const int *__restrict
 // partials (fixed order, optionally stored to y), its exponent and its digits.
 // Sixteen elements lie 17 doubles apart in shared memory: their readers meet
 // different banks (8192 rows of 1024 with shifts and block exponents: 93 us,
-// 101 without the gap).
+// 101 without the gap).  LIFT: with src.shift, and block exponents to blk.
+template <bool LIFT>
 __global__ void __launch_bounds__(256) k_oz_rows(const double *__restrict__ x, int splits,
                                                  size_t part, Src src, double *__restrict__ y,
                                                  int *__restrict__ e, uint16_t *__restrict__ out,
@@ -493,15 +506,14 @@ __global__ void __launch_bounds__(256) k_oz_rows(const double *__restrict__ x, i
     if (r < src.nr && i < src.nc) {
       const size_t o = (size_t)r * src.ld + i;
       for (int p = 0; p < splits; ++p) s += x[(size_t)p * part + o];
-      if (src.scale) s *= src.scale[i];
       if (y) y[o] = s;
+      if (src.scale) s *= src.scale[i];
     }
     v[i + (i >> 4)] = s;
-    int f = exp_field(s);
-    // the power of two is added to the exponents (a multiplication would take
-    // the FP64 pipe, which the factorisation beside this kernel needs)
-    if (src.shift && i < src.nc && nonzero_bits(s)) f = max(f, 1) + src.shift[i];
-    m = max(m, f);
+    if (LIFT)
+      m = max(m, lifted_field(s, i < src.nc ? src.shift[i] : 0));
+    else
+      m = max(m, exp_field(s));
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -516,15 +528,60 @@ __global__ void __launch_bounds__(256) k_oz_rows(const double *__restrict__ x, i
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
       const double s = v[g * 17 + k];
-      const int sh = src.shift && g * 16 + k < src.nc ? src.shift[g * 16 + k] : 0;
+      const int sh = LIFT && g * 16 + k < src.nc ? src.shift[g * 16 + k] : 0;
       u[k] = fixed56(s, m - sh);
-      if (nonzero_bits(s)) mb = max(mb, max(exp_field(s), 1) + sh);
+      if (LIFT) mb = max(mb, lifted_field(s, sh));
     }
-    if (blk) {
-      store_block_exp(mb, g & 3, blk + (size_t)r * nkb + (g >> 2));
-    }
+    if (LIFT) store_block_exp(mb, g & 3, blk + (size_t)r * nkb + (g >> 2));
     store_digits16(u, out + ((size_t)(g >> 2) * rows + r) * 64 + (g & 3) * 16,
                    (size_t)nkb * rows * 64);
+  }
+}
+
+// Largest exponent fields of the rows and of the columns of x [nr][nc] in one
+// pass, with the rows' and columns' own shifts: row[r] of x 2^shift[c], col[c]
+// of x 2^rshift[r].  nc a multiple of 64; a block takes 256 rows by 64 columns.
+__global__ void __launch_bounds__(256) k_oz_max_both(const double *__restrict__ x, int nr, int nc,
+                                                     const int *__restrict__ shift,
+                                                     const int *__restrict__ rshift,
+                                                     int *__restrict__ row, int *__restrict__ col) {
+  pdl_wait();
+  const int c = blockIdx.x * 64 + (threadIdx.x & 63), r0 = blockIdx.y * 256;
+  const int sc = shift ? shift[c] : 0;
+  int m = 0;
+#pragma unroll 4
+  for (int r = r0 + (threadIdx.x >> 6); r < min(nr, r0 + 256); r += 4) {   // alike in a warp
+    const double v = x[(size_t)r * nc + c];
+    m = max(m, lifted_field(v, rshift ? rshift[r] : 0));
+    const int mr = __reduce_max_sync(0xffffffffu, lifted_field(v, sc));
+    if ((threadIdx.x & 31) == 0 && mr > 0) atomicMax(&row[r], mr);
+  }
+  if (m > 0) atomicMax(&col[c], m);
+}
+
+// Balance of a factor along one index, from its largest exponent fields e_k:
+// shifts s_k = max e - e_k that even the factor out, and the vectors' factors
+// 2^-s_k (0 where the factor is zero) and base_k 2^-s_k.  Shifts end at 400.
+__global__ void __launch_bounds__(1024) k_oz_factors(const int *__restrict__ e, int n,
+                                                     const double *__restrict__ base,
+                                                     int *__restrict__ shift,
+                                                     double *__restrict__ down,
+                                                     double *__restrict__ based) {
+  pdl_wait();
+  __shared__ int top;
+  if (threadIdx.x == 0) top = 0;
+  __syncthreads();
+  int m = 0;
+  for (int k = threadIdx.x; k < n; k += 1024) m = max(m, e[k]);
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(&top, m);
+  __syncthreads();
+  for (int k = threadIdx.x; k < n; k += 1024) {
+    const int s = e[k] > 0 ? min(top - e[k], 400) : 0;
+    const double f = e[k] > 0 ? __hiloint2double((1023 - s) << 20, 0) : 0.0;
+    shift[k] = s;
+    down[k] = f;
+    if (base) based[k] = base[k] * f;
   }
 }
 
@@ -687,15 +744,16 @@ static void launch(const CUtensorMap &A, const CUtensorMap &B, int M, int Ncols,
   launch_pdl(k_oz_gemm<NT>, grid, dim3(NTHREADS), Cfg<NT>::SMEM, st, A, B, M, Ncols, nkb, per, e);
 }
 
+template <bool LIFT>
 static void launch_rows(const double *x, int splits, size_t part, const Src &src, double *y,
                         const OzOperand &o, cudaStream_t st) {
   static bool attr = false;
   if (!attr) {
-    cudaFuncSetAttribute(k_oz_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(k_oz_rows<LIFT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          OZ_ROW_MAX / 16 * 17 * (int)sizeof(double));
     attr = true;
   }
-  launch_pdl(k_oz_rows, dim3(o.rows), dim3(256), (size_t)o.nkb * 68 * sizeof(double), st, x,
+  launch_pdl(k_oz_rows<LIFT>, dim3(o.rows), dim3(256), (size_t)o.nkb * 68 * sizeof(double), st, x,
              splits, part, src, y, o.e, o.d, o.rows, o.nkb, o.blk);
 }
 
@@ -757,11 +815,14 @@ bool launch_oz_gemm(const OzOperand &A, const OzOperand &B, int M, int Ncols, in
 void launch_oz_slice(const double *x, size_t ld, int nr, int nc, const double *scale, bool cols,
                      const OzOperand &o, cudaStream_t st, const double *rscale,
                      const int *shift) {
-  const oz::Src src{x, scale, rscale, shift, ld, nr, nc};
+  const oz::Src src{x, scale, rscale, shift, nullptr, ld, nr, nc};
   // short rows: one kernel, a block per row (4.7 us at 160 rows of 256); longer
   // ones spread each row over many blocks (64 rows of 32768: 12 + 20 us)
   if (!cols && !rscale && o.nkb * 64 <= 4096) {
-    oz::launch_rows(x, 1, 0, src, nullptr, o, st);
+    if (shift)
+      oz::launch_rows<true>(x, 1, 0, src, nullptr, o, st);
+    else
+      oz::launch_rows<false>(x, 1, 0, src, nullptr, o, st);
     return;
   }
   cudaMemsetAsync(o.e, 0, sizeof(int) * o.rows, st);
@@ -778,11 +839,37 @@ void launch_oz_slice(const double *x, size_t ld, int nr, int nc, const double *s
   }
 }
 
-// y [rows][len] = sum of the split partials, and its digits (len <= OZ_ROW_MAX)
+// y [rows][len] = sum of the split partials, and the digits of o.scale y (len
+// <= OZ_ROW_MAX)
 void launch_oz_reduce(const double *part, int splits, int nr, int len, double *y,
                       const OzOperand &o, cudaStream_t st) {
-  const oz::Src src{part, nullptr, nullptr, nullptr, (size_t)len, nr, len};
-  oz::launch_rows(part, splits, (size_t)nr * len, src, y, o, st);
+  const oz::Src src{part, o.scale, nullptr, nullptr, nullptr, (size_t)len, nr, len};
+  oz::launch_rows<false>(part, splits, (size_t)nr * len, src, y, o, st);
+}
+
+void launch_oz_max_both(const double *x, int nr, int nc, const int *shift, const int *rshift,
+                        int *row, int *col, cudaStream_t st) {
+  cudaMemsetAsync(row, 0, sizeof(int) * nr, st);
+  cudaMemsetAsync(col, 0, sizeof(int) * nc, st);
+  launch_pdl(oz::k_oz_max_both, dim3(nc / 64, (nr + 255) / 256), dim3(256), 0, st, x, nr, nc,
+             shift, rshift, row, col);
+}
+
+void launch_oz_factors(const int *e, int n, const double *base, int *shift, double *down,
+                       double *based, cudaStream_t st) {
+  launch_pdl(oz::k_oz_factors, dim3(1), dim3(1024), 0, st, e, n, base, shift, down, based);
+}
+
+// Digits of x [nr][nc] whose rows' (columns') exponents are in o.e already.
+void launch_oz_digits(const double *x, int nr, int nc, bool cols, const int *shift,
+                      const OzOperand &o, cudaStream_t st) {
+  const oz::Src src{x, nullptr, nullptr, cols ? nullptr : shift, cols ? shift : nullptr,
+                    (size_t)nc, nr, nc};
+  const dim3 grid(cols ? (o.rows + 63) / 64 : o.nkb, cols ? o.nkb : (o.rows + 63) / 64);
+  if (cols)
+    launch_pdl(oz::k_oz_slice<true>, grid, dim3(256), 0, st, src, o.e, o.d, o.rows, o.nkb, o.blk);
+  else
+    launch_pdl(oz::k_oz_slice<false>, grid, dim3(256), 0, st, src, o.e, o.d, o.rows, o.nkb, o.blk);
 }
 
 void launch_oz_col_max(const double *x, size_t ld, int nr, int nc, int *e, cudaStream_t st) {
@@ -790,7 +877,7 @@ void launch_oz_col_max(const double *x, size_t ld, int nr, int nc, int *e, cudaS
   constexpr int ROWS = 1 << 21;   // a grid's second dimension ends at 65535 tiles
   for (int r0 = 0; r0 < nr; r0 += ROWS) {
     const int n = std::min(ROWS, nr - r0);
-    const oz::Src src{x + (size_t)r0 * ld, nullptr, nullptr, nullptr, ld, n, nc};
+    const oz::Src src{x + (size_t)r0 * ld, nullptr, nullptr, nullptr, nullptr, ld, n, nc};
     launch_pdl(oz::k_oz_max<true>, dim3((nc + 63) / 64, (n + 63) / 64), dim3(256), 0, st, src, e,
                true);
   }

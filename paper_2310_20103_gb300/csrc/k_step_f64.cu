@@ -2,7 +2,8 @@
 //   alpha_j = q_j . w,  w <- w - alpha_j q_j,  full Gram-Schmidt against the
 //   stored q_0..q_j (two passes, the second always or by the norm criterion),
 //   beta_{j+1} = ||w||, breakdown test, q_{j+1} = w / beta_{j+1},
-// and, for the tensor-core FP64 products, the digits of Delta^1/2 q_{j+1}.
+// and, for the tensor-core FP64 products, the digits of Delta^1/2 q_{j+1} (on L's
+// row scales, xd.scale).
 //
 // One cluster of nchunks blocks per vector, a block per chunk of VEC_CHUNK
 // elements, w in registers throughout; sums over the vector meet in the
@@ -272,7 +273,7 @@ __global__ void __launch_bounds__(VEC_THREADS, GS ? 2 : 4)
     w[u].y = inv > 0.0 ? w[u].y * inv : 0.0;
     *reinterpret_cast<double2 *>(qn + e) = w[u];
     if (xd.d) {
-      const double2 d = *reinterpret_cast<const double2 *>(c.dsq + e);
+      const double2 d = *reinterpret_cast<const double2 *>(xd.scale + e);
       w[u].x *= d.x;
       w[u].y *= d.y;
       m = max(m, max(oz::exp_field(w[u].x), oz::exp_field(w[u].y)));

@@ -75,6 +75,7 @@ struct lgw_system {
   // Inf or NaN), 0 not asked for yet
   int oz_state = 0;
   void *oz_buf = nullptr;
+  const double *ozx_tda = nullptr;   // SysDev::ozx of the Tamm-Dancoff view
 };
 
 // ---------------------------------------------------------------------------
@@ -189,6 +190,7 @@ void free_digits(lgw_system *sys) {
   sys_free(sys->h, sys->oz_buf);
   sys->oz_buf = nullptr;
   sys->s.ozA = sys->s.ozT = sys->tda.ozA = sys->tda.ozT = OzOperand{};
+  sys->s.ozx = sys->s.ozy = sys->tda.ozx = sys->tda.ozy = sys->ozx_tda = nullptr;
   sys->oz_state = -1;
 }
 
@@ -522,7 +524,7 @@ void make_fp8(lgw_handle *h, SysDev &s, const double *src, int ld, int nr, int n
 }
 
 // Digits of L for the FP64 products (32 bytes per element of L), made on the
-// first FP64 request.  They may take a third of the free memory at most, and
+// first FP64 request, of L evened out along each contraction.  They may take a third of the free memory at most, and
 // are given back when a workspace allocation fails (drop_digits); without
 // them the products run on the CUDA cores.  One synchronisation, once.
 void ensure_digits(lgw_handle *h, lgw_system *sys) {
@@ -530,24 +532,33 @@ void ensure_digits(lgw_handle *h, lgw_system *sys) {
   SysDev &s = sys->s;
   sys->oz_state = -1;
   if (!s.L64 || !tc_available() || s.A > OZ_ROW_MAX) return;
-  const size_t plane = OzOperand::digits((size_t)s.N, (size_t)s.A / 64) * sizeof(uint16_t);
-  const size_t ints = ((size_t)s.N + s.A + 64) * sizeof(int);
+  const size_t N = (size_t)s.N, A = (size_t)s.A;
+  const size_t plane = OzOperand::digits(N, A / 64) * sizeof(uint16_t);
+  const size_t rest = (2 * N + A) * sizeof(double) + (2 * (N + A) + 64) * sizeof(int);
   size_t fr = 0, tot = 0;
   LGW_TRY_CUDA(h, cudaMemGetInfo(&fr, &tot));
-  if (2 * plane + ints > (fr + h->spare_bytes) / 3) return;
-  void *p = sys_alloc(h, 2 * plane + ints);
+  if (2 * plane + rest > (fr + h->spare_bytes) / 3) return;
+  void *p = sys_alloc(h, 2 * plane + rest);
   if (!p) return;
   sys->oz_buf = p;
   uint16_t *d = static_cast<uint16_t *>(p);
-  int *e = reinterpret_cast<int *>(static_cast<uint8_t *>(p) + 2 * plane);
+  double *x1 = reinterpret_cast<double *>(static_cast<uint8_t *>(p) + 2 * plane);   // 2^-s_vc
+  double *xd = x1 + N, *ys = xd + N;
+  int *e = reinterpret_cast<int *>(ys + A), *sx = e + N + A, *sy = sx + N;
   const OzOperand a{d, e, s.N, s.A / 64};
   const OzOperand t{d + plane / sizeof(uint16_t), e + s.N, s.A, s.N / 64};
-  unsigned *bad = reinterpret_cast<unsigned *>(e + s.N + s.A);
+  unsigned *bad = reinterpret_cast<unsigned *>(sy + A);
   cudaStream_t st = h->stream;
   LGW_TRY_CUDA(h, cudaMemsetAsync(bad, 0, sizeof(unsigned), st));
-  launch_oz_slice(s.L64, s.A, s.N, s.A, nullptr, false, a, st);
-  launch_oz_slice(s.L64, s.A, s.N, s.A, nullptr, true, t, st);
+  // L's scales by pair and by auxiliary function, then its digits on them: over
+  // vc, L 2^s_vc meets x Delta^1/2 2^-s_vc, over mu, L 2^t_mu meets y 2^-t_mu
+  launch_oz_max_both(s.L64, s.N, s.A, nullptr, nullptr, a.e, t.e, st);
   launch_oz_check(t, bad, st);
+  launch_oz_factors(a.e, s.N, s.dsq, sx, x1, xd, st);
+  launch_oz_factors(t.e, s.A, nullptr, sy, ys, nullptr, st);
+  launch_oz_max_both(s.L64, s.N, s.A, sy, sx, a.e, t.e, st);
+  launch_oz_digits(s.L64, s.N, s.A, false, sy, a, st);
+  launch_oz_digits(s.L64, s.N, s.A, true, sx, t, st);
   check_launch(h, "oz_slice(L)");
   h->launches--;   // the system's preparation, not this call's
   unsigned hb = 1;
@@ -559,6 +570,9 @@ void ensure_digits(lgw_handle *h, lgw_system *sys) {
   }
   s.ozA = a;
   s.ozT = t;
+  s.ozx = xd;
+  s.ozy = ys;
+  sys->ozx_tda = x1;
   sys->oz_state = 1;
   h->sliced.push_back(sys);
 }
@@ -704,6 +718,8 @@ F64Work f64_work(lgw_handle *h, const SysDev &s, int rows, const std::string &ow
     if (pp) {
       f.x = OzOperand{d, e, r, s.N / 64};
       f.y = OzOperand{d + nx, e + r, r, s.A / 64};
+      f.x.scale = s.ozx;
+      f.y.scale = s.ozy;
       f.part = pp;
       f.part_n = op;
       return f;
@@ -760,7 +776,7 @@ void f64_contract1(lgw_handle *h, const SysDev &s, const F64Work &f, const doubl
     OzOperand x = f.x, y = f.y;
     x.rows = y.rows = nr;
     if (!ready) {
-      launch_oz_slice(q + (size_t)r0 * s.N, (size_t)s.N, nr, s.N, s.dsq, false, x, st);
+      launch_oz_slice(q + (size_t)r0 * s.N, (size_t)s.N, nr, s.N, x.scale, false, x, st);
       check_launch(h, "oz_slice(x)");
     }
     const int splits = oz_splits(s.A, nr, s.N / 64);
@@ -1816,6 +1832,7 @@ const SysDev &tda_view(lgw_handle *h, const lgw_system *csys) {
   t = s;
   t.kf = 0.5 * s.kf;
   t.dsq = ones;
+  t.ozx = sys->ozx_tda;
   t.Delta2 = s.Delta;
   t.cd = cd;
   t.dsqf = onesf;

@@ -44,6 +44,7 @@ struct OzOperand {
   int *e = nullptr;
   int rows = 0, nkb = 0;
   short *blk = nullptr;   // [rows][nkb] largest exponent field of each K block (optional)
+  const double *scale = nullptr;   // vectors: factor of each K element (NULL: 1)
   static size_t digits(size_t rows, size_t nkb) { return OZ_SLICES * rows * nkb * 64; }
 };
 
@@ -74,8 +75,11 @@ struct SysDev {
   uint8_t *L8t;     // [A][N]   its transpose, K-block-major (kblk_e4m3)
   float *sL;        // [A]      s_mu
   // digits of L64, made on the first FP64 request: rows vc (contraction over
-  // mu) and rows mu (contraction over vc); absent where memory is short
+  // mu) and rows mu (contraction over vc); absent where memory is short.  The
+  // digits are of L evened out along the contraction; ozx, ozy carry L's scales
+  // to the vectors: Delta^1/2 2^-s_vc for x, 2^-t_mu for y
   OzOperand ozA, ozT;
+  const double *ozx, *ozy;
 };
 
 // ---------------------------------------------------------------------------
@@ -317,6 +321,12 @@ bool launch_oz_gemm(const OzOperand &A, const OzOperand &B, int M, int Ncols, in
 void launch_oz_slice(const double *x, size_t ld, int nr, int nc, const double *scale, bool cols,
                      const OzOperand &o, cudaStream_t st, const double *rscale = nullptr,
                      const int *shift = nullptr);
+void launch_oz_max_both(const double *x, int nr, int nc, const int *shift, const int *rshift,
+                        int *row, int *col, cudaStream_t st);
+void launch_oz_factors(const int *e, int n, const double *base, int *shift, double *down,
+                       double *based, cudaStream_t st);
+void launch_oz_digits(const double *x, int nr, int nc, bool cols, const int *shift,
+                      const OzOperand &o, cudaStream_t st);
 // largest finite exponent field of each column of x [nr][nc] (e: nc rounded up to 64)
 void launch_oz_col_max(const double *x, size_t ld, int nr, int nc, int *e, cudaStream_t st);
 void launch_oz_balance(const int *e, int n, double *down, int *up, unsigned *unbalanced,
@@ -437,7 +447,7 @@ void launch_band_combine(const double *sig, int p, int F, double *out, cudaStrea
 
 // k_step_f64.cu : alpha, axpy, Gram-Schmidt, beta and q_{j+1} of one FP64 step
 // in one kernel, one cluster per vector; with x.d also the digits of
-// Delta^1/2 q_{j+1}.  False (nothing launched) beyond its limits.
+// x.scale q_{j+1}.  False (nothing launched) beyond its limits.
 constexpr int STEP_MAX_K1 = 4096;     // k + 1: three rows of coefficients in shared memory
 bool launch_step_f64(const VecCtx &c, int j, const OzOperand &x, cudaStream_t st);
 

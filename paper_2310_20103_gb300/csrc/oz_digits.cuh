@@ -20,10 +20,10 @@ __device__ __forceinline__ unsigned long long fixed56(double x, int f) {
   const int ex = (int)((b >> 52) & 0x7ff);
   long long m = b & 0xfffffffffffffLL;
   if (ex != 0) m |= 1LL << 52;
-  const int sh = max(ex, 1) - f + 2;   // at most 2: |x| < 2^(f - 1022)
+  const int sh = max(ex, 1) - f + 2;   // at most 2: |x| < 2^(f - 1022), or x is 0
   long long v = 0;
   if (sh >= 0)
-    v = m << sh;
+    v = m << min(sh, 2);
   else if (sh > -56)
     v = (m + (1LL << (-sh - 1))) >> -sh;
   if (b < 0) v = -v;

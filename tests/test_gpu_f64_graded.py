@@ -101,3 +101,40 @@ def test_fit_factors_of_infinities(L):
     others = np.arange(70) != 5
     assert np.abs(B[others] - clean[others]).max() <= 1e-13 * np.abs(clean).max()
     assert not np.isfinite(B[5]).any()
+
+
+@pytest.mark.parametrize("pairs,aux", [(0, 0), (10, 0), (0, 12), (10, 12), (16, 16)])
+@pytest.mark.parametrize("x_scale", ["flat", "inverse"])
+@pytest.mark.parametrize("n_v,n_c,A", [(8, 32, 96), (13, 80, 130)])
+def test_apply_casida_of_a_graded_factor(L, n_v, n_c, A, pairs, aux, x_scale):
+    """L = D1 K D2, vectors without grading or as 1 / D1."""
+    rng = np.random.default_rng(pairs + aux + A)
+    wl = gw_inputs.make_workload("p", n_v, n_c, A, [0], [0], 1, 3)
+    N, n_vec = n_v * n_c, 20
+    d1 = 10.0 ** (-pairs * rng.uniform(0, 1, N))
+    d2 = 10.0 ** (-aux * rng.uniform(0, 1, A))
+    Lm = rng.standard_normal((N, A)) * d1[:, None] * d2[None, :]
+    X = rng.standard_normal((n_vec, N)) / (d1 if x_scale == "inverse" else 1.0)
+    Y = np.zeros_like(X)
+    h = L.lgw_create(0)
+    try:
+        s = L.lgw_prepare_system(h, n_v, n_c, A, torch.from_numpy(wl.eps).to(DEV),
+                                 torch.from_numpy(Lm).to(DEV))
+        L.lgw_apply_casida(h, s, np.ascontiguousarray(X), Y, "fp64")
+        L.lgw_release_system(s)
+    finally:
+        L.lgw_destroy(h)
+
+    def apply(dt):
+        e = wl.eps.astype(dt)
+        D = (e[None, n_v:] - e[:n_v, None]).reshape(-1)
+        y = (X.astype(dt) * np.sqrt(D)) @ Lm.astype(dt)
+        return X.astype(dt) * D ** 2 + dt(4.0) * np.sqrt(D) * (y @ Lm.astype(dt).T), D, y
+
+    ref, D, y = apply(LD)
+    own, err = np.abs(apply(np.float64)[0] - ref), np.abs(Y - ref)
+    D = D.astype(np.float64)
+    # terms of the low-rank part, by their typical size over the vectors
+    xt = (np.abs(X) * np.sqrt(D)).mean(0)
+    scale = np.abs(X).mean(0) * D ** 2 + 4 * np.sqrt(D) * ((xt @ np.abs(Lm)) @ np.abs(Lm).T)
+    assert (err / scale).max() <= 4 * (own / scale).max() + 2.0 ** -50
