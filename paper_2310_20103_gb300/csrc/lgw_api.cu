@@ -71,8 +71,8 @@ struct lgw_system {
   // Tamm-Dancoff view (A = Delta + (c_K/2) L L^T in place of C), made on first use
   SysDev tda{};
   void *tda_buf = nullptr;
-  // digits of L for the FP64 products: 1 made, -1 not (no memory, or L holds
-  // Inf or NaN), 0 not asked for yet
+  // digits of L for the FP64 products: 1 made, 0 not (not asked for yet, or no
+  // memory when last asked), -1 never (L holds Inf or NaN)
   int oz_state = 0;
   void *oz_buf = nullptr;
   const double *ozx_tda = nullptr;   // SysDev::ozx of the Tamm-Dancoff view
@@ -191,7 +191,7 @@ void free_digits(lgw_system *sys) {
   sys->oz_buf = nullptr;
   sys->s.ozA = sys->s.ozT = sys->tda.ozA = sys->tda.ozT = OzOperand{};
   sys->s.ozx = sys->s.ozy = sys->tda.ozx = sys->tda.ozy = sys->ozx_tda = nullptr;
-  sys->oz_state = -1;
+  sys->oz_state = 0;
 }
 
 // Gives back every system's digits of L, the workspace of the digits (oz_*
@@ -524,13 +524,17 @@ void make_fp8(lgw_handle *h, SysDev &s, const double *src, int ld, int nr, int n
 }
 
 // Digits of L for the FP64 products (32 bytes per element of L), made on the
-// first FP64 request, of L evened out along each contraction.  They may take a third of the free memory at most, and
-// are given back when a workspace allocation fails (drop_digits); without
-// them the products run on the CUDA cores.  One synchronisation, once.
+// first FP64 request, of L evened out along each contraction.  They may take a
+// third of the free memory at most, and are given back when a workspace
+// allocation fails (drop_digits); without them the products run on the CUDA
+// cores, and the next request asks again.  One synchronisation, once.
 void ensure_digits(lgw_handle *h, lgw_system *sys) {
   if (sys->oz_state != 0) return;
   SysDev &s = sys->s;
-  sys->oz_state = -1;
+  if (sys->oz_buf) {   // of an attempt that ended in an error
+    cudaDeviceSynchronize();
+    free_digits(sys);
+  }
   if (!s.L64 || !tc_available() || s.A > OZ_ROW_MAX) return;
   const size_t N = (size_t)s.N, A = (size_t)s.A;
   const size_t plane = OzOperand::digits(N, A / 64) * sizeof(uint16_t);
@@ -566,6 +570,7 @@ void ensure_digits(lgw_handle *h, lgw_system *sys) {
   LGW_TRY_CUDA(h, cudaStreamSynchronize(st));
   if (hb != 0) {
     free_digits(sys);
+    sys->oz_state = -1;
     return;
   }
   s.ozA = a;
@@ -575,6 +580,7 @@ void ensure_digits(lgw_handle *h, lgw_system *sys) {
   sys->ozx_tda = x1;
   sys->oz_state = 1;
   h->sliced.push_back(sys);
+  h->drop_graphs();   // captured without them
 }
 
 // The copies of L a request needs must exist; the E4M3 copies are made on
