@@ -271,7 +271,10 @@ lgw_status lgw_last_error(lgw_handle *h, char *buf, size_t n);
  * workspace may hold (0: no cap, the default).  A call whose next
  * workspace allocation would pass the cap returns LGW_ERR_OOM before that
  * allocation; nothing already held is freed and the handle stays usable
- * (work queued earlier in the call completes on valid buffers).  A failed
+ * (work queued earlier in the call completes on valid buffers).  Setting a cap
+ * waits for the device and frees what the FP64 products keep to be faster (the
+ * digits of every system's L, 32 bytes per element, and their workspace), and
+ * a handle with a cap makes no more of it.  A failed
  * cudaMalloc gives LGW_ERR_OOM the same way.  lgw_workspace_bytes reports
  * the bytes held; lgw_release_workspace waits for the handle's stream and
  * frees the whole workspace (later calls allocate it again). */

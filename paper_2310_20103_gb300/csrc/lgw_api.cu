@@ -527,9 +527,10 @@ void make_fp8(lgw_handle *h, SysDev &s, const double *src, int ld, int nr, int n
 // first FP64 request, of L evened out along each contraction.  They may take a
 // third of the free memory at most, and are given back when a workspace
 // allocation fails (drop_digits); without them the products run on the CUDA
-// cores, and the next request asks again.  One synchronisation, once.
+// cores, and the next request asks again.  None on a handle with a byte limit.
+// One synchronisation, once.
 void ensure_digits(lgw_handle *h, lgw_system *sys) {
-  if (sys->oz_state != 0) return;
+  if (sys->oz_state != 0 || h->ws_limit) return;   // f64_work takes no buffers there
   SysDev &s = sys->s;
   if (sys->oz_buf) {   // of an attempt that ended in an error
     cudaDeviceSynchronize();
@@ -2188,7 +2189,7 @@ lgw_status lgw_set_workspace_limit(lgw_handle *h, size_t bytes) {
   lgw_status g = guard_handle(h);
   if (g != LGW_OK) return g;
   h->ws_limit = bytes;
-  if (bytes) spare_free(h);
+  if (bytes) drop_digits(h);   // and the spare blocks
   return LGW_OK;
 }
 

@@ -41,6 +41,27 @@ def _apply(L, h, s, inputs):
     return inputs[3].clone()
 
 
+def test_a_limited_handle_makes_none(L, inputs):
+    h = L.lgw_create(0)
+    try:
+        L.lgw_set_workspace_limit(h, 8 * GB)
+        s = L.lgw_prepare_system(h, N_V, N_C, A, inputs[0], inputs[1], 4.0)
+        before = _free()
+        y0 = _apply(L, h, s, inputs)
+        assert before - _free() < L.lgw_workspace_bytes(h) + GB // 8
+        # with the limit lifted the next request makes them, and a new limit frees them
+        L.lgw_set_workspace_limit(h, 0)
+        y1 = _apply(L, h, s, inputs)
+        assert before - _free() > GB
+        L.lgw_set_workspace_limit(h, 8 * GB)
+        assert before - _free() < L.lgw_workspace_bytes(h) + GB // 8
+        assert torch.equal(_apply(L, h, s, inputs), y0)
+        assert float((y0 - y1).norm() / y0.norm()) <= 1e-14
+        L.lgw_release_system(s)
+    finally:
+        L.lgw_destroy(h)
+
+
 def test_made_again_once_memory_has_come_back(L, inputs):
     """A shortage at one request does not keep a system on the CUDA cores for good."""
     h = L.lgw_create(0)
