@@ -66,8 +66,9 @@ typedef enum {
  * are FP64 in the FP64 mode and split BF16 (three products) otherwise. */
 typedef enum {
   LGW_FP64 = 0,   /* FP64 products: the plain FP64 path (on the tensor cores
-                     by error-free slicing where the digits of L fit the
-                     device's memory, else on the CUDA cores)              */
+                     by error-free slicing where the digits of L, 32 bytes
+                     per element, fit a third of the free device memory,
+                     else on the CUDA cores)                               */
   LGW_BF16 = 1,   /* BF16 tcgen05 tensor-core GEMMs, FP32 accumulate      */
   LGW_FP8 = 3,    /* E4M3 tcgen05 GEMMs (kind::f8f6f4), FP32 accumulate:
                      L with one power-of-two scale per column (max -> (224,
@@ -276,8 +277,10 @@ lgw_status lgw_last_error(lgw_handle *h, char *buf, size_t n);
  * digits of every system's L, 32 bytes per element, and their workspace), and
  * a handle with a cap makes no more of it.  A failed
  * cudaMalloc gives LGW_ERR_OOM the same way.  lgw_workspace_bytes reports
- * the bytes held; lgw_release_workspace waits for the handle's stream and
- * frees the whole workspace (later calls allocate it again). */
+ * the bytes held, without the systems' own memory: the copies of L and the
+ * digits.  lgw_release_workspace waits for the handle's work and frees the
+ * whole workspace, every system's digits and the memory kept from released
+ * systems (later calls allocate and make them again). */
 lgw_status lgw_set_workspace_limit(lgw_handle *h, size_t bytes);
 lgw_status lgw_workspace_bytes(lgw_handle *h, size_t *bytes);
 lgw_status lgw_release_workspace(lgw_handle *h);

@@ -2206,13 +2206,13 @@ lgw_status lgw_release_workspace(lgw_handle *h) {
   if (g != LGW_OK) return g;
   if (cudaStreamSynchronize(h->stream) != cudaSuccess)
     return set_err(h, LGW_ERR_CUDA, "stream synchronisation before the release failed");
+  drop_digits(h);   // and the spare blocks
   h->drop_graphs();
   for (auto &kv : h->bufs)
     if (kv.second.p) cudaFree(kv.second.p);
   h->bufs.clear();
   h->ws_bytes = 0;
   h->ws_gen++;
-  spare_free(h);
   return LGW_OK;
 }
 

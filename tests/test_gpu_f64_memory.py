@@ -62,6 +62,22 @@ def test_a_limited_handle_makes_none(L, inputs):
         L.lgw_destroy(h)
 
 
+def test_release_workspace_gives_them_back(L, inputs):
+    h = L.lgw_create(0)
+    try:
+        s = L.lgw_prepare_system(h, N_V, N_C, A, inputs[0], inputs[1], 4.0)
+        before = _free()
+        y0 = _apply(L, h, s, inputs)
+        assert before - _free() > GB
+        L.lgw_release_workspace(h)
+        assert before - _free() < GB // 8
+        assert torch.equal(_apply(L, h, s, inputs), y0)
+        assert before - _free() > GB
+        L.lgw_release_system(s)
+    finally:
+        L.lgw_destroy(h)
+
+
 def test_made_again_once_memory_has_come_back(L, inputs):
     """A shortage at one request does not keep a system on the CUDA cores for good."""
     h = L.lgw_create(0)
