@@ -2804,14 +2804,19 @@ lgw_status lgw_sigma_c_batched(lgw_handle *h, int32_t n_sys, const lgw_system *c
   if (rep) std::memset(rep, 0, sizeof *rep);
   if (n_sys == 0) return LGW_OK;
   const cudaStream_t caller = h->stream;
-  // every exit restores the caller's stream and the default workspace names
+  // every exit restores the caller's stream and the default workspace names; one
+  // that leaves before the lanes are joined waits for what they still run (the
+  // caller may release those systems next)
   struct Restore {
     lgw_handle *h;
     cudaStream_t st;
+    bool joined = false;
     ~Restore() {
       h->stream = st;
       h->ws_prefix.clear();
       h->timing = false;
+      if (!joined)
+        for (cudaStream_t l : h->lanes) cudaStreamSynchronize(l);
     }
   } restore{h, caller};
   try {
@@ -2869,6 +2874,7 @@ lgw_status lgw_sigma_c_batched(lgw_handle *h, int32_t n_sys, const lgw_system *c
       LGW_TRY_CUDA(h, cudaEventRecord(fork, h->lanes[l]));
       LGW_TRY_CUDA(h, cudaStreamWaitEvent(caller, fork, 0));
     }
+    restore.joined = true;
     cudaEventDestroy(fork);
     if (rep) {
       LGW_TRY_CUDA(h, cudaEventRecord(t1, caller));
