@@ -947,15 +947,14 @@ int adj_max_k() {
 
 void launch_eig_full(const AdjCtx &a, cudaStream_t st) {
   const size_t smem = (size_t)6 * a.k * sizeof(double);
-  static bool attr = false;
-  if (!attr) {
+  static DeviceOnce once;
+  once(current_device(), [] {
     cudaFuncSetAttribute(k_eig_full, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     // the GEMM that runs beside it needs an SM's shared memory, which is split
     // from the L1 when the first block arrives
     cudaFuncSetAttribute(k_eig_full, cudaFuncAttributePreferredSharedMemoryCarveout,
                          cudaSharedmemCarveoutMaxShared);
-    attr = true;
-  }
+  });
   launch_pdl(k_eig_full, dim3(a.Bs), dim3(EIG_THREADS), smem, st, a);
 }
 void launch_adj_coeffs(const AdjCtx &a, cudaStream_t st) {
@@ -964,23 +963,16 @@ void launch_adj_coeffs(const AdjCtx &a, cudaStream_t st) {
 }
 void launch_adj_rows(const AdjCtx &a, BasisRef basis, double *Y, double *Gd, cudaStream_t st) {
   const size_t smem = (size_t)a.k * ROW_THREADS * sizeof(double);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_adj_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    attr = true;
-  }
+  static DeviceOnce once;
+  allow_smem(once, k_adj_rows, 200 * 1024);
   dim3 grid((a.N + ROW_THREADS - 1) / ROW_THREADS, a.Bs);
   launch_pdl(k_adj_rows, grid, dim3(ROW_THREADS), smem, st, a, basis, Y, Gd);
 }
 void launch_adj_rows_f32(const AdjCtx &a, BasisRef basis, double *Y, double *Gd,
                          cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_adj_rows_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(k_adj_rows_f32_deep, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         200 * 1024);
-    attr = true;
-  }
+  static DeviceOnce once, once_deep;
+  allow_smem(once, k_adj_rows_f32, 200 * 1024);
+  allow_smem(once_deep, k_adj_rows_f32_deep, 200 * 1024);
   const size_t tables = (size_t)2 * a.k * RF_ELEMS * sizeof(float);
   if (tables <= 200 * 1024)   // k up to 200
     launch_pdl(k_adj_rows_f32, dim3((a.N + RF_ELEMS - 1) / RF_ELEMS, a.Bs), dim3(32 * RF_WARPS),

@@ -734,12 +734,8 @@ static bool encode(CUtensorMap *tm, const OzOperand &o, int box_rows, int box_sl
 template <int NT>
 static void launch(const CUtensorMap &A, const CUtensorMap &B, int M, int Ncols, int nkb, int per,
                    int splits, const Epi &e, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_oz_gemm<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         Cfg<NT>::SMEM);
-    attr = true;
-  }
+  static DeviceOnce once;
+  allow_smem(once, k_oz_gemm<NT>, Cfg<NT>::SMEM);
   const dim3 grid((Ncols + NT - 1) / NT, (M + BM - 1) / BM, splits);
   launch_pdl(k_oz_gemm<NT>, grid, dim3(NTHREADS), Cfg<NT>::SMEM, st, A, B, M, Ncols, nkb, per, e);
 }
@@ -747,32 +743,18 @@ static void launch(const CUtensorMap &A, const CUtensorMap &B, int M, int Ncols,
 template <bool LIFT>
 static void launch_rows(const double *x, int splits, size_t part, const Src &src, double *y,
                         const OzOperand &o, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_oz_rows<LIFT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         OZ_ROW_MAX / 16 * 17 * (int)sizeof(double));
-    attr = true;
-  }
+  static DeviceOnce once;
+  allow_smem(once, k_oz_rows<LIFT>, OZ_ROW_MAX / 16 * 17 * sizeof(double));
   launch_pdl(k_oz_rows<LIFT>, dim3(o.rows), dim3(256), (size_t)o.nkb * 68 * sizeof(double), st, x,
              splits, part, src, y, o.e, o.d, o.rows, o.nkb, o.blk);
 }
 
-static int sm_count() {
-  static int n = [] {
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-    return v > 0 ? v : 152;
-  }();
-  return n;
-}
-
 }  // namespace oz
 
-int oz_splits(int M, int ncols, int nkb) { return oz::k_splits(M, ncols, nkb, oz::sm_count()); }
+int oz_splits(int M, int ncols, int nkb) { return oz::k_splits(M, ncols, nkb, device_sms()); }
 
 size_t oz_part_rows(int M, int rows, int slice, int nkb) {
-  return oz::part_rows(M, rows, slice, nkb, oz::sm_count());
+  return oz::part_rows(M, rows, slice, nkb, device_sms());
 }
 
 bool launch_oz_gemm(const OzOperand &A, const OzOperand &B, int M, int Ncols, int splits,
@@ -796,7 +778,7 @@ bool launch_oz_gemm(const OzOperand &A, const OzOperand &B, int M, int Ncols, in
   const int nkb = A.nkb, per = (nkb + splits - 1) / splits;
   const int m_tiles = (M + oz::BM - 1) / oz::BM;
   const int nt =
-      oz::tile_cols(m_tiles, Ncols, o.mode == OZ_PART ? std::min(64, nkb) : 1, oz::sm_count());
+      oz::tile_cols(m_tiles, Ncols, o.mode == OZ_PART ? std::min(64, nkb) : 1, device_sms());
   CUtensorMap ta, tb;
   if (A.rows < oz::BM || B.rows < nt || A.nkb != B.nkb || !oz::encode(&ta, A, oz::BM, 1) ||
       !oz::encode(&tb, B, nt, nt == 64 ? oz::Cfg<64>::BOX : OZ_SLICES))

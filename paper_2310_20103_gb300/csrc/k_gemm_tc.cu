@@ -896,12 +896,8 @@ template <int BN, int EPI, int EB = 2, int HALF = 0>
 static void launch_tc(const CUtensorMap &A, const CUtensorMap &B, int M, int Ncols, int num_kb,
                       int kb_per_split, int splits, const tc::EpiArgs &ea, cudaStream_t st) {
   using C = tc::Cfg<BN, HALF, EB == 3>;
-  static bool attr_done = false;
-  if (!attr_done) {
-    cudaFuncSetAttribute(tc::k_gemm_tc<BN, EPI, EB, HALF>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    attr_done = true;
-  }
+  static DeviceOnce once;
+  allow_smem(once, tc::k_gemm_tc<BN, EPI, EB, HALF>, C::SMEM);
   dim3 grid((M + tc::BM - 1) / tc::BM, (Ncols + BN - 1) / BN, splits);
   launch_pdl(tc::k_gemm_tc<BN, EPI, EB, HALF>, grid, dim3(tc::NTHREADS), C::SMEM, st, A, B, M,
              Ncols, num_kb,
@@ -912,18 +908,10 @@ template <int BN, int EB>
 static void launch_persist(const CUtensorMap &A, const CUtensorMap &B, int M, int Ncols,
                            int num_kb, const tc::EpiArgs &ea, cudaStream_t st) {
   using C = tc::Cfg<BN, 0>;
-  static bool attr_done = false;
-  static int nsm = 0;
-  if (!attr_done) {
-    cudaFuncSetAttribute(tc::k_gemm_persist<BN, EB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         C::SMEM);
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    attr_done = true;
-  }
+  static DeviceOnce once;
+  allow_smem(once, tc::k_gemm_persist<BN, EB>, C::SMEM);
   const int total = ((M + tc::BM - 1) / tc::BM) * ((Ncols + BN - 1) / BN);
-  const int grid = std::max(1, std::min(total, nsm > 0 ? nsm : 148));
+  const int grid = std::max(1, std::min(total, device_sms()));
   launch_pdl(tc::k_gemm_persist<BN, EB>, dim3(grid), dim3(tc::NTHREADS), C::SMEM, st, A, B, M,
              Ncols, num_kb, ea);
 }
@@ -1063,12 +1051,8 @@ template <int BN>
 static void launch_coupling(const TcPlan *p, const CUtensorMap &bhi, const CUtensorMap &blo,
                             float *vf, unsigned *status, cudaStream_t st) {
   using C = tc::CplCfg<BN>;
-  static bool attr_done = false;
-  if (!attr_done) {
-    cudaFuncSetAttribute(tc::k_gemm_coupling<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         C::SMEM);
-    attr_done = true;
-  }
+  static DeviceOnce once;
+  allow_smem(once, tc::k_gemm_coupling<BN>, C::SMEM);
   const dim3 grid((p->Bs + BN - 1) / BN, (p->N + tc::BM - 1) / tc::BM);
   launch_pdl(tc::k_gemm_coupling<BN>, grid, dim3(tc::NTHREADS), C::SMEM, st, p->g2A, p->g2Alo,
              bhi, blo, p->N, p->Bs, p->A / tc::BK, vf, status);

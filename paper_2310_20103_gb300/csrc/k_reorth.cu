@@ -1221,20 +1221,11 @@ __global__ void __launch_bounds__(256) k_p2_reduce_dcgs(VecCtx c, int j) {
   c.sinv[b] = (stop || !(beta > 0.0)) ? 0.0 : 1.0 / beta;
 }
 
-// Dynamic shared memory above 48 KB needs the attribute, set once per kernel.
-template <class K>
-static void allow_smem(K kern, size_t bytes) {
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <bool LO, bool F64U>
 static void sweep_one(const VecCtx &c, int j, cudaStream_t st) {
-  static bool attr = false;
+  static DeviceOnce once;
   constexpr size_t max_sh = sweep_stage_bytes<LO>() + (size_t)4096 * sizeof(float2);
-  if (!attr) {
-    allow_smem(k_sweep_dcgs<LO, F64U>, max_sh);
-    attr = true;
-  }
+  allow_smem(once, k_sweep_dcgs<LO, F64U>, max_sh);
   const size_t sh = sweep_stage_bytes<LO>() + (size_t)(j > 0 ? j : 1) * sizeof(float2);
   launch_pdl(k_sweep_dcgs<LO, F64U>, dim3(c.nchunks, c.Bs), dim3(VEC_THREADS), sh, st, c, j);
 }
@@ -1255,11 +1246,8 @@ void launch_reduce_dcgs(const VecCtx &c, int j, cudaStream_t st) {
 }
 template <bool LO>
 static void pass2_one(const VecCtx &c, int j, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    allow_smem(k_p2_dcgs<LO>, sweep_stage_bytes<LO>() + (size_t)4096 * sizeof(double));
-    attr = true;
-  }
+  static DeviceOnce once;
+  allow_smem(once, k_p2_dcgs<LO>, sweep_stage_bytes<LO>() + (size_t)4096 * sizeof(double));
   const dim3 grid(c.nchunks, c.Bs < 16 ? c.Bs : 16);
   launch_pdl(k_p2_dcgs<LO>, grid, dim3(VEC_THREADS),
              sweep_stage_bytes<LO>() + (size_t)(j + 1) * sizeof(double), st, c, j);

@@ -343,11 +343,8 @@ void launch_spectral_impl(const double *alpha, const double *beta, const double 
                           const int *k_eff, int B, int k, JacobiBufs jb,
                           unsigned long long *min_theta_bits, unsigned *status, cudaStream_t st) {
   // 40 k bytes of shared memory per block: 164 KB at the largest depth
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_spectral, cudaFuncAttributeMaxDynamicSharedMemorySize, 164 * 1024);
-    attr = true;
-  }
+  static DeviceOnce once;
+  allow_smem(once, k_spectral, 164 * 1024);
   const int threads = std::min(SPEC_THREADS, (k + 31) / 32 * 32);
   const size_t sh = (size_t)k * (sizeof(double2) + sizeof(float2) + 2 * sizeof(double));
   launch_pdl(k_spectral, dim3(B), dim3(threads), sh, st, alpha, beta, beta0, k_eff, k, jb,

@@ -297,13 +297,12 @@ __global__ void __launch_bounds__(VEC_THREADS, GS ? 2 : 4)
 
 template <bool GS>
 void launch_one(const VecCtx &c, int j, const OzOperand &x, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
+  static DeviceOnce once;
+  once(current_device(), [] {
     cudaFuncSetAttribute(k_step_f64<GS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaFuncSetAttribute(k_step_f64<GS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          STEP_MAX_K1 * 3 * (int)sizeof(double));
-    attr = true;
-  }
+  });
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(c.nchunks, c.Bs);
   cfg.blockDim = dim3(VEC_THREADS);

@@ -8,6 +8,7 @@
 
 #include "fp_bits.cuh"
 #include "lgw.h"
+#include "per_device.cuh"
 
 namespace lgw {
 
@@ -207,6 +208,28 @@ void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaSt
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+inline int current_device() {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  return dev;
+}
+inline int device_sms() {
+  static DeviceValue sms;
+  const int dev = current_device();
+  return sms(dev, [&] {
+    int v = 0;
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    return v > 0 ? v : 152;
+  });
+}
+// Dynamic shared memory above 48 KB has to be allowed, per kernel and device.
+template <class K>
+void allow_smem(DeviceOnce &once, K kernel, size_t bytes) {
+  once(current_device(), [&] {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  });
 }
 
 // x != 0 on the integer pipe (NaN counts as nonzero).
