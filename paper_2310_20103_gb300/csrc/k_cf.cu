@@ -14,6 +14,7 @@
 
 #include <algorithm>
 
+#include "fp_iter.cuh"
 #include "lgw_internal.cuh"
 
 namespace lgw {
@@ -52,19 +53,6 @@ __device__ __forceinline__ void cf_eval(const double *__restrict__ a, const doub
     dG.re = -W * pr;
     dG.im = -W * pi;
   }
-}
-
-// 1/d for the positive |zeta - Omega|^2 of a pole: the hardware's estimate
-// (about 20 bits) and one third-order Newton step, y (1 + e + e^2) with
-// e = 1 - d y, 60 bits: 3 FP64 operations where the division takes about 10.
-// Exponents where the estimate could leave the normal range divide.
-__device__ __forceinline__ double pole_rcp(double d) {
-  if ((unsigned)(__double2hiint(d) - (32 << 20)) >= (unsigned)(1980 << 20)) return 1.0 / d;
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-  double e = fma(-d, y, 1.0);
-  e = fma(e, e, e);
-  return fma(y, e, y);
 }
 
 // One thread per (target, frequency, slice of the summed set): loops over its

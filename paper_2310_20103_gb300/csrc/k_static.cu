@@ -10,6 +10,7 @@
 // (Cholesky, R lower) gives the factors B = C R.  FP64 throughout.
 #include <algorithm>
 
+#include "fp_iter.cuh"
 #include "lgw_internal.cuh"
 
 namespace lgw {
@@ -34,27 +35,6 @@ __global__ void k_sigma_x(const double *__restrict__ M, int n_m, int n_aux,
 // triangle of a [n][n] row-major matrix.
 // --------------------------------------------------------------------------
 constexpr int NB = 64;
-
-// sqrt(d) and x / s to the last place or so from r ~ 1 / s: one Newton
-// correction each, instead of a square root and a division (a serial chain of
-// tens of FP64 operations) per column.
-__device__ __forceinline__ double sqrt_from(double d, double r) {
-  const double s = d * r;
-  return fma(fma(-s, s, d), 0.5 * r, s);
-}
-__device__ __forceinline__ double div_from(double x, double s, double r) {
-  const double q = x * r;
-  return fma(fma(-q, s, x), r, q);
-}
-
-// 1 / sqrt(d), 1e-280 < d < 1e280: the hardware's approximation and one cubic
-// Newton step.
-__device__ __forceinline__ double rsqrt_newton(double d) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-  const double e = fma(-d * y, y, 1.0);
-  return fma(y * e, fma(e, 0.375, 0.5), y);
-}
 
 // Factor the diagonal block at (j0, j0): one CTA, columns in panels of eight.
 // A warp's FP64 instruction holds its scheduler's pipe for 76 clocks whatever
@@ -96,7 +76,7 @@ __global__ void __launch_bounds__(POTRF_THREADS) k_potrf_diag(double *A, int n, 
       }
       double x, s;
       if (d > 1e-280 && d < 1e280) {
-        const double r = rsqrt_newton(d);
+        const double r = rsqrt_iter(d);
         s = sqrt_from(d, r);
         x = div_from(v[j], s, r);
       } else {   // infinities too
