@@ -433,8 +433,8 @@ lgw_status lgw_sigma_x(lgw_handle *h, const lgw_system *s, const lgw_problem *p,
  * the system's L, those of the (t, m) pairs the request's M.  Host or device
  * pointers; LGW_ERR_NOT_SPD if the metric is not positive definite.  The
  * auxiliary functions may have any normalisation: their scales in C are moved
- * to R by exact powers of two before the product, and where that does not even
- * out the operands it runs on the CUDA cores. */
+ * to R by exact powers of two before the product, and tiles of B for which that
+ * does not even out the operands are formed by FP64 multiplications. */
 lgw_status lgw_fit_factors(lgw_handle *h, int32_t n_pairs, int32_t n_aux, const double *C,
                            const double *metric, double *B);
 

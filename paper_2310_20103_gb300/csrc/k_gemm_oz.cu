@@ -125,9 +125,99 @@ struct Epi {
   const double *Delta2, *dsq, *cd, *q, *qprev, *betaj;
   double *alpha_part;      // [M / 64][Ncols] partials of q . w, or NULL
   unsigned *status;
+  // CHECK: the K blocks' exponents of A's and B's rows, and the matrices
+  // themselves, A's row i the column i of xa
+  const short *ba, *bb;
+  const double *xa, *xb;
+  int ldxa, ldxb, K;
 };
 
+// Whether eight digits are enough for a tile's products.  What they lose is
+// relative to max |a_i| max |b_j|, so an output (i, j) is as good as FP64's
+// while some K block's largest |a| times its largest |b| comes near that.  False
+// where more than an eighth of the tile's outputs miss it by more than 2^6: a
+// chance small element in a short last block is not counted, operands graded
+// against one another are.  Where in some K block no row falls far below its own
+// largest element, as usual, the outputs need not be looked at one by one.  The
+// epilogue's warps ask while the products run.
+constexpr int LOSS_BITS = 6;
+struct LossShared {
+  int da[32], db[32];   // by K block: the rows' largest distance from their maxima
+  int bad, all;
+};
+__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+
 template <int NT>
+__device__ bool digits_do(const Epi &e, int m0, int n0, int M, int Ncols, int nkb,
+                          LossShared &sh) {
+  const int t = threadIdx.x - 64, kfirst = e.lower ? m0 / KB : 0;
+  if (t == 0) sh.bad = sh.all = 0;
+  for (int k0 = kfirst; k0 < nkb; k0 += 32) {
+    epi_sync();
+    if (t < 32) sh.da[t] = sh.db[t] = k0 + t < nkb ? 0 : 1 << 20;
+    epi_sync();
+    const int k = t & 31, part = t >> 5;
+    if (k0 + k < nkb) {
+      int xa = 0, xb = 0;   // rows of zeros have no say
+#pragma unroll
+      for (int i = 0; i < BM / 8; ++i) {
+        const int r = m0 + part * (BM / 8) + i, f = r < M ? e.ea[r] : 0;
+        const int d = r < M ? f - e.ba[(size_t)r * nkb + k0 + k] : 0;
+        if (f > 0) xa = max(xa, d);
+      }
+#pragma unroll
+      for (int i = 0; i < NT / 8; ++i) {
+        const int r = n0 + part * (NT / 8) + i, f = r < Ncols ? e.eb[r] : 0;
+        const int d = r < Ncols ? f - e.bb[(size_t)r * nkb + k0 + k] : 0;
+        if (f > 0) xb = max(xb, d);
+      }
+      atomicMax(&sh.da[k], xa);
+      atomicMax(&sh.db[k], xb);
+    }
+    epi_sync();
+    for (int i = 0; i < 32; ++i)
+      if (sh.da[i] + sh.db[i] <= LOSS_BITS) return true;
+  }
+  const int row = m0 + (t & 127);
+  int bad = 0, all = 0;
+  if (row < M)
+    for (int j = (t >> 7) * (NT / 2); j < ((t >> 7) + 1) * (NT / 2) && n0 + j < Ncols; ++j) {
+      int best = 2 * OZ_ZERO;
+      for (int k = kfirst; k < nkb; ++k)
+        best = max(best, e.ba[(size_t)row * nkb + k] + e.bb[(size_t)(n0 + j) * nkb + k]);
+      if (best <= 0) continue;   // no product at all: exactly zero
+      ++all;
+      bad += e.ea[row] + e.eb[n0 + j] - best > LOSS_BITS ? 1 : 0;
+    }
+  atomicAdd(&sh.bad, bad);
+  atomicAdd(&sh.all, all);
+  epi_sync();
+  return 8 * sh.bad <= sh.all;
+}
+
+// The tile by FP64 multiplications, one chain over K per output (the order of
+// k_gemm_nn_f64).
+template <int NT>
+__device__ void tile_f64(const Epi &e, int m0, int n0, int M, int Ncols) {
+  const int t = threadIdx.x - 64, row = m0 + (t & 127), c0 = n0 + (t >> 7) * (NT / 2);
+  if (row >= M) return;
+  for (int g = 0; g < NT / 2; g += 8) {
+    double acc[8] = {};
+    for (int k = 0; k < e.K; ++k) {
+      const double x = e.xa[(size_t)k * e.ldxa + row];
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        acc[i] = fma(e.xb[(size_t)min(c0 + g + i, Ncols - 1) * e.ldxb + k], x, acc[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (c0 + g + i < Ncols) e.out[(size_t)(c0 + g + i) * e.ldo + row] = acc[i];
+  }
+}
+
+// CHECK: outputs that the digits are not enough for are formed in FP64 (OZ_PART
+// of one split).
+template <int NT, bool CHECK>
 __global__ void __launch_bounds__(NTHREADS, 1)
     k_oz_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
               int M, int Ncols, int num_kb, int kb_per_split, Epi e) {
@@ -271,6 +361,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       cdr = e.dsq[row];
     }
     double *out = e.out + (e.mode == OZ_PART ? (size_t)split * Ncols * e.ldo : 0);
+    __shared__ LossShared loss;
+    const bool do_f64 =
+        CHECK && !digits_do<NT>(e, m_tile * BM, n_tile * NT, M, Ncols, num_kb, loss);
     for (int c = 0; c < chunks; ++c) {
       if (!mbar_wait(tfull, c & 1, e.status)) break;
       tc_fence_after();
@@ -359,8 +452,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty);
     }
+    if (CHECK && do_f64) {
+      epi_sync();   // the tile's stores come first
+      tile_f64<NT>(e, m_tile * BM, n_tile * NT, M, Ncols);
+    }
     if (e.alpha_part != nullptr && chunks > 0) {
-      asm volatile("bar.sync 1, 256;" ::: "memory");
+      epi_sync();
       for (int i = threadIdx.x - 64; i < 2 * NT; i += 32 * EPI_WARPS) {
         const int hf = i / NT, col = i % NT, b = n_tile * NT + col;
         if (b < Ncols && m_tile * BM + 64 * hf < M)
@@ -395,22 +492,34 @@ __device__ __forceinline__ void store_digits16(const unsigned long long (&u)[16]
   }
 }
 
-// A matrix in memory: element (r, c) = x[r * ld + c], times scale[c] and
-// rscale[r] where given, inside [nr][nc], zero outside; times 2^lift(r, c),
-// which is added to the exponents (a multiplication would take the FP64 pipe).
+// Shift that brings a contraction index whose largest exponent field is e to a
+// common scale, 0 .. 800: up in one operand, down in the other (exactly; indices
+// beyond 2^+-400 come as near as that).
+__device__ __forceinline__ int even_shift(int e) {
+  return e > 0 ? 1423 - min(max(e, 623), 1423) : 0;
+}
+
+// A matrix in memory: element (r, c) = x[r * ld + c], times scale[c] where
+// given, inside [nr][nc], zero outside; times 2^lift(r, c), which is added to
+// the exponents (a multiplication would take the FP64 pipe).  shift and rshift
+// are shifts by column and by row; even: shift holds exponent fields instead,
+// for even_shift up; reven: exponent fields by row, for even_shift down.
 struct Src {
-  const double *x, *scale, *rscale;
-  const int *shift, *rshift;   // by column, by row
+  const double *x, *scale;
+  const int *shift, *rshift, *reven;
+  bool even;
   size_t ld;
   int nr, nc;
   __device__ __forceinline__ double at(int r, int c) const {
     if (r >= nr || c >= nc) return 0.0;
-    double v = x[(size_t)r * ld + c];
-    if (scale) v *= scale[c];
-    return rscale ? rscale[r] * v : v;
+    const double v = x[(size_t)r * ld + c];
+    return scale ? scale[c] * v : v;
   }
   __device__ __forceinline__ int lift(int r, int c) const {
-    return (shift && c < nc ? shift[c] : 0) + (rshift && r < nr ? rshift[r] : 0);
+    int s = rshift && r < nr ? rshift[r] : 0;
+    if (reven && r < nr) s -= even_shift(reven[r]);
+    if (shift && c < nc) s += even ? even_shift(shift[c]) : shift[c];
+    return s;
   }
 };
 
@@ -426,21 +535,23 @@ __device__ __forceinline__ int lifted_field(double x, int sh) {
 template <bool COLS>
 __global__ void __launch_bounds__(256) k_oz_max(Src src, int *__restrict__ e, bool finite) {
   pdl_wait();
-  auto field = [&](int r, int c) {
-    const double v = src.at(r, c);
-    return finite && exp_field(v) == 2047 ? 0 : lifted_field(v, src.lift(r, c));
-  };
   const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
+  const int r = COLS ? r0 + (threadIdx.x >> 6) : r0 + (threadIdx.x >> 2);
+  const int c = COLS ? c0 + (threadIdx.x & 63) : c0 + (threadIdx.x & 3) * 16;
+  constexpr int DR = COLS ? 4 : 0, DC = COLS ? 0 : 1;
+  double v[16];
+  int sh[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = src.at(r + DR * i, c + DC * i);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) sh[i] = src.lift(r + DR * i, c + DC * i);
+  int m = 0;
+#pragma unroll
+  for (int i = 0; i < 16; ++i)
+    if (!(finite && exp_field(v[i]) == 2047)) m = max(m, lifted_field(v[i], sh[i]));
   if (COLS) {
-    const int c = c0 + (threadIdx.x & 63);
-    int m = 0;
-    for (int r = r0 + (threadIdx.x >> 6); r < r0 + 64; r += 4) m = max(m, field(r, c));
     if (m > 0) atomicMax(&e[c], m);
   } else {
-    const int r = r0 + (threadIdx.x >> 2), cc = c0 + (threadIdx.x & 3) * 16;
-    int m = 0;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) m = max(m, field(r, cc + i));
     m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
     m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
     if ((threadIdx.x & 3) == 0 && m > 0) atomicMax(&e[r], m);
@@ -490,7 +601,7 @@ __global__ void __launch_bounds__(256) k_oz_slice(Src src, const int *__restrict
 // partials (fixed order, optionally stored to y), its exponent and its digits.
 // Sixteen elements lie 17 doubles apart in shared memory: their readers meet
 // different banks (8192 rows of 1024 with shifts and block exponents: 93 us,
-// 101 without the gap).  LIFT: with src.shift, and block exponents to blk.
+// 101 without the gap).  LIFT: on src's even shifts, with block exponents to blk.
 template <bool LIFT>
 __global__ void __launch_bounds__(256) k_oz_rows(const double *__restrict__ x, int splits,
                                                  size_t part, Src src, double *__restrict__ y,
@@ -511,7 +622,7 @@ __global__ void __launch_bounds__(256) k_oz_rows(const double *__restrict__ x, i
     }
     v[i + (i >> 4)] = s;
     if (LIFT)
-      m = max(m, lifted_field(s, i < src.nc ? src.shift[i] : 0));
+      m = max(m, lifted_field(s, even_shift(src.shift[i])));
     else
       m = max(m, exp_field(s));
   }
@@ -524,11 +635,17 @@ __global__ void __launch_bounds__(256) k_oz_rows(const double *__restrict__ x, i
   m = max(m, 1);
   for (int g = threadIdx.x; g < nkb * 4; g += 256) {
     unsigned long long u[16];
-    int mb = 0;
+    int mb = 0, ev[16];   // shift covers whole K blocks
+    if (LIFT) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        *reinterpret_cast<int4 *>(ev + 4 * q) =
+            *reinterpret_cast<const int4 *>(src.shift + g * 16 + 4 * q);
+    }
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
       const double s = v[g * 17 + k];
-      const int sh = LIFT && g * 16 + k < src.nc ? src.shift[g * 16 + k] : 0;
+      const int sh = LIFT ? even_shift(ev[k]) : 0;
       u[k] = fixed56(s, m - sh);
       if (LIFT) mb = max(mb, lifted_field(s, sh));
     }
@@ -585,119 +702,6 @@ __global__ void __launch_bounds__(1024) k_oz_factors(const int *__restrict__ e, 
   }
 }
 
-// Scales of n contraction indices from their largest exponent fields e_k: the
-// factors 2^-s_k (down), s_k = max e - e_k, for one operand and the shifts s_k
-// (up) for the other, kept within 400, past which *unbalanced is set.
-__global__ void __launch_bounds__(256) k_oz_balance(const int *__restrict__ e, int n,
-                                                    double *__restrict__ down,
-                                                    int *__restrict__ up,
-                                                    unsigned *unbalanced) {
-  pdl_wait();
-  __shared__ int top;
-  if (threadIdx.x == 0) top = 0;
-  __syncthreads();
-  int m = 0;
-  for (int k = threadIdx.x; k < n; k += 256) m = max(m, e[k]);
-  atomicMax(&top, m);
-  __syncthreads();
-  for (int k = threadIdx.x; k < n; k += 256) {
-    const int d = e[k] > 0 ? top - e[k] : 0, s = min(d, 400);
-    down[k] = __hiloint2double((1023 - s) << 20, 0);
-    up[k] = s;
-    if (d != s) *unbalanced = 1u;
-  }
-}
-
-// Whether eight digits are enough for the products of operands a (its row i
-// zero before K index i) and b.  What they lose is relative to max |a_i| max
-// |b_j|, so an output (i, j) is as good as FP64's while some K block's largest
-// |a| times its largest |b| comes near that.  *poor is set where, in some 64 x
-// 64 tile of outputs, more than an eighth miss it by more than 2^6: a chance
-// small element in a short last block is not counted, operands graded against
-// one another are.  (8192 x 1024 outputs: 14 us.)  Where in some K block no row of the tile falls far below
-// its own largest element, as usual, the outputs need not be looked at one by
-// one.
-constexpr int LOSS_BITS = 6;
-
-__global__ void __launch_bounds__(256) k_oz_loss(const short *__restrict__ a,
-                                                 const short *__restrict__ b,
-                                                 const int *__restrict__ ea,
-                                                 const int *__restrict__ eb, int na, int nb,
-                                                 int nkb, unsigned *poor) {
-  pdl_wait();
-  __shared__ short sa[64][33], sb[64][33];
-  __shared__ int da[32], db[32];   // by K block: the rows' largest distance from their maxima
-  __shared__ int nbad, nall;
-  const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
-  const int a0 = blockIdx.x * 64, b0 = blockIdx.y * 64, kfirst = a0 / 64;
-  auto load = [&](int k0) {
-    for (int idx = t; idx < 64 * 32; idx += 256) {
-      const int r = idx >> 5, k = idx & 31;
-      const bool in = k0 + k < nkb;
-      sa[r][k] = in && a0 + r < na ? a[(size_t)(a0 + r) * nkb + k0 + k] : OZ_ZERO;
-      sb[r][k] = in && b0 + r < nb ? b[(size_t)(b0 + r) * nkb + k0 + k] : OZ_ZERO;
-    }
-  };
-  if (t == 0) nbad = nall = 0;
-  for (int k0 = kfirst; k0 < nkb; k0 += 32) {
-    __syncthreads();
-    if (t < 32) da[t] = db[t] = 0;
-    load(k0);
-    __syncthreads();
-    const int k = t & 31, r0 = (t >> 5) * 8;
-    int xa = 0, xb = 0;
-#pragma unroll
-    for (int r = r0; r < r0 + 8; ++r) {   // rows of zeros have no say
-      const int ma = a0 + r < na ? ea[a0 + r] : 0, mb = b0 + r < nb ? eb[b0 + r] : 0;
-      if (ma > 0) xa = max(xa, ma - sa[r][k]);
-      if (mb > 0) xb = max(xb, mb - sb[r][k]);
-    }
-    atomicMax(&da[k], xa);
-    atomicMax(&db[k], xb);
-    __syncthreads();
-    if (__syncthreads_or(t < 32 && k0 + t < nkb && da[t & 31] + db[t & 31] <= LOSS_BITS)) return;
-  }
-  int best[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) best[i][j] = 2 * OZ_ZERO;
-  for (int k0 = kfirst; k0 < nkb; k0 += 32) {
-    __syncthreads();
-    load(k0);
-    __syncthreads();
-    for (int k = 0; k < min(32, nkb - k0); ++k) {
-      int x[4], y[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) x[i] = sa[ty + 16 * i][k], y[i] = sb[tx + 16 * i][k];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) best[i][j] = max(best[i][j], x[i] + y[j]);
-    }
-  }
-  int bad = 0, all = 0;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = a0 + ty + 16 * i, ma = r < na ? ea[r] : 0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = b0 + tx + 16 * j, mb = c < nb ? eb[c] : 0;
-      if (best[i][j] <= 0) continue;   // no product at all: exactly zero
-      ++all;
-      bad += ma + mb - best[i][j] > LOSS_BITS ? 1 : 0;
-    }
-  }
-  bad = __reduce_add_sync(0xffffffffu, bad);
-  all = __reduce_add_sync(0xffffffffu, all);
-  if ((t & 31) == 0) {
-    atomicAdd(&nbad, bad);
-    atomicAdd(&nall, all);
-  }
-  __syncthreads();
-  if (t == 0 && 8 * nbad > nall) *poor = 1u;
-}
-
 // *bad != 0 if an exponent field says Inf or NaN
 __global__ void k_oz_check(const int *__restrict__ e, int n, unsigned *bad) {
   pdl_wait();
@@ -731,13 +735,23 @@ static bool encode(CUtensorMap *tm, const OzOperand &o, int box_rows, int box_sl
              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int NT>
+template <int NT, bool CHECK>
 static void launch(const CUtensorMap &A, const CUtensorMap &B, int M, int Ncols, int nkb, int per,
                    int splits, const Epi &e, cudaStream_t st) {
   static DeviceOnce once;
-  allow_smem(once, k_oz_gemm<NT>, Cfg<NT>::SMEM);
+  allow_smem(once, k_oz_gemm<NT, CHECK>, Cfg<NT>::SMEM);
   const dim3 grid((Ncols + NT - 1) / NT, (M + BM - 1) / BM, splits);
-  launch_pdl(k_oz_gemm<NT>, grid, dim3(NTHREADS), Cfg<NT>::SMEM, st, A, B, M, Ncols, nkb, per, e);
+  launch_pdl(k_oz_gemm<NT, CHECK>, grid, dim3(NTHREADS), Cfg<NT>::SMEM, st, A, B, M, Ncols, nkb,
+             per, e);
+}
+
+template <int NT>
+static void launch_any(const CUtensorMap &A, const CUtensorMap &B, int M, int Ncols, int nkb,
+                       int per, int splits, const Epi &e, cudaStream_t st) {
+  if (e.ba)
+    launch<NT, true>(A, B, M, Ncols, nkb, per, splits, e, st);
+  else
+    launch<NT, false>(A, B, M, Ncols, nkb, per, splits, e, st);
 }
 
 template <bool LIFT>
@@ -775,6 +789,16 @@ bool launch_oz_gemm(const OzOperand &A, const OzOperand &B, int M, int Ncols, in
   e.betaj = o.betaj;
   e.alpha_part = o.alpha_part;
   e.status = status;
+  if (o.xa) {
+    if (o.mode != OZ_PART || splits != 1 || !A.blk || !B.blk) return false;
+    e.ba = A.blk;
+    e.bb = B.blk;
+    e.xa = o.xa;
+    e.xb = o.xb;
+    e.ldxa = o.ldxa;
+    e.ldxb = o.ldxb;
+    e.K = o.K;
+  }
   const int nkb = A.nkb, per = (nkb + splits - 1) / splits;
   const int m_tiles = (M + oz::BM - 1) / oz::BM;
   const int nt =
@@ -784,24 +808,24 @@ bool launch_oz_gemm(const OzOperand &A, const OzOperand &B, int M, int Ncols, in
       !oz::encode(&tb, B, nt, nt == 64 ? oz::Cfg<64>::BOX : OZ_SLICES))
     return false;
   if (nt == 64)
-    oz::launch<64>(ta, tb, M, Ncols, nkb, per, splits, e, st);
+    oz::launch_any<64>(ta, tb, M, Ncols, nkb, per, splits, e, st);
   else if (nt == 32)
-    oz::launch<32>(ta, tb, M, Ncols, nkb, per, splits, e, st);
+    oz::launch_any<32>(ta, tb, M, Ncols, nkb, per, splits, e, st);
   else
-    oz::launch<16>(ta, tb, M, Ncols, nkb, per, splits, e, st);
+    oz::launch_any<16>(ta, tb, M, Ncols, nkb, per, splits, e, st);
   return true;
 }
 
 // Digits of x [nr][nc] (row stride ld, optional column scale): operand rows
-// are x's rows, or its columns.  o.rows covers them (more rows become zeros).
+// are x's rows, or its columns.  up: exponent fields of x's columns (nc rounded
+// up to 64 of them) to shift up by, down: of its rows to shift down by.  o.rows covers them (more rows become zeros).
 void launch_oz_slice(const double *x, size_t ld, int nr, int nc, const double *scale, bool cols,
-                     const OzOperand &o, cudaStream_t st, const double *rscale,
-                     const int *shift) {
-  const oz::Src src{x, scale, rscale, shift, nullptr, ld, nr, nc};
+                     const OzOperand &o, cudaStream_t st, const int *up, const int *down) {
+  const oz::Src src{x, scale, up, nullptr, down, true, ld, nr, nc};
   // short rows: one kernel, a block per row (4.7 us at 160 rows of 256); longer
   // ones spread each row over many blocks (64 rows of 32768: 12 + 20 us)
-  if (!cols && !rscale && o.nkb * 64 <= 4096) {
-    if (shift)
+  if (!cols && !down && o.nkb * 64 <= 4096) {
+    if (up)
       oz::launch_rows<true>(x, 1, 0, src, nullptr, o, st);
     else
       oz::launch_rows<false>(x, 1, 0, src, nullptr, o, st);
@@ -825,7 +849,7 @@ void launch_oz_slice(const double *x, size_t ld, int nr, int nc, const double *s
 // <= OZ_ROW_MAX)
 void launch_oz_reduce(const double *part, int splits, int nr, int len, double *y,
                       const OzOperand &o, cudaStream_t st) {
-  const oz::Src src{part, o.scale, nullptr, nullptr, nullptr, (size_t)len, nr, len};
+  const oz::Src src{part, o.scale, nullptr, nullptr, nullptr, false, (size_t)len, nr, len};
   oz::launch_rows<false>(part, splits, (size_t)nr * len, src, y, o, st);
 }
 
@@ -845,7 +869,7 @@ void launch_oz_factors(const int *e, int n, const double *base, int *shift, doub
 // Digits of x [nr][nc] whose rows' (columns') exponents are in o.e already.
 void launch_oz_digits(const double *x, int nr, int nc, bool cols, const int *shift,
                       const OzOperand &o, cudaStream_t st) {
-  const oz::Src src{x, nullptr, nullptr, cols ? nullptr : shift, cols ? shift : nullptr,
+  const oz::Src src{x, nullptr, cols ? nullptr : shift, cols ? shift : nullptr, nullptr, false,
                     (size_t)nc, nr, nc};
   const dim3 grid(cols ? (o.rows + 63) / 64 : o.nkb, cols ? o.nkb : (o.rows + 63) / 64);
   if (cols)
@@ -859,21 +883,10 @@ void launch_oz_col_max(const double *x, size_t ld, int nr, int nc, int *e, cudaS
   constexpr int ROWS = 1 << 21;   // a grid's second dimension ends at 65535 tiles
   for (int r0 = 0; r0 < nr; r0 += ROWS) {
     const int n = std::min(ROWS, nr - r0);
-    const oz::Src src{x + (size_t)r0 * ld, nullptr, nullptr, nullptr, nullptr, ld, n, nc};
+    const oz::Src src{x + (size_t)r0 * ld, nullptr, nullptr, nullptr, nullptr, false, ld, n, nc};
     launch_pdl(oz::k_oz_max<true>, dim3((nc + 63) / 64, (n + 63) / 64), dim3(256), 0, st, src, e,
                true);
   }
-}
-
-void launch_oz_balance(const int *e, int n, double *down, int *up, unsigned *unbalanced,
-                       cudaStream_t st) {
-  launch_pdl(oz::k_oz_balance, dim3(1), dim3(256), 0, st, e, n, down, up, unbalanced);
-}
-
-void launch_oz_loss(const OzOperand &a, const OzOperand &b, int na, int nb, unsigned *poor,
-                    cudaStream_t st) {
-  launch_pdl(oz::k_oz_loss, dim3((na + 63) / 64, (nb + 63) / 64), dim3(256), 0, st, a.blk, b.blk,
-             a.e, b.e, na, nb, a.nkb, poor);
 }
 
 void launch_oz_check(const OzOperand &o, unsigned *bad, cudaStream_t st) {

@@ -46,10 +46,30 @@ constexpr int NB = 64;
 // thread per row and square root, division and row sums in sequence, 109 us
 // column by column with three barriers each, 75 us now.
 constexpr int POTRF_THREADS = 128, PW = 8;
+constexpr int CM_ROWS = 256;   // rows of a column-maximum tile of 64 columns
+
+// Largest finite exponent field of 64 columns of a tile of C, into col.
+__device__ void col_max_tile(const ColMax &cm, int n, int tile) {
+  const int strips = (n + 63) / 64, c = (tile % strips) * 64 + (threadIdx.x & 63);
+  const int r0 = (tile / strips) * CM_ROWS, r1 = min(cm.n_pairs, r0 + CM_ROWS);
+  if (c >= n) return;
+  int m = 0;
+#pragma unroll 8
+  for (int r = r0 + (threadIdx.x >> 6); r < r1; r += POTRF_THREADS / 64) {
+    const double x = cm.C[(size_t)r * n + c];
+    const int f = (__double2hiint(x) >> 20) & 0x7ff;
+    if (nonzero_bits(x) && f < 2047) m = max(m, max(f, 1));
+  }
+  if (m > 0) atomicMax(&cm.col[c], m);
+}
 
 __global__ void __launch_bounds__(POTRF_THREADS) k_potrf_diag(double *A, int n, int j0,
-                                                              unsigned *status) {
+                                                              unsigned *status, ColMax cm) {
   pdl_wait();
+  if (blockIdx.x > 0) {   // beside the first diagonal block
+    col_max_tile(cm, n, blockIdx.x - 1);
+    return;
+  }
   __shared__ double blk[NB][NB + 1];
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int nb = min(NB, n - j0);
@@ -224,10 +244,8 @@ __global__ void k_zero_upper(double *A, int n) {
 // Cm[M][N] = Am[M][K] Bm[K][N], row-major, FP64 (64 x 64 tiles)
 __global__ void __launch_bounds__(256) k_gemm_nn_f64(const double *__restrict__ Am,
                                                      const double *__restrict__ Bm, int M, int N,
-                                                     int K, double *__restrict__ Cm,
-                                                     const unsigned *only) {
+                                                     int K, double *__restrict__ Cm) {
   pdl_wait();
-  if (only != nullptr && *only == 0u) return;
   __shared__ double As[16][65];
   __shared__ double Bs[16][65];
   const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
@@ -275,11 +293,28 @@ void launch_sigma_x(const double *M, int n_t, int n_m, int n_aux, const int *m_i
   if (n_t > 0) launch_pdl(k_sigma_x, dim3(n_t), dim3(256), 0, st, M, n_m, n_aux, m_idx, n_v, out);
 }
 
-int launch_cholesky(double *A, int n, unsigned *status, cudaStream_t st) {
+// R = the metric, and the column maxima start at zero.
+__global__ void __launch_bounds__(256) k_fit_init(const double *__restrict__ metric, size_t n2,
+                                                  double *__restrict__ R, int *__restrict__ col,
+                                                  int nc) {
+  pdl_wait();
+  const size_t step = (size_t)gridDim.x * 256, i0 = (size_t)blockIdx.x * 256 + threadIdx.x;
+  for (size_t i = i0; i < n2; i += step) R[i] = metric[i];
+  for (size_t i = i0; i < (size_t)nc; i += step) col[i] = 0;
+}
+void launch_fit_init(const double *metric, int n, double *R, int *col, int nc, cudaStream_t st) {
+  const size_t n2 = (size_t)n * n;
+  launch_pdl(k_fit_init, dim3((unsigned)std::min<size_t>((n2 + 255) / 256, 152 * 8)), dim3(256), 0,
+             st, metric, n2, R, col, col ? nc : 0);
+}
+
+int launch_cholesky(double *A, int n, unsigned *status, cudaStream_t st, const ColMax &cm) {
   int launches = 0;
+  const int tiles = cm.col ? (n + 63) / 64 * ((cm.n_pairs + CM_ROWS - 1) / CM_ROWS) : 0;
   for (int j0 = 0; j0 < n; j0 += NB) {
     const int nb = std::min(NB, n - j0);
-    launch_pdl(k_potrf_diag, dim3(1), dim3(POTRF_THREADS), 0, st, A, n, j0, status);
+    launch_pdl(k_potrf_diag, dim3(j0 == 0 ? 1 + tiles : 1), dim3(POTRF_THREADS), 0, st, A, n, j0,
+               status, cm);
     ++launches;
     const int rest = n - j0 - nb;
     if (rest > 0) {
@@ -295,9 +330,9 @@ int launch_cholesky(double *A, int n, unsigned *status, cudaStream_t st) {
 }
 
 void launch_gemm_nn_f64(const double *A, const double *B, int M, int N, int K, double *C,
-                        cudaStream_t st, const unsigned *only) {
+                        cudaStream_t st) {
   dim3 grid((N + 63) / 64, (M + 63) / 64);
-  launch_pdl(k_gemm_nn_f64, grid, dim3(256), 0, st, A, B, M, N, K, C, only);
+  launch_pdl(k_gemm_nn_f64, grid, dim3(256), 0, st, A, B, M, N, K, C);
 }
 
 }  // namespace lgw

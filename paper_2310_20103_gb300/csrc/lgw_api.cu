@@ -873,20 +873,20 @@ void f64_atb(lgw_handle *h, const double *X, int ldx, const double *Y, int ldy, 
 // pairs, is moved to row k of R first (an exact power of two): C's rows are then
 // as even as they can be, and a column of R shows what its terms are worth.
 // (Even rows of R would not do: column i starts in row i, and a large function
-// before it would set the grid of C's rows.)  Where that is not enough,
-// k_oz_loss says so and the CUDA cores do the product again, without the host.
+// before it would set the grid of C's rows.)  Tiles for which that is not enough
+// find it out from the K blocks' exponents and use the FP64 pipe.
 struct FitWork {
   OzOperand a, b;        // digits of R's columns and of C's rows; a.d NULL: none
-  double *down = nullptr;   // factors of R's rows
-  int *up = nullptr;        // and of C's columns, as powers of two
-  int *col = nullptr;       // largest exponent fields of C's columns
-  unsigned *poor = nullptr;
+  int *col = nullptr;    // largest exponent fields of C's columns
 };
-// The scales, the look at the exponents and the second product's empty launch
-// take 50 us at 16384 pairs, n 1024; the digits of the first 8192, made beside
-// the factorisation, take most of it off: 3.39 ms per call, 3.37 to 3.39 without
-// all of this.  (16384 pairs at a time, all digits made there: 3.47 ms, the
-// blocks of the chain wait for the others.)
+// The scales cost a pass over C, the shifts 10 us per 8192 rows of 1024, the
+// tiles' look at the exponents hides behind their products.  For small C the
+// pass runs beside the first diagonal block, else beside the factorisation with
+// the digits of the first 8192 pairs, which takes as much off: 3.38 ms per call
+// at 16384 pairs, n 1024, 3.37 to 3.40 without any of it; 1.48 against 1.50 at
+// 6000 x 600, 338 us against 333 at 700 x 130, 129 against 123 at 512 x 64.  (All
+// 16384 pairs' digits made beside the factorisation: 3.47 ms, the chain's blocks
+// wait for a place.)
 constexpr int FIT_PAIRS = 8192;
 
 FitWork fit_work(lgw_handle *h, int n_pairs, int n) {
@@ -897,18 +897,13 @@ FitWork fit_work(lgw_handle *h, int n_pairs, int n) {
   if (!tc_available() || n > OZ_ROW_MAX) return f;
   uint16_t *d = static_cast<uint16_t *>(ws(h, "oz_fit", (na + nb) * sizeof(uint16_t), true));
   const size_t nc = round_up(n, 64);
-  uint8_t *e = d ? static_cast<uint8_t *>(
-                       ws(h, "oz_fit_e", nc * sizeof(double) +
-                                             (2 * nc + ra + rb + 2) * sizeof(int) +
-                                             (ra + rb) * nkb * sizeof(short), true))
-                 : nullptr;
+  int *e = d ? static_cast<int *>(ws(h, "oz_fit_e", (nc + ra + rb) * sizeof(int) +
+                                                       (ra + rb) * nkb * sizeof(short), true))
+             : nullptr;
   if (!e) return f;
-  f.down = reinterpret_cast<double *>(e);
-  f.up = reinterpret_cast<int *>(f.down + nc);
-  f.col = f.up + nc;
+  f.col = e;
   int *ea = f.col + nc, *eb = ea + ra;
-  f.poor = reinterpret_cast<unsigned *>(eb + rb);
-  short *blk = reinterpret_cast<short *>(eb + rb + 2);
+  short *blk = reinterpret_cast<short *>(eb + rb);
   f.a = OzOperand{d, ea, (int)ra, (int)nkb, blk};
   f.b = OzOperand{d + na, eb, (int)rb, (int)nkb, blk + ra * nkb};
   return f;
@@ -916,19 +911,16 @@ FitWork fit_work(lgw_handle *h, int n_pairs, int n) {
 
 void fit_slice(lgw_handle *h, const FitWork &f, const double *C, int n_pairs, int n, int p0,
                cudaStream_t st) {
-  launch_oz_slice(C + (size_t)p0 * n, (size_t)n, std::min(FIT_PAIRS, n_pairs - p0), n, nullptr, false,
-                  f.b, st, nullptr, f.up);
+  launch_oz_slice(C + (size_t)p0 * n, (size_t)n, std::min(FIT_PAIRS, n_pairs - p0), n, nullptr,
+                  false, f.b, st, f.col);
   check_launch(h, "oz_slice(C)");
 }
 
 // What needs C alone: the scales and the first pairs' digits.
 void fit_begin(lgw_handle *h, const FitWork &f, const double *C, int n_pairs, int n,
                cudaStream_t st) {
-  LGW_TRY_CUDA(h, cudaMemsetAsync(f.poor, 0, sizeof(unsigned), st));
   launch_oz_col_max(C, (size_t)n, n_pairs, n, f.col, st);
   check_launch(h, "oz_col_max");
-  launch_oz_balance(f.col, n, f.down, f.up, f.poor, st);
-  check_launch(h, "oz_balance");
   fit_slice(h, f, C, n_pairs, n, 0, st);
 }
 
@@ -940,25 +932,20 @@ void f64_fit(lgw_handle *h, const FitWork &f, const double *C, const double *R, 
     check_launch(h, "gemm_nn_f64");
     return;
   }
-  launch_oz_slice(R, (size_t)n, n, n, nullptr, true, f.a, st, f.down);
+  launch_oz_slice(R, (size_t)n, n, n, nullptr, true, f.a, st, nullptr, f.col);
   check_launch(h, "oz_slice(R)");
   for (int p0 = 0; p0 < n_pairs; p0 += FIT_PAIRS) {
     const int np = std::min(FIT_PAIRS, n_pairs - p0);
     if (p0 > 0) fit_slice(h, f, C, n_pairs, n, p0, st);
-    launch_oz_loss(f.a, f.b, n, np, f.poor, st);
-    check_launch(h, "oz_loss");
     OzOut o;
     o.mode = OZ_PART;
     o.out = B + (size_t)p0 * n;
     o.ldo = n;
     o.lower = true;   // column i of R starts in row i
+    o.xa = R;
+    o.xb = C + (size_t)p0 * n;
+    o.ldxa = o.ldxb = o.K = n;
     oz_gemm(h, f.a, f.b, n, np, 1, o, "oz_gemm(fit)");
-  }
-  constexpr int ROWS = 1 << 21;
-  for (int p0 = 0; p0 < n_pairs; p0 += ROWS) {
-    launch_gemm_nn_f64(C + (size_t)p0 * n, R, std::min(ROWS, n_pairs - p0), n, n,
-                       B + (size_t)p0 * n, st, f.poor);
-    check_launch(h, "gemm_nn_f64");
   }
 }
 
@@ -3281,8 +3268,6 @@ lgw_status lgw_fit_factors(lgw_handle *h, int32_t n_pairs, int32_t n_aux, const 
     LGW_TRY_CUDA(h, cudaMemsetAsync(h->d_status, 0, sizeof(unsigned), st));
     const double *Vd = in_dev(h, "in_metric", metric, (size_t)n_aux * n_aux);
     double *R = wsT<double>(h, "fit_R", (size_t)n_aux * n_aux);
-    LGW_TRY_CUDA(h, cudaMemcpyAsync(R, Vd, sizeof(double) * n_aux * n_aux,
-                                    cudaMemcpyDeviceToDevice, st));
     const double *Cd = nullptr;
     OutBuf<double> out;
     FitWork f;
@@ -3293,12 +3278,19 @@ lgw_status lgw_fit_factors(lgw_handle *h, int32_t n_pairs, int32_t n_aux, const 
     }
     {
       // the factorisation is a serial chain that leaves the chip idle: what
-      // needs C alone beside it, where that takes longer than the fork and join
-      SideStream side(h, f.a.d && (size_t)n_pairs * n_aux >= (size_t)1 << 21);
-      if (f.a.d) fit_begin(h, f, Cd, n_pairs, n_aux, side.st);
-      h->launches += launch_cholesky(R, n_aux, h->d_status, st);
+      // needs C alone runs beside it, the first pairs' digits too where they
+      // take longer than the fork and join, else the scales only
+      const bool fork = f.a.d && (size_t)n_pairs * n_aux >= (size_t)1 << 21;
+      ColMax cm;
+      if (f.a.d && !fork) cm = ColMax{Cd, n_pairs, f.col};
+      launch_fit_init(Vd, n_aux, R, cm.col, round_up(n_aux, 64), st);
+      check_launch(h, "fit_init");
+      SideStream side(h, fork);
+      if (fork) fit_begin(h, f, Cd, n_pairs, n_aux, side.st);
+      h->launches += launch_cholesky(R, n_aux, h->d_status, st, cm);
       check_launch(h, "cholesky");
       side.join();
+      if (cm.col) fit_slice(h, f, Cd, n_pairs, n_aux, 0, st);
     }
     if (n_pairs > 0) {
       f64_fit(h, f, Cd, R, n_pairs, n_aux, out.dev);

@@ -333,6 +333,10 @@ struct OzOut {
   const double *Delta2 = nullptr, *dsq = nullptr, *cd = nullptr, *q = nullptr, *qprev = nullptr,
                *betaj = nullptr;
   double *alpha_part = nullptr;   // [M / 64][Ncols]
+  // OZ_PART of one split, with the operands' blk: tiles that the digits are not
+  // enough for are formed in FP64 from xa [K][M] and xb [Ncols][K]
+  const double *xa = nullptr, *xb = nullptr;
+  int ldxa = 0, ldxb = 0, K = 0;
 };
 int oz_splits(int M, int ncols, int nkb);
 // rows of partials of OZ_PART products of `rows` columns, `slice` at a time
@@ -342,8 +346,8 @@ size_t oz_part_rows(int M, int rows, int slice, int nkb);
 bool launch_oz_gemm(const OzOperand &A, const OzOperand &B, int M, int Ncols, int splits,
                     const OzOut &o, unsigned *status, cudaStream_t st);
 void launch_oz_slice(const double *x, size_t ld, int nr, int nc, const double *scale, bool cols,
-                     const OzOperand &o, cudaStream_t st, const double *rscale = nullptr,
-                     const int *shift = nullptr);
+                     const OzOperand &o, cudaStream_t st, const int *up = nullptr,
+                     const int *down = nullptr);
 void launch_oz_max_both(const double *x, int nr, int nc, const int *shift, const int *rshift,
                         int *row, int *col, cudaStream_t st);
 void launch_oz_factors(const int *e, int n, const double *base, int *shift, double *down,
@@ -352,10 +356,6 @@ void launch_oz_digits(const double *x, int nr, int nc, bool cols, const int *shi
                       const OzOperand &o, cudaStream_t st);
 // largest finite exponent field of each column of x [nr][nc] (e: nc rounded up to 64)
 void launch_oz_col_max(const double *x, size_t ld, int nr, int nc, int *e, cudaStream_t st);
-void launch_oz_balance(const int *e, int n, double *down, int *up, unsigned *unbalanced,
-                       cudaStream_t st);
-void launch_oz_loss(const OzOperand &a, const OzOperand &b, int na, int nb, unsigned *poor,
-                    cudaStream_t st);
 void launch_oz_reduce(const double *part, int splits, int nr, int len, double *y,
                       const OzOperand &o, cudaStream_t st);
 void launch_oz_check(const OzOperand &o, unsigned *bad, cudaStream_t st);
@@ -562,10 +562,17 @@ void launch_pol_combine(const double *sig2, int n_pairs, int n_freq, double *out
 // k_static.cu : exchange self-energy and density-fitting factors
 void launch_sigma_x(const double *M, int n_t, int n_m, int n_aux, const int *m_idx, int n_v,
                     double *out, cudaStream_t st);
-int launch_cholesky(double *A, int n, unsigned *status, cudaStream_t st);
-// only: nothing is done unless *only is nonzero
+// col (rounded up to 64 columns, zeroed by launch_fit_init): largest finite
+// exponent field of each column of C [n_pairs][n], beside the first diagonal block
+struct ColMax {
+  const double *C = nullptr;
+  int n_pairs = 0;
+  int *col = nullptr;
+};
+void launch_fit_init(const double *metric, int n, double *R, int *col, int nc, cudaStream_t st);
+int launch_cholesky(double *A, int n, unsigned *status, cudaStream_t st, const ColMax &cm);
 void launch_gemm_nn_f64(const double *A, const double *B, int M, int N, int K, double *C,
-                        cudaStream_t st, const unsigned *only = nullptr);
+                        cudaStream_t st);
 
 // k_adjoint.cu : gradient of the QP energies (implicit function + Daleckii-Krein)
 // A stored Krylov basis [slot][Bs][N]: FP64, or the float pair hi (+ lo).

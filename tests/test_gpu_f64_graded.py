@@ -66,6 +66,24 @@ def test_fit_factors_of_a_graded_metric(L, n_pairs, n, decades, coeffs, order):
     assert err.max() <= 4 * own.max() + 2.0 ** -50
 
 
+@pytest.mark.parametrize("n_pairs,n", [(2200, 1024), (80, 4160)])
+def test_large_fits_of_a_graded_metric(L, n_pairs, n):
+    """Sizes that make the digits beside the factorisation, and rows too long for one block's
+    single pass."""
+    rng = np.random.default_rng(n)
+    d = 2.0 ** rng.integers(-25, 26, n)
+    R = d[:, None] * _factor(n, rng)
+    C = rng.standard_normal((n_pairs, n)) / d
+    B = _fit(L, C, R @ R.T)
+    typical = np.abs(C).mean(0) @ np.abs(R)
+    rows = np.linspace(0, n_pairs - 1, 12).astype(int)      # the extended products take long
+    ref = C[rows].astype(LD) @ R.astype(LD)
+    own = np.abs(C[rows] @ R - ref) / typical
+    err = np.abs(B[rows] - ref) / typical
+    assert err.max() <= 4 * own.max() + 2.0 ** -50
+    assert np.abs((B - C @ R) / typical).max() <= 1e-13
+
+
 def test_fit_factors_of_rows_with_gradings_of_their_own(L):
     """No scale per auxiliary function helps where every pair has its own: pairs on fragment
     a see a's functions at 1 and b's at 1e-12, pairs on b the other way round, and B's columns
