@@ -68,7 +68,10 @@ typedef enum {
   LGW_FP64 = 0,   /* FP64 products: the plain FP64 path (on the tensor cores
                      by error-free slicing where the digits of L, 32 bytes
                      per element, fit a third of the free device memory,
-                     else on the CUDA cores)                               */
+                     else on the CUDA cores).  The digits' errors, 2^-56
+                     each, are relative to the largest of the terms of a sum
+                     once the scales of L's rows and columns are evened out,
+                     the CUDA cores' to each term                          */
   LGW_BF16 = 1,   /* BF16 tcgen05 tensor-core GEMMs, FP32 accumulate      */
   LGW_FP8 = 3,    /* E4M3 tcgen05 GEMMs (kind::f8f6f4), FP32 accumulate:
                      L with one power-of-two scale per column (max -> (224,

@@ -830,7 +830,10 @@ void f64_contract2(lgw_handle *h, const SysDev &s, const F64Work &f, const doubl
 }
 
 // S [Ni][Nmu] += scale * X^T Y over R rows (X row stride ldx, Y row stride
-// ldy), 1024 rows at a time on the tensor cores.
+// ldy), 1024 rows at a time on the tensor cores.  Rows need no balance here: of
+// the pairs (X, Y) one holds unit vectors, bounded polynomials of C on them or
+// images of those under L, or (Y, M) both scale with the vector's weight, so a
+// row that is small in one factor is small in the sum.
 void f64_atb(lgw_handle *h, const double *X, int ldx, const double *Y, int ldy, int R, int Ni,
              int Nmu, double *S, double scale = 1.0) {
   cudaStream_t st = h->stream;
