@@ -531,8 +531,9 @@ __device__ __forceinline__ int lifted_field(double x, int sh) {
 
 // Largest exponent field of each operand row: the operand's rows are the
 // matrix's rows (COLS = false, contraction along c) or its columns.  finite:
-// Inf and NaN do not count.
-template <bool COLS>
+// Inf and NaN do not count.  LIFT: with src's shifts (the vectors of every step
+// have none: 12 us for 64 of 32768 elements, 17 with the questions for them).
+template <bool COLS, bool LIFT>
 __global__ void __launch_bounds__(256) k_oz_max(Src src, int *__restrict__ e, bool finite) {
   pdl_wait();
   const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
@@ -544,11 +545,13 @@ __global__ void __launch_bounds__(256) k_oz_max(Src src, int *__restrict__ e, bo
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = src.at(r + DR * i, c + DC * i);
 #pragma unroll
-  for (int i = 0; i < 16; ++i) sh[i] = src.lift(r + DR * i, c + DC * i);
+  for (int i = 0; i < 16; ++i) sh[i] = LIFT ? src.lift(r + DR * i, c + DC * i) : 0;
   int m = 0;
 #pragma unroll
-  for (int i = 0; i < 16; ++i)
-    if (!(finite && exp_field(v[i]) == 2047)) m = max(m, lifted_field(v[i], sh[i]));
+  for (int i = 0; i < 16; ++i) {
+    const int f = LIFT ? lifted_field(v[i], sh[i]) : exp_field(v[i]);
+    if (!(finite && exp_field(v[i]) == 2047)) m = max(m, f);
+  }
   if (COLS) {
     if (m > 0) atomicMax(&e[c], m);
   } else {
@@ -568,7 +571,8 @@ __device__ __forceinline__ void store_block_exp(int m, int part, short *blk) {
 }
 
 // Digits of a 64 x 64 tile; the operand has `rows` rows and nkb K blocks.
-template <bool COLS>
+// LIFT: with src's shifts and, where asked for, block exponents.
+template <bool COLS, bool LIFT>
 __global__ void __launch_bounds__(256) k_oz_slice(Src src, const int *__restrict__ e,
                                                   uint16_t *__restrict__ out, int rows, int nkb,
                                                   short *__restrict__ blk) {
@@ -589,11 +593,11 @@ __global__ void __launch_bounds__(256) k_oz_slice(Src src, const int *__restrict
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
     const double x = COLS ? tile[k0 + k][i] : src.at(row, c0 + k0 + k);
-    const int sh = COLS ? src.lift(r0 + k0 + k, row) : src.lift(row, c0 + k0 + k);
+    const int sh = !LIFT ? 0 : COLS ? src.lift(r0 + k0 + k, row) : src.lift(row, c0 + k0 + k);
     u[k] = fixed56(x, f - sh);
-    if (blk) m = max(m, lifted_field(x, sh));
+    if (LIFT) m = max(m, lifted_field(x, sh));
   }
-  if (blk) store_block_exp(m, threadIdx.x & 3, blk + (size_t)row * nkb + kb);
+  if (LIFT && blk) store_block_exp(m, threadIdx.x & 3, blk + (size_t)row * nkb + kb);
   store_digits16(u, out + ((size_t)kb * rows + row) * 64 + k0, (size_t)nkb * rows * 64);
 }
 
@@ -676,37 +680,32 @@ __global__ void __launch_bounds__(256) k_oz_max_both(const double *__restrict__ 
   if (m > 0) atomicMax(&col[c], m);
 }
 
-// Balance of a factor along one index, from its largest exponent fields e_k:
-// shifts s_k = max e - e_k that even the factor out, and the vectors' factors
-// 2^-s_k (0 where the factor is zero) and base_k 2^-s_k.  Shifts end at 400.
-__global__ void __launch_bounds__(1024) k_oz_factors(const int *__restrict__ e, int n,
-                                                     const double *__restrict__ base,
-                                                     int *__restrict__ shift,
-                                                     double *__restrict__ down,
-                                                     double *__restrict__ based) {
+// Balance of a factor along its rows (block 0) and its columns (block 1), from
+// their largest exponent fields e_k: shifts s_k = max e - e_k that even the
+// factor out, and the vectors' factors 2^-s_k (0 where the factor is zero) and
+// base_k 2^-s_k.  Shifts end at 400.  The fields are left at zero for the next
+// pass; *bad != 0 if one says Inf or NaN.
+__global__ void __launch_bounds__(1024) k_oz_factors(OzBalance rows, OzBalance cols,
+                                                     unsigned *bad) {
   pdl_wait();
+  const OzBalance o = blockIdx.x == 0 ? rows : cols;
   __shared__ int top;
   if (threadIdx.x == 0) top = 0;
   __syncthreads();
   int m = 0;
-  for (int k = threadIdx.x; k < n; k += 1024) m = max(m, e[k]);
+  for (int k = threadIdx.x; k < o.n; k += 1024) m = max(m, o.e[k]);
   m = __reduce_max_sync(0xffffffffu, m);
   if ((threadIdx.x & 31) == 0) atomicMax(&top, m);
   __syncthreads();
-  for (int k = threadIdx.x; k < n; k += 1024) {
-    const int s = e[k] > 0 ? min(top - e[k], 400) : 0;
-    const double f = e[k] > 0 ? __hiloint2double((1023 - s) << 20, 0) : 0.0;
-    shift[k] = s;
-    down[k] = f;
-    if (base) based[k] = base[k] * f;
+  if (threadIdx.x == 0 && top >= 2047) atomicOr(bad, 1u);
+  for (int k = threadIdx.x; k < o.n; k += 1024) {
+    const int e = o.e[k], s = e > 0 ? min(top - e, 400) : 0;
+    const double f = e > 0 ? __hiloint2double((1023 - s) << 20, 0) : 0.0;
+    o.e[k] = 0;
+    o.shift[k] = s;
+    o.down[k] = f;
+    if (o.base) o.based[k] = o.base[k] * f;
   }
-}
-
-// *bad != 0 if an exponent field says Inf or NaN
-__global__ void k_oz_check(const int *__restrict__ e, int n, unsigned *bad) {
-  pdl_wait();
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n && e[i] >= 2047) atomicOr(bad, 1u);
 }
 
 static PFN_cuTensorMapEncodeTiled_v12000 encoder() {
@@ -761,6 +760,16 @@ static void launch_rows(const double *x, int splits, size_t part, const Src &src
   allow_smem(once, k_oz_rows<LIFT>, OZ_ROW_MAX / 16 * 17 * sizeof(double));
   launch_pdl(k_oz_rows<LIFT>, dim3(o.rows), dim3(256), (size_t)o.nkb * 68 * sizeof(double), st, x,
              splits, part, src, y, o.e, o.d, o.rows, o.nkb, o.blk);
+}
+
+// Exponents (into zeros), then digits, by tiles of 64 x 64.
+template <bool COLS, bool LIFT>
+static void launch_tiles(const Src &src, const OzOperand &o, cudaStream_t st) {
+  const int kr = COLS ? o.nkb : (o.rows + 63) / 64, kc = COLS ? (o.rows + 63) / 64 : o.nkb;
+  launch_pdl(k_oz_max<COLS, LIFT>, dim3((src.nc + 63) / 64, (src.nr + 63) / 64), dim3(256), 0, st,
+             src, o.e, false);
+  launch_pdl(k_oz_slice<COLS, LIFT>, dim3(kc, kr), dim3(256), 0, st, src, o.e, o.d, o.rows, o.nkb,
+             o.blk);
 }
 
 }  // namespace oz
@@ -832,17 +841,14 @@ void launch_oz_slice(const double *x, size_t ld, int nr, int nc, const double *s
     return;
   }
   cudaMemsetAsync(o.e, 0, sizeof(int) * o.rows, st);
-  const int kr = cols ? o.nkb : (o.rows + 63) / 64, kc = cols ? (o.rows + 63) / 64 : o.nkb;
-  const dim3 grid(kc, kr), data((nc + 63) / 64, (nr + 63) / 64);
-  if (cols) {
-    launch_pdl(oz::k_oz_max<true>, data, dim3(256), 0, st, src, o.e, false);
-    launch_pdl(oz::k_oz_slice<true>, grid, dim3(256), 0, st, src, o.e, o.d, o.rows, o.nkb,
-               o.blk);
-  } else {
-    launch_pdl(oz::k_oz_max<false>, data, dim3(256), 0, st, src, o.e, false);
-    launch_pdl(oz::k_oz_slice<false>, grid, dim3(256), 0, st, src, o.e, o.d, o.rows, o.nkb,
-               o.blk);
-  }
+  if (cols && (up || down))
+    oz::launch_tiles<true, true>(src, o, st);
+  else if (cols)
+    oz::launch_tiles<true, false>(src, o, st);
+  else if (up || down)
+    oz::launch_tiles<false, true>(src, o, st);
+  else
+    oz::launch_tiles<false, false>(src, o, st);
 }
 
 // y [rows][len] = sum of the split partials, and the digits of o.scale y (len
@@ -855,15 +861,13 @@ void launch_oz_reduce(const double *part, int splits, int nr, int len, double *y
 
 void launch_oz_max_both(const double *x, int nr, int nc, const int *shift, const int *rshift,
                         int *row, int *col, cudaStream_t st) {
-  cudaMemsetAsync(row, 0, sizeof(int) * nr, st);
-  cudaMemsetAsync(col, 0, sizeof(int) * nc, st);
   launch_pdl(oz::k_oz_max_both, dim3(nc / 64, (nr + 255) / 256), dim3(256), 0, st, x, nr, nc,
              shift, rshift, row, col);
 }
 
-void launch_oz_factors(const int *e, int n, const double *base, int *shift, double *down,
-                       double *based, cudaStream_t st) {
-  launch_pdl(oz::k_oz_factors, dim3(1), dim3(1024), 0, st, e, n, base, shift, down, based);
+void launch_oz_factors(const OzBalance &rows, const OzBalance &cols, unsigned *bad,
+                       cudaStream_t st) {
+  launch_pdl(oz::k_oz_factors, dim3(2), dim3(1024), 0, st, rows, cols, bad);
 }
 
 // Digits of x [nr][nc] whose rows' (columns') exponents are in o.e already.
@@ -873,9 +877,9 @@ void launch_oz_digits(const double *x, int nr, int nc, bool cols, const int *shi
                     (size_t)nc, nr, nc};
   const dim3 grid(cols ? (o.rows + 63) / 64 : o.nkb, cols ? o.nkb : (o.rows + 63) / 64);
   if (cols)
-    launch_pdl(oz::k_oz_slice<true>, grid, dim3(256), 0, st, src, o.e, o.d, o.rows, o.nkb, o.blk);
+    launch_pdl(oz::k_oz_slice<true, true>, grid, dim3(256), 0, st, src, o.e, o.d, o.rows, o.nkb, o.blk);
   else
-    launch_pdl(oz::k_oz_slice<false>, grid, dim3(256), 0, st, src, o.e, o.d, o.rows, o.nkb, o.blk);
+    launch_pdl(oz::k_oz_slice<false, true>, grid, dim3(256), 0, st, src, o.e, o.d, o.rows, o.nkb, o.blk);
 }
 
 void launch_oz_col_max(const double *x, size_t ld, int nr, int nc, int *e, cudaStream_t st) {
@@ -884,13 +888,9 @@ void launch_oz_col_max(const double *x, size_t ld, int nr, int nc, int *e, cudaS
   for (int r0 = 0; r0 < nr; r0 += ROWS) {
     const int n = std::min(ROWS, nr - r0);
     const oz::Src src{x + (size_t)r0 * ld, nullptr, nullptr, nullptr, nullptr, false, ld, n, nc};
-    launch_pdl(oz::k_oz_max<true>, dim3((nc + 63) / 64, (n + 63) / 64), dim3(256), 0, st, src, e,
+    launch_pdl(oz::k_oz_max<true, false>, dim3((nc + 63) / 64, (n + 63) / 64), dim3(256), 0, st, src, e,
                true);
   }
-}
-
-void launch_oz_check(const OzOperand &o, unsigned *bad, cudaStream_t st) {
-  launch_pdl(oz::k_oz_check, dim3((o.rows + 255) / 256), dim3(256), 0, st, o.e, o.rows, bad);
 }
 
 }  // namespace lgw

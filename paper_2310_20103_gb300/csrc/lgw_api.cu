@@ -549,18 +549,17 @@ void ensure_digits(lgw_handle *h, lgw_system *sys) {
   uint16_t *d = static_cast<uint16_t *>(p);
   double *x1 = reinterpret_cast<double *>(static_cast<uint8_t *>(p) + 2 * plane);   // 2^-s_vc
   double *xd = x1 + N, *ys = xd + N;
-  int *e = reinterpret_cast<int *>(ys + A), *sx = e + N + A, *sy = sx + N;
+  int *e = reinterpret_cast<int *>(ys + A), *sx = e + N + A + 1, *sy = sx + N;
   const OzOperand a{d, e, s.N, s.A / 64};
   const OzOperand t{d + plane / sizeof(uint16_t), e + s.N, s.A, s.N / 64};
-  unsigned *bad = reinterpret_cast<unsigned *>(sy + A);
+  unsigned *bad = reinterpret_cast<unsigned *>(e + N + A);
   cudaStream_t st = h->stream;
-  LGW_TRY_CUDA(h, cudaMemsetAsync(bad, 0, sizeof(unsigned), st));
+  LGW_TRY_CUDA(h, cudaMemsetAsync(e, 0, (N + A + 1) * sizeof(int), st));
   // L's scales by pair and by auxiliary function, then its digits on them: over
   // vc, L 2^s_vc meets x Delta^1/2 2^-s_vc, over mu, L 2^t_mu meets y 2^-t_mu
   launch_oz_max_both(s.L64, s.N, s.A, nullptr, nullptr, a.e, t.e, st);
-  launch_oz_check(t, bad, st);
-  launch_oz_factors(a.e, s.N, s.dsq, sx, x1, xd, st);
-  launch_oz_factors(t.e, s.A, nullptr, sy, ys, nullptr, st);
+  launch_oz_factors(OzBalance{a.e, s.N, s.dsq, sx, x1, xd},
+                    OzBalance{t.e, s.A, nullptr, sy, ys, nullptr}, bad, st);
   launch_oz_max_both(s.L64, s.N, s.A, sy, sx, a.e, t.e, st);
   launch_oz_digits(s.L64, s.N, s.A, false, sy, a, st);
   launch_oz_digits(s.L64, s.N, s.A, true, sx, t, st);

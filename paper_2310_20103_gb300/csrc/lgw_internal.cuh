@@ -348,17 +348,23 @@ bool launch_oz_gemm(const OzOperand &A, const OzOperand &B, int M, int Ncols, in
 void launch_oz_slice(const double *x, size_t ld, int nr, int nc, const double *scale, bool cols,
                      const OzOperand &o, cudaStream_t st, const int *up = nullptr,
                      const int *down = nullptr);
+// row, col: zeros before
 void launch_oz_max_both(const double *x, int nr, int nc, const int *shift, const int *rshift,
                         int *row, int *col, cudaStream_t st);
-void launch_oz_factors(const int *e, int n, const double *base, int *shift, double *down,
-                       double *based, cudaStream_t st);
+struct OzBalance {
+  int *e, n;            // largest exponent fields of n contraction indices
+  const double *base;   // or NULL
+  int *shift;
+  double *down, *based;
+};
+void launch_oz_factors(const OzBalance &rows, const OzBalance &cols, unsigned *bad,
+                       cudaStream_t st);
 void launch_oz_digits(const double *x, int nr, int nc, bool cols, const int *shift,
                       const OzOperand &o, cudaStream_t st);
 // largest finite exponent field of each column of x [nr][nc] (e: nc rounded up to 64)
 void launch_oz_col_max(const double *x, size_t ld, int nr, int nc, int *e, cudaStream_t st);
 void launch_oz_reduce(const double *part, int splits, int nr, int len, double *y,
                       const OzOperand &o, cudaStream_t st);
-void launch_oz_check(const OzOperand &o, unsigned *bad, cudaStream_t st);
 
 // k_gemm_tc.cu : BF16 tcgen05 contractions
 struct TcPlan;
