@@ -156,3 +156,31 @@ def test_apply_casida_of_a_graded_factor(L, n_v, n_c, A, pairs, aux, x_scale):
     xt = (np.abs(X) * np.sqrt(D)).mean(0)
     scale = np.abs(X).mean(0) * D ** 2 + 4 * np.sqrt(D) * ((xt @ np.abs(Lm)) @ np.abs(Lm).T)
     assert (err / scale).max() <= 4 * (own / scale).max() + 2.0 ** -50
+
+
+def test_coupling_vectors_of_a_graded_basis(L):
+    """V = L M with auxiliary functions of any normalisation, L's columns as d and M as 1 / d:
+    against the FP64 pipe (a handle with a byte limit), within the bounds of the ungraded
+    comparison (1e-11 eV for E, 1e-9 of the largest self-energy)."""
+    wl = gw_inputs.tiny(k=12)
+    d = 10.0 ** (-12 * np.random.default_rng(5).uniform(0, 1, wl.n_aux))
+    t = lambda x: torch.from_numpy(np.ascontiguousarray(x)).to(DEV)
+    res = []
+    for limit in (0, 1 << 40):
+        h = L.lgw_create(0)
+        try:
+            L.lgw_set_workspace_limit(h, limit)
+            s = L.lgw_prepare_system(h, wl.n_v, wl.n_c, wl.n_aux, t(wl.eps), t(wl.L * d), 4.0)
+            prob = L.Problem(targets=t(wl.targets), m_idx=t(wl.m_idx), omega=t(wl.omega),
+                             delta=wl.delta, M=t(wl.M / d))
+            sig = torch.zeros(wl.n_t, wl.omega.size, 2, dtype=torch.float64, device=DEV)
+            e = torch.zeros(wl.n_t, dtype=torch.float64, device=DEV)
+            L.lgw_sigma_c(h, s, prob, L.Options(k=12, precision="fp64", reorth="cgs2"), sig, e)
+            torch.cuda.synchronize()
+            res.append((sig.cpu().numpy(), e.cpu().numpy()))
+            L.lgw_release_system(s)
+        finally:
+            L.lgw_destroy(h)
+    (s0, e0), (s1, e1) = res
+    assert np.abs(s0 - s1).max() <= 1e-9 * np.abs(s1).max()
+    assert np.abs(e0 - e1).max() <= 1e-11
